@@ -279,7 +279,10 @@ smpm_status smpm_factor_host_only(smpm_handle h, const smpm_opts* o);
  * "x1d","w1d","D" (Sec. 1.2), "T" (nel*(4n)^2, T_e row-major), "G", "X"
  * (block-Jacobi, per black element), "black" (black element ids as doubles),
  * "C","H","c0","uC" (coarse, Sec. 2), "uS","B1" (kp), "uL","what" (r),
- * "null_iterations" (1 value). */
+ * "null_iterations" (1 value), and the strips of the coarse inverse:
+ * "strips_shape" (h, p, m, ns, ldn, lds, ldw; all 0 when not built),
+ * "strips_N", "strips_Hs", "strips_W", "strips_z", for the adjoint system
+ * "stripsa_...". */
 smpm_status smpm_host_factor(smpm_handle h, const char* name, double* out, long long count, long long* len);
 
 /* y = P v exactly as smpm_apply_deflation, for callers that cannot allocate

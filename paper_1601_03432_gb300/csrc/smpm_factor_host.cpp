@@ -815,6 +815,96 @@ static int coarse_memory_check(const Geometry& g, bool adjoint, std::string* err
   return SMPM_ENOMEM;
 }
 
+// Strip height with the fewest products, and its factors, for the coarse
+// system A y = r - u (u^T r) with pseudo-inverse Hp and left null vector u (A =
+// C, u = u_C; transposed: A = C^T, u = c0^).  The interiors are cut out of C,
+// the separators' inverse Schur complement is Hp's own block, and the
+// couplings are banded, so the factors hold O(d (h mx)) entries.
+static void strip_factors(const Geometry& g, const std::vector<double>& C, const std::vector<double>& Hp,
+                          const double* u, bool transpose, StripFactors* out) {
+  *out = StripFactors();
+  const int d = static_cast<int>(g.d), mx = g.mx, row = 2 * mx - 1;
+  if (d < 128) return;
+  int hbest = 0;
+  double best = 0.5 * static_cast<double>(d) * d;  // at least half of the dense products saved
+  auto count = [&](int h) {
+    const double p = (g.my + h - 1) / h, m = static_cast<double>(h) * row - mx, ns = (p - 1) * mx;
+    return p * (m + 2.0 * mx) * m + (ns + 1) * ns + p * m * 2.0 * mx;
+  };
+  for (int h = 1; 2 * h <= g.my; ++h) {
+    const int p = (g.my + h - 1) / h;
+    if ((p + 1) * mx > d + 1) continue;  // the staging buffer holds d + 1 entries
+    if (count(h) < best) { best = count(h); hbest = h; }
+  }
+  if (!hbest) return;
+  StripFactors& f = *out;
+  const int h = hbest, p = (g.my + h - 1) / h, m = h * row - mx, srow = h * row;
+  auto pad = [](int v) { return (v + 3) & ~3; };
+  f.h = h; f.m = m; f.ns = (p - 1) * mx;
+  f.ldn = pad(m); f.lds = pad(f.ns); f.ldw = pad(2 * mx);
+  f.products = best;
+  const size_t RS = static_cast<size_t>(m) + 2 * mx;
+  f.N.assign(p * RS * f.ldn, 0.0);
+  f.W.assign(static_cast<size_t>(p) * m * f.ldw, 0.0);
+  f.z.assign(static_cast<size_t>(p) * m, 0.0);
+  f.Hs.assign(static_cast<size_t>(f.ns + 1) * f.lds, 0.0);
+  auto at = [&](int i, int j) { return transpose ? C[static_cast<size_t>(j) * d + i] : C[static_cast<size_t>(i) * d + j]; };
+  auto sep = [&](int sp, int q) { return (sp + 1) * srow - mx + q; };  // entry q of separator sp
+  bool ok = true;
+#pragma omp parallel for schedule(dynamic, 1)
+  for (int i = 0; i < p; ++i) {
+    const int b = i * srow, mi = std::min(m, d - b), nr = mi + 2 * mx + 1;
+    std::vector<double> A(static_cast<size_t>(mi) * mi), B(static_cast<size_t>(mi) * nr, 0.0);
+    for (int r = 0; r < mi; ++r) {
+      for (int c = 0; c < mi; ++c) A[static_cast<size_t>(r) * mi + c] = at(b + r, b + c);
+      double* Br = B.data() + static_cast<size_t>(r) * nr;
+      Br[r] = 1.0;
+      for (int q = 0; q < mx; ++q) {
+        if (i > 0) Br[mi + q] = at(b + r, sep(i - 1, q));
+        if (i < p - 1) Br[mi + mx + q] = at(b + r, sep(i, q));
+      }
+      Br[nr - 1] = u[b + r];
+    }
+    DenseLU lu = lu_factor_move(std::move(A), mi);
+    if (!lu.ok) {
+#pragma omp atomic write
+      ok = false;
+      continue;
+    }
+    lu_solve_multi(lu, B.data(), nr);
+    for (int r = 0; r < mi; ++r) {
+      const double* Br = B.data() + static_cast<size_t>(r) * nr;
+      std::copy(Br, Br + mi, f.N.begin() + (i * RS + r) * f.ldn);
+      std::copy(Br + mi, Br + mi + 2 * mx, f.W.begin() + (static_cast<size_t>(i) * m + r) * f.ldw);
+      f.z[static_cast<size_t>(i) * m + r] = Br[nr - 1];
+    }
+    for (int side = 0; side < 2; ++side) {
+      if (side == 0 ? i == 0 : i == p - 1) continue;
+      for (int q = 0; q < mx; ++q) {  // C_si C_ii^-1
+        double* Nr = f.N.data() + (i * RS + m + side * mx + q) * f.ldn;
+        const int js = sep(side == 0 ? i - 1 : i, q);
+        for (int k = 0; k < mi; ++k) {
+          const double c = at(js, b + k);
+          if (c == 0.0) continue;
+          const double* Bk = B.data() + static_cast<size_t>(k) * nr;
+          for (int r = 0; r < mi; ++r) Nr[r] += c * Bk[r];
+        }
+      }
+    }
+  }
+  if (!ok) {  // a singular interior: the dense form is used
+    *out = StripFactors();
+    return;
+  }
+  for (int r = 0; r < f.ns; ++r) {
+    const int jr = sep(r / mx, r % mx);
+    for (int c = 0; c < f.ns; ++c)
+      f.Hs[static_cast<size_t>(r) * f.lds + c] = Hp[static_cast<size_t>(jr) * d + sep(c / mx, c % mx)];
+    f.Hs[static_cast<size_t>(f.ns) * f.lds + r] = u[jr];
+  }
+  f.p = p;
+}
+
 static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, std::string* err) {
   const bool op_only = (o.flags & SMPM_FLAG_OPERATOR_ONLY) != 0;
   if (!op_only) {
@@ -1016,6 +1106,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
       for (int j = 0; j < d; ++j) Hd[static_cast<size_t>(i) * d + j] = Kinv[static_cast<size_t>(i) * d + j] - s * f->uC[j];
     }
     if (!keep) f->H = std::move(Kinv);
+    if (o.precond == 2) strip_factors(g, f->C, f->H, f->uC.data(), false, &f->cs);
   }
 
   // null vectors of S and L
@@ -1120,6 +1211,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
       for (int j = 0; j < d; ++j)
         f->Ha[static_cast<size_t>(i) * d + j] =
             Kinv[static_cast<size_t>(j) * d + i] - v[i] * ch[j] - f->uC[i] * w[j];
+    if (o.precond == 2) strip_factors(g, f->C, f->Ha, ch.data(), true, &f->csa);
     // left null vector of the permuted S^T: Phi B1 (Phi swaps the two slots
     // facing each other across an interface; Phi B1 = B1 where B1 is constant
     // on each interface), normalised

@@ -84,6 +84,10 @@ struct GmresArgs {
   int fused;           // 1: use HT / chatd in the Arnoldi steps
   const double* HT;    // d*d, H column-major (HT[j d + r] = H[r][j])
   double* chatd;       // 2 d: c_hat of even / odd steps (accumulated with atomics)
+  // C^+ by element-row strips (strips.p > 0 and use_strips): see coarse_solve
+  CoarseStrips<typename std::conditional<sizeof(S) == 4, float, double>::type> strips;
+  double* gsep;        // strips: 2 p mx + 1 doubles per column (sums pushed onto the separators, alpha)
+  int use_strips;      // 1: the strips are the cheaper form for this team size
 };
 
 // rank of this CTA within the team that works on a solve
@@ -174,7 +178,7 @@ struct Smem {
   double *h1, *h2, *hs1, *hs2, *gcs, *gsn, *gg, *col, *invb, *misc, *cs;
   S *p, *r1, *av, *z, *red;
   S *w, *w2;
-  double* cst;  // staged coarse vector c (d)
+  double* cst;  // staged coarse vector c (d, and two entries of padding)
   double* cpv;  // fused coarse: c_j of the owned white elements' interfaces (4 per element)
   int* cpj;     // and their interface indices (-1: none)
   S* V;     // (m+1) * ES when resident
@@ -200,7 +204,7 @@ __device__ Smem<S> carve(const GmresArgs<S>& a, unsigned char* raw) {
   s.invb = d; d += m + 3;
   s.misc = d; d += 16;
   s.cs = d; d += M;
-  s.cst = d; d += a.g.d + 1;
+  s.cst = d; d += a.g.d + 3;
   s.cpv = d; d += 4 * (size_t)a.nown_w;
   s.cpj = reinterpret_cast<int*>(d); d += 2 * (size_t)a.nown_w;
   S* q = reinterpret_cast<S*>(d);
@@ -234,7 +238,7 @@ template <typename S>
 inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown_w, int basis_smem, int mats_smem,
                                long long d, int stream_elems = 0, bool w_global = false, int nbuf = 2,
                                bool warp_elems = false) {
-  size_t dbl = kMaxStreamBufs + 9 * (size_t)(m + 3) + 16 + M + (size_t)d + 1 + 6 * (size_t)nown_w;
+  size_t dbl = kMaxStreamBufs + 9 * (size_t)(m + 3) + 16 + M + (size_t)d + 3 + 6 * (size_t)nown_w;
   size_t sel = 4 * (size_t)M + 256 + (w_global ? 0 : 2 * (size_t)(ES + 1));
   if (warp_elems) sel += (size_t)(kGmresThreads / 32) * warp_scratch(M) + 16 / sizeof(S);
   if (basis_smem) sel += (size_t)(m + 1) * ES;
@@ -614,6 +618,167 @@ __device__ void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s) {
   }
 }
 
+// ---- C^+ by strips ----------------------------------------------------------
+// C couples two interfaces only when they share an element, so the horizontal
+// interfaces between two element rows separate the grid.  With a separator
+// every h element rows, c_hat = C^+ c is, for the strips' interiors i and the
+// separators s (all factors from the host factor step):
+//   P1  y_i = C_ii^-1 c_i, and the sums C_si y_i it pushes onto its separators
+//   P2  c_s' = c_s - sum_i C_si y_i;  x_s = H_ss c_s';  alpha = u_C,s . c_s'
+//   P3  x_i = y_i - alpha C_ii^-1 u_C,i - C_ii^-1 C_is x_s
+// (alpha = u_C . c: the left projection (I - u_C u_C^T); H_ss, the separators'
+// block of H, inverts the Schur complement; the result differs from H c by a
+// multiple of c0, which S Z maps to zero and the zero mean of u removes).
+// About d^2 / 7 products instead of d^2, in three phases of short dot
+// products with two more barriers (see strips_pay on when that is less).
+__device__ __forceinline__ void ld_vec(const double* p, double (&v)[2]) {
+  const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+  v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+
+// For rows r0 <= r < r1: get(r, &row, &x, &len) names a row (16-byte aligned,
+// zero-padded to whole 16-byte groups) and the staged vector (readable to the
+// padded length); put(r, sum) takes the dot product (len 0: no call).  P lanes
+// per row, P as large as the rows leave threads for, but 4 at least: each
+// halving step of the final sums costs as much FP64 time as a product.
+template <typename T, typename Get, typename Put>
+__device__ __forceinline__ void row_dots(int r0, int r1, Get&& get, Put&& put) {
+  constexpr int V = 16 / (int)sizeof(T), U = 4;
+  const int rows = r1 - r0;
+  int P = 32;
+  while (P > 4 && P * rows > (int)blockDim.x) P >>= 1;
+  const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
+  for (int rb = 0; rb < rows; rb += ngrp) {  // uniform trip count per warp
+    const int r = r0 + rb + grp;
+    const T* a = nullptr;
+    const T* x = nullptr;
+    int len = 0;
+    if (r < r1) get(r, a, x, len);
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    int j = V * lane;
+    for (; j + V * P * (U - 1) < len; j += V * P * U) {
+      T h[U][V];
+#pragma unroll
+      for (int u = 0; u < U; ++u) ld_vec(a + j + u * V * P, h[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[u] += h[u][v] * x[j + u * V * P + v];
+    }
+    for (; j < len; j += V * P) {
+      T h[V];
+      ld_vec(a + j, h);
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[v & 3] += h[v] * x[j + v];
+    }
+    T sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, P);
+    if (lane == 0 && len > 0) put(r, sum);
+  }
+}
+
+// c_hat = C^+ c (a.c -> a.chat), complete after the final barrier; false when a
+// barrier timed out.  cst: staging for at least d + 1 entries.
+template <typename S>
+__device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsigned& epoch) {
+  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+  constexpr int V = 16 / (int)sizeof(T);
+  T* xs = reinterpret_cast<T*>(cst);
+  const auto& k = a.strips;
+  const int G = a.G, rank = team_rank(a), d = (int)a.g.d;
+  const int srow = k.h * k.row, RS = k.m + 2 * k.mx;  // interfaces of a strip with its upper separator; rows of N
+  double* alpha = a.gsep + 2 * (size_t)k.p * k.mx;
+  {  // P1
+    const int n1 = k.p * RS, per = (n1 + G - 1) / G, r0 = min(n1, rank * per), r1 = min(n1, r0 + per);
+    if (r0 < r1) {
+      const int b0 = (r0 / RS) * srow, b1 = min(d, ((r1 - 1) / RS + 1) * srow);
+      for (int j = threadIdx.x; j < b1 - b0 + V; j += blockDim.x) xs[j] = b0 + j < b1 ? (T)__ldcg(a.c + b0 + j) : T(0);
+      __syncthreads();
+      row_dots<T>(
+          r0, r1,
+          [&](int r, const T*& row, const T*& x, int& len) {
+            const int i = r / RS, l = r - i * RS, mi = min(k.m, d - i * srow);
+            const bool on = l < k.m ? l < mi : (l < k.m + k.mx ? i > 0 : i < k.p - 1);
+            row = k.N + (size_t)r * k.ldn;
+            x = xs + i * srow - b0;
+            len = on ? mi : 0;
+          },
+          [&](int r, T sum) {
+            const int i = r / RS, l = r - i * RS;
+            if (l < k.m) a.chat[i * srow + l] = (double)sum;
+            else a.gsep[2 * (size_t)i * k.mx + (l - k.m)] = (double)sum;
+          });
+    }
+    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+  }
+  {  // P2: rows 0 .. ns-1 of H_ss, row ns: u_C on the separators
+    const int n2 = k.ns + 1, per = (n2 + G - 1) / G, r0 = min(n2, rank * per), r1 = min(n2, r0 + per);
+    if (r0 < r1) {
+      for (int j = threadIdx.x; j < k.ns + V; j += blockDim.x) {
+        T v = T(0);
+        if (j < k.ns) {
+          const int sp = j / k.mx, q = j - sp * k.mx;
+          const double* up = a.gsep + (2 * (size_t)sp + 1) * k.mx + q;  // strip below; lower sums of the one above
+          v = (T)(__ldcg(a.c + (sp + 1) * srow - k.mx + q) - __ldcg(up) - __ldcg(up + k.mx));
+        }
+        xs[j] = v;
+      }
+      __syncthreads();
+      row_dots<T>(
+          r0, r1,
+          [&](int r, const T*& row, const T*& x, int& len) {
+            row = k.Hs + (size_t)r * k.lds;
+            x = xs;
+            len = k.ns;
+          },
+          [&](int r, T sum) {
+            if (r == k.ns) *alpha = (double)sum;
+            else a.chat[(r / k.mx + 1) * srow - k.mx + r % k.mx] = (double)sum;
+          });
+    }
+    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+  }
+  {  // P3: rows of W: 2 mx coefficients of the separators below and above, then C_ii^-1 u_C,i
+    const int n3 = k.p * k.m, per = (n3 + G - 1) / G, r0 = min(n3, rank * per), r1 = min(n3, r0 + per);
+    if (r0 < r1) {
+      const int i0 = r0 / k.m, i1 = (r1 - 1) / k.m;  // separators i0 - 1 .. i1
+      for (int j = threadIdx.x; j < (i1 - i0 + 2) * k.mx + V; j += blockDim.x) {
+        const int sp = i0 - 1 + j / k.mx;
+        xs[j] = (sp >= 0 && sp < k.p - 1 && sp <= i1) ? (T)__ldcg(a.chat + (sp + 1) * srow - k.mx + j % k.mx) : T(0);
+      }
+      const double al = __ldcg(alpha);
+      __syncthreads();
+      row_dots<T>(
+          r0, r1,
+          [&](int r, const T*& row, const T*& x, int& len) {
+            const int i = r / k.m;
+            row = k.W + (size_t)r * k.ldw;
+            x = xs + (i - i0) * k.mx;
+            len = (r - i * k.m) < min(k.m, d - i * srow) ? 2 * k.mx : 0;
+          },
+          [&](int r, T sum) {
+            const int i = r / k.m;
+            double* out = a.chat + i * srow + (r - i * k.m);
+            *out = __ldcg(out) - al * (double)k.z[r] - (double)sum;
+          });
+    }
+  }
+  return grid_sync(a.bar, a.err, epoch, G);
+}
+
+// c_hat = C^+ c by all CTAs of the team (strips or dense rows), complete after
+// its last barrier; false when a barrier timed out
+template <typename S>
+__device__ __forceinline__ bool coarse_solve(const GmresArgs<S>& a, const Smem<S>& s, unsigned& epoch) {
+  if (a.use_strips) return coarse_strips(a, s.cst, epoch);
+  coarse_rows(a, s);
+  return grid_sync(a.bar, a.err, epoch, a.G);
+}
+
 // w = y - S Z chat for one slot (pull form); chat == nullptr gives w = y.
 template <typename S>
 __device__ __forceinline__ double deflate_slot_cg(const DevGeo& g, const S* y, const double* chat,
@@ -960,9 +1125,7 @@ __device__ bool apply_op(const GmresArgs<S>& a, const Smem<S>& s, const S* src, 
   if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
   GM_TRACE(23);
   if (a.precond == 2 && !fuse) {
-    coarse_rows(a, s);
-    GM_TRACE(24);
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!coarse_solve(a, s, epoch)) return false;
     GM_TRACE(25);
   }
   return true;
@@ -1032,7 +1195,7 @@ __device__ __forceinline__ void store_rcol(const GmresArgs<S>& a, const Smem<S>&
 // epoch: the team barrier's epoch, carried across consecutive bodies.
 // Returns false when a barrier or copy wait timed out (err set).
 template <typename S>
-__device__ bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw, unsigned& epoch) {
+__device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw, unsigned& epoch) {
   const Smem<S> s = carve(a, smraw);
   const DevGeo& g = a.g;
   const int M = g.M, n = g.n, m = a.m;
@@ -1311,12 +1474,4 @@ __device__ bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw, unsigned
   ms_drain(a, s, msd);
   return true;
 #undef GM_FAIL
-}
-
-template <typename S>
-__global__ void __launch_bounds__(256, 1) k_gmres(GmresArgs<S> a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  if (a.skip && *((volatile const int*)a.skip)) return;
-  unsigned epoch = 0;
-  gmres_body(a, smraw, epoch);
 }

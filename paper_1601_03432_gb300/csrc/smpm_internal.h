@@ -73,6 +73,16 @@ struct Geometry {
   }
 };
 
+// C^+ by strips of h element rows (see coarse_strips on the device): the
+// dense factors of the strips' interiors, the separators' block of H and the
+// couplings, rows padded to ld (a multiple of 4) with zeros.  p = 0: not built
+// (a grid too small for it to pay).
+struct StripFactors {
+  int h = 0, p = 0, m = 0, ns = 0, ldn = 0, lds = 0, ldw = 0;
+  std::vector<double> N, Hs, W, z;
+  double products = 0;  // multiplications of one C^+ c
+};
+
 // Everything the factor step produces, in host memory (FP64).
 struct Factors {
   // face data per element column (W/E faces) and row (S/N faces), three
@@ -100,6 +110,7 @@ struct Factors {
   // grid, where z_j is the indicator of Sec. 2); zwa: the adjoint system's
   // weights, zwa[4e + F] = zw[4 nbr(e,F) + opp F]
   std::vector<double> zw, zwa;
+  StripFactors cs, csa;  // C^+ by strips, and the adjoint system's
   bool operator_only = false;  // only T_e and its row sums (SMPM_FLAG_OPERATOR_ONLY)
   int null_iterations = 0;   // GMRES steps of the u_S bordered solve
   double null_relres = 0;

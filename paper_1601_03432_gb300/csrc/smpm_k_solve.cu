@@ -1,0 +1,48 @@
+// Kernels of a solve of one right-hand side (one team spanning the grid).
+#include "smpm_device.cuh"
+
+namespace {
+
+#include "smpm_gmres.cuh"
+#include "smpm_prepost.cuh"
+#include "smpm_refine.cuh"
+
+template <typename S>
+__global__ void __launch_bounds__(256, 1) k_gmres(GmresArgs<S> a) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  if (a.skip && *((volatile const int*)a.skip)) return;
+  unsigned epoch = 0;
+  gmres_body(a, smraw, epoch);
+}
+
+__global__ void __launch_bounds__(256, 1) k_pre(PrePostArgs P) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned epoch = 0;
+  pre_body(P, smraw, epoch);
+}
+
+__global__ void __launch_bounds__(256, 1) k_post(PrePostArgs P) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  unsigned epoch = 0;
+  post_body(P, smraw, epoch);
+}
+
+__global__ void __launch_bounds__(256, 1) k_refine(RefineArgs R) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  if (*((volatile const int*)R.done)) return;
+  unsigned epoch = 0;
+  refine_body(R, smraw, epoch);
+}
+
+}  // namespace
+
+namespace smpm {
+
+const void* fn_pre() { return (const void*)k_pre; }
+const void* fn_post() { return (const void*)k_post; }
+const void* fn_gmres64() { return (const void*)k_gmres<double>; }
+const void* fn_gmres32() { return (const void*)k_gmres<float>; }
+const void* fn_refine() { return (const void*)k_refine; }
+cudaError_t set_spin_solve(long long v) { return cudaMemcpyToSymbol(g_barrier_spin_limit, &v, sizeof(v)); }
+
+}  // namespace smpm

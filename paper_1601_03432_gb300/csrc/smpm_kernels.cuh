@@ -29,6 +29,19 @@ struct DevGeo {
   int pad_;
 };
 
+// C^+ by strips of h element rows (device pointers, T = FP64 or its FP32
+// copy); interfaces in their natural order: strip i's interior starts at
+// i h row and holds m entries (the last strip fewer), the separator above it
+// follows with mx entries.
+template <typename T>
+struct CoarseStrips {
+  const T* N;   // p (m + 2 mx) rows of ldn: C_ii^-1, then what it pushes onto the separator below and above
+  const T* Hs;  // ns + 1 rows of lds: the separators' block of H, then u_C on the separators
+  const T* W;   // p m rows of ldw: C_ii^-1 C_is for the separators below and above
+  const T* z;   // p m: C_ii^-1 u_C,i
+  int h, p, row, m, mx, ns, ldn, lds, ldw, pad_;
+};
+
 __device__ __forceinline__ double dev_zw(const DevGeo& g, int e, int F) {
   return g.zw ? __ldg(g.zw + 4 * (size_t)e + F) : 1.0;
 }

@@ -192,7 +192,9 @@ __device__ __forceinline__ void warp_gemm_rc(int RC, const S* Amat, const S* X, 
     case 1: warp_gemm<S, 1>(Amat, X, Z, M, lane); break;
     case 2: warp_gemm<S, 2>(Amat, X, Z, M, lane); break;
     case 4: warp_gemm<S, 4>(Amat, X, Z, M, lane); break;
-    default: warp_gemm<S, 8>(Amat, X, Z, M, lane); break;
+    default:  // FP32 only (lock_rc gives FP64 columns at most 4 per item)
+      if constexpr (sizeof(S) == 4) warp_gemm<S, 8>(Amat, X, Z, M, lane);
+      break;
   }
 }
 
@@ -422,17 +424,200 @@ __device__ void lk_coarse32_staged(const LockArgs<S>& A, float* cf, int dc) {
   }
 }
 
+// As row_dots for NC columns at a time: eight lanes per row, lane l of the
+// group ends with column l's sum (the partial sums are exchanged halving the
+// columns each time: 7 adds per row and lane instead of 24).  x: column c of
+// the staged vectors at c * xld.
+template <typename T, int NC, typename Get, typename Put>
+__device__ __forceinline__ void row_dots_cols(int r0, int r1, int xld, Get&& get, Put&& put) {
+  constexpr int V = 16 / (int)sizeof(T), P = 8;
+  const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
+  for (int rb = 0; rb < r1 - r0; rb += ngrp) {  // uniform trip count per warp
+    const int r = r0 + rb + grp;
+    const T* a = nullptr;
+    const T* x = nullptr;
+    int len = 0;
+    if (r < r1) get(r, a, x, len);
+    T acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = T(0);
+    for (int j = V * lane; j < len; j += 2 * V * P) {
+      T h[2][V];
+      ld_vec(a + j, h[0]);
+      const bool two = j + V * P < len;
+      if (two) ld_vec(a + j + V * P, h[1]);
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[c] += h[0][v] * x[(size_t)c * xld + j + v];
+      if (two) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[c] += h[1][v] * x[(size_t)c * xld + j + V * P + v];
+      }
+    }
+    // lane keeps the half of the columns that its bit o selects; lanes beyond
+    // the columns add the halves that are left
+    int w = NC;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const int half = w > 1 ? w / 2 : 1;
+      const bool up = (lane & o) != 0;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        if (c >= half) break;
+        const T keep = (w > 1 && up) ? acc[(c + half) % NC] : acc[c];
+        const T give = (w > 1 && !up) ? acc[(c + half) % NC] : acc[c];
+        const T got = __shfl_xor_sync(0xffffffffu, give, o, P);
+        acc[c] = keep + got;
+      }
+      if (w > 1) w = half;
+    }
+    // column of this lane: the top log2(NC) bits of lane
+    constexpr int S3 = NC == 8 ? 0 : NC == 4 ? 1 : NC == 2 ? 2 : 3;
+    if (len > 0 && (lane & ((1 << S3) - 1)) == 0) put(r, lane >> S3, acc[0]);
+  }
+}
+
+// C^+ by strips (coarse_strips) for all columns, NC of them at a time staged
+// in st (each phase's stretch of every column, xld entries apart).
+template <typename S, int NC>
+__device__ bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& epoch) {
+  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+  constexpr int V = 16 / (int)sizeof(T);
+  const GmresArgs<S>& a = A.a;
+  const auto& k = a.strips;
+  T* xs = reinterpret_cast<T*>(st);
+  const int G = a.G, rank = team_rank(a), d = (int)a.g.d, R = A.R;
+  const int srow = k.h * k.row, RS = k.m + 2 * k.mx;
+  const size_t gst = 2 * (size_t)k.p * k.mx + 1;  // gsep per column
+  {
+    const int n1 = k.p * RS, per = (n1 + G - 1) / G, r0 = min(n1, rank * per), r1 = min(n1, r0 + per);
+    if (r0 < r1) {
+      const int b0 = (r0 / RS) * srow, b1 = min(d, ((r1 - 1) / RS + 1) * srow), xld = b1 - b0 + V;
+      for (int c0 = 0; c0 < R; c0 += NC) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < NC * xld; q += blockDim.x) {
+          const int c = q / xld, j = q - c * xld;
+          xs[q] = (c0 + c < R && b0 + j < b1) ? (T)__ldcg(a.c + (c0 + c) * A.ds + b0 + j) : T(0);
+        }
+        __syncthreads();
+        row_dots_cols<T, NC>(
+            r0, r1, xld,
+            [&](int r, const T*& row, const T*& x, int& len) {
+              const int i = r / RS, l = r - i * RS, mi = min(k.m, d - i * srow);
+              const bool on = l < k.m ? l < mi : (l < k.m + k.mx ? i > 0 : i < k.p - 1);
+              row = k.N + (size_t)r * k.ldn;
+              x = xs + i * srow - b0;
+              len = on ? mi : 0;
+            },
+            [&](int r, int c, T sum) {
+              if (c0 + c >= R) return;
+              const int i = r / RS, l = r - i * RS;
+              if (l < k.m) a.chat[(c0 + c) * A.ds + i * srow + l] = (double)sum;
+              else a.gsep[(c0 + c) * gst + 2 * (size_t)i * k.mx + (l - k.m)] = (double)sum;
+            });
+      }
+    }
+    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+  }
+  {
+    const int n2 = k.ns + 1, per = (n2 + G - 1) / G, r0 = min(n2, rank * per), r1 = min(n2, r0 + per);
+    if (r0 < r1) {
+      const int xld = k.ns + V;
+      for (int c0 = 0; c0 < R; c0 += NC) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < NC * xld; q += blockDim.x) {
+          const int c = q / xld, j = q - c * xld;
+          T v = T(0);
+          if (c0 + c < R && j < k.ns) {
+            const int sp = j / k.mx, e = j - sp * k.mx;
+            const double* up = a.gsep + (c0 + c) * gst + (2 * (size_t)sp + 1) * k.mx + e;
+            v = (T)(__ldcg(a.c + (c0 + c) * A.ds + (sp + 1) * srow - k.mx + e) - __ldcg(up) - __ldcg(up + k.mx));
+          }
+          xs[q] = v;
+        }
+        __syncthreads();
+        row_dots_cols<T, NC>(
+            r0, r1, xld,
+            [&](int r, const T*& row, const T*& x, int& len) {
+              row = k.Hs + (size_t)r * k.lds;
+              x = xs;
+              len = k.ns;
+            },
+            [&](int r, int c, T sum) {
+              if (c0 + c >= R) return;
+              if (r == k.ns) a.gsep[(c0 + c) * gst + gst - 1] = (double)sum;
+              else a.chat[(c0 + c) * A.ds + (r / k.mx + 1) * srow - k.mx + r % k.mx] = (double)sum;
+            });
+      }
+    }
+    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+  }
+  {
+    const int n3 = k.p * k.m, per = (n3 + G - 1) / G, r0 = min(n3, rank * per), r1 = min(n3, r0 + per);
+    if (r0 < r1) {
+      const int i0 = r0 / k.m, i1 = (r1 - 1) / k.m, len0 = (i1 - i0 + 2) * k.mx, xld = len0 + V;
+      for (int c0 = 0; c0 < R; c0 += NC) {
+        __syncthreads();
+        for (int q = threadIdx.x; q < NC * xld; q += blockDim.x) {
+          const int c = q / xld, j = q - c * xld, sp = i0 - 1 + j / k.mx;
+          xs[q] = (c0 + c < R && sp >= 0 && sp < k.p - 1 && sp <= i1)
+                      ? (T)__ldcg(a.chat + (c0 + c) * A.ds + (sp + 1) * srow - k.mx + j % k.mx)
+                      : T(0);
+        }
+        __syncthreads();
+        row_dots_cols<T, NC>(
+            r0, r1, xld,
+            [&](int r, const T*& row, const T*& x, int& len) {
+              const int i = r / k.m;
+              row = k.W + (size_t)r * k.ldw;
+              x = xs + (i - i0) * k.mx;
+              len = (r - i * k.m) < min(k.m, d - i * srow) ? 2 * k.mx : 0;
+            },
+            [&](int r, int c, T sum) {
+              if (c0 + c >= R) return;
+              const int i = r / k.m;
+              double* out = a.chat + (c0 + c) * A.ds + i * srow + (r - i * k.m);
+              *out = __ldcg(out) - __ldcg(a.gsep + (c0 + c) * gst + gst - 1) * (double)k.z[r] - (double)sum;
+            });
+      }
+    }
+  }
+  return grid_sync(a.bar, a.err, epoch, G);
+}
+
+// longest stretch of a coarse vector that a CTA of a team of G stages
+template <typename T>
+__host__ __device__ inline int strips_stage(const CoarseStrips<T>& k, int G) {
+  const int RS = k.m + 2 * k.mx, per1 = (k.p * RS + G - 1) / G, per3 = (k.p * k.m + G - 1) / G;
+  const int s1 = ((per1 + RS - 2) / RS + 1) * k.h * k.row, s3 = ((per3 + k.m - 2) / k.m + 2) * k.mx;
+  int m = s1 > s3 ? s1 : s3;
+  if (k.ns > m) m = k.ns;
+  return m + 16 / (int)sizeof(T);
+}
+
+// c_hat = C^+ c for all columns, complete after its last barrier.
 template <typename S>
-__device__ void lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s) {
+__device__ bool lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s, unsigned& epoch) {
+  const int room = (int)((size_t)(blockDim.x / 32) * lock_tile_elems(A.a.g.M, A.RC));  // the idle warp tiles
+  if (A.a.use_strips) {
+    const int nc = room / strips_stage(A.a.strips, A.a.G);
+    if (nc >= 8 && A.R > 4) return lk_coarse_strips_nc<S, 8>(A, s.wb, epoch);
+    if (nc >= 4 && A.R > 2) return lk_coarse_strips_nc<S, 4>(A, s.wb, epoch);
+    if (nc >= 2) return lk_coarse_strips_nc<S, 2>(A, s.wb, epoch);
+  }
+  bool done = false;
   if constexpr (sizeof(S) == 4) {
-    const int room = (int)((size_t)(blockDim.x / 32) * lock_tile_elems(A.a.g.M, A.RC));
     const int dc = (room / A.R) & ~31;  // entries per column and chunk
     if (dc >= 256) {
       lk_coarse32_staged(A, reinterpret_cast<float*>(s.wb), dc);
-      return;
+      done = true;
     }
   }
-  lk_coarse_h(A, A.a.H);
+  if (!done) lk_coarse_h(A, A.a.H);
+  return grid_sync(A.a.bar, A.a.err, epoch, A.a.G);
 }
 
 // op(sc * src) -> y (and c, chat) for all columns; with own_j >= 0 the block
@@ -450,9 +635,7 @@ __device__ bool lk_apply(const LockArgs<S>& A, const LockSmem<S>& s, const S* sr
   if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
   GM_TRACE(34);
   if (a.precond == 2) {
-    lk_coarse(A, s);
-    GM_TRACE(35);
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!lk_coarse(A, s, epoch)) return false;
     GM_TRACE(36);
   }
   return true;
@@ -883,43 +1066,4 @@ __device__ __forceinline__ bool lock_all_done(const LockArgs<S>& A) {
   for (int c = 0; c < A.R; ++c)
     if (!*((volatile const int*)(A.done + (size_t)c * A.done_stride))) return false;
   return true;
-}
-
-template <typename S>
-__global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  if (lock_all_done(A)) return;
-  unsigned epoch = 0;
-  lock_body(A, smraw, epoch);
-}
-
-// The right-hand-side and recovery bodies of R columns, one launch each: the
-// bodies run one column after another (their barrier epoch carries on), each
-// with its own arguments; the scratch vectors they share (t, y, c, c_hat)
-// are only touched after a barrier that every CTA passes once it is done with
-// the previous column.
-__global__ void __launch_bounds__(256, 1) k_pre_cols(const PrePostArgs* __restrict__ Ps, int R) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  for (int c = 0; c < R; ++c)
-    if (!pre_body(Ps[c], smraw, epoch)) return;
-}
-
-__global__ void __launch_bounds__(256, 1) k_post_cols(const PrePostArgs* __restrict__ Ps, int R) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  for (int c = 0; c < R; ++c)
-    if (!post_body(Ps[c], smraw, epoch)) return;
-}
-
-// One refinement step (refine_body) for every column not yet done, one
-// column after another.  A column's done flag is read before its body starts;
-// only its own body (rank 0, after a barrier every CTA passed) sets it.
-__global__ void __launch_bounds__(256, 1) k_refine_cols(const RefineArgs* __restrict__ Rs, int R) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  for (int c = 0; c < R; ++c) {
-    if (*((volatile const int*)Rs[c].done)) continue;
-    if (refine_body(Rs[c], smraw, epoch) < 0) return;
-  }
 }

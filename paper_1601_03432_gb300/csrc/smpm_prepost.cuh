@@ -80,7 +80,7 @@ __device__ void elem_fd(const PrePostArgs& P, int e, double* B, double* U, doubl
   elem_solve_dev(g.n, fd_x(g, P.fdx, e), fd_y(g, P.fdy, e), B, U, t1);
 }
 
-__device__ bool pre_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
+__device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<double>& a = P.ga;
   const Smem<double> s = carve(a, smraw);
   const DevGeo& g = a.g;
@@ -181,9 +181,7 @@ __device__ bool pre_body(const PrePostArgs& P, unsigned char* smraw, unsigned& e
     GM_TRACE(55);
     if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
     GM_TRACE(56);
-    coarse_rows(a, s);  // a.c -> a.chat
-    GM_TRACE(57);
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!coarse_solve(a, s, epoch)) return false;  // a.c -> a.chat
     GM_TRACE(58);
     for (int j = rank * blockDim.x + threadIdx.x; j < (int)g.d; j += G * blockDim.x)
       P.chatb[j] = __ldcg(a.chat + j);
@@ -228,13 +226,7 @@ __device__ bool pre_body(const PrePostArgs& P, unsigned char* smraw, unsigned& e
   return true;
 }
 
-__global__ void __launch_bounds__(256, 1) k_pre(PrePostArgs P) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  pre_body(P, smraw, epoch);
-}
-
-__device__ bool post_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
+__device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<double>& a = P.ga;
   const Smem<double> s = carve(a, smraw);
   const DevGeo& g = a.g;
@@ -370,12 +362,6 @@ __device__ bool post_body(const PrePostArgs& P, unsigned char* smraw, unsigned& 
     for (int q = threadIdx.x; q < nn; q += blockDim.x) P.u[e * nn + q] -= mean * P.uL[e * nn + q];
   }
   return true;
-}
-
-__global__ void __launch_bounds__(256, 1) k_post(PrePostArgs P) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  post_body(P, smraw, epoch);
 }
 
 inline size_t prepost_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown_w, long long d,

@@ -40,7 +40,7 @@ inline size_t refine_smem_bytes(int m, int M, int n, int ES, int nown_b, int now
 
 // One refinement step by the CTAs of a team; returns 1 when converged (done
 // set), 0 when another inner solve follows, -1 when a barrier timed out.
-__device__ int refine_body(const RefineArgs& R, unsigned char* smraw, unsigned& epoch) {
+__device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<float>& a = R.ga;
   const Smem<float> s = carve(a, smraw);
   double* p64 = reinterpret_cast<double*>(s.mats);
@@ -134,9 +134,8 @@ __device__ int refine_body(const RefineArgs& R, unsigned char* smraw, unsigned& 
     GmresArgs<float> b = a;
     b.c = R.cr;
     b.chat = R.chat_r;
-    coarse_rows(b, s);
+    if (!coarse_solve(b, s, epoch)) return -1;
   }
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return -1;
   // ---- R7: next inner right-hand side P r (FP32); Z^T r back to zero
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
     const long long sl = entry_slot(a, i);
@@ -146,11 +145,4 @@ __device__ int refine_body(const RefineArgs& R, unsigned char* smraw, unsigned& 
   for (long long j = (long long)rank * blockDim.x + threadIdx.x; j < g.d; j += (long long)G * blockDim.x)
     R.cr[j] = 0.0;
   return 0;
-}
-
-__global__ void __launch_bounds__(256, 1) k_refine(RefineArgs R) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  if (*((volatile const int*)R.done)) return;
-  unsigned epoch = 0;
-  refine_body(R, smraw, epoch);
 }

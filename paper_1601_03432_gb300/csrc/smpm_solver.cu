@@ -45,41 +45,11 @@
 #include <string>
 #include <vector>
 
-#include "smpm_internal.h"
-#include "smpm_kernels.cuh"
-
-using namespace smpm;
+#include "smpm_device.cuh"
 
 namespace {
 
 thread_local std::string g_last_error;
-
-constexpr int kSlotsPerBlock = 256;   // slots per CTA in the vector kernels
-constexpr int kElemThreads = 256;     // threads per element CTA
-constexpr int kTraceCap = 1 << 16;    // entries of the optional phase trace
-constexpr int kGmresThreads = 256;    // threads per CTA of the persistent GMRES kernel
-// per-solve control block (zeroed by one memset): 64 barrier counters |
-// err, done, nref | 8 accumulators | 32 refinement residual norms
-constexpr size_t kCtlBytes = 720;  // + 32 inner iteration counts
-constexpr int kMaxRefine = 8;        // FP64 refinement steps of the mixed-precision path
-constexpr int kMaxStreamBufs = 4;    // shared-memory buffers of the GMRES kernel's matrix stream
-constexpr int kWarpElemsMin = 4;     // owned blocks per CTA from which each warp takes its own element
-constexpr double kInnerTol = 1e-4;   // relative tolerance of each FP32 inner GMRES
-// the coarse solve is fused into the white-element phase when the atomic adds
-// it costs per Arnoldi step (d per CTA) stay below this
-constexpr long long kFusedCoarseMaxAdds = 1LL << 17;
-
-struct GState {
-  double tolabs, beta0, beta, wnorm0sq, resid;
-  int j, converged, breakdown, nan;
-  double g[kMaxRestart + 1];
-  double cs[kMaxRestart], sn[kMaxRestart];
-  double R[(kMaxRestart + 1) * kMaxRestart];  // column j at R[j*(kMaxRestart+1)]
-  double h1[kMaxRestart + 2], h2[kMaxRestart + 2];
-  double y[kMaxRestart];
-  double scal[8];
-};
-
 
 // ------------------------------------------------------------ reductions
 __device__ bool last_block_done(unsigned* cnt) {
@@ -127,79 +97,7 @@ __device__ void block_multidot(const S* __restrict__ V, long long kp, int nvec, 
   }
 }
 
-// ------------------------------------------------------- element solves
-// U = A_e^-1 B by fast diagonalisation (the Kronecker-sum structure of A_e):
-// U = Vy ((Vy^-1 B Vx^-T) ./ (lx_i + ly_j)) Vx^T.  B, U, t1: n*n in shared.
-__device__ void elem_solve_dev(int n, const double* __restrict__ fx, const double* __restrict__ fy, const double* B,
-                               double* U, double* t1) {
-  const double *Vx = fx, *Vxi = fx + n * n, *lx = fx + 2 * n * n;
-  const double *Vy = fy, *Vyi = fy + n * n, *ly = fy + 2 * n * n;
-  const int nn = n * n;
-  for (int q = threadIdx.x; q < nn; q += blockDim.x) {  // t1 = Vyi B
-    int j = q / n, a = q % n;
-    double s = 0;
-    for (int b = 0; b < n; ++b) s += __ldg(Vyi + j * n + b) * B[b * n + a];
-    t1[q] = s;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nn; q += blockDim.x) {  // U = t1 Vxi^T ./ (lx + ly)
-    int j = q / n, i = q % n;
-    double s = 0;
-    for (int a = 0; a < n; ++a) s += t1[j * n + a] * __ldg(Vxi + i * n + a);
-    U[q] = s / (__ldg(lx + i) + __ldg(ly + j));
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nn; q += blockDim.x) {  // t1 = U Vx^T
-    int j = q / n, a = q % n;
-    double s = 0;
-    for (int i = 0; i < n; ++i) s += U[j * n + i] * __ldg(Vx + a * n + i);
-    t1[q] = s;
-  }
-  __syncthreads();
-  for (int q = threadIdx.x; q < nn; q += blockDim.x) {  // U = Vy t1
-    int b = q / n, a = q % n;
-    double s = 0;
-    for (int j = 0; j < n; ++j) s += __ldg(Vy + b * n + j) * t1[j * n + a];
-    U[q] = s;
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ void face_node(int n, int F, int t, int* a, int* b) {
-  switch (F) {
-    case 0: *a = 0; *b = t; break;
-    case 1: *a = n - 1; *b = t; break;
-    case 2: *a = t; *b = 0; break;
-    default: *a = t; *b = n - 1; break;
-  }
-}
-
-// n_F . grad U at face node t (U in shared memory, D in global).
-// n_F . grad U at face node t of face F (sc = 2/h of the element across F).
-__device__ double normal_deriv(const DevGeo& g, const double* __restrict__ D, const double* U, int F, int t,
-                               double sc) {
-  const int n = g.n;
-  double acc = 0;
-  switch (F) {
-    case 0: for (int c = 0; c < n; ++c) acc += __ldg(D + c) * U[t * n + c]; return -sc * acc;
-    case 1: for (int c = 0; c < n; ++c) acc += __ldg(D + (n - 1) * n + c) * U[t * n + c]; return sc * acc;
-    case 2: for (int c = 0; c < n; ++c) acc += __ldg(D + c) * U[c * n + t]; return -sc * acc;
-    default: for (int c = 0; c < n; ++c) acc += __ldg(D + (n - 1) * n + c) * U[c * n + t]; return sc * acc;
-  }
-}
-
-// fast-diagonalisation entry: face-type class, or the column / row on a graded grid
-__device__ __forceinline__ const double* fd_x(const DevGeo& g, const double* fdx, int e) {
-  int ix = e % g.mx;
-  int cls = g.graded ? ix : ((ix > 0 ? 1 : 0) | (ix < g.mx - 1 ? 2 : 0));
-  return fdx + (size_t)cls * (2 * g.n * g.n + g.n);
-}
-__device__ __forceinline__ const double* fd_y(const DevGeo& g, const double* fdy, int e) {
-  int iy = e / g.mx;
-  int cls = g.graded ? iy : ((iy > 0 ? 1 : 0) | (iy < g.my - 1 ? 2 : 0));
-  return fdy + (size_t)cls * (2 * g.n * g.n + g.n);
-}
-
+// ------------------------------------------------------- element operators
 // b_S = B A^-1 b (Eq. schur_complement_system): one CTA per element; the flux of
 // w = A_e^-1 b_e into the slot (nbr, opp F, t) is -tau' (p' w - n_F.grad w),
 // tau' and p' those of the neighbour's face opp F.
@@ -1017,6 +915,12 @@ struct smpm_handle_s {
   float* dTcls32 = nullptr;
   int* dtiles = nullptr;     // ntiles * (class, first, count) into dclsel
   int* dclsel = nullptr;     // nel: elements sorted by class
+  // C^+ by strips (StripFactors) on the device, forward and adjoint, and the
+  // scratch of its phases (2 p mx + 1 doubles)
+  CoarseStrips<double> st{}, sta{};
+  CoarseStrips<float> st32{};
+  double st_products = 0, sta_products = 0;
+  double* wgsep = nullptr;
   double* dHT = nullptr;     // H column-major, for the fused coarse solve of the Arnoldi steps
   double* wchatd = nullptr;  // 2 d: its two c_hat buffers
   Factors f;
@@ -1079,6 +983,7 @@ struct smpm_handle_s {
     double *b = nullptr, *bS = nullptr, *rg = nullptr, *cb = nullptr, *chatb = nullptr, *xs = nullptr;
     double *x = nullptr, *t = nullptr, *y = nullptr, *vg = nullptr, *c = nullptr, *chat = nullptr;
     double *V = nullptr, *W = nullptr, *acc = nullptr, *Rh = nullptr, *yv = nullptr;
+    double* gsep = nullptr;        // strips' scratch per column
     LockColState* cs = nullptr;
     unsigned char* ctl = nullptr;  // barrier counters | err | per column: acc8, done, nref, rn
     PrePostArgs* dP = nullptr;     // 2 cap argument blocks (pre, post)
@@ -1149,6 +1054,18 @@ smpm_status upload(smpm_handle h, P** p, const std::vector<P>& src, cudaStream_t
   smpm_status s = dalloc(h, p, src.size() ? src.size() : 1);
   if (s != SMPM_OK) return s;
   if (!src.empty()) CU(cudaMemcpyAsync(*p, src.data(), src.size() * sizeof(P), cudaMemcpyHostToDevice, st));
+  return SMPM_OK;
+}
+
+template <typename T>
+smpm_status upload_strips(smpm_handle h, const StripFactors& f, CoarseStrips<T>* out, cudaStream_t st) {
+  T *N = nullptr, *Hs = nullptr, *W = nullptr, *z = nullptr;
+  auto conv = [](const std::vector<double>& v) { return std::vector<T>(v.begin(), v.end()); };
+  smpm_status s;
+  if ((s = upload(h, &N, conv(f.N), st)) || (s = upload(h, &Hs, conv(f.Hs), st)) || (s = upload(h, &W, conv(f.W), st)) ||
+      (s = upload(h, &z, conv(f.z), st)))
+    return s;
+  *out = {N, Hs, W, z, f.h, f.p, 2 * h->g.mx - 1, f.m, h->g.mx, f.ns, f.ldn, f.lds, f.ldw, 0};
   return SMPM_OK;
 }
 
@@ -1396,6 +1313,21 @@ Layout choose_layout(const Geometry& g, int m, int ES, int nown_b, int nown_w, i
   return L;
 }
 
+// Whether C^+ by strips is the cheaper form for R columns on a team of G CTAs:
+// its two extra team barriers and phase starts cost about 9,000 cycles, the
+// dense rows one cycle per product and CTA in FP64, 0.37 in FP32.  Measured
+// (SM cycles per Arnoldi step, G = 152): see the comment of coarse_solve.
+bool strips_pay(long long d, double products, int G, int R, bool fp32) {
+  return R * ((double)d * d - products) / G >= (fp32 ? 24000.0 : 9000.0);
+}
+
+// Form of the coarse solve for a solve of R columns by a.G CTAs.
+template <typename S>
+void choose_coarse(GmresArgs<S>& a, double products, int R) {
+  a.use_strips = a.precond == 2 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4);
+  a.fused = a.HT && !a.use_strips;
+}
+
 // Kernel arguments shared by the three cooperative kernels of a solve
 // (adj: the operator of the slot-swapped transposed system).
 GmresArgs<double> gmres_args(smpm_handle h, double tol, bool adj = false) {
@@ -1420,9 +1352,11 @@ GmresArgs<double> gmres_args(smpm_handle h, double tol, bool adj = false) {
   a.skip = nullptr;
   a.G = h->gm.grid;
   a.base = 0;
-  a.fused = (!adj && h->dHT) ? 1 : 0;
   a.HT = adj ? nullptr : h->dHT;
   a.chatd = h->wchatd;
+  a.strips = adj ? h->sta : h->st;
+  a.gsep = h->wgsep;
+  choose_coarse(a, adj ? h->sta_products : h->st_products, 1);
   return a;
 }
 
@@ -1447,9 +1381,11 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.skip = h->wdone;
   a.G = h->gm.grid;
   a.base = 0;
-  a.fused = h->dHT ? 1 : 0;
   a.HT = h->dHT;
   a.chatd = h->wchatd;
+  a.strips = h->st32;
+  a.gsep = h->wgsep;
+  choose_coarse(a, h->st_products, 1);
   return a;
 }
 
@@ -1525,7 +1461,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   {
     P.ga.bar = h->wbar + 0;
     void* args[] = {&P};
-    CU(cudaLaunchCooperativeKernel((const void*)k_pre, dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
+    CU(cudaLaunchCooperativeKernel(fn_pre(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
     CHECK_LAUNCH();
   }
@@ -1540,7 +1476,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
     }
     {
       void* args[] = {&a};
-      CU(cudaLaunchCooperativeKernel((const void*)k_gmres<float>, dim3(h->gm.grid), dim3(kGmresThreads), args,
+      CU(cudaLaunchCooperativeKernel(fn_gmres32(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                      h->gm32.smem, st));
       CHECK_LAUNCH();
     }
@@ -1548,7 +1484,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
     RA.ga.bar = h->wbar + 3 + 2 * ref;
     RA.rn = h->wrn + ref;
     void* args[] = {&RA};
-    CU(cudaLaunchCooperativeKernel((const void*)k_refine, dim3(h->gm.grid), dim3(kGmresThreads), args,
+    CU(cudaLaunchCooperativeKernel(fn_refine(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm32.smem_ref, st));
     CHECK_LAUNCH();
   }
@@ -1557,7 +1493,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
     P.ga.bar = h->wbar + 1;
     P.assembled = 1;
     void* args[] = {&P};
-    CU(cudaLaunchCooperativeKernel((const void*)k_post, dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
+    CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
     CHECK_LAUNCH();
     CU(cudaEventRecord(h->evq, st));
@@ -1627,7 +1563,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   {
     void* args[] = {&P};
     CU(cudaEventRecord(h->evp, st));
-    CU(cudaLaunchCooperativeKernel((const void*)k_pre, dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
+    CU(cudaLaunchCooperativeKernel(fn_pre(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
     CHECK_LAUNCH();
   }
@@ -1636,7 +1572,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
     GmresArgs<double> a = gmres_args(h, tol, adj);
     a.bar = h->wbar + 1;
     void* args[] = {&a};
-    CU(cudaLaunchCooperativeKernel((const void*)k_gmres<double>, dim3(h->gm.grid), dim3(kGmresThreads), args,
+    CU(cudaLaunchCooperativeKernel(fn_gmres64(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm.smem, st));
     CHECK_LAUNCH();
   }
@@ -1645,7 +1581,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
     P.ga.bar = h->wbar + 2;
     if (h->wtrace) P.ga.trace = h->wtrace + 3 * (kTraceCap / 4);
     void* args[] = {&P};
-    CU(cudaLaunchCooperativeKernel((const void*)k_post, dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
+    CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
     CHECK_LAUNCH();
     CU(cudaEventRecord(h->evq, st));
@@ -1729,6 +1665,7 @@ smpm_status lock_prepare(smpm_handle h, int R) {
   if ((s = lalloc(h, &L.b, cap * r)) || (s = lalloc(h, &L.bS, cap * kp)) || (s = lalloc(h, &L.rg, cap * kp)) ||
       (s = lalloc(h, &L.cb, cap * d)) || (s = lalloc(h, &L.chatb, cap * d)) || (s = lalloc(h, &L.xs, cap * kp)) ||
       (s = lalloc(h, &L.c, cap * d)) || (s = lalloc(h, &L.chat, cap * d)) ||
+      (h->st.p > 0 && (s = lalloc(h, &L.gsep, cap * (2 * (size_t)h->st.p * g.mx + 1)))) ||
       (s = lalloc(h, &L.acc, (2 * m + 1) * cap * (m + 3))) || (s = lalloc(h, &L.Rh, cap * m * (m + 1))) ||
       (s = lalloc(h, &L.yv, cap * m)) || (s = lalloc(h, &L.cs, (size_t)cap)) ||
       (s = lalloc(h, &L.ctl, kLockCtlBytes + kLockColBytes * (size_t)cap)) ||
@@ -1768,7 +1705,7 @@ smpm_status lock_shape(smpm_handle h, int R, int optin, int* RC, int* mats, size
     *smem = lock_smem_bytes<S>(m, g.M, g.n, R, *RC, h->gm.nown_b, h->gm.nown_w, false);
   }
   if (*smem > (size_t)optin) return fail(SMPM_EINVAL, "lockstep layout does not fit in shared memory");
-  CU(set_smem_limit(k_gmres_lock<S>, optin));
+  CU(set_smem_limit(sizeof(S) == 8 ? fn_lock64() : fn_lock32(), optin));
   return SMPM_OK;
 }
 
@@ -1793,8 +1730,8 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   if ((s = mixed ? lock_shape<float>(h, R, optin, &RC, &mats, &smem) : lock_shape<double>(h, R, optin, &RC, &mats,
                                                                                           &smem)))
     return s;
-  CU(set_smem_limit(k_pre_cols, optin));
-  CU(set_smem_limit(k_post_cols, optin));
+  CU(set_smem_limit(fn_pre_cols(), optin));
+  CU(set_smem_limit(fn_post_cols(), optin));
   unsigned* bar = reinterpret_cast<unsigned*>(L.ctl);
   int* err = reinterpret_cast<int*>(L.ctl + 128);
   auto colblk = [&](int k) { return L.ctl + kLockCtlBytes + kLockColBytes * (size_t)k; };
@@ -1877,7 +1814,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     const PrePostArgs* Ps = L.dP;
     int RR = R;
     void* args[] = {&Ps, &RR};
-    CU(cudaLaunchCooperativeKernel((const void*)k_pre_cols, dim3(h->gm.grid), dim3(kGmresThreads), args,
+    CU(cudaLaunchCooperativeKernel(fn_pre_cols(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm.smem_pp, st));
     CHECK_LAUNCH();
   }
@@ -1886,7 +1823,8 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     A.a.err = err;
     A.a.mats_smem = mats; A.a.basis_smem = 0; A.a.stream_mats = 0; A.a.warp_elems = 1;
     A.a.trace = nullptr; A.a.trace_cap = 0; A.a.skip = nullptr; A.a.its_out = nullptr; A.a.wscr = nullptr;
-    A.a.c = L.c; A.a.chat = L.chat; A.a.acc = L.acc;
+    A.a.c = L.c; A.a.chat = L.chat; A.a.acc = L.acc; A.a.gsep = L.gsep;
+    choose_coarse(A.a, h->st_products, R);
     A.R = R; A.RC = RC; A.vs = g.kp; A.ds = g.d;
     A.cs = L.cs; A.Rh = L.Rh; A.yv = L.yv;
   };
@@ -1903,11 +1841,11 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       A.a.trace_cap = kTraceCap / 2;
     }
     void* args[] = {&A};
-    CU(cudaLaunchCooperativeKernel((const void*)k_gmres_lock<double>, dim3(h->gm.grid), dim3(kGmresThreads), args,
+    CU(cudaLaunchCooperativeKernel(fn_lock64(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    smem, st));
     CHECK_LAUNCH();
   } else {
-    CU(set_smem_limit(k_refine_cols, optin));
+    CU(set_smem_limit(fn_refine_cols(), optin));
     for (int ref = 0; ref < kMaxRefine; ++ref) {
       LockArgs<float> A{};
       A.a = gmres_args32(h, kInnerTol);
@@ -1923,7 +1861,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       }
       {
         void* args[] = {&A};
-        CU(cudaLaunchCooperativeKernel((const void*)k_gmres_lock<float>, dim3(h->gm.grid), dim3(kGmresThreads),
+        CU(cudaLaunchCooperativeKernel(fn_lock32(), dim3(h->gm.grid), dim3(kGmresThreads),
                                        args, smem, st));
         CHECK_LAUNCH();
       }
@@ -1931,7 +1869,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
         const RefineArgs* Rs = L.dR + (size_t)ref * R;
         int RR = R;
         void* args[] = {&Rs, &RR};
-        CU(cudaLaunchCooperativeKernel((const void*)k_refine_cols, dim3(h->gm.grid), dim3(kGmresThreads), args,
+        CU(cudaLaunchCooperativeKernel(fn_refine_cols(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                        h->gm32.smem_ref, st));
         CHECK_LAUNCH();
       }
@@ -1942,7 +1880,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     const PrePostArgs* Ps = L.dP + R;
     int RR = R;
     void* args[] = {&Ps, &RR};
-    CU(cudaLaunchCooperativeKernel((const void*)k_post_cols, dim3(h->gm.grid), dim3(kGmresThreads), args,
+    CU(cudaLaunchCooperativeKernel(fn_post_cols(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm.smem_pp, st));
     CHECK_LAUNCH();
   }
@@ -2187,7 +2125,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
     begin[t] = (int)tasks.size();
     // ---- the team's lockstep workspace: the largest group it runs
     struct {
-      size_t R = 0, r = 0, kp = 0, d = 0, acc = 0, Rh = 0, yv = 0, V64 = 0, W64 = 0, V32 = 0, W32 = 0;
+      size_t R = 0, r = 0, kp = 0, d = 0, gs = 0, acc = 0, Rh = 0, yv = 0, V64 = 0, W64 = 0, V32 = 0, W32 = 0;
       bool f64 = false, f32 = false;
     } need;
     for (int p : plist[t]) {
@@ -2200,6 +2138,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
       need.r = std::max(need.r, (size_t)g.r);
       need.kp = std::max(need.kp, (size_t)g.kp);
       need.d = std::max(need.d, (size_t)g.d);
+      need.gs = std::max(need.gs, R * (2 * (size_t)h->st.p * g.mx + 1));
       need.acc = std::max(need.acc, (2 * m + 1) * R * (m + 3));
       need.Rh = std::max(need.Rh, R * m * (m + 1));
       need.yv = std::max(need.yv, R * m);
@@ -2214,7 +2153,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
       }
     }
     double *wb = nullptr, *wbS = nullptr, *wrg = nullptr, *wcb = nullptr, *wchatb = nullptr, *wxs = nullptr;
-    double *wc = nullptr, *wchat = nullptr, *wacc = nullptr, *wRh = nullptr, *wyv = nullptr;
+    double *wgs = nullptr, *wc = nullptr, *wchat = nullptr, *wacc = nullptr, *wRh = nullptr, *wyv = nullptr;
     double *wx = nullptr, *wt = nullptr, *wy = nullptr, *wvg = nullptr, *wV = nullptr, *wW = nullptr, *wcr = nullptr;
     float *wx32 = nullptr, *wt32 = nullptr, *wy32 = nullptr, *wvg32 = nullptr, *wrg32 = nullptr, *wV32 = nullptr,
           *wW32 = nullptr;
@@ -2226,6 +2165,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
           (st = balloc(b, &wrg, R * need.kp)) || (st = balloc(b, &wcb, R * need.d)) ||
           (st = balloc(b, &wchatb, R * need.d)) || (st = balloc(b, &wxs, R * need.kp)) ||
           (st = balloc(b, &wc, R * need.d)) || (st = balloc(b, &wchat, R * need.d)) ||
+          (st = balloc(b, &wgs, need.gs)) ||
           (st = balloc(b, &wacc, need.acc)) || (st = balloc(b, &wRh, need.Rh)) || (st = balloc(b, &wyv, need.yv)) ||
           (st = balloc(b, &wcs, R)) || (st = balloc(b, &wctl, R * kLockColBytes)))
         return st;
@@ -2264,6 +2204,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
         a.trace_cap = 0;
         a.skip = nullptr;
         a.its_out = nullptr;
+        choose_coarse(a, h->st_products, 1);
       };
       auto layout_fields = [&](auto& a) {
         a.mats_smem = L.lay.mats_smem;
@@ -2276,33 +2217,9 @@ smpm_status batch_layout(smpm_batch b, int T) {
       auto single_task = [&](int k) {
         BatchTask bt{};
         bt.P = prepost_args(h, tol, nullptr, nullptr, nullptr, mixed);
-        auto team_fields = [&](auto& a) {
-          a.G = T;
-          a.base = t * T;
-          a.nown_b = L.nown_b;
-          a.nown_w = L.nown_w;
-          a.ES = L.ES;
-          a.mats_smem = 0;
-          a.basis_smem = 0;
-          a.stream_mats = 0;
-          a.bar = b->dbars + t;
-          a.err = b->derr;
-          a.trace = nullptr;
-          a.trace_cap = 0;
-          a.skip = nullptr;
-          a.its_out = nullptr;
-        };
         team_fields(bt.P.ga);
         bt.P.ga.vown = nullptr;
         bt.P.ga.wscr = L.wscr64;
-        auto layout_fields = [&](auto& a) {
-          a.mats_smem = L.lay.mats_smem;
-          a.basis_smem = L.lay.basis_smem;
-          a.stream_mats = L.lay.stream_mats;
-          a.buf_elems = L.lay.buf_elems;
-          a.nbuf = L.lay.nbuf;
-          a.warp_elems = L.lay.warp_elems;
-        };
         if (mixed) {
           bt.a32 = gmres_args32(h, kInnerTol);
           team_fields(bt.a32);
@@ -2400,6 +2317,8 @@ smpm_status batch_layout(smpm_batch b, int T) {
           A.a.c = wc;
           A.a.chat = wchat;
           A.a.acc = wacc;
+          A.a.gsep = wgs;
+          choose_coarse(A.a, h->st_products, R);
           A.R = R;
           A.RC = lock_rc(R, L.nown_b, maxrc, kGmresThreads / 32);
           A.vs = g.kp;
@@ -2478,9 +2397,9 @@ smpm_status batch_layout(smpm_batch b, int T) {
   CU(cudaMemcpy(b->dbegin, begin.data(), begin.size() * sizeof(int), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(b->dteam, team_of.data(), team_of.size() * sizeof(int), cudaMemcpyHostToDevice));
   b->smem = smem;
-  CU(set_smem_limit(k_batch, optin));
+  CU(set_smem_limit(fn_batch(), optin));
   int per = 0;
-  CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_batch, kGmresThreads, smem));
+  CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn_batch(), kGmresThreads, smem));
   if (per < 1) return fail(SMPM_ECUDA, "the batch kernel does not fit on an SM");
   return SMPM_OK;
 }
@@ -2537,9 +2456,13 @@ smpm_status batch_enqueue(smpm_batch b, cudaStream_t st) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int ctl = (int)kCtlBytes;
-  CU(cudaLaunchKernelEx(&cfg, k_batch, (const BatchTask*)b->dtasks, (const int*)b->dbegin, (const int*)b->dteam,
-                        (const BatchIO*)b->dio, b->drep, ctl));
+  const BatchTask* tasks = b->dtasks;
+  const int *begin = b->dbegin, *team = b->dteam;
+  const BatchIO* io = b->dio;
+  TaskReport* rep = b->drep;
+  int ctl = (int)kCtlBytes;
+  void* args[] = {&tasks, &begin, &team, &io, &rep, &ctl};
+  CU(cudaLaunchKernelExC(&cfg, fn_batch(), args));
   CU(cudaMemcpyAsync(b->hrep, b->drep, sizeof(TaskReport) * b->ntasks, cudaMemcpyDeviceToHost, st));
   CU(cudaMemcpyAsync(b->herr, b->derr, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
   return SMPM_OK;
@@ -2939,9 +2862,9 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       gm.warp_elems = L.warp_elems;
       gm.smem = L.smem;
     }
-    CU(set_smem_limit(k_gmres<double>, smem_optin));
+    CU(set_smem_limit(fn_gmres64(), smem_optin));
     int per_sm = 0;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gmres<double>, kGmresThreads, gm.smem));
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_gmres64(), kGmresThreads, gm.smem));
     if (per_sm < 1) return fail(SMPM_ECUDA, "the GMRES kernel does not fit on an SM");
     if (opts.precision == 1) {
       // FP32 inner GMRES: FP32 copies of the operator, its own layout, the
@@ -2956,13 +2879,13 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       g32.nbuf = L.nbuf;
       g32.warp_elems = L.warp_elems;
       g32.smem = L.smem;
-      CU(set_smem_limit(k_gmres<float>, smem_optin));
-      CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gmres<float>, kGmresThreads, g32.smem));
+      CU(set_smem_limit(fn_gmres32(), smem_optin));
+      CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_gmres32(), kGmresThreads, g32.smem));
       if (per_sm < 1) return fail(SMPM_ECUDA, "the FP32 GMRES kernel does not fit on an SM");
       g32.smem_ref = refine_smem_bytes(m, g.M, g.n, gm.ES, gm.nown_b, gm.nown_w, g.d, false, g32.warp_elems != 0);
       if (g32.smem_ref > (size_t)smem_optin) return fail(SMPM_EINVAL, "grid too large for the refinement kernel");
-      CU(set_smem_limit(k_refine, smem_optin));
-      CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_refine, kGmresThreads, g32.smem_ref));
+      CU(set_smem_limit(fn_refine(), smem_optin));
+      CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_refine(), kGmresThreads, g32.smem_ref));
       if (per_sm < 1) return fail(SMPM_ECUDA, "the refinement kernel does not fit on an SM");
       auto to32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
       if ((s = upload(h, &h->dT32, to32(Tc), st)) || (s = upload(h, &h->dG32, to32(Gc), st)) ||
@@ -2977,9 +2900,9 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     }
     gm.smem_pp = prepost_smem_bytes(m, g.M, g.n, gm.ES, gm.nown_b, gm.nown_w, g.d);
     if (gm.smem_pp > (size_t)smem_optin) return fail(SMPM_EINVAL, "grid too large for the solve kernels");
-    CU(set_smem_limit(k_pre, smem_optin));
-    CU(set_smem_limit(k_post, smem_optin));
-    for (const void* fn : {(const void*)k_pre, (const void*)k_post}) {
+    CU(set_smem_limit(fn_pre(), smem_optin));
+    CU(set_smem_limit(fn_post(), smem_optin));
+    for (const void* fn : {fn_pre(), fn_post()}) {
       int per = 0;
       CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kGmresThreads, gm.smem_pp));
       if (per < 1) return fail(SMPM_ECUDA, "the solve kernels do not fit on an SM");
@@ -3037,6 +2960,17 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
           (s = upload(h, &h->dZtuSa, ztusa, st)))
         return s;
     }
+    if (h->f.cs.p > 0) {
+      if ((s = upload_strips(h, h->f.cs, &h->st, st))) return s;
+      h->st_products = h->f.cs.products;
+      if (opts.precision == 1 && (s = upload_strips(h, h->f.cs, &h->st32, st))) return s;
+    }
+    if (h->f.csa.p > 0) {
+      if ((s = upload_strips(h, h->f.csa, &h->sta, st))) return s;
+      h->sta_products = h->f.csa.products;
+    }
+    if (const int p = std::max(h->f.cs.p, h->f.csa.p); p > 0 && (s = dalloc(h, &h->wgsep, 2 * (size_t)p * g.mx + 1)))
+      return s;
     if ((s = dalloc(h, &h->wctl, kCtlBytes)) || (s = dalloc(h, &h->wxs, g.kp))) return s;
     h->wbar = reinterpret_cast<unsigned*>(h->wctl);
     h->werr = reinterpret_cast<int*>(h->wctl + 256);
@@ -3412,6 +3346,18 @@ smpm_status smpm_host_factor(smpm_handle h, const char* name, double* out, long 
   else if (nm == "uSa") src = &f.uSa;
   else if (nm == "fdx") src = &f.fdx;
   else if (nm == "fdxT") src = &f.fdxT;
+  else if (nm.rfind("strips_", 0) == 0 || nm.rfind("stripsa_", 0) == 0) {  // C^+ by strips, forward / adjoint
+    const StripFactors& k = nm[6] == 'a' ? f.csa : f.cs;
+    const std::string part = nm.substr(nm.find('_') + 1);
+    if (part == "N") src = &k.N;
+    else if (part == "Hs") src = &k.Hs;
+    else if (part == "W") src = &k.W;
+    else if (part == "z") src = &k.z;
+    else if (part == "shape") {
+      tmp = {(double)k.h, (double)k.p, (double)k.m, (double)k.ns, (double)k.ldn, (double)k.lds, (double)k.ldw};
+      src = &tmp;
+    } else return fail(SMPM_EINVAL, "unknown factor name " + nm);
+  }
   else if (nm == "black") { tmp.assign(f.black.begin(), f.black.end()); src = &tmp; }
   else if (nm == "null_iterations") { tmp.assign(1, (double)f.null_iterations); src = &tmp; }
   else return fail(SMPM_EINVAL, "unknown factor name " + nm);
@@ -3671,6 +3617,9 @@ smpm_status smpm_batch_task_times(smpm_batch b, int* team, double* begin_ms, dou
 smpm_status smpm_set_barrier_spin_limit(long long spins) try {
   const long long v = spins > 0 ? spins : (1LL << 28);
   CU(cudaMemcpyToSymbol(g_barrier_spin_limit, &v, sizeof(v)));
+  CU(set_spin_solve(v));
+  CU(set_spin_lock(v));
+  CU(set_spin_batch(v));
   return SMPM_OK;
 } catch (...) {
   return host_exception();
