@@ -1,0 +1,410 @@
+// Exact fixed-point products on the tensor cores ("digits"): y = A x for small
+// dense A in FP64 or FP32 accuracy, where the FP64 pipe of this part (2 FMA
+// per clock and SM) or the FP32 pipe's shared-memory loads are the bound.
+//
+// A number is held as a signed integer X = v 2^(B-e) (|X| < 2^B; B = 62 for
+// FP64, 30 for FP32) relative to an exponent e shared by a row of A or a
+// column of x, and cut into base-256 digits in [-128, 127] (ND = 8 or 4): with
+// the bias 0x80..80 added, the digits are the bytes of X, less 128.  Digits
+// are exact in fp16, their products are integers of at most 2^14, and up to
+// 8 x 128 of them add exactly in the FP32 accumulators of mma.sync (at most
+// 2^24; checked on this part).  Products of digits i and j weigh 256^(i+j);
+// those of one weight share an accumulator, and the weights below 256^GMIN
+// are left out.  The sums are put together in integers and rounded once.
+//
+// Error: the operands carry 2^-62 (2^-30) relative to the largest of their row
+// or column, the left-out weights about 2^-59 (2^-35) of row maximum times
+// column maximum; a chain of K FP64 FMAs loses up to K 2^-53 of the sum of
+// magnitudes.  mma.sync m16n8k16 rather than tcgen05: the operands are one
+// element's 4n x 4n matrix and eight columns (or the eight digits of one
+// column), far below a tcgen05 tile, and each warp works on its own element.
+//
+// Fragments of A (host: pack_digits): tile (mt, kt) of 16 x 16 entries, lane
+// (g = lane / 4, q = lane % 4) holds rows g, g + 8 and columns 2q, 2q+1, 2q+8,
+// 2q+9; 8 bytes per digit (the biased digits in the order of the mma
+// registers), two digits per 16-byte word: [mt][kt][digit / 2][lane].
+#pragma once
+#include <cuda_fp16.h>
+#include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+namespace {
+
+template <typename S>
+struct Digits;
+template <>
+struct Digits<double> {
+  static constexpr int ND = 8, GMIN = 7, NG = 8, B = 62;
+};
+template <>
+struct Digits<float> {
+  static constexpr int ND = 4, GMIN = 2, NG = 5, B = 30;
+};
+
+constexpr short kBadRow = 32767;  // row exponent of a matrix row with an Inf or NaN
+
+__host__ __device__ constexpr int digit_tiles(int m) { return (m + 15) / 16; }
+// uint4 words of one packed rows x cols matrix
+template <typename S>
+__host__ __device__ constexpr size_t digit_words(int rows, int cols) {
+  return (size_t)digit_tiles(rows) * digit_tiles(cols) * (Digits<S>::ND / 2) * 32;
+}
+// uint4 words of the packed eight columns of a vector of `len` entries
+template <typename S>
+__host__ __device__ constexpr int digit_bwords(int len) {
+  return digit_tiles(len) * (Digits<S>::ND / 2) * 32;
+}
+
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3},{%4,%5,%6,%7},{%8,%9},{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// two biased digits (bytes in halves 0x64dd: the fp16 number 1024 + byte) less 1152
+__device__ __forceinline__ uint32_t digit_half2(uint32_t w) {
+  const uint32_t bias = 0x64806480u;
+  const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&w), *reinterpret_cast<const __half2*>(&bias));
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// A registers of one digit from its 8 bytes
+__device__ __forceinline__ void digit_a(uint32_t w0, uint32_t w1, uint32_t (&a)[4]) {
+  a[0] = digit_half2(__byte_perm(w0, 0x64646464u, 0x4140));
+  a[1] = digit_half2(__byte_perm(w0, 0x64646464u, 0x4342));
+  a[2] = digit_half2(__byte_perm(w1, 0x64646464u, 0x4140));
+  a[3] = digit_half2(__byte_perm(w1, 0x64646464u, 0x4342));
+}
+
+// biased exponent field of v (0 for zero and subnormals, the largest value for Inf and NaN)
+__device__ __forceinline__ int exp_field(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+__device__ __forceinline__ int exp_field(float v) { return (__float_as_int(v) >> 23) & 0xff; }
+
+// biased fixed-point digits of v relative to a column whose largest exponent field is E (>= 1)
+__device__ __forceinline__ uint64_t to_digits(double v, int E) {
+  const long long bits = __double_as_longlong(v);
+  const int ev = (int)((bits >> 52) & 0x7ff);
+  long long m = bits & 0xfffffffffffffLL;
+  if (ev) m |= 1LL << 52;
+  const int sh = 9 - (E - (ev ? ev : 1));  // m < 2^53 -> below 2^62
+  long long x;
+  if (sh >= 0) x = m << sh;
+  else x = -sh < 60 ? (m + (1LL << (-sh - 1))) >> -sh : 0;
+  x = bits < 0 ? -x : x;
+  return (uint64_t)x + 0x8080808080808080ull;
+}
+__device__ __forceinline__ uint32_t to_digits(float v, int E) {
+  const int bits = __float_as_int(v);
+  const int ev = (bits >> 23) & 0xff;
+  int m = bits & 0x7fffff;
+  if (ev) m |= 1 << 23;
+  const int sh = 6 - (E - (ev ? ev : 1));  // m < 2^24 -> below 2^30
+  int x;
+  if (sh >= 0) x = m << sh;
+  else x = -sh < 28 ? (m + (1 << (-sh - 1))) >> -sh : 0;
+  x = bits < 0 ? -x : x;
+  return (uint32_t)x + 0x80808080u;
+}
+
+// byte j of a and b as the two low halves' digits
+template <typename U>
+__device__ __forceinline__ uint32_t digit_pair(U a, U b, int j) {
+  uint32_t wa, wb;
+  if constexpr (sizeof(U) == 8) {
+    wa = j < 4 ? (uint32_t)a : (uint32_t)(a >> 32);
+    wb = j < 4 ? (uint32_t)b : (uint32_t)(b >> 32);
+  } else {
+    wa = a;
+    wb = b;
+  }
+  const uint32_t p = __byte_perm(wa, wb, (uint32_t)((j & 3) | ((4 + (j & 3)) << 8)));  // bytes 0 and 2
+  return digit_half2((p & 0x00ff00ffu) | 0x64006400u);
+}
+
+// value 2^s of the integer hi 2^32 + lo (|hi| < 2^62, |lo| < 2^62), rounded to
+// nearest; s such that the result is a normal number unless it is zero
+__device__ __forceinline__ double digits_value(long long hi, long long lo, int s) {
+  hi += lo >> 32;
+  uint32_t l = (uint32_t)lo;  // value = hi 2^32 + l
+  const bool neg = hi < 0;
+  if (neg) {
+    hi = ~hi;
+    l = ~l;  // magnitude - 1; the missing unit is far below the rounding unless hi is 0
+    if (++l == 0) ++hi;
+  }
+  unsigned long long h = (unsigned long long)hi;
+  int e = 32;
+  if (h == 0) {
+    if (l == 0) return 0.0;
+    h = (unsigned long long)l << 32;
+    l = 0;
+    e = -32;
+  }
+  const int z = __clzll((long long)h);
+  if (z) h = (h << z) | (z < 32 ? (unsigned long long)(l >> (32 - z)) : ((unsigned long long)l << (z - 32)));
+  e -= z;
+  unsigned long long m = (h >> 11) + ((h >> 10) & 1);  // 53 bits, nearest
+  // value = m 2^(e + 11): the exponent field of m (implicit bit included) is added below
+  const long long bits = (long long)m + ((long long)(e + 11 + s + 1023 + 52 - 1) << 52);
+  return __longlong_as_double(neg ? (bits | (1LL << 63)) : bits);
+}
+
+// v 2^s for any s (two exact factors where the scale itself is out of range)
+__device__ __forceinline__ double scale2(double v, int s) {
+  if (s < -1000 || s > 1000) {
+    const int h = s / 2;
+    return v * __longlong_as_double((long long)(1023 + max(-1022, min(1023, h))) << 52) *
+           __longlong_as_double((long long)(1023 + max(-1022, min(1023, s - h))) << 52);
+  }
+  return v * __longlong_as_double((long long)(1023 + s) << 52);
+}
+
+// Result from the summed weights hi 2^32 + lo (units of 256^GMIN); er: exponent
+// of A's row, E: the column's largest exponent field.  Inf or NaN in the column
+// gives NaN, as does a row marked kBadRow.
+__device__ __forceinline__ double digits_result(long long hi, long long lo, int er, int E, double) {
+  const int s = er + E - 1022 + 56 - 124;  // 256^7 2^(er - 62) 2^(E - 1022 - 62)
+  if (E >= 600 && E <= 1400 && er != kBadRow) return digits_value(hi, lo, s);
+  if (E == 0x7ff || er == kBadRow) return __longlong_as_double(0x7ff8000000000000LL);
+  return scale2(digits_value(hi, lo, 0), s);
+}
+__device__ __forceinline__ float digits_result(long long hi, long long lo, int er, int E, float) {
+  if (E == 0xff || er == kBadRow) return __int_as_float(0x7fc00000);
+  return (float)digits_value(hi, lo, er + E - 126 + 16 - 60);  // 256^2 2^(er - 30) 2^(E - 126 - 30), FP64 exponents
+}
+
+// ---- eight columns -----------------------------------------------------------
+// Packs the eight columns x(k, c), k < len, into Bf (digit_bwords words) and
+// returns the largest exponent field (>= 1) of column g = lane / 4.  get(k, c):
+// the entry.  One warp (it packs the k tiles part, part + parts, ...: several
+// warps share the work, each finding the exponents itself).
+template <typename S, typename Get>
+__device__ __forceinline__ int pack_cols(uint4* Bf, int len, int lane, Get&& get, int part = 0, int parts = 1) {
+  constexpr int ND = Digits<S>::ND;
+  const int g = lane >> 2, q = lane & 3, kt_n = digit_tiles(len);
+  int E = 1;
+  for (int kt = 0; kt < kt_n; ++kt)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
+      if (k < len) E = max(E, exp_field((S)get(k, g)));
+    }
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+  for (int kt = part; kt < kt_n; kt += parts) {
+    decltype(to_digits(S(0), 1)) Y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
+      Y[u] = to_digits(k < len ? (S)get(k, g) : S(0), E);
+    }
+#pragma unroll
+    for (int j = 0; j < ND; j += 2)
+      Bf[(kt * (ND / 2) + j / 2) * 32 + lane] =
+          make_uint4(digit_pair(Y[0], Y[1], j), digit_pair(Y[2], Y[3], j), digit_pair(Y[0], Y[1], j + 1),
+                     digit_pair(Y[2], Y[3], j + 1));
+  }
+  __syncwarp();
+  return E;
+}
+
+// Row tile mt of A times the packed columns: put(row g or g + 8, column, value)
+// for rows < rows.  Af: A's fragments (L1/L2), er: its row exponents, E: the
+// exponent field of column lane / 4 (from pack_cols).
+template <typename S, typename Put>
+__device__ __forceinline__ void digits_tile8(const uint4* __restrict__ Af, const short* __restrict__ er,
+                                             const uint4* Bf, int rows, int kt_n, int mt, int lane, int E, Put&& put) {
+  constexpr int ND = Digits<S>::ND, GMIN = Digits<S>::GMIN, NG = Digits<S>::NG;
+  float acc[NG][4];
+#pragma unroll
+  for (int c = 0; c < NG; ++c)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[c][v] = 0.f;
+  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
+  uint4 an[ND / 2];
+#pragma unroll
+  for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + p * 32);
+  for (int kt = 0; kt < kt_n; ++kt) {
+    uint4 av[ND / 2], bv[ND / 2];
+#pragma unroll
+    for (int p = 0; p < ND / 2; ++p) {
+      av[p] = an[p];
+      bv[p] = Bf[(kt * (ND / 2) + p) * 32 + lane];
+    }
+    if (kt + 1 < kt_n) {
+#pragma unroll
+      for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + ((kt + 1) * (ND / 2) + p) * 32);
+    }
+#pragma unroll
+    for (int i = 0; i < ND; ++i) {
+      uint32_t a[4];
+      const uint4 w = av[i / 2];
+      digit_a((i & 1) ? w.z : w.x, (i & 1) ? w.w : w.y, a);
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        if (i + j < GMIN) continue;
+        const uint4 b = bv[j / 2];
+        mma_16816(acc[i + j - GMIN], a, (j & 1) ? b.z : b.x, (j & 1) ? b.w : b.y);
+      }
+    }
+  }
+  // lane holds rows g, g + 8 of columns 2q, 2q + 1 (their E is with lanes 8q, 8q + 4)
+  const int g = lane >> 2, q = lane & 3;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const int row = mt * 16 + g + 8 * (v >> 1), col = 2 * q + (v & 1);
+    const int Ec = __shfl_sync(0xffffffffu, E, 4 * col);
+    if (row < rows) {
+      long long lo = 0, hi = 0;
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const long long t = (long long)__float2int_rn(acc[k][v]) << (8 * (k & 3));
+        if (k < 4) lo += t;
+        else hi += t;
+      }
+      put(row, col, digits_result(hi, lo, er[row], Ec, S(0)));
+    }
+  }
+}
+
+// ---- one column --------------------------------------------------------------
+// The eight mma columns are the weights: digit i of A meets digit n + GMIN - i
+// of x in column n, so the digits of A share one accumulator tile (two, by
+// parity, for shorter chains).  Bf: one fragment per digit i of A
+// (digit_bwords words).  get(k): entry k < len; returns the largest exponent
+// field (>= 1).  One warp packs the k tiles part, part + parts, ...
+template <typename S, typename Get>
+__device__ __forceinline__ int pack_one(uint4* Bf, int len, int lane, Get&& get, int part = 0, int parts = 1) {
+  constexpr int ND = Digits<S>::ND, GMIN = Digits<S>::GMIN, NG = Digits<S>::NG, OFF = ND - 1 - GMIN;
+  const int g = lane >> 2, q = lane & 3, kt_n = digit_tiles(len);
+  int E = 1;
+  for (int k = lane; k < len; k += 32) E = max(E, exp_field((S)get(k)));
+  E = __reduce_max_sync(0xffffffffu, E);
+  constexpr unsigned long long kFill = 0x8080808080808080ull;
+  for (int kt = part; kt < kt_n; kt += parts) {
+    unsigned long long Y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
+      unsigned long long y = to_digits(k < len ? (S)get(k) : S(0), E);
+      if (sizeof(S) == 4) y = ((y | (kFill << 32)) << (8 * OFF)) | (kFill >> (64 - 8 * (OFF > 0 ? OFF : 1)));
+      // digits moved down by g places, zeros moved in at the top
+      if (g > 0) y = (y >> (8 * g)) | (kFill << (64 - 8 * g));
+      Y[u] = y;
+    }
+    uint32_t r[ND][2];
+#pragma unroll
+    for (int i = 0; i < ND; ++i) {  // digit g + GMIN - i of x is now at place GMIN - i + OFF = ND - 1 - i
+      r[i][0] = g < NG ? digit_pair(Y[0], Y[1], ND - 1 - i) : 0u;
+      r[i][1] = g < NG ? digit_pair(Y[2], Y[3], ND - 1 - i) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < ND; i += 2)
+      Bf[(kt * (ND / 2) + i / 2) * 32 + lane] = make_uint4(r[i][0], r[i][1], r[i + 1][0], r[i + 1][1]);
+  }
+  __syncwarp();
+  return E;
+}
+
+// Row tile mt of A times the packed column: put(row, value) for rows < rows.
+template <typename S, typename Put>
+__device__ __forceinline__ void digits_tile1(const uint4* __restrict__ Af, const short* __restrict__ er,
+                                             const uint4* Bf, int rows, int kt_n, int mt, int lane, int E, Put&& put) {
+  constexpr int ND = Digits<S>::ND;
+  float acc[2][4];
+#pragma unroll
+  for (int v = 0; v < 8; ++v) acc[v >> 2][v & 3] = 0.f;
+  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
+  uint4 an[ND / 2];
+#pragma unroll
+  for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + p * 32);
+  for (int kt = 0; kt < kt_n; ++kt) {
+    uint4 av[ND / 2];
+#pragma unroll
+    for (int p = 0; p < ND / 2; ++p) av[p] = an[p];
+    if (kt + 1 < kt_n) {
+#pragma unroll
+      for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + ((kt + 1) * (ND / 2) + p) * 32);
+    }
+#pragma unroll
+    for (int p = 0; p < ND / 2; ++p) {
+      const uint4 b = Bf[(kt * (ND / 2) + p) * 32 + lane];
+      uint32_t a[4];
+      digit_a(av[p].x, av[p].y, a);
+      mma_16816(acc[0], a, b.x, b.y);
+      digit_a(av[p].z, av[p].w, a);
+      mma_16816(acc[1], a, b.z, b.w);
+    }
+  }
+  // lane holds weights 2q, 2q + 1 of rows g and g + 8; the quad adds them up:
+  // row g ends in lane q = 0, row g + 8 in lane q = 2
+  const int g = lane >> 2, q = lane & 3;
+  long long w[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const long long a0 = (long long)__float2int_rn(acc[0][2 * h]) + __float2int_rn(acc[1][2 * h]);
+    const long long a1 = (long long)__float2int_rn(acc[0][2 * h + 1]) + __float2int_rn(acc[1][2 * h + 1]);
+    w[h] = a0 + (a1 << 8);
+    if (q & 1) w[h] <<= 16;
+    w[h] += __shfl_xor_sync(0xffffffffu, w[h], 1);
+  }
+  const long long got = __shfl_xor_sync(0xffffffffu, q < 2 ? w[1] : w[0], 2);
+  const int row = mt * 16 + g + (q < 2 ? 0 : 8);
+  if (!(q & 1) && row < rows)
+    put(row, q < 2 ? digits_result(got, w[0], er[row], E, S(0)) : digits_result(w[1], got, er[row], E, S(0)));
+}
+
+// Packs count row-major rows x cols matrices: fragments (digit_words each) and
+// row exponents (rows each, within +-400: the results' exponents are formed
+// without checks).  A row with an Inf or NaN, or above 2^400, is marked.
+template <typename S>
+void pack_digits(const double* A, int rows, int cols, size_t count, std::vector<uint4>* frag, std::vector<short>* er) {
+  constexpr int ND = Digits<S>::ND, B = Digits<S>::B;
+  const int mt_n = digit_tiles(rows), kt_n = digit_tiles(cols);
+  frag->assign(count * digit_words<S>(rows, cols), make_uint4(0, 0, 0, 0));
+  er->assign(count * rows, 0);
+  constexpr uint64_t kBias = ND == 8 ? 0x8080808080808080ull : 0x80808080ull;
+#pragma omp parallel for schedule(static) if (count > 16)
+  for (long long c = 0; c < (long long)count; ++c) {
+    const double* a = A + c * rows * cols;
+    std::vector<uint64_t> Y((size_t)mt_n * 16 * kt_n * 16, kBias);
+    for (int r = 0; r < rows; ++r) {
+      double mx = 0;
+      bool ok = true;
+      for (int k = 0; k < cols; ++k) {
+        const double v = std::fabs(a[(size_t)r * cols + k]);
+        ok = ok && v < 0x1p400;
+        if (v > mx) mx = v;
+      }
+      int e = 0;
+      if (ok && mx > 0) std::frexp(mx, &e);
+      e = std::max(e, -400);
+      (*er)[c * rows + r] = ok ? (short)e : kBadRow;
+      if (!ok) continue;
+      for (int k = 0; k < cols; ++k)
+        Y[(size_t)r * kt_n * 16 + k] = kBias + (uint64_t)std::llrint(std::ldexp(a[(size_t)r * cols + k], B - e));
+    }
+    uint4* f = frag->data() + c * digit_words<S>(rows, cols);
+    for (int mt = 0; mt < mt_n; ++mt)
+      for (int kt = 0; kt < kt_n; ++kt)
+        for (int p = 0; p < ND / 2; ++p)
+          for (int lane = 0; lane < 32; ++lane) {
+            const int g = lane / 4, q = lane % 4;
+            uint32_t w[4];
+            for (int h = 0; h < 4; ++h) {  // h: digit 2p + (h / 2), columns 2q + 8 (h % 2) of rows g, g + 8
+              w[h] = 0;
+              for (int b = 0; b < 4; ++b) {
+                const int row = mt * 16 + g + 8 * (b / 2), col = kt * 16 + 2 * q + (b % 2) + 8 * (h % 2);
+                const uint64_t y = Y[(size_t)row * kt_n * 16 + col];
+                w[h] |= (uint32_t)((y >> (8 * (2 * p + h / 2))) & 0xff) << (8 * b);
+              }
+            }
+            f[((size_t)(mt * kt_n + kt) * (ND / 2) + p) * 32 + lane] = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+  }
+}
+
+}  // namespace

@@ -659,7 +659,7 @@ void row_sums(const Geometry& g, const std::vector<double>& T, const std::vector
 // inversion.
 int block_factors(const Geometry& g, const std::vector<int>& black, const std::vector<double>& T,
                   const std::vector<int>& tcls, std::vector<double>* Gout, std::vector<double>* Xout,
-                  std::string* err) {
+                  std::vector<int>* repout, std::string* err) {
   const int n = g.n, M = g.M;
   const size_t nb = black.size();
   Gout->assign(nb * M * M, 0.0);
@@ -717,6 +717,8 @@ int block_factors(const Geometry& g, const std::vector<int>& black, const std::v
 #pragma omp parallel for schedule(static)
   for (long long ib = 0; ib < static_cast<long long>(nb); ++ib)
     std::memcpy(Gout->data() + ib * M * M, ginv[rep[ib]].data(), sizeof(double) * M * M);
+  repout->resize(nb);
+  for (size_t ib = 0; ib < nb; ++ib) (*repout)[ib] = reps[rep[ib]];
   return SMPM_OK;
 }
 
@@ -1022,7 +1024,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
   f->white.clear();
   for (long long e = 0; e < g.nel; ++e) (g.black(static_cast<int>(e)) ? f->black : f->white).push_back(static_cast<int>(e));
   {
-    int st = block_factors(g, f->black, f->T, f->tcls, &f->G, &f->X, err);
+    int st = block_factors(g, f->black, f->T, f->tcls, &f->G, &f->X, &f->grep, err);
     if (st != SMPM_OK) return st;
   }
 
@@ -1177,7 +1179,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
         for (int j = 0; j < M; ++j) Ae[i * M + j] = Te[j * M + i];
     }
     row_sums(g, f->Ta, f->zwa, &f->Rsa);
-    int sta = block_factors(g, f->black, f->Ta, f->tcls, &f->Ga, &f->Xa, err);
+    int sta = block_factors(g, f->black, f->Ta, f->tcls, &f->Ga, &f->Xa, &f->grep, err);
     if (sta != SMPM_OK) return sta;
     transpose_fd(n, f->fdx, &f->fdxT);
     transpose_fd(n, f->fdy, &f->fdyT);

@@ -44,7 +44,17 @@ struct GmresArgs {
   const S* Tc;      // nel * M*M, column-major T_e
   const S* Gc;      // nblack * M*M, column-major G_b
   const S* Xc;      // nblack * 4*n*n, column-major X_F blocks
-  const S* Rs;      // nel * M*4 row sums of T_e (deflation)
+  // identical matrices (one class of face types and sizes) are read from one
+  // copy: T_e from element tr[e]'s, G_b and X_b from block gr[ib]'s.  A CTA's
+  // elements are mostly of one class, so the matrices come from L1 instead of
+  // once per element from L2 or HBM
+  const int* tr;
+  const int* gr;
+  // per entry of a black block (2M per block: own slots, then facing slots):
+  // {slot or -1, element that pushes into it, its interface or -1, 4 e + F of the slot}
+  const int4* bt;
+  const int4* if4;   // interfaces of each element (0 where there is none; its weight is 0)
+  const double* Rd;  // kp * 4: S Z at each slot, the coefficients of c_hat on the pusher's interfaces
   // d*d row-major coarse inverse: FP64, or its FP32 copy for the FP32 inner
   // solves of the mixed-precision path
   const typename std::conditional<sizeof(S) == 4, float, double>::type* H;
@@ -158,15 +168,10 @@ __device__ bool grid_sync(unsigned* bar, int* err, unsigned& epoch, int G) {
   return grid_sync_with(bar, err, epoch, G, [] {});
 }
 
-// slot of entry i (< 2M) of the block of black element e: own slots first,
-// then the neighbours' slots facing e; -1 where a face has no neighbour.
-__device__ __forceinline__ long long block_slot(const DevGeo& g, int e, int i) {
-  const int M = g.M, n = g.n;
-  if (i < M) return (long long)e * M + i;
-  i -= M;
-  int F = i / n, t = i % n;
-  int e2 = dev_neighbour(g, e, F);
-  return e2 >= 0 ? (long long)e2 * M + (F ^ 1) * n + t : -1;
+// entry i (< 2M) of black block ib
+template <typename S>
+__device__ __forceinline__ int4 block_entry(const GmresArgs<S>& a, int ib, int i) {
+  return __ldg(a.bt + (size_t)ib * 2 * a.g.M + i);
 }
 
 // per-warp scratch of the warp-per-element phases: p, q (the block's own and
@@ -251,23 +256,23 @@ inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown
 template <typename S>
 __device__ __forceinline__ const S* mat_G(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib) {
   const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) : a.Gc + (size_t)ib * M * M;
+  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) : a.Gc + (size_t)__ldg(a.gr + ib) * M * M;
 }
 template <typename S>
 __device__ __forceinline__ const S* mat_Tb(const GmresArgs<S>& a, const Smem<S>& s, int k, int e) {
   const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + M * M : a.Tc + (size_t)e * M * M;
+  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + M * M : a.Tc + (size_t)__ldg(a.tr + e) * M * M;
 }
 template <typename S>
 __device__ __forceinline__ const S* mat_X(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib) {
   const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + 2 * M * M : a.Xc + (size_t)ib * 4 * n * n;
+  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + 2 * M * M : a.Xc + (size_t)__ldg(a.gr + ib) * 4 * n * n;
 }
 template <typename S>
 __device__ __forceinline__ const S* mat_Tw(const GmresArgs<S>& a, const Smem<S>& s, int k, int e) {
   const int M = a.g.M, n = a.g.n;
   return a.mats_smem ? s.mats + (size_t)a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M
-                     : a.Tc + (size_t)e * M * M;
+                     : a.Tc + (size_t)__ldg(a.tr + e) * M * M;
 }
 
 template <typename S>
@@ -330,16 +335,17 @@ __device__ void ms_issue(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>& 
     if ((it & 1) == 0) {
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm + xx)
                    : "memory");
-      bulk_g2s(dst, a.Gc + (size_t)ib * M * M, mm, bar);
-      bulk_g2s(dst + (size_t)M * M, a.Xc + (size_t)ib * 4 * n * n, xx, bar);
+      const size_t ir = __ldg(a.gr + ib);
+      bulk_g2s(dst, a.Gc + ir * M * M, mm, bar);
+      bulk_g2s(dst + (size_t)M * M, a.Xc + ir * 4 * n * n, xx, bar);
     } else {
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm) : "memory");
-      bulk_g2s(dst, a.Tc + (size_t)a.black[ib] * M * M, mm, bar);
+      bulk_g2s(dst, a.Tc + (size_t)__ldg(a.tr + a.black[ib]) * M * M, mm, bar);
     }
   } else {
     const int k = it - 2 * ms.nb, iw = rank + k * G;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm) : "memory");
-    bulk_g2s(dst, a.Tc + (size_t)a.white[iw] * M * M, mm, bar);
+    bulk_g2s(dst, a.Tc + (size_t)__ldg(a.tr + a.white[iw]) * M * M, mm, bar);
   }
 }
 
@@ -417,11 +423,11 @@ __device__ void block_solve_a(const GmresArgs<S>& a, const Smem<S>& s, const S* 
 }
 
 template <typename S>
-__device__ void block_solve_b(const GmresArgs<S>& a, const Smem<S>& s, int e, const S* T, const S* vb) {
+__device__ void block_solve_b(const GmresArgs<S>& a, const Smem<S>& s, int ib, const S* T, const S* vb) {
   const int M = a.g.M;
   gemv_split(T, M, s.av, s.z, M, M, s.red);
   for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) {
-    long long sl = block_slot(a.g, e, i);
+    const int sl = block_entry(a, ib, i).x;
     if (sl < 0) continue;
     a.t[sl] = i < M ? s.av[i] : (S)(vb[i] - s.z[i - M]);
   }
@@ -431,7 +437,7 @@ __device__ void block_solve_b(const GmresArgs<S>& a, const Smem<S>& s, int e, co
 template <typename S>
 __device__ void block_solve(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib, int e, const S* vb) {
   block_solve_a(a, s, mat_G(a, s, k, ib), mat_X(a, s, k, ib), vb);
-  block_solve_b(a, s, e, mat_Tb(a, s, k, e), vb);
+  block_solve_b(a, s, ib, mat_Tb(a, s, k, e), vb);
 }
 
 // White element: y = S t on the black slots facing e, y = sc*v on e's slots,
@@ -481,7 +487,7 @@ __device__ void push_step(const GmresArgs<S>& a, const Smem<S>& s, int e, const 
   const int M = g.M, n = g.n;
   for (int i = threadIdx.x; i < M; i += blockDim.x) s.p[i] = (S)(sc * (double)ldcg(v + (size_t)e * M + i));
   __syncthreads();
-  gemv_split(a.Tc + (size_t)e * M * M, M, s.p, s.z, M, M, s.red);
+  gemv_split(a.Tc + (size_t)__ldg(a.tr + e) * M * M, M, s.p, s.z, M, M, s.red);
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     int F = i / n, tt = i % n;
     int e2 = dev_neighbour(g, e, F);
@@ -779,25 +785,21 @@ __device__ __forceinline__ bool coarse_solve(const GmresArgs<S>& a, const Smem<S
   return grid_sync(a.bar, a.err, epoch, a.G);
 }
 
-// w = y - S Z chat for one slot (pull form); chat == nullptr gives w = y.
-template <typename S>
-__device__ __forceinline__ double deflate_slot_cg(const DevGeo& g, const S* y, const double* chat,
-                                                  const S* __restrict__ Rs, long long sl) {
-  const int M = g.M, n = g.n;
-  int e = (int)(sl / M), i = (int)(sl % M), F = i / n, t = i % n;
-  int e2 = dev_neighbour(g, e, F);
-  if (e2 < 0) return 0.0;
-  double ys = (double)ldcg(y + sl);
+// ys - (S Z chat) at an entry (pull form); 0 on the physical boundary, ys
+// itself when chat is null.
+template <typename A>
+__device__ __forceinline__ double deflate_value(const GmresArgs<A>& a, double ys, const double* chat, int4 en) {
+  if (en.z < 0) return 0.0;
   if (!chat) return ys;
-  double acc = __ldcg(chat + dev_iface(g, e, F));
-  if (g.zw) acc *= dev_zw(g, e, F);  // uniform grids: weight 1, no FP64 multiply
-  const S* R = Rs + ((size_t)e2 * M + (F ^ 1) * n + t) * 4;
-#pragma unroll
-  for (int G = 0; G < 4; ++G) {
-    int jj = dev_iface(g, e2, G);
-    if (jj >= 0) acc += (double)__ldg(R + G) * __ldcg(chat + jj);
-  }
-  return ys - acc;
+  const int4 J = __ldg(a.if4 + en.y);
+  const double2* R = reinterpret_cast<const double2*>(a.Rd + 4 * (size_t)en.x);
+  const double2 r0 = __ldg(R), r1 = __ldg(R + 1);
+  const double c0 = __ldcg(chat + J.x), c1 = __ldcg(chat + J.y), c2 = __ldcg(chat + J.z), c3 = __ldcg(chat + J.w);
+  return (ys - (r0.x * c0 + r0.y * c1)) - (r1.x * c2 + r1.y * c3);
+}
+template <typename S, typename A>
+__device__ __forceinline__ double deflate_entry(const GmresArgs<A>& a, const S* y, const double* chat, int4 en) {
+  return deflate_value(a, en.x >= 0 ? (double)ldcg(y + en.x) : 0.0, chat, en);
 }
 
 // Dot products of the owned basis slice with vec (ES entries) for l < nl,
@@ -877,13 +879,16 @@ __device__ __forceinline__ double basis_combo(const GmresArgs<S>& a, const Smem<
   }
 }
 
+// owned entry i of the CTA: block rank + k G, entry i - 2M k of it
 template <typename S>
-__device__ __forceinline__ long long entry_slot(const GmresArgs<S>& a, int i) {
-  const int M2 = 2 * a.g.M;
-  int k = i / M2, ii = i % M2;
-  int ib = team_rank(a) + k * a.G;
-  if (k >= a.nown_b || ib >= a.nblack) return -1;
-  return block_slot(a.g, a.black[ib], ii);
+__device__ __forceinline__ int4 owned_entry(const GmresArgs<S>& a, int i) {
+  const int M2 = 2 * a.g.M, k = i / M2, ib = team_rank(a) + k * a.G;
+  if (k >= a.nown_b || ib >= a.nblack) return make_int4(-1, 0, -1, 0);
+  return block_entry(a, ib, i - k * M2);
+}
+template <typename S>
+__device__ __forceinline__ int entry_slot(const GmresArgs<S>& a, int i) {
+  return owned_entry(a, i).x;
 }
 
 // ---- warp-per-element phases -------------------------------------------
@@ -959,7 +964,7 @@ __device__ void black_phase_warps(const GmresArgs<S>& a, const Smem<S>& s, const
       if (own) {
         v = (S)(sc * (double)own[k * 2 * M + i]);
       } else {
-        const long long sl = block_slot(g, e, i);
+        const int sl = block_entry(a, ib, i).x;
         v = sl >= 0 ? (S)(sc * (double)ldcg(src + sl)) : S(0);
       }
       p[i] = v;  // p and q are contiguous: q = p + M
@@ -977,7 +982,7 @@ __device__ void black_phase_warps(const GmresArgs<S>& a, const Smem<S>& s, const
     warp_gemv(mat_G(a, s, k, ib), r1, av, M, lane);
     warp_gemv(mat_Tb(a, s, k, e), av, z, M, lane);
     for (int i = lane; i < 2 * M; i += 32) {
-      const long long sl = block_slot(g, e, i);
+      const int sl = block_entry(a, ib, i).x;
       if (sl >= 0) a.t[sl] = i < M ? av[i] : (S)(q[i - M] - z[i - M]);
     }
     __syncwarp();
@@ -1053,7 +1058,7 @@ __device__ bool black_phase(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S
       if (own) {
         s.w[i] = (S)(sc * (double)own[k * 2 * M + i]);
       } else {
-        long long sl = block_slot(g, e, i);
+        const int sl = block_entry(a, ib, i).x;
         s.w[i] = sl >= 0 ? (S)(sc * (double)ldcg(src + sl)) : S(0);
       }
     }
@@ -1065,7 +1070,7 @@ __device__ bool black_phase(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S
       ms_release(a, s, *ms);
       const S* T = ms_acquire(a, s, *ms);
       if (!T) return false;
-      block_solve_b(a, s, e, T, s.w);
+      block_solve_b(a, s, ib, T, s.w);
       ms_release(a, s, *ms);
     } else {
       block_solve(a, s, k, ib, e, s.w);
@@ -1238,17 +1243,18 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       int e = a.black[ib];
       S* dst = s.mats + (size_t)k * (2 * M * M + 4 * n * n);
       for (int i = threadIdx.x; i < M * M; i += blockDim.x) {
-        dst[i] = a.Gc[(size_t)ib * M * M + i];
-        dst[M * M + i] = a.Tc[(size_t)e * M * M + i];
+        dst[i] = a.Gc[(size_t)a.gr[ib] * M * M + i];
+        dst[M * M + i] = a.Tc[(size_t)a.tr[e] * M * M + i];
       }
-      for (int i = threadIdx.x; i < 4 * n * n; i += blockDim.x) dst[2 * M * M + i] = a.Xc[(size_t)ib * 4 * n * n + i];
+      for (int i = threadIdx.x; i < 4 * n * n; i += blockDim.x)
+        dst[2 * M * M + i] = a.Xc[(size_t)a.gr[ib] * 4 * n * n + i];
     }
     for (int k = 0; k < a.nown_w; ++k) {
       int iw = rank + k * G;
       if (iw >= a.nwhite) break;
       int e = a.white[iw];
       S* dst = s.mats + (size_t)a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M;
-      for (int i = threadIdx.x; i < M * M; i += blockDim.x) dst[i] = a.Tc[(size_t)e * M * M + i];
+      for (int i = threadIdx.x; i < M * M; i += blockDim.x) dst[i] = a.Tc[(size_t)a.tr[e] * M * M + i];
     }
   }
 
@@ -1266,11 +1272,12 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       S* v0 = basis(a, s, 0);
       double nn = 0;
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-        long long sl = entry_slot(a, i);
+        const int4 en = owned_entry(a, i);
+        const int sl = en.x;
         S rv = 0;
         if (sl >= 0) {
           double r = (double)ldcg(a.rhs + sl);
-          if (cycle > 0) r -= deflate_slot_cg(g, a.y, a.precond == 2 ? a.chat : nullptr, a.Rs, sl);
+          if (cycle > 0) r -= deflate_entry(a, a.y, a.precond == 2 ? a.chat : nullptr, en);
           rv = (S)r;
           a.vglob[sl] = rv;
         }
@@ -1310,7 +1317,7 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
         for (int i = threadIdx.x; i < ES; i += blockDim.x) {
           S rv = (S)basis_combo(a, s, (double)s.w2[i], s.hs2, j, i);
           vj[i] = rv;
-          long long sl = entry_slot(a, i);
+          const int sl = entry_slot(a, i);
           if (sl >= 0) a.vglob[sl] = rv;
         }
         __syncthreads();
@@ -1335,8 +1342,7 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       // ---- D: w = y - S Z chat on owned entries; V^T w, ||w||^2
       const double* chat_d = a.precond == 2 ? (fused ? chat_j : a.chat) : nullptr;
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-        long long sl = entry_slot(a, i);
-        s.w[i] = sl >= 0 ? (S)deflate_slot_cg(g, a.y, chat_d, a.Rs, sl) : S(0);
+        s.w[i] = (S)deflate_entry(a, a.y, chat_d, owned_entry(a, i));
       }
       __syncthreads();
       owned_dots(a, s, s.w, j + 2, accD);
@@ -1450,7 +1456,7 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
     for (int l = threadIdx.x; l < j; l += blockDim.x) s.hs1[l] = -__ldcg(a.gs->y + l) * s.invb[l];
     __syncthreads();
     for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-      long long sl = entry_slot(a, i);
+      const int sl = entry_slot(a, i);
       if (sl < 0) continue;
       a.x[sl] = (S)basis_combo(a, s, (double)ldcg(a.x + sl), s.hs1, j, i);
     }

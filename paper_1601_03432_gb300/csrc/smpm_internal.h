@@ -97,6 +97,7 @@ struct Factors {
   std::vector<int> tcls;     // nel : class of T_e (elements of one class hold identical T_e)
   std::vector<double> Rs;    // nel * M*4 : row sums of T_e per input face
   std::vector<int> black, white;
+  std::vector<int> grep;     // nblack : first block that holds the same G_b and X_b
   std::vector<double> G;     // nblack * M*M : (I - X Y)^-1
   std::vector<double> X;     // nblack * 4*n*n : X_F blocks
   std::vector<double> C;     // d*d coarse matrix

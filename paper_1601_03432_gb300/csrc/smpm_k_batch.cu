@@ -2,6 +2,7 @@
 // lockstep solves task by task.
 #define SMPM_BODY __noinline__
 #include "smpm_device.cuh"
+#include "smpm_digits.cuh"
 
 namespace {
 

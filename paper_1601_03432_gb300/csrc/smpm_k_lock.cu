@@ -1,5 +1,6 @@
 // Kernels of a lockstep solve of several right-hand sides of one grid.
 #include "smpm_device.cuh"
+#include "smpm_digits.cuh"
 
 namespace {
 

@@ -46,6 +46,9 @@ __device__ __forceinline__ double dev_zw(const DevGeo& g, int e, int F) {
   return g.zw ? __ldg(g.zw + 4 * (size_t)e + F) : 1.0;
 }
 
+// deflation weight of the slot of a block entry (w: 4 e + F of the slot)
+__device__ __forceinline__ double entry_zw(const DevGeo& g, int4 en) { return g.zw ? __ldg(g.zw + en.w) : 1.0; }
+
 // [tau, p, 2/h] of face F of element e
 __device__ __forceinline__ const double* face_geo(const DevGeo& g, int e, int F) {
   return F < 2 ? g.cgeo + 3 * (e % g.mx) : g.rgeo + 3 * (e / g.mx);

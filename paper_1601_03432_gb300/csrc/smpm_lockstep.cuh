@@ -3,8 +3,8 @@
 // together, one step at a time, in ONE persistent cooperative launch, so that
 // every operator matrix (G_b, X_b, T_e, the coarse C^+) is read once per step
 // for all R columns and the five grid barriers of a step are shared.  Each
-// element product becomes a small dense GEMM: the M x M matrix times an
-// M x RC tile of columns.
+// element product becomes a small dense GEMM: the M x M matrix times a tile of
+// eight columns.
 //
 // Per column, everything of the single-column kernel is kept: its own basis,
 // Hessenberg column, FP64 Givens rotations, residual estimate, convergence,
@@ -20,9 +20,9 @@
 // base + rho * ds.  The basis lives in global memory (L2 / HBM): CTA rank's
 // slice of basis vector l, column rho at V + ((rank (m+1) + l) R + rho) ES;
 // w and w2 likewise (W + (rank 2R + rho) (ES+1), w2 at + R (ES+1)).
-// Element work items are (owned element, chunk of RC columns); warp w takes
-// items w, w + 8, ...; an item's tile of slot values lives in the warp's
-// shared scratch as X[i * RC + rho].
+// Element work items are (owned element, eight columns); a group of W warps
+// takes items grp, grp + ngrp, ...; an item's tiles live in the group's
+// shared scratch.
 #pragma once
 // Included inside the anonymous namespace of smpm_solver.cu, after smpm_gmres.cuh.
 
@@ -39,8 +39,14 @@ struct LockArgs {
   GmresArgs<S> a;  // geometry, ownership, matrices, team, barrier, err, precond, m, maxit, tol;
                    // rhs, x, t, y, vglob: column 0 (stride vs); c, chat: column 0 (stride ds);
                    // acc: (2m+1) R (m+3) FP64 accumulators (zero on entry)
-  int R;           // columns (a multiple of RC, <= kLockMaxCols)
-  int RC;          // columns per element work item (1, 2, 4 or 8)
+  int R;           // columns (<= kLockMaxCols)
+  int W_item, ngrp;  // warps per element work item (eight columns of an element), groups of that many warps
+  size_t wb_bytes;   // shared scratch of the groups
+  // packed matrices of the classes (smpm_digits.cuh) and the class of each
+  // block / element: G_b and X_b (4 per block class), T_e
+  const uint4 *Gd, *Xd, *Td;
+  const short *Ge, *Xe, *Te;
+  const int *bcls, *tcls;
   long long vs, ds;
   S* V;            // basis, G (m+1) R ES
   S* W;            // w, w2: G 2R (ES+1)
@@ -59,20 +65,43 @@ struct LockSmem {
   int* jc;                                                     // steps of the column in this cycle
   int* active;
   int* flags;  // [0]: any column active
-  S* wb;       // per-warp tiles: 4 M RC entries per warp
-  S* mats;     // resident matrices (a.mats_smem)
+  unsigned char* wb;  // group scratch (lock_group_bytes each)
 };
 
-__host__ __device__ inline size_t lock_tile_elems(int M, int RC) { return 4 * (size_t)M * RC; }
-
+// entries from one column of a staged tile to the next: 8 modulo 16, so the
+// lanes of a pack (eight columns, consecutive rows) spread over the banks
+__host__ __device__ constexpr int lock_ld(int len) { return (len + 7) / 16 * 16 + 8; }
+// scratch of a group: packed columns (of M rows, or of the four faces), the
+// tiles [p; q] and r1 of eight columns (a white item: contributions to c)
 template <typename S>
-inline size_t lock_smem_bytes(int m, int M, int n, int R, int RC, int nown_b, int nown_w, bool mats_smem) {
-  const size_t m3 = m + 3;
-  size_t dbl = 9 * m3 * R + 9 * (size_t)R;
-  size_t ints = 2 * (size_t)R + 4;
-  size_t sel = (size_t)(kGmresThreads / 32) * lock_tile_elems(M, RC) + 16;
-  if (mats_smem) sel += (size_t)nown_b * (2 * (size_t)M * M + 4 * (size_t)n * n) + (size_t)nown_w * M * M;
-  return dbl * sizeof(double) + ints * sizeof(int) + 16 + sel * sizeof(S) + 128;
+__host__ __device__ constexpr size_t lock_bf_bytes(int M, int n) {
+  const int a = digit_bwords<S>(M), b = 4 * digit_bwords<S>(n);
+  return sizeof(uint4) * (size_t)(a > b ? a : b);
+}
+template <typename S>
+__host__ __device__ constexpr size_t lock_group_bytes(int M, int n) {
+  const size_t black = 8 * sizeof(S) * (size_t)(lock_ld(2 * M) + lock_ld(M)), white = 8 * sizeof(double) * (size_t)lock_ld(M);
+  return lock_bf_bytes<S>(M, n) + (black > white ? black : white);
+}
+
+// shared memory beside the group scratch
+inline size_t lock_fixed_bytes(int m, int R) {
+  const size_t m3 = m + 3, dbl = 9 * m3 * R + 9 * (size_t)R, ints = 2 * (size_t)R + 4;
+  return dbl * sizeof(double) + ints * sizeof(int) + 16 + 128;
+}
+
+// Warps per item and groups for `items` items per CTA: every warp busy, as many
+// groups as `room` bytes of scratch hold.  Returns the scratch bytes (0: not
+// even one group fits).
+template <typename S>
+inline size_t lock_groups(int M, int n, long long items, size_t room, int* W, int* ngrp) {
+  const int warps = kGmresThreads / 32;
+  const size_t per = lock_group_bytes<S>(M, n);
+  int w = 1;
+  while (w < warps && (items * w * 2 <= warps || (warps / w) * per > room)) w *= 2;
+  *W = w;
+  *ngrp = warps / w;
+  return *ngrp * per <= room ? *ngrp * per : 0;
 }
 
 template <typename S>
@@ -95,35 +124,8 @@ __device__ LockSmem<S> lock_carve(const LockArgs<S>& A, unsigned char* raw) {
   s.jc = ip; ip += R;
   s.active = ip; ip += R;
   s.flags = ip; ip += 4;
-  S* q = reinterpret_cast<S*>((reinterpret_cast<size_t>(ip) + 15) & ~size_t(15));
-  s.wb = q;
-  q += (size_t)(blockDim.x / 32) * lock_tile_elems(A.a.g.M, A.RC);
-  q = reinterpret_cast<S*>((reinterpret_cast<size_t>(q) + 15) & ~size_t(15));
-  s.mats = q;
+  s.wb = reinterpret_cast<unsigned char*>((reinterpret_cast<size_t>(ip) + 15) & ~size_t(15));
   return s;
-}
-
-// matrices of owned block k / white element k: resident copies or global
-template <typename S>
-__device__ __forceinline__ const S* lk_G(const LockArgs<S>& A, const LockSmem<S>& s, int k, int ib) {
-  const int M = A.a.g.M, n = A.a.g.n;
-  return A.a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) : A.a.Gc + (size_t)ib * M * M;
-}
-template <typename S>
-__device__ __forceinline__ const S* lk_Tb(const LockArgs<S>& A, const LockSmem<S>& s, int k, int e) {
-  const int M = A.a.g.M, n = A.a.g.n;
-  return A.a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + M * M : A.a.Tc + (size_t)e * M * M;
-}
-template <typename S>
-__device__ __forceinline__ const S* lk_X(const LockArgs<S>& A, const LockSmem<S>& s, int k, int ib) {
-  const int M = A.a.g.M, n = A.a.g.n;
-  return A.a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + 2 * M * M : A.a.Xc + (size_t)ib * 4 * n * n;
-}
-template <typename S>
-__device__ __forceinline__ const S* lk_Tw(const LockArgs<S>& A, const LockSmem<S>& s, int k, int e) {
-  const int M = A.a.g.M, n = A.a.g.n;
-  return A.a.mats_smem ? s.mats + (size_t)A.a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M
-                       : A.a.Tc + (size_t)e * M * M;
 }
 
 template <typename S>
@@ -139,113 +141,75 @@ __device__ __forceinline__ S* lk_w2(const LockArgs<S>& A, int rho) {
   return A.W + ((size_t)team_rank(A.a) * 2 * A.R + A.R + rho) * (A.a.ES + 1);
 }
 
-// Z[r * RC + c] = sum_k Amat[k * M + r] X[k * RC + c] for r < M, c < RC by one
-// warp: lane l owns rows l, l+32, l+64, l+96 (M <= 128); Amat column-major in
-// shared or global memory; X, Z in the warp's shared scratch.  Every product
-// is a plain FMA into one of 4 RC independent accumulators.  Ends with
-// __syncwarp.
-template <typename S, int RC>
-__device__ __forceinline__ void warp_gemm(const S* Amat, const S* X, S* Z, int M, int lane) {
-  constexpr int U = sizeof(S) == 4 ? (RC >= 8 ? 4 : 8) : 2;  // columns of A per step (registers: 4 RC + 4 U)
-  S acc[4][RC];
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-#pragma unroll
-    for (int c = 0; c < RC; ++c) acc[j][c] = S(0);
-  const int nr = (M - lane + 31) / 32;
-  int k = 0;
-  for (; k + U <= M; k += U) {
-    S av[U][4];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) av[u][j] = j < nr ? Amat[(size_t)(k + u) * M + lane + 32 * j] : S(0);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-#pragma unroll
-      for (int c = 0; c < RC; ++c) {
-        const S xc = X[(k + u) * RC + c];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j][c] += av[u][j] * xc;
-      }
-    }
-  }
-  for (; k < M; ++k) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const S av = j < nr ? Amat[(size_t)k * M + lane + 32 * j] : S(0);
-#pragma unroll
-      for (int c = 0; c < RC; ++c) acc[j][c] += av * X[k * RC + c];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (j < nr)
-#pragma unroll
-      for (int c = 0; c < RC; ++c) Z[(lane + 32 * j) * RC + c] = acc[j][c];
-  __syncwarp();
+// The W warps of a group (named barrier of their own) work on one item.
+__device__ __forceinline__ void lk_group_sync(int grp, int W) {
+  if (W == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * W) : "memory");
 }
 
-template <typename S>
-__device__ __forceinline__ void warp_gemm_rc(int RC, const S* Amat, const S* X, S* Z, int M, int lane) {
-  switch (RC) {
-    case 1: warp_gemm<S, 1>(Amat, X, Z, M, lane); break;
-    case 2: warp_gemm<S, 2>(Amat, X, Z, M, lane); break;
-    case 4: warp_gemm<S, 4>(Amat, X, Z, M, lane); break;
-    default:  // FP32 only (lock_rc gives FP64 columns at most 4 per item)
-      if constexpr (sizeof(S) == 4) warp_gemm<S, 8>(Amat, X, Z, M, lane);
-      break;
-  }
-}
-
-// Black block solves for all columns: items (owned block k, chunk q of RC
-// columns).  Column rho's input is sc[rho] * (the basis slice when own, else
-// the global vector src).  t = M^-1 v on the block: r1 = p - X q,
-// a = G r1, z = T_e a, t = [a; q - z].
+// Black block solves for all columns: items (owned block k, eight columns), a
+// group of W warps each.  Column rho's input is sc[rho] * (the basis slice when
+// own, else the global vector src).  t = M^-1 v on the block: r1 = p - X q,
+// a = G r1, z = T_e a, t = [a; q - z]; the products run on the tensor cores
+// (smpm_digits.cuh), eight columns to a tile.
 template <typename S>
 __device__ void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int jbasis) {
   const GmresArgs<S>& a = A.a;
   const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), RC = A.RC, Q = A.R / A.RC;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  S* P = s.wb + (size_t)warp * lock_tile_elems(M, RC);  // [p; q]: 2M x RC
-  S* Rr = P + 2 * M * RC;                                // r1, later z: M x RC
-  S* Aa = Rr + M * RC;                                   // a: M x RC
-  for (int it = warp; it < a.nown_b * Q; it += nwarps) {
-    const int k = it / Q, c0 = (it % Q) * RC;
+  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), R = A.R, Q = (R + 7) / 8, W = A.W_item;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int ldp = lock_ld(2 * M), ldr = lock_ld(M), kt_n = digit_tiles(M), kf_n = digit_tiles(n);
+  unsigned char* base = s.wb + (size_t)grp * lock_group_bytes<S>(M, n);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  S* P = reinterpret_cast<S*>(base + lock_bf_bytes<S>(M, n));  // [p; q]: column c at c ldp
+  S* Rr = P + 8 * ldp;                                         // r1, then a: column c at c ldr
+  for (int it = grp; it < a.nown_b * Q; it += A.ngrp) {
+    const int k = it / Q, c0 = (it % Q) * 8, nc = min(8, R - c0);
     const int ib = rank + k * G;
     if (ib >= a.nblack) continue;
-    const int e = a.black[ib];
-    for (int idx = lane; idx < 2 * M * RC; idx += 32) {
+    const int e = a.black[ib], cb = A.bcls[ib], ct = A.tcls[e];
+    for (int idx = part * 32 + lane; idx < 2 * M * 8; idx += 32 * W) {
       const int c = idx / (2 * M), i = idx % (2 * M), rho = c0 + c;
       S v = S(0);
-      if (jbasis >= 0) {
-        v = (S)(sc[rho] * (double)lk_basis(A, jbasis, rho)[k * 2 * M + i]);
-      } else {
-        const long long sl = block_slot(g, e, i);
-        if (sl >= 0) v = (S)(sc[rho] * (double)ldcg(src + rho * A.vs + sl));
+      if (c < nc) {
+        if (jbasis >= 0) {
+          v = (S)(sc[rho] * (double)lk_basis(A, jbasis, rho)[k * 2 * M + i]);
+        } else {
+          const int sl = block_entry(a, ib, i).x;
+          if (sl >= 0) v = (S)(sc[rho] * (double)ldcg(src + rho * A.vs + sl));
+        }
       }
-      P[i * RC + c] = v;
+      P[c * ldp + i] = v;
     }
-    __syncwarp();
-    const S* X = lk_X(A, s, k, ib);
-    for (int idx = lane; idx < M * RC; idx += 32) {
-      const int i = idx / RC, c = idx % RC, F = i / n, t = i % n;
-      const S* xf = X + (size_t)F * n * n;
-      const S* qf = P + (size_t)(M + F * n) * RC + c;
-      S acc = 0;
-      for (int cc = 0; cc < n; ++cc) acc += xf[cc * n + t] * qf[cc * RC];
-      Rr[idx] = P[idx] - acc;
+    lk_group_sync(grp, W);
+    for (int F = part; F < 4; F += W) {  // r1 = p - X q, face by face
+      uint4* Bq = Bf + F * digit_bwords<S>(n);
+      const S* q = P + M + F * n;
+      const int E = pack_cols<S>(Bq, n, lane, [&](int kk, int c) { return q[c * ldp + kk]; });
+      __syncwarp();
+      for (int mt = 0; mt < kf_n; ++mt)
+        digits_tile8<S>(A.Xd + ((size_t)cb * 4 + F) * digit_words<S>(n, n), A.Xe + ((size_t)cb * 4 + F) * n, Bq, n, kf_n,
+                        mt, lane, E, [&](int row, int c, S v) { Rr[c * ldr + F * n + row] = P[c * ldp + F * n + row] - v; });
     }
-    __syncwarp();
-    warp_gemm_rc(RC, lk_G(A, s, k, ib), Rr, Aa, M, lane);
-    warp_gemm_rc(RC, lk_Tb(A, s, k, e), Aa, Rr, M, lane);
-    for (int idx = lane; idx < 2 * M * RC; idx += 32) {
-      const int c = idx / (2 * M), i = idx % (2 * M), rho = c0 + c;
-      const long long sl = block_slot(g, e, i);
-      if (sl >= 0) a.t[rho * A.vs + sl] = i < M ? Aa[i * RC + c] : (S)(P[i * RC + c] - Rr[(i - M) * RC + c]);
-    }
-    __syncwarp();
+    lk_group_sync(grp, W);
+    int E = pack_cols<S>(Bf, M, lane, [&](int kk, int c) { return Rr[c * ldr + kk]; }, part, W);
+    lk_group_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W)  // a = G r1
+      digits_tile8<S>(A.Gd + (size_t)cb * digit_words<S>(M, M), A.Ge + (size_t)cb * M, Bf, M, kt_n, mt, lane, E,
+                      [&](int row, int c, S v) {
+                        Rr[c * ldr + row] = v;
+                        if (c < nc) a.t[(c0 + c) * A.vs + (size_t)e * M + row] = v;
+                      });
+    lk_group_sync(grp, W);
+    E = pack_cols<S>(Bf, M, lane, [&](int kk, int c) { return Rr[c * ldr + kk]; }, part, W);
+    lk_group_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W)  // z = T_e a, t = q - z on the facing slots
+      digits_tile8<S>(A.Td + (size_t)ct * digit_words<S>(M, M), A.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E,
+                      [&](int row, int c, S z) {
+                        const int sl = block_entry(a, ib, M + row).x;
+                        if (c < nc && sl >= 0) a.t[(c0 + c) * A.vs + sl] = P[c * ldp + M + row] - z;
+                      });
+    lk_group_sync(grp, W);
   }
   __syncthreads();
 }
@@ -256,46 +220,49 @@ template <typename S>
 __device__ void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v, const double* sc, bool with_c) {
   const GmresArgs<S>& a = A.a;
   const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), RC = A.RC, Q = A.R / A.RC;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  S* P = s.wb + (size_t)warp * lock_tile_elems(M, RC);  // t on e's slots: M x RC
-  S* Z = P + M * RC;                                     // T_e t: M x RC
-  double* ci = reinterpret_cast<double*>(Z + M * RC + (sizeof(S) == 4 ? (M * RC) & 1 : 0));  // M x RC doubles
-  for (int it = warp; it < a.nown_w * Q; it += nwarps) {
-    const int k = it / Q, c0 = (it % Q) * RC;
+  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), R = A.R, Q = (R + 7) / 8, W = A.W_item;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int kt_n = digit_tiles(M), ldc = lock_ld(M);
+  unsigned char* base = s.wb + (size_t)grp * lock_group_bytes<S>(M, n);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  double* ci = reinterpret_cast<double*>(base + lock_bf_bytes<S>(M, n));  // contributions to c: column c at c ldc
+  for (int it = grp; it < a.nown_w * Q; it += A.ngrp) {
+    const int k = it / Q, c0 = (it % Q) * 8, nc = min(8, R - c0);
     const int iw = rank + k * G;
     if (iw >= a.nwhite) continue;
-    const int e = a.white[iw];
-    for (int idx = lane; idx < M * RC; idx += 32) {
-      const int c = idx / M, i = idx % M;
-      P[i * RC + c] = ldcg(a.t + (c0 + c) * A.vs + (size_t)e * M + i);
-    }
-    __syncwarp();
-    warp_gemm_rc(RC, lk_Tw(A, s, k, e), P, Z, M, lane);
-    for (int idx = lane; idx < M * RC; idx += 32) {
-      const int c = idx / M, i = idx % M, rho = c0 + c;
-      const int F = i / n, tt = i % n, e2 = dev_neighbour(g, e, F);
-      const S vo = (S)(sc[rho] * (double)ldcg(v + rho * A.vs + (size_t)e * M + i));
-      a.y[rho * A.vs + (size_t)e * M + i] = vo;
-      double c1 = 0;
-      if (e2 >= 0) {
-        const size_t sl = (size_t)e2 * M + (F ^ 1) * n + tt;
-        const S ys = ldcg(a.t + rho * A.vs + sl) + Z[i * RC + c];
-        a.y[rho * A.vs + sl] = ys;
-        c1 = g.zw ? dev_zw(g, e, F) * (double)vo + dev_zw(g, e2, F ^ 1) * (double)ys : (double)vo + (double)ys;
-      }
-      ci[c * M + i] = c1;
-    }
-    __syncwarp();
-    if (with_c && lane < 4 * RC) {  // face F of column c summed by lane c * 4 + F
+    const int e = a.white[iw], ct = A.tcls[e];
+    const S* te = a.t + (size_t)e * M;
+    const int E = pack_cols<S>(
+        Bf, M, lane, [&](int kk, int c) { return c < nc ? ldcg(te + (c0 + c) * A.vs + kk) : S(0); }, part, W);
+    lk_group_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W)
+      digits_tile8<S>(A.Td + (size_t)ct * digit_words<S>(M, M), A.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E,
+                      [&](int row, int c, S z) {
+                        if (c >= nc) return;
+                        const int rho = c0 + c, F = row / n, tt = row - F * n, e2 = dev_neighbour(g, e, F);
+                        const size_t own = rho * A.vs + (size_t)e * M + row;
+                        const S vo = (S)(sc[rho] * (double)ldcg(v + own));
+                        a.y[own] = vo;
+                        double c1 = 0;
+                        if (e2 >= 0) {
+                          const size_t sl = rho * A.vs + (size_t)e2 * M + (F ^ 1) * n + tt;
+                          const S ys = ldcg(a.t + sl) + z;
+                          a.y[sl] = ys;
+                          c1 = g.zw ? dev_zw(g, e, F) * (double)vo + dev_zw(g, e2, F ^ 1) * (double)ys
+                                    : (double)vo + (double)ys;
+                        }
+                        ci[c * ldc + row] = c1;
+                      });
+    lk_group_sync(grp, W);
+    if (with_c && part == 0 && lane < 4 * nc) {  // face F of column c summed by lane c * 4 + F
       const int c = lane / 4, F = lane % 4, j = dev_iface(g, e, F);
       if (j >= 0) {
         double sum = 0;
-        for (int tt = 0; tt < n; ++tt) sum += ci[c * M + F * n + tt];
+        for (int tt = 0; tt < n; ++tt) sum += ci[c * ldc + F * n + tt];
         a.c[(c0 + c) * A.ds + j] = sum;
       }
     }
-    __syncwarp();
+    lk_group_sync(grp, W);
   }
   __syncthreads();
 }
@@ -601,7 +568,7 @@ __host__ __device__ inline int strips_stage(const CoarseStrips<T>& k, int G) {
 // c_hat = C^+ c for all columns, complete after its last barrier.
 template <typename S>
 __device__ bool lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s, unsigned& epoch) {
-  const int room = (int)((size_t)(blockDim.x / 32) * lock_tile_elems(A.a.g.M, A.RC));  // the idle warp tiles
+  const int room = (int)(A.wb_bytes / sizeof(S));  // the groups' scratch is idle here
   if (A.a.use_strips) {
     const int nc = room / strips_stage(A.a.strips, A.a.G);
     if (nc >= 8 && A.R > 4) return lk_coarse_strips_nc<S, 8>(A, s.wb, epoch);
@@ -747,7 +714,7 @@ __device__ void lk_combo_pass(const LockArgs<S>& A, bool from_w2, const double* 
         lk_w2(A, rho_[q])[i_[q]] = val;
       }
       if (to_vg) {
-        const long long sl = entry_slot(a, i_[q]);
+        const int sl = entry_slot(a, i_[q]);
         if (sl >= 0) a.vglob[rho_[q] * A.vs + sl] = val;
       }
     }
@@ -774,32 +741,10 @@ template <typename S>
 __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smraw, unsigned& epoch) {
   const LockSmem<S> s = lock_carve(A, smraw);
   const GmresArgs<S>& a = A.a;
-  const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, m = a.m, m3 = m + 3, R = A.R;
+  const int m = a.m, m3 = m + 3, R = A.R;
   const int ES = a.ES, G = a.G, rank = team_rank(a);
   int trace_n = 0;
 
-  // resident copies of the owned matrices
-  if (a.mats_smem) {
-    for (int k = 0; k < a.nown_b; ++k) {
-      const int ib = rank + k * G;
-      if (ib >= a.nblack) break;
-      const int e = a.black[ib];
-      S* dst = s.mats + (size_t)k * (2 * M * M + 4 * n * n);
-      for (int i = threadIdx.x; i < M * M; i += blockDim.x) {
-        dst[i] = a.Gc[(size_t)ib * M * M + i];
-        dst[M * M + i] = a.Tc[(size_t)e * M * M + i];
-      }
-      for (int i = threadIdx.x; i < 4 * n * n; i += blockDim.x) dst[2 * M * M + i] = a.Xc[(size_t)ib * 4 * n * n + i];
-    }
-    for (int k = 0; k < a.nown_w; ++k) {
-      const int iw = rank + k * G;
-      if (iw >= a.nwhite) break;
-      const int e = a.white[iw];
-      S* dst = s.mats + (size_t)a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M;
-      for (int i = threadIdx.x; i < M * M; i += blockDim.x) dst[i] = a.Tc[(size_t)e * M * M + i];
-    }
-  }
   // misc per column: 0 ||w||^2, 1 ||w2||^2, 2 residual estimate, 3 state (0 running,
   // 1 converged, 2 breakdown, 3 NaN), 5 Arnoldi steps (all cycles), 6 beta0, 7 tol * beta0
   for (int c = threadIdx.x; c < R; c += blockDim.x) {
@@ -824,12 +769,13 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       S* v0 = lk_basis(A, 0, rho);
       double nn = 0;
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-        const long long sl = entry_slot(a, i);
+        const int4 en = owned_entry(a, i);
+        const int sl = en.x;
         S rv = 0;
         if (sl >= 0 && s.active[rho]) {
           double r = (double)ldcg(a.rhs + rho * A.vs + sl);
           if (cycle > 0)
-            r -= deflate_slot_cg(g, a.y + rho * A.vs, a.precond == 2 ? a.chat + rho * A.ds : nullptr, a.Rs, sl);
+            r -= deflate_entry(a, a.y + rho * A.vs, a.precond == 2 ? a.chat + rho * A.ds : nullptr, en);
           rv = (S)r;
         }
         if (sl >= 0) a.vglob[rho * A.vs + sl] = rv;
@@ -880,22 +826,35 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       __syncthreads();
       GM_TRACE(37);
       if (!lk_apply(A, s, a.vglob, s.scl, j, epoch, trace_n)) return false;
-      // ---- D: w = y - S Z chat on owned entries; V^T w, ||w||^2 (four
-      // (column, entry) pairs per thread at a time, their loads interleaved)
-      for (int p0 = threadIdx.x; p0 < R * ES; p0 += 4 * blockDim.x) {
-        double wv[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int p = p0 + q * blockDim.x, rho = p / ES, i = p % ES;
-          const long long sl = p < R * ES ? entry_slot(a, i) : -1;
-          wv[q] = sl >= 0 ? deflate_slot_cg(g, a.y + rho * A.vs, a.precond == 2 ? a.chat + rho * A.ds : nullptr,
-                                            a.Rs, sl)
-                          : 0.0;
+      // ---- D: w = y - S Z chat on owned entries; V^T w, ||w||^2.  A thread
+      // takes an entry through the columns, four at a time: the entry's
+      // indices and coefficients are read once
+      for (int i = threadIdx.x; i < ES; i += blockDim.x) {
+        const int4 en = owned_entry(a, i);
+        if (en.z < 0 || a.precond != 2) {
+          for (int c = 0; c < R; ++c) lk_w(A, c)[i] = en.z < 0 ? S(0) : ldcg(a.y + c * A.vs + en.x);
+          continue;
         }
+        const int4 J = __ldg(a.if4 + en.y);
+        const double2* Rp = reinterpret_cast<const double2*>(a.Rd + 4 * (size_t)en.x);
+        const double2 r0 = __ldg(Rp), r1 = __ldg(Rp + 1);
+        for (int c0 = 0; c0 < R; c0 += 4) {
+          double yv[4], h[4][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int p = p0 + q * blockDim.x;
-          if (p < R * ES) lk_w(A, p / ES)[p % ES] = (S)wv[q];
+          for (int q = 0; q < 4; ++q) {
+            const int c = min(c0 + q, R - 1);
+            const double* ch = a.chat + c * A.ds;
+            yv[q] = (double)ldcg(a.y + c * A.vs + en.x);
+            h[q][0] = __ldcg(ch + J.x);
+            h[q][1] = __ldcg(ch + J.y);
+            h[q][2] = __ldcg(ch + J.z);
+            h[q][3] = __ldcg(ch + J.w);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (c0 + q < R)
+              lk_w(A, c0 + q)[i] =
+                  (S)((yv[q] - (r0.x * h[q][0] + r0.y * h[q][1])) - (r1.x * h[q][2] + r1.y * h[q][3]));
         }
       }
       __syncthreads();
@@ -1029,7 +988,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       const int jj = s.jc[rho];
       if (jj == 0) continue;
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-        const long long sl = entry_slot(a, i);
+        const int sl = entry_slot(a, i);
         if (sl < 0) continue;
         S* xp = a.x + rho * A.vs + sl;
         *xp = (S)lk_combo(A, (double)ldcg(xp), s.hs1 + rho * m3, jj, rho, i);

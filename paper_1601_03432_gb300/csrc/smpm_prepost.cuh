@@ -189,30 +189,19 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
   // ---- P4: owner entries: project b_S, rhs = P b_S
   double bsn = 0, rgn = 0;
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-    const long long sl = entry_slot(a, i);
+    const int4 en = owned_entry(a, i);
+    const int sl = en.x;
     if (sl < 0) continue;
-    const int e = (int)(sl / M), F = (int)(sl % M) / n;
-    if (dev_neighbour(g, e, F) < 0) {
+    if (en.z < 0) {  // slot on the physical boundary
       P.bS[sl] = 0.0;
       P.rg[sl] = 0.0;
       if (P.rg32) P.rg32[sl] = 0.f;
       continue;
     }
-    double v = __ldcg(P.bS + sl) - beta * P.uS[sl];
+    const double v = __ldcg(P.bS + sl) - beta * P.uS[sl];
     P.bS[sl] = v;
     bsn += v * v;
-    double r = v;
-    if (a.precond == 2) {
-      // - (S Z c_hat_b) at the slot (pull form), as in the GMRES deflation
-      const int ii = (int)(sl % M), t = ii % n, e2 = dev_neighbour(g, e, F);
-      double acc = dev_zw(g, e, F) * __ldcg(a.chat + dev_iface(g, e, F));
-      const double* R = a.Rs + ((size_t)e2 * M + (F ^ 1) * n + t) * 4;
-      for (int G2 = 0; G2 < 4; ++G2) {
-        const int jj = dev_iface(g, e2, G2);
-        if (jj >= 0) acc += __ldg(R + G2) * __ldcg(a.chat + jj);
-      }
-      r -= acc;
-    }
+    const double r = deflate_value(a, v, a.precond == 2 ? a.chat : nullptr, en);  // b_S - S Z c_hat_b
     P.rg[sl] = r;
     if (P.rg32) P.rg32[sl] = (float)r;
     rgn += r * r;
@@ -240,7 +229,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
     // x_S given (iterative refinement)
   } else if (a.precond == 0) {
     for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-      const long long sl = entry_slot(a, i);
+      const int sl = entry_slot(a, i);
       if (sl >= 0) P.xs[sl] = __ldcg(a.x + sl);
     }
   } else {
@@ -249,7 +238,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
       if (ib >= a.nblack) break;
       const int e = a.black[ib];
       for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) {
-        const long long sl = block_slot(g, e, i);
+        const int sl = block_entry(a, ib, i).x;
         s.w[i] = sl >= 0 ? __ldcg(a.x + sl) : 0.0;
       }
       __syncthreads();
@@ -260,17 +249,16 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
       if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
       GM_TRACE(62);
       for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-        const long long sl = entry_slot(a, i);
+        const int sl = entry_slot(a, i);
         if (sl >= 0) P.xs[sl] = __ldcg(a.t + sl);
       }
     } else {
       // white step and coarse solve of y = S t, then x_S = t - Z (c_hat - c_hat_b)
       if (!apply_op(a, s, a.x, 1.0, true, trace_n, epoch)) return false;
       for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-        const long long sl = entry_slot(a, i);
-        if (sl < 0) continue;
-        const int e = (int)(sl / M), F = (int)(sl % M) / n, j = dev_iface(g, e, F);
-        P.xs[sl] = j < 0 ? 0.0 : __ldcg(a.t + sl) - dev_zw(g, e, F) * (__ldcg(a.chat + j) - P.chatb[j]);
+        const int4 en = owned_entry(a, i);
+        if (en.x < 0) continue;
+        P.xs[en.x] = en.z < 0 ? 0.0 : __ldcg(a.t + en.x) - entry_zw(g, en) * (__ldcg(a.chat + en.z) - P.chatb[en.z]);
       }
     }
   }
@@ -319,7 +307,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
       pm += (P.adjoint ? P.uL[e * nn + q] : P.what[e * nn + q]) * U[q];
     }
     // (S x_S) on the slots facing e: x_S + T_e x_S,e
-    gemv_split(a.Tc + (size_t)e * M * M, M, s.p, s.z, M, M, s.red);
+    gemv_split(a.Tc + (size_t)__ldg(a.tr + e) * M * M, M, s.p, s.z, M, M, s.red);
     for (int i = threadIdx.x; i < M; i += blockDim.x) {
       const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
       if (e2 < 0) continue;

@@ -18,7 +18,6 @@
 struct alignas(16) RefineArgs {  // 16-byte multiple: staged with 16-byte copies in batched solves
   GmresArgs<float> ga;   // FP32 operator and vectors: x = inner y, t, y, c, chat, rhs (next inner rhs)
   const double* Tc64;    // nel * M*M, FP64 T_e (column-major)
-  const double* Rs64;    // FP64 row sums for the deflation of r
   double* xS;            // kp, FP64 Schur iterate
   const double* bS;      // kp, projected b_S
   double* r;             // kp, FP64 residual
@@ -54,11 +53,11 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
   if (!apply_op(a, s, a.x, 1.0, true, trace_n, epoch)) return -1;
   // ---- R4: x_S += t - Z (c_hat - c_hat_r); y <- 0 for the next inner solve
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-    const long long sl = entry_slot(a, i);
-    if (sl < 0) continue;
-    const int e = (int)(sl / M), F = (int)(sl % M) / n, j = dev_iface(g, e, F);
-    if (j >= 0) R.xS[sl] += (double)__ldcg(a.t + sl) - dev_zw(g, e, F) * (__ldcg(a.chat + j) - R.chat_r[j]);
-    a.x[sl] = 0.f;
+    const int4 en = owned_entry(a, i);
+    if (en.x < 0) continue;
+    if (en.z >= 0)
+      R.xS[en.x] += (double)__ldcg(a.t + en.x) - entry_zw(g, en) * (__ldcg(a.chat + en.z) - R.chat_r[en.z]);
+    a.x[en.x] = 0.f;
   }
   if (!grid_sync(a.bar, a.err, epoch, a.G)) return -1;
   // ---- R5: r = b_S - S x_S (FP64), ||r||^2, Z^T r
@@ -70,7 +69,7 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
     for (long long e = rank + (long long)warp * G; e < g.nel; e += (long long)nwarps * G) {
       for (int i = lane; i < M; i += 32) pw[i] = __ldcg(R.xS + e * M + i);
       __syncwarp();
-      warp_gemv(R.Tc64 + (size_t)e * M * M, pw, zw, M, lane);
+      warp_gemv(R.Tc64 + (size_t)__ldg(a.tr + e) * M * M, pw, zw, M, lane);
       for (int i = lane; i < M; i += 32) {  // pw is free again: it takes the residual entries
         const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
         double rr = 0;
@@ -96,7 +95,7 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
   for (long long e = rank; e < (a.warp_elems ? 0 : g.nel); e += G) {
     for (int i = threadIdx.x; i < M; i += blockDim.x) p64[i] = __ldcg(R.xS + e * M + i);
     __syncthreads();
-    gemv_split(R.Tc64 + (size_t)e * M * M, M, p64, z64, M, M, red64);
+    gemv_split(R.Tc64 + (size_t)__ldg(a.tr + e) * M * M, M, p64, z64, M, M, red64);
     for (int i = threadIdx.x; i < M; i += blockDim.x) {
       const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
       double rr = 0;
@@ -138,9 +137,8 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
   }
   // ---- R7: next inner right-hand side P r (FP32); Z^T r back to zero
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
-    const long long sl = entry_slot(a, i);
-    if (sl < 0) continue;
-    R.rhs32[sl] = (float)deflate_slot_cg(g, (const double*)R.r, R.chat_r, R.Rs64, sl);
+    const int4 en = owned_entry(a, i);
+    if (en.x >= 0) R.rhs32[en.x] = (float)deflate_entry(a, (const double*)R.r, R.chat_r, en);
   }
   for (long long j = (long long)rank * blockDim.x + threadIdx.x; j < g.d; j += (long long)G * blockDim.x)
     R.cr[j] = 0.0;

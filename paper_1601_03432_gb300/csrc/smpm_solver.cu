@@ -46,6 +46,7 @@
 #include <vector>
 
 #include "smpm_device.cuh"
+#include "smpm_digits.cuh"
 
 namespace {
 
@@ -281,9 +282,10 @@ __global__ void k_coarse(const double* __restrict__ H, const double* __restrict_
   if (lane == 0) out[row] = acc;
 }
 
-// w = y - (S Z) chat on one slot (pull form); chat == nullptr gives w = y.
-template <typename S>
-__device__ __forceinline__ double deflate_slot(const DevGeo& g, const S* __restrict__ y, const double* __restrict__ chat,
+// w = y - (S Z) chat on one slot (pull form); chat == nullptr gives w = y.  CG:
+// chat is written by other CTAs of the same kernel (read from L2).
+template <typename S, bool CG = false>
+__device__ __forceinline__ double deflate_slot(const DevGeo& g, const S* __restrict__ y, const double* chat,
                                                const S* __restrict__ Rs, long long s) {
   const int M = g.M, n = g.n;
   int e = (int)(s / M), i = (int)(s % M), F = i / n, t = i % n;
@@ -291,12 +293,13 @@ __device__ __forceinline__ double deflate_slot(const DevGeo& g, const S* __restr
   if (e2 < 0) return 0.0;
   double ys = (double)y[s];
   if (!chat) return ys;
-  double acc = dev_zw(g, e, F) * chat[dev_iface(g, e, F)];
+  auto ch = [&](int j) { return CG ? __ldcg(chat + j) : __ldg(chat + j); };
+  double acc = dev_zw(g, e, F) * ch(dev_iface(g, e, F));
   const S* R = Rs + ((size_t)e2 * M + (F ^ 1) * n + t) * 4;
 #pragma unroll
   for (int G = 0; G < 4; ++G) {
     int jj = dev_iface(g, e2, G);
-    if (jj >= 0) acc += (double)R[G] * chat[jj];
+    if (jj >= 0) acc += (double)__ldg(R + G) * ch(jj);
   }
   return ys - acc;
 }
@@ -791,101 +794,43 @@ cudaError_t launch_schur_warp(const ElemMeta<S>* tab, long long nelem, const S* 
 // Element-class-shared apply y = S v.  On an axis-aligned uniform grid T_e
 // depends only on which of the element's four faces are interfaces (at most
 // 9 classes: interior, 4 edges, 4 corners), so y = v + scatter(T_c X_c) with
-// X_c the M x n_c matrix of the own slots of all elements of class c: a real
-// dense contraction.  One CTA per tile of up to kClassTile elements of one
-// class: thread 0 stages T_c and the tile's element slot vectors in shared
-// memory with 1-D bulk copies (all in flight at once, one mbarrier; plain
-// loads when v is not 16-byte aligned), thread (rg, eg) accumulates rows
-// rg + 16 i (i < ceil(M/16)) of elements eg + 16 j (j < 4) in registers, and
-// the products go straight to the neighbours' facing slots.  HBM traffic is
-// the vectors only (plus the class matrices once).  A copy that does not
-// complete within the bounded wait leaves the tile's outputs NaN.
-constexpr int kClassTile = 64;  // elements per CTA tile
-inline size_t class_smem(int M, size_t elem) {
-  return 16 + ((size_t)M * M + (size_t)(M + 16 / elem) * kClassTile) * elem;
+// X_c the M x n_c matrix of the own slots of all elements of class c: a dense
+// contraction on the tensor cores (smpm_digits.cuh), with the vectors as the
+// only traffic from HBM.  One CTA per tile of up to kClassTile elements of one
+// class, one warp per eight of them: the warp cuts their slot vectors into
+// digits (in its shared scratch) and walks the row tiles of T_c, whose packed
+// digits all warps of the CTA read from L1.
+constexpr int kClassTile = 32, kClassThreads = 32 * (kClassTile / 8);
+template <typename S>
+inline size_t class_smem(int M) {
+  return (size_t)(kClassTile / 8) * digit_bwords<S>(M) * sizeof(uint4);
 }
 
 template <typename S>
-__global__ void __launch_bounds__(256) k_schur_class(DevGeo g, const S* __restrict__ Tcls, const int* __restrict__ tiles,
-                                                     const int* __restrict__ elems, const S* __restrict__ v, S* y,
-                                                     int bulk) {
+__global__ void __launch_bounds__(kClassThreads) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
+                                                               const short* __restrict__ Texp,
+                                                               const int* __restrict__ tiles,
+                                                               const int* __restrict__ elems, const S* v, S* y) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const int M = g.M, n = g.n;
-  unsigned long long* bar = reinterpret_cast<unsigned long long*>(raw);
-  S* Ts = reinterpret_cast<S*>(raw + 16);  // M x M column-major
-  const int XS = M + 16 / (int)sizeof(S);  // element stride of Xs: 16 bytes of padding (banks, bulk alignment)
-  S* Xs = Ts + (size_t)M * M;              // element-major: Xs[t * XS + k]
+  const int M = g.M, n = g.n, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cls = tiles[3 * blockIdx.x], start = tiles[3 * blockIdx.x + 1], cnt = tiles[3 * blockIdx.x + 2];
-  const S* T = Tcls + (size_t)cls * M * M;
-  __shared__ int ok;
-  if (bulk) {
-    // warp 0 issues the copies: lane 0 arms the mbarrier with the tile's
-    // byte count, then every lane copies its own elements (their indices are
-    // loaded in parallel, not one after another)
-    if (threadIdx.x < 32) {
-      const unsigned mm = (unsigned)(M * M * sizeof(S)), col = (unsigned)(M * sizeof(S));
-      if (threadIdx.x == 0) {
-        mbar_init(bar);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                     "r"(mm + (unsigned)cnt * col)
-                     : "memory");
-        bulk_g2s(Ts, T, mm, bar);
-      }
-      __syncwarp();
-      for (int t = threadIdx.x; t < cnt; t += 32)
-        bulk_g2s(Xs + (size_t)t * XS, v + (size_t)__ldg(elems + start + t) * M, col, bar);
-      if (threadIdx.x == 0) ok = mbar_wait(bar, 0) ? 1 : 0;
-    }
-    __syncthreads();
-  } else {
-    for (int i = threadIdx.x; i < M * M; i += blockDim.x) Ts[i] = T[i];
-    for (int i = threadIdx.x; i < M * cnt; i += blockDim.x)
-      Xs[(size_t)(i / M) * XS + i % M] = v[(size_t)elems[start + i / M] * M + i % M];
-    if (threadIdx.x == 0) ok = 1;
-    __syncthreads();
-  }
-  const int rg = threadIdx.x & 15, eg = threadIdx.x >> 4;  // 16 x 16 thread grid
-  constexpr int RT = 8;                                    // rows per thread (M <= 128)
-  S acc[RT][4];
-#pragma unroll
-  for (int i = 0; i < RT; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = S(0);
-  const int nr = (M - rg + 15) / 16;
-  const S* xb = Xs + (size_t)eg * XS;
-  for (int k = 0; k < M; ++k) {
-    S b[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) b[j] = xb[(size_t)16 * j * XS + k];
-#pragma unroll
-    for (int i = 0; i < RT; ++i) {
-      if (i < nr) {
-        const S a = Ts[(size_t)k * M + rg + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += a * b[j];
-      }
-    }
-  }
-  const S bad = ok ? S(0) : S(nan(""));
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int t = eg + 16 * j;
-    if (t >= cnt) continue;
-    const int e = elems[start + t];
-#pragma unroll
-    for (int i = 0; i < RT; ++i) {
-      const int r = rg + 16 * i;
-      if (i >= nr) continue;
-      const int F = r / n, tt = r % n, e2 = dev_neighbour(g, e, F);
-      if (e2 >= 0) {
-        const size_t sl = (size_t)e2 * M + (F ^ 1) * n + tt;
-        y[sl] = v[sl] + acc[i][j] + bad;
-      } else {
-        y[(size_t)e * M + r] = Xs[(size_t)t * XS + r] + bad;
-      }
-    }
-  }
+  if (warp * 8 >= cnt) return;
+  uint4* Bf = reinterpret_cast<uint4*>(raw) + (size_t)warp * digit_bwords<S>(M);
+  const int left = cnt - warp * 8;  // elements of this warp (of 8)
+  const int* el = elems + start + warp * 8;
+  const int mine = __ldg(el + min(lane >> 2, left - 1));
+  const S* vm = v + (size_t)mine * M;
+  const bool live = (lane >> 2) < left;
+  const int E = pack_cols<S>(Bf, M, lane, [&](int k, int) { return live ? __ldg(vm + k) : S(0); });
+  const uint4* A = Tdig + (size_t)cls * digit_words<S>(M, M);
+  const short* er = Texp + (size_t)cls * M;
+  for (int mt = 0; mt < kt_n; ++mt)
+    digits_tile8<S>(A, er, Bf, M, kt_n, mt, lane, E, [&](int row, int col, S z) {
+      if (col >= left) return;
+      const int e = __ldg(el + col), F = row / n, tt = row - F * n, e2 = dev_neighbour(g, e, F);
+      const size_t sl = e2 >= 0 ? (size_t)e2 * M + (F ^ 1) * n + tt : (size_t)e * M + row;
+      y[sl] = e2 >= 0 ? v[sl] + z : v[sl];
+    });
 }
 
 template <typename S>
@@ -909,12 +854,22 @@ struct smpm_handle_s {
   bool factored = false;
   bool op_factored = false;  // operator-only factor step (SMPM_FLAG_OPERATOR_ONLY): S can be applied
   // element classes (face-type masks) for the class-shared apply
-  int ncls = 0, ntiles = 0, cls_ok = 0;  // cls_ok: the kernel's shared-memory limit is set
+  int ncls = 0, ntiles = 0, cls_ok = 0;  // cls_ok: packed, and the kernel's shared-memory limit is set
   int apply_kind = 0;                     // kernel of smpm_apply_schur(32): SMPM_APPLY_*
-  double* dTcls = nullptr;   // ncls * M*M, column-major
-  float* dTcls32 = nullptr;
+  // packed digits (smpm_digits.cuh) of one T_e per class, G_b and the four X_F
+  // per block class, their row exponents, and the class of each element / block
+  struct DigitSet {
+    uint4 *T = nullptr, *G = nullptr, *X = nullptr;
+    short *Te = nullptr, *Ge = nullptr, *Xe = nullptr;
+  } dig, dig32;
+  int *dtcls = nullptr, *dbcls = nullptr;
   int* dtiles = nullptr;     // ntiles * (class, first, count) into dclsel
   int* dclsel = nullptr;     // nel: elements sorted by class
+  // tables of the solve kernels (GmresArgs): class representatives, block
+  // entries, interfaces per element, S Z per slot (forward, adjoint)
+  int *dtr = nullptr, *dgr = nullptr;
+  int4 *dbt = nullptr, *dif4 = nullptr;
+  double *dRd = nullptr, *dRda = nullptr;
   // C^+ by strips (StripFactors) on the device, forward and adjoint, and the
   // scratch of its phases (2 p mx + 1 doubles)
   CoarseStrips<double> st{}, sta{};
@@ -949,7 +904,7 @@ struct smpm_handle_s {
   double* wvown = nullptr;
   double* wacc = nullptr;
   // mixed precision: FP32 operator copies and work vectors, FP64 residual
-  float *dT32 = nullptr, *dG32 = nullptr, *dX32 = nullptr, *dRs32 = nullptr;
+  float *dT32 = nullptr, *dG32 = nullptr, *dX32 = nullptr;
   float* dH32 = nullptr;  // FP32 copy of the coarse inverse, for the FP32 inner solves
   float *wx32 = nullptr, *wt32 = nullptr, *wy32 = nullptr, *wV32 = nullptr, *wrg32 = nullptr, *wvown32 = nullptr;
   double *wr = nullptr, *wcr = nullptr, *wrn = nullptr;
@@ -960,7 +915,7 @@ struct smpm_handle_s {
   } gm32;
   double *wacc8 = nullptr, *wxs = nullptr, *dZtuS = nullptr;
   // transposed system for the adjoint solve (SMPM_FLAG_ADJOINT)
-  double *dTa = nullptr, *dRsa = nullptr, *dGa = nullptr, *dXa = nullptr, *dHa = nullptr;
+  double *dTa = nullptr, *dGa = nullptr, *dXa = nullptr, *dHa = nullptr;
   // element tables of the register-streamed apply (k_schur_warp_batch / k_schur_warpk)
   ElemMeta<double>* dtab64 = nullptr;
   ElemMeta<float>* dtab32 = nullptr;
@@ -978,8 +933,7 @@ struct smpm_handle_s {
   // up to `cap` columns): per-column pre/post state and GMRES vectors,
   // basis, w/w2, column reports and the launch shape
   struct {
-    int cap = 0, RC = 1, mats_smem = 0;
-    size_t smem = 0;
+    int cap = 0;
     double *b = nullptr, *bS = nullptr, *rg = nullptr, *cb = nullptr, *chatb = nullptr, *xs = nullptr;
     double *x = nullptr, *t = nullptr, *y = nullptr, *vg = nullptr, *c = nullptr, *chat = nullptr;
     double *V = nullptr, *W = nullptr, *acc = nullptr, *Rh = nullptr, *yv = nullptr;
@@ -1155,7 +1109,7 @@ smpm_status launch_schur_stream(smpm_handle h, const S* T, const S* v, S* y, cud
 }
 
 template <typename S>
-smpm_status launch_schur_class(smpm_handle h, const S* T, const S* v, S* y, cudaStream_t st);
+smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st);
 
 // Whether apply kernel kind (SMPM_APPLY_*) can run on h's grid.
 bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
@@ -1163,7 +1117,7 @@ bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
     case SMPM_APPLY_AUTO: case SMPM_APPLY_STREAM: return true;
     case SMPM_APPLY_WARP: case SMPM_APPLY_WARP2: case SMPM_APPLY_WARP4:
       return h->g.M <= 96 && (fp32 ? h->dtab32 != nullptr : h->dtab64 != nullptr);
-    case SMPM_APPLY_CLASS: return h->cls_ok && (fp32 ? h->dTcls32 != nullptr : h->dTcls != nullptr);
+    case SMPM_APPLY_CLASS: return h->cls_ok && (fp32 ? h->dig32.T != nullptr : h->dig.T != nullptr);
     default: return false;
   }
 }
@@ -1179,8 +1133,7 @@ smpm_status launch_schur_kind(smpm_handle h, int kind, const S* v, S* y, cudaStr
   if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
   if (kind == SMPM_APPLY_STREAM) return launch_schur_stream<S>(h, T, v, y, st);
   if (kind == SMPM_APPLY_CLASS) {
-    const S* Tc = reinterpret_cast<const S*>(fp32 ? (const void*)h->dTcls32 : (const void*)h->dTcls);
-    return launch_schur_class<S>(h, Tc, v, y, st);
+    return launch_schur_class<S>(h, v, y, st);
   }
   int dev = 0, sms = 0;
   CU(cudaGetDevice(&dev));
@@ -1337,8 +1290,9 @@ GmresArgs<double> gmres_args(smpm_handle h, double tol, bool adj = false) {
   a.white = h->dwhite;
   a.nblack = (int)h->f.black.size();
   a.nwhite = (int)h->f.white.size();
-  a.Tc = h->dT; a.Gc = h->dG; a.Xc = h->dX; a.Rs = h->dRs; a.H = h->dH;
-  if (adj) { a.Tc = h->dTa; a.Gc = h->dGa; a.Xc = h->dXa; a.Rs = h->dRsa; a.H = h->dHa; a.g.zw = h->dzwa; }
+  a.Tc = h->dT; a.Gc = h->dG; a.Xc = h->dX; a.Rd = h->dRd; a.H = h->dH;
+  if (adj) { a.Tc = h->dTa; a.Gc = h->dGa; a.Xc = h->dXa; a.Rd = h->dRda; a.H = h->dHa; a.g.zw = h->dzwa; }
+  a.tr = h->dtr; a.gr = h->dgr; a.bt = h->dbt; a.if4 = h->dif4;
   a.vglob = h->wV; a.vown = h->wvown; a.t = h->wt; a.y = h->wy;
   a.c = h->wc; a.chat = h->wchat; a.rhs = h->wrg; a.x = h->wx;
   a.acc = h->wacc; a.gs = h->wgs; a.bar = h->wbar; a.err = h->werr;
@@ -1367,7 +1321,8 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.white = h->dwhite;
   a.nblack = (int)h->f.black.size();
   a.nwhite = (int)h->f.white.size();
-  a.Tc = h->dT32; a.Gc = h->dG32; a.Xc = h->dX32; a.Rs = h->dRs32; a.H = h->dH32;
+  a.Tc = h->dT32; a.Gc = h->dG32; a.Xc = h->dX32; a.Rd = h->dRd; a.H = h->dH32;
+  a.tr = h->dtr; a.gr = h->dgr; a.bt = h->dbt; a.if4 = h->dif4;
   a.vglob = h->wV32; a.vown = h->wvown32; a.t = h->wt32; a.y = h->wy32;
   a.c = h->wc; a.chat = h->wchat; a.rhs = h->wrg32; a.x = h->wx32;
   a.acc = h->wacc; a.gs = h->wgs; a.bar = h->wbar; a.err = h->werr;
@@ -1432,7 +1387,6 @@ RefineArgs refine_args(smpm_handle h, const GmresArgs<float>& a, double tol) {
   RA.ga.stream_mats = 0;
   RA.ga.rhs = h->wrg32;
   RA.Tc64 = h->dT;
-  RA.Rs64 = h->dRs;
   RA.xS = h->wxs;
   RA.bS = h->wbS;
   RA.r = h->wr;
@@ -1641,15 +1595,6 @@ smpm_status lalloc(smpm_handle h, P** p, size_t count) {
 // +64) | rn[kMaxRefine] at +128
 constexpr size_t kLockCtlBytes = 256;  // (kLockColBytes, the column block size, is shared with the batch)
 
-// columns per element work item: the largest of maxrc, ..., 2, 1 that
-// divides R and still gives `warps` warps of a CTA an item (all warps busy:
-// FP64 needs at least 4 per SM for its pipe, FP32 its loads in flight).
-int lock_rc(int R, int nown_b, int maxrc, int warps) {
-  for (int c = maxrc; c >= 2; c /= 2)
-    if (R % c == 0 && (long long)nown_b * (R / c) >= warps) return c;
-  return 1;
-}
-
 // Workspace of the lockstep kernels for up to R columns (FP32 inner buffers
 // too when the handle is factored for mixed precision).
 smpm_status lock_prepare(smpm_handle h, int R) {
@@ -1692,21 +1637,22 @@ smpm_status lock_prepare(smpm_handle h, int R) {
   return SMPM_OK;
 }
 
-// Launch shape of the lockstep kernel: resident operator matrices when they fit.
+// Fields of a lockstep solve of R columns by teams of CTAs that own nown_b
+// blocks each: packed matrices, warps per item and group scratch within
+// `budget` bytes of shared memory.  Returns the kernel's shared memory (0: it
+// does not fit).
 template <typename S>
-smpm_status lock_shape(smpm_handle h, int R, int optin, int* RC, int* mats, size_t* smem) {
-  const Geometry& g = h->g;
-  const int m = h->opts.restart;
-  *RC = lock_rc(R, h->gm.nown_b, sizeof(S) == 4 ? 8 : 4, kGmresThreads / 32);
-  *mats = 1;
-  *smem = lock_smem_bytes<S>(m, g.M, g.n, R, *RC, h->gm.nown_b, h->gm.nown_w, true);
-  if ((h->opts.flags & SMPM_FLAG_NO_SMEM_RESIDENCY) || *smem > (size_t)optin) {
-    *mats = 0;
-    *smem = lock_smem_bytes<S>(m, g.M, g.n, R, *RC, h->gm.nown_b, h->gm.nown_w, false);
-  }
-  if (*smem > (size_t)optin) return fail(SMPM_EINVAL, "lockstep layout does not fit in shared memory");
-  CU(set_smem_limit(sizeof(S) == 8 ? fn_lock64() : fn_lock32(), optin));
-  return SMPM_OK;
+size_t lock_shape(smpm_handle h, LockArgs<S>& A, int R, int nown_b, size_t budget) {
+  const auto& D = sizeof(S) == 8 ? h->dig : h->dig32;
+  A.Gd = D.G; A.Xd = D.X; A.Td = D.T;
+  A.Ge = D.Ge; A.Xe = D.Xe; A.Te = D.Te;
+  A.bcls = h->dbcls;
+  A.tcls = h->dtcls;
+  A.R = R;
+  const size_t fixed = lock_fixed_bytes(h->opts.restart, R);
+  if (fixed >= budget) return 0;
+  A.wb_bytes = lock_groups<S>(h->g.M, h->g.n, (long long)nown_b * ((R + 7) / 8), budget - fixed, &A.W_item, &A.ngrp);
+  return A.wb_bytes ? fixed + A.wb_bytes : 0;
 }
 
 // R right-hand sides of one grid in lockstep.  FP64: k_pre_cols,
@@ -1725,11 +1671,11 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   int dev = 0, optin = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  int RC = 1, mats = 0;
-  size_t smem = 0;
-  if ((s = mixed ? lock_shape<float>(h, R, optin, &RC, &mats, &smem) : lock_shape<double>(h, R, optin, &RC, &mats,
-                                                                                          &smem)))
-    return s;
+  LockArgs<double> A64{};
+  LockArgs<float> A32{};
+  const size_t smem = mixed ? lock_shape(h, A32, R, h->gm.nown_b, optin) : lock_shape(h, A64, R, h->gm.nown_b, optin);
+  if (!smem) return fail(SMPM_EINVAL, "lockstep layout does not fit in shared memory");
+  CU(set_smem_limit(mixed ? fn_lock32() : fn_lock64(), optin));
   CU(set_smem_limit(fn_pre_cols(), optin));
   CU(set_smem_limit(fn_post_cols(), optin));
   unsigned* bar = reinterpret_cast<unsigned*>(L.ctl);
@@ -1821,15 +1767,15 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   CU(cudaEventRecord(h->ev0, st));
   auto lock_fields = [&](auto& A) {
     A.a.err = err;
-    A.a.mats_smem = mats; A.a.basis_smem = 0; A.a.stream_mats = 0; A.a.warp_elems = 1;
+    A.a.mats_smem = 0; A.a.basis_smem = 0; A.a.stream_mats = 0; A.a.warp_elems = 1;
     A.a.trace = nullptr; A.a.trace_cap = 0; A.a.skip = nullptr; A.a.its_out = nullptr; A.a.wscr = nullptr;
     A.a.c = L.c; A.a.chat = L.chat; A.a.acc = L.acc; A.a.gsep = L.gsep;
     choose_coarse(A.a, h->st_products, R);
-    A.R = R; A.RC = RC; A.vs = g.kp; A.ds = g.d;
+    A.vs = g.kp; A.ds = g.d;
     A.cs = L.cs; A.Rh = L.Rh; A.yv = L.yv;
   };
   if (!mixed) {
-    LockArgs<double> A{};
+    LockArgs<double>& A = A64;
     A.a = gmres_args(h, tol);
     lock_fields(A);
     A.a.rhs = L.rg; A.a.x = L.x; A.a.t = L.t; A.a.y = L.y; A.a.vglob = L.vg;
@@ -1847,7 +1793,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   } else {
     CU(set_smem_limit(fn_refine_cols(), optin));
     for (int ref = 0; ref < kMaxRefine; ++ref) {
-      LockArgs<float> A{};
+      LockArgs<float> A = A32;
       A.a = gmres_args32(h, kInnerTol);
       lock_fields(A);
       A.a.rhs = L.rg32; A.a.x = L.x32; A.a.t = L.t32; A.a.y = L.y32; A.a.vglob = L.vg32;
@@ -2039,6 +1985,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
     size_t lsmem;   // shared memory of its lockstep body (bound over its groups)
   };
   std::vector<PL> pl(np);
+  const int budget_all = optin - kBatchHdr - 1024;
   size_t smem = 0;
   smpm_status st;
   for (int p = 0; p < np; ++p) {
@@ -2054,7 +2001,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
     // the all-global needs of pre/post and refinement, then the richest
     // GMRES layout that fits beside the argument header (resident or
     // streamed operator matrices, resident basis)
-    const int budget = optin - kBatchHdr - 1024;
+    const int budget = budget_all;
     auto need_fixed = [&](bool wg) {
       size_t a = prepost_smem_bytes(m, g.M, g.n, L.ES, L.nown_b, L.nown_w, g.d, wg);
       if (mixed) a = std::max(a, refine_smem_bytes(m, g.M, g.n, L.ES, L.nown_b, L.nown_w, g.d, wg));
@@ -2078,9 +2025,18 @@ smpm_status batch_layout(smpm_batch b, int T) {
     L.lsmem = 0;
     if (b->nrhs[p] >= 2 && precond > 0 && !(h->opts.flags & SMPM_FLAG_NO_LOCKSTEP)) {
       const int Rg = std::min(b->nrhs[p], kLockMaxCols);
-      L.lsmem = mixed ? lock_smem_bytes<float>(m, g.M, g.n, Rg, 8, L.nown_b, L.nown_w, false)
-                      : lock_smem_bytes<double>(m, g.M, g.n, Rg, 4, L.nown_b, L.nown_w, false);
-      if (std::max(need_fixed(L.wg), L.lsmem) <= (size_t)budget) L.lock = 1;
+      L.lsmem = 0;
+      bool fits = true;
+      for (int k0 = 0; k0 < b->nrhs[p]; k0 += kLockMaxCols) {
+        const int Rg = std::min(kLockMaxCols, b->nrhs[p] - k0);
+        if (Rg < 2) continue;
+        LockArgs<double> A64{};
+        LockArgs<float> A32{};
+        const size_t q = mixed ? lock_shape(h, A32, Rg, L.nown_b, budget) : lock_shape(h, A64, Rg, L.nown_b, budget);
+        fits = fits && q > 0;
+        L.lsmem = std::max(L.lsmem, q);
+      }
+      if (fits && need_fixed(L.wg) <= (size_t)budget) L.lock = 1;
     }
     const size_t nd = kBatchHdr + std::max(need_fixed(L.wg), L.lock ? L.lsmem : L.lay.smem);
     if (nd > (size_t)optin - 1024)
@@ -2305,7 +2261,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
         hPc.insert(hPc.end(), pre.begin(), pre.end());
         hPc.insert(hPc.end(), post.begin(), post.end());
         hRc.resize(hRc.size() + (size_t)kMaxRefine * R);
-        auto lock_fields = [&](auto& A, int maxrc) {
+        auto lock_fields = [&](auto& A) {
           team_fields(A.a);
           A.a.mats_smem = 0;
           A.a.basis_smem = 0;
@@ -2319,8 +2275,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
           A.a.acc = wacc;
           A.a.gsep = wgs;
           choose_coarse(A.a, h->st_products, R);
-          A.R = R;
-          A.RC = lock_rc(R, L.nown_b, maxrc, kGmresThreads / 32);
+          lock_shape(h, A, R, L.nown_b, (size_t)budget_all);
           A.vs = g.kp;
           A.ds = g.d;
           A.cs = wcs;
@@ -2329,7 +2284,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
         };
         if (!mixed) {
           bt.L64.a = gmres_args(h, tol);
-          lock_fields(bt.L64, 4);
+          lock_fields(bt.L64);
           bt.L64.a.rhs = wrg;
           bt.L64.a.x = wx;
           bt.L64.a.t = wt;
@@ -2341,7 +2296,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
           bt.L64.done_stride = 0;
         } else {
           bt.L32.a = gmres_args32(h, kInnerTol);
-          lock_fields(bt.L32, 8);
+          lock_fields(bt.L32);
           bt.L32.a.rhs = wrg32;
           bt.L32.a.x = wx32;
           bt.L32.a.t = wt32;
@@ -2699,10 +2654,49 @@ smpm_status smpm_factor_many(const smpm_handle* hs, int count, const smpm_opts* 
 
 namespace {
 
+// Packed digits of the square row-major matrices in A (b x b each).
+template <typename S>
+smpm_status upload_digits(smpm_handle h, const std::vector<double>& A, int b, uint4** frag, short** er,
+                          cudaStream_t st) {
+  std::vector<uint4> f;
+  std::vector<short> e;
+  pack_digits<S>(A.data(), b, b, A.size() / ((size_t)b * b), &f, &e);
+  smpm_status s;
+  if ((s = upload(h, frag, f, st)) || (s = upload(h, er, e, st))) return s;
+  CU(cudaStreamSynchronize(st));  // f and e go out of scope
+  return SMPM_OK;
+}
+
+// Packed digits of the block classes' G_b and X_F, for the lockstep solves.
+smpm_status upload_block_digits(smpm_handle h, cudaStream_t st) {
+  const Geometry& g = h->g;
+  const size_t MM = (size_t)g.M * g.M, XX = 4 * (size_t)g.n * g.n, nb = h->f.black.size();
+  std::vector<int> idx(nb), of(nb, -1);
+  std::vector<double> Gc, Xc;
+  int n = 0;
+  for (size_t ib = 0; ib < nb; ++ib) {
+    const int r = h->f.grep[ib];
+    if (of[r] < 0) {
+      of[r] = n++;
+      Gc.insert(Gc.end(), h->f.G.begin() + r * MM, h->f.G.begin() + (r + 1) * MM);
+      Xc.insert(Xc.end(), h->f.X.begin() + r * XX, h->f.X.begin() + (r + 1) * XX);
+    }
+    idx[ib] = of[r];
+  }
+  smpm_status s;
+  if ((s = upload(h, &h->dbcls, idx, st)) || (s = upload_digits<double>(h, Gc, g.M, &h->dig.G, &h->dig.Ge, st)) ||
+      (s = upload_digits<double>(h, Xc, g.n, &h->dig.X, &h->dig.Xe, st)))
+    return s;
+  if (h->opts.precision == 1 && ((s = upload_digits<float>(h, Gc, g.M, &h->dig32.G, &h->dig32.Ge, st)) ||
+                                 (s = upload_digits<float>(h, Xc, g.n, &h->dig32.X, &h->dig32.Xe, st))))
+    return s;
+  return SMPM_OK;
+}
+
 // Class tables of the class-shared apply: one T per T class of the factor
 // step (face types, and on a graded grid the sizes; the copies of T_e within
 // a class are identical), tiles of kClassTile elements.
-smpm_status upload_classes(smpm_handle h, const std::vector<double>& Tc, cudaStream_t st) {
+smpm_status upload_classes(smpm_handle h, cudaStream_t st) {
   const Geometry& g = h->g;
   const size_t MM = (size_t)g.M * g.M;
   std::vector<int> cls_of(g.nel, -1), first;
@@ -2716,9 +2710,10 @@ smpm_status upload_classes(smpm_handle h, const std::vector<double>& Tc, cudaStr
     }
     members[cls_of[key]].push_back((int)e);
   }
-  std::vector<double> Tcls(members.size() * MM);
+  std::vector<double> Tcls(members.size() * MM);  // row-major
   for (size_t c = 0; c < members.size(); ++c)
-    std::copy(Tc.begin() + (size_t)first[c] * MM, Tc.begin() + (size_t)(first[c] + 1) * MM, Tcls.begin() + c * MM);
+    std::copy(h->f.T.begin() + (size_t)first[c] * MM, h->f.T.begin() + (size_t)(first[c] + 1) * MM,
+              Tcls.begin() + c * MM);
   std::vector<int> sel, tiles;
   for (size_t c = 0; c < members.size(); ++c) {
     const int base = (int)sel.size();
@@ -2730,17 +2725,19 @@ smpm_status upload_classes(smpm_handle h, const std::vector<double>& Tc, cudaStr
     }
   }
   smpm_status s;
-  if ((s = upload(h, &h->dTcls, Tcls, st)) || (s = upload(h, &h->dtiles, tiles, st)) ||
-      (s = upload(h, &h->dclsel, sel, st)))
+  std::vector<int> cidx(g.nel);
+  for (long long e = 0; e < g.nel; ++e) cidx[e] = cls_of[h->f.tcls[e]];
+  if ((s = upload(h, &h->dtiles, tiles, st)) || (s = upload(h, &h->dclsel, sel, st)) ||
+      (s = upload(h, &h->dtcls, cidx, st)))
     return s;
-  if (h->opts.precision == 1 && (s = upload(h, &h->dTcls32, std::vector<float>(Tcls.begin(), Tcls.end()), st)))
-    return s;
+  if ((s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
+  if (h->opts.precision == 1 && (s = upload_digits<float>(h, Tcls, g.M, &h->dig32.T, &h->dig32.Te, st))) return s;
   h->ncls = (int)members.size();
   h->ntiles = (int)(tiles.size() / 3);
   int dev = 0, optin = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (g.M <= 128 && class_smem(g.M, sizeof(double)) <= (size_t)optin) {
+  if (class_smem<double>(g.M) <= (size_t)optin) {
     CU(set_smem_limit(k_schur_class<double>, optin));
     CU(set_smem_limit(k_schur_class<float>, optin));
     h->cls_ok = 1;
@@ -2776,11 +2773,67 @@ smpm_status factor_device_operator(smpm_handle h, cudaStream_t st) {
   }
   if ((s = upload(h, &h->dtab64, t64, st))) return s;
   if (h->dT32 && (s = upload(h, &h->dtab32, t32, st))) return s;
-  if ((s = upload_classes(h, Tc, st))) return s;
+  if ((s = upload_classes(h, st))) return s;
   CU(cudaStreamSynchronize(st));
   h->f.T.clear();
   h->f.T.shrink_to_fit();
   h->op_factored = true;
+  return SMPM_OK;
+}
+
+// S Z at every slot from the row sums of the pushed products: slot (e, F, t)
+// takes row (opp F, t) of the neighbour's Rs, and its own weight in z_j as
+// the identity's share (zw: weights of the 4 faces of each element).
+std::vector<double> pulled_row_sums(const Geometry& g, const std::vector<double>& Rs, const std::vector<double>& zw) {
+  std::vector<double> out(4 * (size_t)g.kp, 0.0);
+  for (long long e = 0; e < g.nel; ++e)
+    for (int F = 0; F < 4; ++F) {
+      const int e2 = g.neighbour((int)e, F), Fo = opposite(F);
+      if (e2 < 0) continue;
+      for (int t = 0; t < g.n; ++t) {
+        double* o = out.data() + 4 * ((size_t)e * g.M + F * g.n + t);
+        const double* r = Rs.data() + 4 * ((size_t)e2 * g.M + Fo * g.n + t);
+        for (int G = 0; G < 4; ++G)
+          if (g.iface(e2, G) >= 0) o[G] = r[G];
+        o[Fo] += zw[4 * e + F];
+      }
+    }
+  return out;
+}
+
+// Tables of the solve kernels (see GmresArgs).
+smpm_status upload_tables(smpm_handle h, cudaStream_t st) {
+  const Geometry& g = h->g;
+  std::vector<int> tr(g.nel), first;
+  for (long long e = 0; e < g.nel; ++e) {
+    const size_t c = h->f.tcls[e];
+    if (first.size() <= c) first.resize(c + 1, -1);
+    if (first[c] < 0) first[c] = (int)e;
+    tr[e] = first[c];
+  }
+  std::vector<int4> if4(g.nel), bt(h->f.black.size() * 2 * (size_t)g.M);
+  for (long long e = 0; e < g.nel; ++e) {
+    int j[4];
+    for (int F = 0; F < 4; ++F) j[F] = std::max(0, g.iface((int)e, F));
+    if4[e] = make_int4(j[0], j[1], j[2], j[3]);
+  }
+  for (size_t ib = 0; ib < h->f.black.size(); ++ib) {
+    const int e = h->f.black[ib];
+    for (int F = 0; F < 4; ++F) {
+      const int e2 = g.neighbour(e, F), Fo = opposite(F);
+      for (int t = 0; t < g.n; ++t) {
+        const int i = F * g.n + t;
+        int4* o = bt.data() + ib * 2 * g.M;
+        o[i] = make_int4(e * g.M + i, std::max(0, e2), g.iface(e, F), 4 * e + F);
+        o[g.M + i] = e2 >= 0 ? make_int4(e2 * g.M + Fo * g.n + t, e, g.iface(e, F), 4 * e2 + Fo) : make_int4(-1, 0, -1, 0);
+      }
+    }
+  }
+  smpm_status s;
+  if ((s = upload(h, &h->dtr, tr, st)) || (s = upload(h, &h->dgr, h->f.grep, st)) || (s = upload(h, &h->dif4, if4, st)) ||
+      (s = upload(h, &h->dbt, bt, st)) || (s = upload(h, &h->dRd, pulled_row_sums(g, h->f.Rs, h->f.zw), st)))
+    return s;
+  if (h->f.has_adjoint && (s = upload(h, &h->dRda, pulled_row_sums(g, h->f.Rsa, h->f.zwa), st))) return s;
   return SMPM_OK;
 }
 
@@ -2811,6 +2864,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     if (h->f.has_adjoint && (s = upload(h, &h->dzwa, h->f.zwa, st))) return s;
   }
   dg.zw = h->dzw;
+  if ((s = upload_tables(h, st))) return s;
   const size_t kp = g.kp, r = g.r, d = g.d, m = opts.restart;
   const size_t nbs = blocks_for(g.kp, kSlotsPerBlock);
   if ((s = dalloc(h, &h->wb, r)) || (s = dalloc(h, &h->wbS, kp)) || (s = dalloc(h, &h->wV, (m + 1) * kp)) ||
@@ -2889,7 +2943,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       if (per_sm < 1) return fail(SMPM_ECUDA, "the refinement kernel does not fit on an SM");
       auto to32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
       if ((s = upload(h, &h->dT32, to32(Tc), st)) || (s = upload(h, &h->dG32, to32(Gc), st)) ||
-          (s = upload(h, &h->dX32, to32(Xc), st)) || (s = upload(h, &h->dRs32, to32(h->f.Rs), st)) ||
+          (s = upload(h, &h->dX32, to32(Xc), st)) ||
           (s = upload(h, &h->dH32, to32(h->f.H), st)))
         return s;
       if ((s = dalloc(h, &h->wx32, g.kp)) || (s = dalloc(h, &h->wt32, g.kp)) || (s = dalloc(h, &h->wy32, g.kp)) ||
@@ -2940,7 +2994,8 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       }
       if ((s = upload(h, &h->dtab64, t64, st))) return s;
       if (h->dT32 && (s = upload(h, &h->dtab32, t32, st))) return s;
-      if ((s = upload_classes(h, Tc, st))) return s;
+      if ((s = upload_classes(h, st))) return s;
+      if (opts.precond > 0 && (s = upload_block_digits(h, st))) return s;
     }
     if (h->f.has_adjoint) {
       // T~_e = T_e^T: its column-major device copy is T_e row-major
@@ -2953,7 +3008,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
           if (j < 0) continue;
           for (int t = 0; t < g.n; ++t) ztusa[j] += h->f.zwa[4 * e + F] * h->f.uSa[e * g.M + F * g.n + t];
         }
-      if ((s = upload(h, &h->dTa, h->f.T, st)) || (s = upload(h, &h->dRsa, h->f.Rsa, st)) ||
+      if ((s = upload(h, &h->dTa, h->f.T, st)) ||
           (s = upload(h, &h->dGa, Gca, st)) || (s = upload(h, &h->dXa, Xca, st)) ||
           (s = upload(h, &h->dHa, h->f.Ha, st)) || (s = upload(h, &h->dfdxT, h->f.fdxT, st)) ||
           (s = upload(h, &h->dfdyT, h->f.fdyT, st)) || (s = upload(h, &h->duSa, h->f.uSa, st)) ||
@@ -3181,11 +3236,11 @@ smpm_status smpm_autotune_apply(smpm_handle h, int precision, int reps, int flus
 namespace {
 
 template <typename S>
-smpm_status launch_schur_class(smpm_handle h, const S* T, const S* v, S* y, cudaStream_t st) {
-  if (!h->cls_ok) return fail(SMPM_EINVAL, "the class-shared apply needs n <= 32 and its tile in shared memory");
-  const int bulk = (reinterpret_cast<uintptr_t>(v) % 16 == 0) ? 1 : 0;  // bulk copies need 16-byte alignment
-  k_schur_class<S><<<(unsigned)h->ntiles, 256, class_smem(h->g.M, sizeof(S)), st>>>(h->dg, T, h->dtiles, h->dclsel,
-                                                                                      v, y, bulk);
+smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st) {
+  if (!h->cls_ok) return fail(SMPM_EINVAL, "the class-shared apply needs its packed matrices and tile in shared memory");
+  const bool fp32 = sizeof(S) == 4;
+  k_schur_class<S><<<(unsigned)h->ntiles, kClassThreads, class_smem<S>(h->g.M), st>>>(
+      h->dg, fp32 ? h->dig32.T : h->dig.T, fp32 ? h->dig32.Te : h->dig.Te, h->dtiles, h->dclsel, v, y);
   CHECK_LAUNCH();
   return SMPM_OK;
 }
@@ -3197,7 +3252,7 @@ extern "C" {
 smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, void* stream) try {
   NEED_OPERATOR();
   if (!v || !y) return fail(SMPM_EINVAL, "null vector");
-  return launch_schur_class<double>(h, h->dTcls, v, y, as_stream(stream));
+  return launch_schur_class<double>(h, v, y, as_stream(stream));
 } catch (...) {
   return host_exception();
 }
@@ -3205,8 +3260,8 @@ smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, vo
 smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, void* stream) try {
   NEED_OPERATOR();
   if (!v || !y) return fail(SMPM_EINVAL, "null vector");
-  if (!h->dTcls32) return fail(SMPM_ESTATE, "FP32 factors exist only after schur_factor with precision = 1");
-  return launch_schur_class<float>(h, h->dTcls32, v, y, as_stream(stream));
+  if (!h->dT32) return fail(SMPM_ESTATE, "FP32 factors exist only after schur_factor with precision = 1");
+  return launch_schur_class<float>(h, v, y, as_stream(stream));
 } catch (...) {
   return host_exception();
 }
@@ -3723,7 +3778,7 @@ __global__ void __launch_bounds__(256) k_deflate_noalloc(DevGeo g, const double*
     }
     ok = grid_sync(bar, err, epoch, (int)gridDim.x);
   }
-  for (long long s = tid; s < g.kp; s += nthr) y[s] = ok ? deflate_slot_cg(g, v, chat, Rs, s) : nan("");
+  for (long long s = tid; s < g.kp; s += nthr) y[s] = ok ? deflate_slot<double, true>(g, v, chat, Rs, s) : nan("");
 }
 
 }  // namespace
