@@ -71,15 +71,16 @@ typedef struct {
   int flags;           /* SMPM_FLAG_* bits (default 0)                        */
 } smpm_opts;
 
-/* flags: keep the GMRES operator matrices and Krylov basis in global memory
- * even when they fit in shared memory; stream the operator matrices through
- * shared memory with bulk copies even when they would fit resident (the
- * large-grid layouts, selectable for testing). */
+/* flags: keep the GMRES kernel's matrices, tables and Krylov basis in global
+ * memory even when they fit in shared memory (the large-grid layout, selectable
+ * for testing).  STREAM_MATRICES and WARP_ELEMS are accepted and change
+ * nothing: the matrices are packed once per element or block class and read
+ * from L1 and L2, and a group of warps per block or element is sized by the
+ * number a CTA owns. */
 #define SMPM_FLAG_NO_SMEM_RESIDENCY 1
 #define SMPM_FLAG_STREAM_MATRICES 2
 #define SMPM_FLAG_ADJOINT 4        /* also build the transposed system for schur_solve_adjoint */
-#define SMPM_FLAG_WARP_ELEMS 8     /* one warp per block / element in the GMRES phases even when few
-                                      are owned per CTA (the default from 4 per CTA; for testing) */
+#define SMPM_FLAG_WARP_ELEMS 8
 #define SMPM_FLAG_ROBIN_LITERAL 16 /* Robin flux R = I + n.grad with identity weight p_F = 1 on every face
                                       (the literal form of Sec. 1.2); robin_scale is then unused */
 #define SMPM_FLAG_NO_LOCKSTEP 32    /* solve several right-hand sides one after another instead of in
@@ -235,9 +236,10 @@ smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, vo
 smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, void* stream);
 
 /* Kernels of y = S v (smpm_apply_schur, smpm_apply_schur32 and the S apply
- * inside the deflation entry points): AUTO picks by thresholds (one warp per
- * element for 4n <= 96, 1, 2 or 4 elements per warp by the element count, else
- * the shared-memory stream); WARP: persistent CTAs, one warp per element,
+ * inside the deflation entry points): AUTO takes CLASS where the elements
+ * fall into few enough classes that its tiles of eight elements are at least 5/8
+ * full on average, else by thresholds one warp per element for 4n <= 96 (1, 2 or
+ * 4 warps by the element count) or the shared-memory stream; WARP: persistent CTAs, one warp per element,
  * T_e read column by column from global memory; WARP2 / WARP4: 2 or 4 warps
  * per element; STREAM: bulk copies of T_e into a shared-memory ring; CLASS:
  * the element-class-shared product (smpm_apply_schur_class). */
@@ -330,9 +332,12 @@ smpm_status smpm_set_barrier_spin_limit(long long spins);
  *
  * smpm_batch_create: hs[count] factored handles (distinct; their device
  * workspaces are used by the batch, so do not solve on them concurrently),
- * nrhs[count] >= 1 right-hand sides each.  team_size <= 0 picks the smallest
- * of 8, 16, 19, 38, 76 that fits (each problem's solve state must fit the
- * shared memory of one CTA at that team size), else all SMs as one team.
+ * nrhs[count] >= 1 right-hand sides each.  team_size <= 0 forms teams of
+ * different sizes, as large as each problem needs for all to finish together
+ * (an estimate from the problems' sizes; smpm_batch_info's team_size is then
+ * the largest); where that does not fit, uniform teams of the smallest of 8,
+ * 16, 19, 38, 76 that fits (each problem's solve state must fit the shared
+ * memory of one CTA at that team size), else all SMs as one team.
  * use_graph != 0 captures the batch's device work (argument copy, barrier
  * resets, the launch, the report copy) in a CUDA graph on the first solve
  * and replays it afterwards.  precision: -1 each handle's own, 0 FP64 for all,

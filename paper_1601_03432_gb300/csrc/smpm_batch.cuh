@@ -15,7 +15,7 @@
 
 struct alignas(16) BatchTask {
   PrePostArgs P;          // FP64 pre/post arguments (all-global layout)
-  GmresArgs<double> a64;  // FP64 GMRES (its own layout: resident or streamed matrices, basis)
+  GmresArgs<double> a64;  // FP64 GMRES (its own layout: resident matrices, basis)
   GmresArgs<float> a32;   // FP32 inner GMRES (mixed precision)
   RefineArgs R;           // refinement step (mixed precision)
   int precision;          // 0 FP64, 1 FP32 inner + FP64 refinement
@@ -62,13 +62,6 @@ constexpr int kBatchTaskBytes = (int)((sizeof(BatchTask) + 127) / 128 * 128);
 // header: the task, then staging for one column's pre/post and refinement arguments
 constexpr int kBatchHdr = (int)((kBatchTaskBytes + sizeof(PrePostArgs) + sizeof(RefineArgs) + 127) / 128 * 128);
 
-// copy n bytes (a multiple of 16) from global memory into shared memory, all threads
-__device__ __forceinline__ void stage16(void* dst, const void* src, int n) {
-  const int4* s = reinterpret_cast<const int4*>(src);
-  int4* d = reinterpret_cast<int4*>(dst);
-  for (int i = threadIdx.x; i < n / 16; i += blockDim.x) d[i] = s[i];
-}
-
 // A lockstep group task: pre bodies of the R columns, the lockstep GMRES
 // (FP64, or up to kMaxRefine rounds of FP32 lockstep GMRES and per-column
 // refinement), post bodies, reports.  Returns the failing body (0: none).
@@ -103,7 +96,7 @@ __device__ __noinline__ int batch_group(BatchTask& T, unsigned char* smraw, unsi
     double* acc = T.precision == 0 ? T.L64.a.acc : T.L32.a.acc;
     for (size_t i = (size_t)rank * blockDim.x + threadIdx.x; i < nacc; i += (size_t)a.G * blockDim.x) acc[i] = 0.0;
   }
-  if (!grid_sync(ga.bar, ga.err, epoch, ga.G)) return 1;
+  if (!team_sync(ga, epoch)) return 1;
   for (int c = 0; c < R; ++c) {
     stage_p(c, c);
     if (!pre_body(Pst, body, epoch)) return 2;
@@ -125,14 +118,14 @@ __device__ __noinline__ int batch_group(BatchTask& T, unsigned char* smraw, unsi
         __syncthreads();
         if (refine_body(Rst, body, epoch) < 0) return 4;
       }
-      if (!grid_sync(ga.bar, ga.err, epoch, ga.G)) return 4;
+      if (!team_sync(ga, epoch)) return 4;
     }
   }
   for (int c = 0; c < R; ++c) {
     stage_p(R + c, c);
     if (!post_body(Pst, body, epoch)) return 5;
   }
-  if (!grid_sync(ga.bar, ga.err, epoch, ga.G)) return 5;
+  if (!team_sync(ga, epoch)) return 5;
   if (rank == 0 && threadIdx.x < R) {
     const int c = threadIdx.x;
     const unsigned char* blk = T.lctl + (size_t)c * kLockColBytes;

@@ -4,12 +4,12 @@
 #pragma once
 #include <cuda_runtime.h>
 
-// How the solve bodies enter a kernel: inlined into the kernels that run one
-// of them; called by the batch kernel, which runs them all (inlined, that one
-// kernel took 154 s to compile and spilled registers).
-#ifndef SMPM_BODY
-#define SMPM_BODY
-#endif
+// The solve bodies and their phases are calls, not inlined: one kernel with all
+// of them inlined spills registers (k_gmres: 1.6 KB per thread) and takes
+// minutes to compile.  The kernels stage their arguments in shared memory, so
+// that a call's reference to them costs no copy.
+#define SMPM_BODY __noinline__
+#define SMPM_PHASE __noinline__
 
 #include <algorithm>
 #include <cmath>
@@ -49,16 +49,11 @@ constexpr int kSlotsPerBlock = 256;   // slots per CTA in the vector kernels
 constexpr int kElemThreads = 256;     // threads per element CTA
 constexpr int kTraceCap = 1 << 16;    // entries of the optional phase trace
 constexpr int kGmresThreads = 256;    // threads per CTA of the persistent GMRES kernel
-// per-solve control block (zeroed by one memset): 64 barrier counters |
+// per-solve control block (zeroed by one memset): barrier counter | (at 256)
 // err, done, nref | 8 accumulators | 32 refinement residual norms
 constexpr size_t kCtlBytes = 720;  // + 32 inner iteration counts
 constexpr int kMaxRefine = 8;        // FP64 refinement steps of the mixed-precision path
-constexpr int kMaxStreamBufs = 4;    // shared-memory buffers of the GMRES kernel's matrix stream
-constexpr int kWarpElemsMin = 4;     // owned blocks per CTA from which each warp takes its own element
 constexpr double kInnerTol = 1e-4;   // relative tolerance of each FP32 inner GMRES
-// the coarse solve is fused into the white-element phase when the atomic adds
-// it costs per Arnoldi step (d per CTA) stay below this
-constexpr long long kFusedCoarseMaxAdds = 1LL << 17;
 
 struct GState {
   double tolabs, beta0, beta, wnorm0sq, resid;

@@ -165,79 +165,134 @@ __device__ __forceinline__ double scale2(double v, int s) {
 // Result from the summed weights hi 2^32 + lo (units of 256^GMIN); er: exponent
 // of A's row, E: the column's largest exponent field.  Inf or NaN in the column
 // gives NaN, as does a row marked kBadRow.
-__device__ __forceinline__ double digits_result(long long hi, long long lo, int er, int E, double) {
-  const int s = er + E - 1022 + 56 - 124;  // 256^7 2^(er - 62) 2^(E - 1022 - 62)
-  if (E >= 600 && E <= 1400 && er != kBadRow) return digits_value(hi, lo, s);
+__device__ __noinline__ double digits_far(long long hi, long long lo, int er, int E) {  // exponents out of the usual range
   if (E == 0x7ff || er == kBadRow) return __longlong_as_double(0x7ff8000000000000LL);
-  return scale2(digits_value(hi, lo, 0), s);
+  return scale2(digits_value(hi, lo, 0), er + E - 1022 + 56 - 124);
+}
+__device__ __forceinline__ double digits_result(long long hi, long long lo, int er, int E, double) {
+  if (E >= 600 && E <= 1400 && er != kBadRow)
+    return digits_value(hi, lo, er + E - 1022 + 56 - 124);  // 256^7 2^(er - 62) 2^(E - 1022 - 62)
+  return digits_far(hi, lo, er, E);
+}
+__device__ __noinline__ float digits_far32(long long hi, long long lo, int er, int E) {
+  return (float)digits_value(hi, lo, er + E - 126 + 16 - 60);
 }
 __device__ __forceinline__ float digits_result(long long hi, long long lo, int er, int E, float) {
   if (E == 0xff || er == kBadRow) return __int_as_float(0x7fc00000);
   return (float)digits_value(hi, lo, er + E - 126 + 16 - 60);  // 256^2 2^(er - 30) 2^(E - 126 - 30), FP64 exponents
 }
 
+// The same in a few FP64 operations (the halves are below 2^53: one rounding),
+// for the one-column products, where few instructions count more than FP64
+// throughput.
+__device__ __forceinline__ double pow2(int s) { return __longlong_as_double((long long)(1023 + s) << 52); }
+__device__ __forceinline__ double digits_short(long long hi, long long lo, int er, int E, double) {
+  const int s = er + E - 1022 + 56 - 124;
+  if (E >= 600 && E <= 1400 && er != kBadRow) return fma((double)hi, pow2(s + 32), (double)lo * pow2(s));
+  return digits_far(hi, lo, er, E);
+}
+__device__ __forceinline__ float digits_short(long long hi, long long lo, int er, int E, float) {
+  // hi 2^32 + lo < 2^57: rounded once from the integer, then scaled exactly
+  if (E == 0xff || er == kBadRow) return __int_as_float(0x7fc00000);
+  const int s = er + E - 126 + 16 - 60;
+  const float t = __ll2float_rn((hi << 32) + lo);
+  return s > -120 && s < 60 ? t * __int_as_float((127 + s) << 23) : digits_far32(hi, lo, er, E);
+}
+
 // ---- eight columns -----------------------------------------------------------
-// Packs the eight columns x(k, c), k < len, into Bf (digit_bwords words) and
-// returns the largest exponent field (>= 1) of column g = lane / 4.  get(k, c):
-// the entry.  One warp (it packs the k tiles part, part + parts, ...: several
-// warps share the work, each finding the exponents itself).
-template <typename S, typename Get>
-__device__ __forceinline__ int pack_cols(uint4* Bf, int len, int lane, Get&& get, int part = 0, int parts = 1) {
+// k tile kt of eight packed columns: the lane's entries of column lane / 4
+template <typename S>
+__device__ __forceinline__ void pack_tile(uint4* Bf, int kt, int lane, const S (&v)[4], int E) {
   constexpr int ND = Digits<S>::ND;
+  decltype(to_digits(S(0), 1)) Y[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) Y[u] = to_digits(v[u], E);
+#pragma unroll
+  for (int j = 0; j < ND; j += 2)
+    Bf[(kt * (ND / 2) + j / 2) * 32 + lane] = make_uint4(digit_pair(Y[0], Y[1], j), digit_pair(Y[2], Y[3], j),
+                                                         digit_pair(Y[0], Y[1], j + 1), digit_pair(Y[2], Y[3], j + 1));
+}
+
+// The routines below are calls, one copy each: the solve kernels run them from
+// a dozen places, each once per phase and a few warps at a time, and inlined
+// there the instruction fetches took longer than the products (a 64 x 64
+// block solve 25 k cycles instead of 12 k).
+//
+// Packs eight columns, entry (k, c) at x[k ldk + c ldc] (shared memory, or
+// global memory that no other CTA writes; columns >= nc are zero), k < len,
+// into Bf (digit_bwords words) and returns the largest exponent field (>= 1) of
+// column g = lane / 4.  One warp (it packs the k tiles part, part + parts, ...:
+// several warps share the work, each finding the exponents itself).
+template <typename S>
+__device__ __noinline__ int pack_cols(uint4* Bf, const S* x, int ldk, int ldc, int len, int nc, int lane, int part,
+                                      int parts) {
   const int g = lane >> 2, q = lane & 3, kt_n = digit_tiles(len);
+  const S* xc = x + (size_t)min(g, nc - 1) * ldc;
+  const int klen = g < nc ? len : 0;
   int E = 1;
   for (int kt = 0; kt < kt_n; ++kt)
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
-      if (k < len) E = max(E, exp_field((S)get(k, g)));
+      if (k < klen) E = max(E, exp_field(xc[k * ldk]));
     }
   E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
   E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
   for (int kt = part; kt < kt_n; kt += parts) {
-    decltype(to_digits(S(0), 1)) Y[4];
+    S v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
-      Y[u] = to_digits(k < len ? (S)get(k, g) : S(0), E);
+      v[u] = k < klen ? xc[k * ldk] : S(0);
     }
-#pragma unroll
-    for (int j = 0; j < ND; j += 2)
-      Bf[(kt * (ND / 2) + j / 2) * 32 + lane] =
-          make_uint4(digit_pair(Y[0], Y[1], j), digit_pair(Y[2], Y[3], j), digit_pair(Y[0], Y[1], j + 1),
-                     digit_pair(Y[2], Y[3], j + 1));
+    pack_tile<S>(Bf, kt, lane, v, E);
   }
   __syncwarp();
   return E;
 }
 
-// Row tile mt of A times the packed columns: put(row g or g + 8, column, value)
-// for rows < rows.  Af: A's fragments (L1/L2), er: its row exponents, E: the
-// exponent field of column lane / 4 (from pack_cols).
-template <typename S, typename Put>
-__device__ __forceinline__ void digits_tile8(const uint4* __restrict__ Af, const short* __restrict__ er,
-                                             const uint4* Bf, int rows, int kt_n, int mt, int lane, int E, Put&& put) {
+// A's fragments of k tile kt of a row tile, ND / 2 words per lane (shared or
+// global memory)
+template <typename S>
+__device__ __forceinline__ void ld_frag(uint4 (&f)[Digits<S>::ND / 2], const uint4* __restrict__ A, int kt) {
+#pragma unroll
+  for (int p = 0; p < Digits<S>::ND / 2; ++p) f[p] = A[(kt * (Digits<S>::ND / 2) + p) * 32];
+}
+
+// The values a lane (g, q) holds of a row tile times eight columns: z[v] is row
+// 16 mt + g + 8 (v >> 1), column 2q + (v & 1).
+template <typename S>
+struct Tile8 {
+  S z[4];
+};
+
+// Row tile mt of A times the packed columns (row indices beyond rows give
+// arbitrary values).  Af: A's fragments (two k tiles ahead), er: its row
+// exponents, E: the exponent field of column lane / 4 (from pack_cols).
+template <typename S>
+__device__ __forceinline__ Tile8<S> tile8_products(const uint4* Af, const short* __restrict__ er,
+                                                   const uint4* Bf, int rows, int kt_n, int mt, int lane, int E) {
   constexpr int ND = Digits<S>::ND, GMIN = Digits<S>::GMIN, NG = Digits<S>::NG;
+  const int g = lane >> 2, q = lane & 3, row0 = mt * 16 + g;
+  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
+  uint4 a0[ND / 2], a1[ND / 2];
+  ld_frag<S>(a0, A, 0);
+  if (kt_n > 1) ld_frag<S>(a1, A, 1);
+  const int er0 = row0 < rows ? __ldg(er + row0) : 0, er1 = row0 + 8 < rows ? __ldg(er + row0 + 8) : 0;
   float acc[NG][4];
 #pragma unroll
   for (int c = 0; c < NG; ++c)
 #pragma unroll
     for (int v = 0; v < 4; ++v) acc[c][v] = 0.f;
-  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
-  uint4 an[ND / 2];
-#pragma unroll
-  for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + p * 32);
   for (int kt = 0; kt < kt_n; ++kt) {
     uint4 av[ND / 2], bv[ND / 2];
 #pragma unroll
     for (int p = 0; p < ND / 2; ++p) {
-      av[p] = an[p];
+      av[p] = a0[p];
+      a0[p] = a1[p];
       bv[p] = Bf[(kt * (ND / 2) + p) * 32 + lane];
     }
-    if (kt + 1 < kt_n) {
-#pragma unroll
-      for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + ((kt + 1) * (ND / 2) + p) * 32);
-    }
+    if (kt + 2 < kt_n) ld_frag<S>(a1, A, kt + 2);
 #pragma unroll
     for (int i = 0; i < ND; ++i) {
       uint32_t a[4];
@@ -251,45 +306,49 @@ __device__ __forceinline__ void digits_tile8(const uint4* __restrict__ Af, const
       }
     }
   }
-  // lane holds rows g, g + 8 of columns 2q, 2q + 1 (their E is with lanes 8q, 8q + 4)
-  const int g = lane >> 2, q = lane & 3;
+  Tile8<S> o;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    const int row = mt * 16 + g + 8 * (v >> 1), col = 2 * q + (v & 1);
-    const int Ec = __shfl_sync(0xffffffffu, E, 4 * col);
-    if (row < rows) {
-      long long lo = 0, hi = 0;
+    const int Ec = __shfl_sync(0xffffffffu, E, 4 * (2 * q + (v & 1)));  // column 2q + (v & 1): lanes 8q, 8q + 4
+    long long lo = 0, hi = 0;
 #pragma unroll
-      for (int k = 0; k < NG; ++k) {
-        const long long t = (long long)__float2int_rn(acc[k][v]) << (8 * (k & 3));
-        if (k < 4) lo += t;
-        else hi += t;
-      }
-      put(row, col, digits_result(hi, lo, er[row], Ec, S(0)));
+    for (int k = 0; k < NG; ++k) {
+      const long long t = (long long)__float2int_rn(acc[k][v]) << (8 * (k & 3));
+      if (k < 4) lo += t;
+      else hi += t;
     }
+    o.z[v] = digits_result(hi, lo, v < 2 ? er0 : er1, Ec, S(0));
   }
+  return o;
+}
+template <typename S>
+__device__ __noinline__ Tile8<S> digits_tile8(const uint4* Af, const short* __restrict__ er,
+                                              const uint4* Bf, int rows, int kt_n, int mt, int lane, int E) {
+  return tile8_products<S>(Af, er, Bf, rows, kt_n, mt, lane, E);
 }
 
 // ---- one column --------------------------------------------------------------
 // The eight mma columns are the weights: digit i of A meets digit n + GMIN - i
 // of x in column n, so the digits of A share one accumulator tile (two, by
 // parity, for shorter chains).  Bf: one fragment per digit i of A
-// (digit_bwords words).  get(k): entry k < len; returns the largest exponent
-// field (>= 1).  One warp packs the k tiles part, part + parts, ...
-template <typename S, typename Get>
-__device__ __forceinline__ int pack_one(uint4* Bf, int len, int lane, Get&& get, int part = 0, int parts = 1) {
+// (digit_bwords words).  x: len entries (as for pack_cols); returns the largest
+// exponent field (>= 1).  One warp packs the k tiles part, part + parts, ...
+template <typename S>
+__device__ __noinline__ int pack_one(uint4* Bf, const S* x, int len, int lane, int part, int parts) {
   constexpr int ND = Digits<S>::ND, GMIN = Digits<S>::GMIN, NG = Digits<S>::NG, OFF = ND - 1 - GMIN;
   const int g = lane >> 2, q = lane & 3, kt_n = digit_tiles(len);
   int E = 1;
-  for (int k = lane; k < len; k += 32) E = max(E, exp_field((S)get(k)));
+#pragma unroll 1
+  for (int k = lane; k < len; k += 32) E = max(E, exp_field(x[k]));
   E = __reduce_max_sync(0xffffffffu, E);
   constexpr unsigned long long kFill = 0x8080808080808080ull;
+#pragma unroll 1
   for (int kt = part; kt < kt_n; kt += parts) {
     unsigned long long Y[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int k = kt * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
-      unsigned long long y = to_digits(k < len ? (S)get(k) : S(0), E);
+      unsigned long long y = to_digits(k < len ? x[k] : S(0), E);
       if (sizeof(S) == 4) y = ((y | (kFill << 32)) << (8 * OFF)) | (kFill >> (64 - 8 * (OFF > 0 ? OFF : 1)));
       // digits moved down by g places, zeros moved in at the top
       if (g > 0) y = (y >> (8 * g)) | (kFill << (64 - 8 * g));
@@ -309,52 +368,62 @@ __device__ __forceinline__ int pack_one(uint4* Bf, int len, int lane, Get&& get,
   return E;
 }
 
-// Row tile mt of A times the packed column: put(row, value) for rows < rows.
-template <typename S, typename Put>
-__device__ __forceinline__ void digits_tile1(const uint4* __restrict__ Af, const short* __restrict__ er,
-                                             const uint4* Bf, int rows, int kt_n, int mt, int lane, int E, Put&& put) {
+// row of a row tile whose value digits_tile1 leaves in this lane, -1: none
+__device__ __forceinline__ int tile1_row(int mt, int lane, int rows) {
+  const int q = lane & 3, row = mt * 16 + (lane >> 2) + (q < 2 ? 0 : 8);
+  return !(q & 1) && row < rows ? row : -1;
+}
+
+// Row tile mt of A times the packed column: the value of row tile1_row.
+template <typename S>
+__device__ __noinline__ S digits_tile1(const uint4* Af, const short* __restrict__ er, const uint4* Bf,
+                                       int rows, int kt_n, int mt, int lane, int E) {
   constexpr int ND = Digits<S>::ND;
+  const int q = lane & 3, row = tile1_row(mt, lane, rows);
+  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
+  uint4 a0[ND / 2], a1[ND / 2];
+  ld_frag<S>(a0, A, 0);
+  if (kt_n > 1) ld_frag<S>(a1, A, 1);
+  const int err = row >= 0 ? __ldg(er + row) : 0;
   float acc[2][4];
 #pragma unroll
   for (int v = 0; v < 8; ++v) acc[v >> 2][v & 3] = 0.f;
-  const uint4* A = Af + (size_t)mt * kt_n * (ND / 2) * 32 + lane;
-  uint4 an[ND / 2];
+  auto step = [&](uint4 (&f)[ND / 2], int kt) {  // k tile kt, whose fragments f then become those of kt + 2
+    uint4 b[ND / 2];
 #pragma unroll
-  for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + p * 32);
-  for (int kt = 0; kt < kt_n; ++kt) {
-    uint4 av[ND / 2];
-#pragma unroll
-    for (int p = 0; p < ND / 2; ++p) av[p] = an[p];
-    if (kt + 1 < kt_n) {
-#pragma unroll
-      for (int p = 0; p < ND / 2; ++p) an[p] = __ldg(A + ((kt + 1) * (ND / 2) + p) * 32);
-    }
+    for (int p = 0; p < ND / 2; ++p) b[p] = Bf[(kt * (ND / 2) + p) * 32 + lane];
+    uint32_t a[ND][4];
 #pragma unroll
     for (int p = 0; p < ND / 2; ++p) {
-      const uint4 b = Bf[(kt * (ND / 2) + p) * 32 + lane];
-      uint32_t a[4];
-      digit_a(av[p].x, av[p].y, a);
-      mma_16816(acc[0], a, b.x, b.y);
-      digit_a(av[p].z, av[p].w, a);
-      mma_16816(acc[1], a, b.z, b.w);
+      digit_a(f[p].x, f[p].y, a[2 * p]);
+      digit_a(f[p].z, f[p].w, a[2 * p + 1]);
     }
+    if (kt + 2 < kt_n) ld_frag<S>(f, A, kt + 2);
+#pragma unroll
+    for (int p = 0; p < ND / 2; ++p) {
+      mma_16816(acc[0], a[2 * p], b[p].x, b[p].y);
+      mma_16816(acc[1], a[2 * p + 1], b[p].z, b[p].w);
+    }
+  };
+#pragma unroll 1
+  for (int kt = 0; kt < kt_n; kt += 2) {
+    step(a0, kt);
+    if (kt + 1 < kt_n) step(a1, kt + 1);
   }
-  // lane holds weights 2q, 2q + 1 of rows g and g + 8; the quad adds them up:
-  // row g ends in lane q = 0, row g + 8 in lane q = 2
-  const int g = lane >> 2, q = lane & 3;
+  // lane holds weights 2q, 2q + 1 of rows g and g + 8 (each accumulator stays
+  // within 2^24, exact, for up to 256 columns); the quad adds them up: row g ends in lane
+  // q = 0, row g + 8 in lane q = 2
+  const int m0 = (q & 1) ? 1 << 16 : 1;
   long long w[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const long long a0 = (long long)__float2int_rn(acc[0][2 * h]) + __float2int_rn(acc[1][2 * h]);
-    const long long a1 = (long long)__float2int_rn(acc[0][2 * h + 1]) + __float2int_rn(acc[1][2 * h + 1]);
-    w[h] = a0 + (a1 << 8);
-    if (q & 1) w[h] <<= 16;
+    const int s0 = __float2int_rn(acc[0][2 * h]) + __float2int_rn(acc[1][2 * h]);
+    const int s1 = __float2int_rn(acc[0][2 * h + 1]) + __float2int_rn(acc[1][2 * h + 1]);
+    w[h] = (long long)s0 * m0 + (long long)s1 * (m0 << 8);
     w[h] += __shfl_xor_sync(0xffffffffu, w[h], 1);
   }
   const long long got = __shfl_xor_sync(0xffffffffu, q < 2 ? w[1] : w[0], 2);
-  const int row = mt * 16 + g + (q < 2 ? 0 : 8);
-  if (!(q & 1) && row < rows)
-    put(row, q < 2 ? digits_result(got, w[0], er[row], E, S(0)) : digits_result(w[1], got, er[row], E, S(0)));
+  return digits_short(q < 2 ? got : w[1], q < 2 ? w[0] : got, err, E, S(0));
 }
 
 // Packs count row-major rows x cols matrices: fragments (digit_words each) and

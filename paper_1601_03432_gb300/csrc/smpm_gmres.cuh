@@ -3,37 +3,55 @@
 //   S M^-1       (Algorithm 2),
 //   P S M^-1     (Algorithm 3),
 // run as ONE cooperative launch per solve: restarted GMRES(m), classical
-// Gram-Schmidt with one re-orthogonalisation (CGS2), FP64 Givens rotations,
-// the convergence test on the rotated residual, restarts from the true
-// residual.
+// Gram-Schmidt with one re-orthogonalisation (CGS2), the convergence test on
+// the least-squares residual, restarts from the true residual.
 //
 // Work is owned, not redistributed per phase: CTA c owns the checkerboard
 // blocks ib = c, c + G, ... (G = grid size) -- the black elements and the
 // slots of their blocks, which partition Gamma -- and the white elements
-// iw = c, c + G, ...  The owner keeps its blocks' operator matrices (G_b, T_e,
-// X_b and the white T_e, column-major) and its slice of the Krylov basis in
-// shared memory when they fit, so an Arnoldi step touches L2/HBM only for the
-// vectors exchanged between neighbouring elements.  One step:
+// iw = c, c + G, ...  The matrices are shared per class of elements or blocks,
+// packed in digits (smpm_digits.cuh); the class a CTA uses most, its slice of
+// the Krylov basis, its entries' table and its rows of C^+ stay in shared
+// memory as far as they fit.  One step:
 //   A  owner: v_j = w2 - V h2 on its block slots (lazy, see E), then the
-//      block solve t = M^-1 v_j: a = G (p - X q), b = q - T_e a
+//      block solve t = M^-1 v_j: a = G (p - X q), b = q - T_e a, in stages
+//      (black_phase) or with the whole inverse (black_block)
 //   B  white elements: y = S t (y = v on white-owned slots), c = Z^T y
-//   C  c_hat = C^+ c (dense FP64 rows spread over all CTAs; Algorithm 3)
+//   C  c_hat = C^+ c (rows over all CTAs, or by element-row strips; Algorithm 3)
 //   D  owner: w = y - S Z c_hat; V^T w and ||w||^2, accumulated with FP64
 //      atomics in L2
 //   E  owner: w2 = w - V h1; V^T w2 and ||w2||^2 likewise; every CTA forms
-//      ||v_{j+1}||^2 = ||w2||^2 - ||h2||^2 and applies the same Givens
-//      rotations to its own copy, so all CTAs take the same decision.
-// Phases are separated by a grid barrier (5 per step for Algorithm 3).  The
-// basis is kept unnormalised with the inverse norms replicated in every CTA.
-// FP64 products are plain per-thread FMA chains (thread per matrix row, per
-// basis vector, per slot): FP64 issue slots are scarce on this part, so the
-// hot path uses no warp-shuffle reduction trees.
+//      ||v_{j+1}||^2 = ||w2||^2 - ||h2||^2 and the residual norm from its own
+//      copy of the Hessenberg column, so all CTAs take the same decision.
+// Phases are separated by a team barrier (5 per step for Algorithm 3, 7 with
+// strips).  The basis is kept unnormalised with the inverse norms replicated
+// in every CTA.
+//
+// What bounds it: on a grid with a block or two per CTA, the chain of one
+// step: five barriers (about 3,000 SM cycles each), a dozen dependent loads
+// from L2 (about 700 each), FP64 sums at 76 cycles per operation, one packing
+// and one product of digits per element phase.  At 16 x 16 elements, n = 16,
+// on 152 CTAs a step takes 59,000 cycles (57,000 with FP64 products and a
+// step more per solve before).  On large grids, the element products, the
+// basis read from L2 and C^+.
 //
 // Data written by other CTAs inside the kernel is read with ld.global.cg: L1
-// is not coherent across SMs.  The grid barrier spins with a bound and raises
-// an error flag instead of hanging.
+// is not coherent across SMs.  The barrier spins with a bound and raises an
+// error flag instead of hanging.
 #pragma once
 // Included inside the anonymous namespace of smpm_solver.cu.
+
+// Packed class matrices of the element products (smpm_digits.cuh): T_e per
+// element class, G_b and the four X_F per block class, with row exponents,
+// and the class of each element / black block.  Elements of one class (face
+// types and sizes) share one copy, so a CTA reads its matrices from L1.
+struct DigitMats {
+  const uint4 *G, *X, *T;
+  const short *Ge, *Xe, *Te;
+  const int *bcls, *tcls;
+  const uint4* B;   // whole block inverses (2M x 2M), or null: see black_block
+  const short* Be;
+};
 
 template <typename S>
 struct GmresArgs {
@@ -41,22 +59,14 @@ struct GmresArgs {
   const int* black;
   const int* white;
   int nblack, nwhite;
-  const S* Tc;      // nel * M*M, column-major T_e
-  const S* Gc;      // nblack * M*M, column-major G_b
-  const S* Xc;      // nblack * 4*n*n, column-major X_F blocks
-  // identical matrices (one class of face types and sizes) are read from one
-  // copy: T_e from element tr[e]'s, G_b and X_b from block gr[ib]'s.  A CTA's
-  // elements are mostly of one class, so the matrices come from L1 instead of
-  // once per element from L2 or HBM
-  const int* tr;
-  const int* gr;
+  DigitMats dm;
   // per entry of a black block (2M per block: own slots, then facing slots):
   // {slot or -1, element that pushes into it, its interface or -1, 4 e + F of the slot}
   const int4* bt;
   const int4* if4;   // interfaces of each element (0 where there is none; its weight is 0)
   const double* Rd;  // kp * 4: S Z at each slot, the coefficients of c_hat on the pusher's interfaces
-  // d*d row-major coarse inverse: FP64, or its FP32 copy for the FP32 inner
-  // solves of the mixed-precision path
+  // coarse inverse, d rows of (d rounded up to a multiple of 4) entries: FP64, or
+  // its FP32 copy for the FP32 inner solves of the mixed-precision path
   const typename std::conditional<sizeof(S) == 4, float, double>::type* H;
   S* vglob;         // kp : current basis vector (raw), exchanged between CTAs
   S* vown;          // G * (m+1) * ES : basis slices when not resident in smem
@@ -68,32 +78,24 @@ struct GmresArgs {
   S* x;             // kp (zero on entry)
   double* acc;      // (2m + 1) * (m + 3) FP64 accumulators (zero on entry)
   GState* gs;
-  unsigned* bar;    // barrier counter (zero on entry)
+  unsigned* bar;    // the team's barrier counter
   int* err;
   int precond, m, maxit;
   double tol;
   int nown_b, nown_w;  // blocks / white elements per CTA (ceil)
-  int ES;              // entries per CTA in the basis slice (odd, >= 2M nown_b)
-  int mats_smem;       // 1: owned matrices resident in shared memory
+  int ES;              // entries per CTA in the basis slice (a multiple of 4, >= 2M nown_b)
   int basis_smem;      // 1: basis slice resident in shared memory
-  int stream_mats;     // 1: owned matrices streamed through two shared buffers (bulk copies)
-  int buf_elems;       // elements of S per stream buffer (>= M*M + 4*n*n, multiple of 16 bytes)
-  int nbuf;            // stream buffers (2..kMaxStreamBufs): nbuf - 1 items in flight while one is used
-  int warp_elems;      // 1: each warp works on its own block / white element (many per CTA); 0: the
-                       // whole CTA works on one element at a time
+  int W_item;          // warps per block / element in the element phases (8 / W_item groups per CTA)
+  int res_T, res_G;    // classes whose matrices the CTA keeps in shared memory: T_e (0 .. 2), G_b with X_b (0, 1)
+  int tab, res_H;      // 1: the owned entries' table / the CTA's rows of H in shared memory
+  int blk;             // 1: black blocks by their whole inverse (dm.B)
   long long* trace;
   int trace_cap;
   const int* skip;  // when non-null and set on entry, the kernel returns at once
   int* its_out;     // when non-null: Arnoldi steps of this launch
   int G;            // CTAs working on this solve (a team; the whole grid for one solve)
   int base;         // first CTA of the team: the CTA's rank is blockIdx.x - base
-  S* wscr;          // when non-null: per-CTA global scratch for w, w2 (2 (ES+1) per rank)
-  // fused coarse solve (Algorithm 3 steps only): each white element adds
-  // H[:, j] c_j for its interfaces j into c_hat as soon as c_j is known, so
-  // the separate coarse phase and its grid barrier disappear
-  int fused;           // 1: use HT / chatd in the Arnoldi steps
-  const double* HT;    // d*d, H column-major (HT[j d + r] = H[r][j])
-  double* chatd;       // 2 d: c_hat of even / odd steps (accumulated with atomics)
+  S* wscr;          // when non-null: per-CTA global scratch for w (ES per rank)
   // C^+ by element-row strips (strips.p > 0 and use_strips): see coarse_solve
   CoarseStrips<typename std::conditional<sizeof(S) == 4, float, double>::type> strips;
   double* gsep;        // strips: 2 p mx + 1 doubles per column (sums pushed onto the separators, alpha)
@@ -106,12 +108,16 @@ __device__ __forceinline__ int team_rank(const GmresArgs<S>& a) {
   return (int)blockIdx.x - a.base;
 }
 
-#define GM_TRACE(tag)                                                                   \
-  do {                                                                                  \
-    if (a.trace && team_rank(a) == 0 && threadIdx.x == 0 && trace_n + 2 <= a.trace_cap) { \
-      a.trace[trace_n++] = (tag);                                                       \
-      a.trace[trace_n++] = clock64();                                                   \
-    }                                                                                   \
+// Phase trace of CTA 0 (SMPM_TRACE); a call, so that the solve's own code stays small.
+__device__ __noinline__ void trace_point(long long* trace, int cap, int rank, int tag, int& n) {
+  if (rank == 0 && threadIdx.x == 0 && n + 2 <= cap) {
+    trace[n++] = tag;
+    trace[n++] = clock64();
+  }
+}
+#define GM_TRACE(tag) \
+  do {                \
+    if (a.trace) trace_point(a.trace, a.trace_cap, team_rank(a), tag, trace_n); \
   } while (0)
 
 template <typename S>
@@ -119,11 +125,6 @@ __device__ __forceinline__ S ldcg(const S* p) {
   return __ldcg(p);
 }
 
-// Team barrier on a monotonic counter: thread 0 of each CTA adds one with
-// release semantics and polls with acquire loads until the counter reaches
-// the CTA's next epoch (a multiple of the team size G; the team is the whole
-// grid for a single solve).  Bounded spin; err is set on timeout and the
-// caller unwinds.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -134,39 +135,41 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
 // of polling; smpm_set_barrier_spin_limit lowers it to exercise the timeout).
 __device__ long long g_barrier_spin_limit = 1LL << 28;
 
-// work: run by thread 0 between its arrival and its wait (serial work of this
-// CTA overlapped with the other CTAs' arrival); it must touch only what no
-// other CTA reads before the barrier completes.
-template <typename Work>
-__device__ bool grid_sync_with(unsigned* bar, int* err, unsigned& epoch, int G, Work&& work) {
-  __shared__ int ok;
+// Team barrier on a monotonic counter: thread 0 of each CTA adds one with
+// release semantics and polls with acquire loads until the counter reaches
+// the CTA's next epoch (the counter's value on entry to a kernel, which all
+// CTAs share, plus the team size G per barrier).  One flag per CTA, polled by
+// a thread each, was four times slower at 152 CTAs (10 k against 2.6 k cycles:
+// the polls of all CTAs crowd the flags' L2 slice).  Bounded spin; err is set
+// on timeout and the caller unwinds.
+__device__ __noinline__ bool team_sync_call(unsigned* bar, int* err, unsigned epoch) {
   __syncthreads();
+  bool ok = true;
   if (threadIdx.x == 0) {
-    ok = 1;
-    epoch += (unsigned)G;
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(1u) : "memory");
-    work();
     long long spins = 0;
     const long long limit = g_barrier_spin_limit;
     while ((int)(ld_acquire(bar) - epoch) < 0) {
       if (++spins > limit) {  // this CTA's own timeout: code 1 unless a failure is recorded
         atomicCAS(err, 0, 1);
-        ok = 0;
+        ok = false;
         break;
       }
       if ((spins & 4095) == 0 && *((volatile int*)err)) {  // another CTA failed: unwind
-        ok = 0;
+        ok = false;
         break;
       }
     }
   }
-  __syncthreads();
-  return ok != 0;
+  return __syncthreads_and(ok);
 }
-
-__device__ bool grid_sync(unsigned* bar, int* err, unsigned& epoch, int G) {
-  return grid_sync_with(bar, err, epoch, G, [] {});
+template <typename S>
+__device__ __forceinline__ bool team_sync(const GmresArgs<S>& a, unsigned& epoch) {
+  epoch += (unsigned)a.G;
+  return team_sync_call(a.bar, a.err, epoch);
 }
+// the epoch on entry to a kernel
+__device__ __forceinline__ unsigned first_epoch(const unsigned* bar) { return __ldcg(bar); }
 
 // entry i (< 2M) of black block ib
 template <typename S>
@@ -174,454 +177,474 @@ __device__ __forceinline__ int4 block_entry(const GmresArgs<S>& a, int ib, int i
   return __ldg(a.bt + (size_t)ib * 2 * a.g.M + i);
 }
 
-// per-warp scratch of the warp-per-element phases: p, q (the block's own and
-// facing slots), r1, a, z
-__host__ __device__ __forceinline__ int warp_scratch(int M) { return 5 * M; }
+// owned entry i of the CTA: block rank + k G, entry i - 2M k of it
+template <typename S>
+__device__ __forceinline__ int4 owned_entry(const GmresArgs<S>& a, int i) {
+  const int M2 = 2 * a.g.M, k = i / M2, ib = team_rank(a) + k * a.G;
+  if (k >= a.nown_b || ib >= a.nblack) return make_int4(-1, 0, -1, 0);
+  return block_entry(a, ib, i - k * M2);
+}
+template <typename S>
+__device__ __forceinline__ int entry_slot(const GmresArgs<S>& a, int i) {
+  return owned_entry(a, i).x;
+}
+
+// ---- shared memory ---------------------------------------------------------
+// A group of W warps works on one block or element; its scratch: the packed
+// vector (M entries, or n on each of the four faces), the block's values
+// [p; q], r1 (then a), and for white elements the contributions to c.
+template <typename S>
+__host__ __device__ constexpr size_t item_bf_bytes(int M, int n, int blk) {
+  const int a = digit_bwords<S>(blk ? 2 * M : M), b = 4 * digit_bwords<S>(n);
+  return sizeof(uint4) * (size_t)(a > b ? a : b);
+}
+template <typename S>
+__host__ __device__ constexpr size_t item_bytes(int M, int n, int blk) {
+  return item_bf_bytes<S>(M, n, blk) + 3 * (size_t)M * sizeof(double);
+}
+// warps per item for `items` items per CTA: every warp busy
+inline int item_warps(long long items) {
+  int w = 1;
+  while (w < kGmresThreads / 32 && items * w * 2 <= kGmresThreads / 32) w *= 2;
+  return w;
+}
+
+// The W warps of a group (named barrier of their own) work on one item.
+__device__ __forceinline__ void item_sync(int grp, int W) {
+  if (W == 1) __syncwarp();
+  else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * W) : "memory");
+}
+
+// Matrices resident in shared memory: the classes most of the CTA's blocks and
+// elements belong to.  L1 does not keep them: the acquiring load of a barrier
+// invalidates it (31 % hits measured in k_gmres), so from global memory every
+// phase reads its matrices from L2 again.
+struct Resident {
+  const uint4 *T, *G, *X;
+  int clsT[2], clsG;  // -1: none
+};
+
+// What the deflation of an owned entry needs besides y and c_hat: its table
+// entry, its pusher's interfaces and the row of S Z (a chain of two dependent
+// loads from L2, 1,300 cycles of every step, when read from global memory).
+struct OwnedEntry {
+  int4 en, J;
+  double2 r0, r1;
+};
 
 template <typename S>
 struct Smem {
-  double *h1, *h2, *hs1, *hs2, *gcs, *gsn, *gg, *col, *invb, *misc, *cs;
-  S *p, *r1, *av, *z, *red;
-  S *w, *w2;
+  double *h1, *h2, *hs1, *hs2, *z, *xi, *gg, *col, *invb, *misc;
   double* cst;  // staged coarse vector c (d, and two entries of padding)
-  double* cpv;  // fused coarse: c_j of the owned white elements' interfaces (4 per element)
-  int* cpj;     // and their interface indices (-1: none)
-  S* V;     // (m+1) * ES when resident
-  S* mats;  // resident matrices, or the two stream buffers
-  S* wb;    // warp_elems: per-warp element scratch, kWarpScratch(M) entries per warp
-  unsigned long long* mbar;  // mbarriers of the matrix stream (kMaxStreamBufs)
+  unsigned char* wb;  // group scratch (item_bytes each)
+  Resident* res;
+  int4* ob;         // owned blocks: {element or -1, block class, T class}
+  int4* ow;         // owned white elements: {element or -1, T class}
+  OwnedEntry* tab;  // ES entries, or null
+  const typename std::conditional<sizeof(S) == 4, float, double>::type* H;  // the CTA's rows of H, or null
+  S* w;     // ES : w, then w2 in its place
+  S* V;     // the CTA's slice of the basis, (m+1) * ES: shared or global memory
+  unsigned char* end;
 };
+
+// bytes of one CTA's rows of H (coarse_rows)
+template <typename S>
+__host__ __device__ inline size_t coarse_row_bytes(long long d, int G) {
+  return (size_t)((d + G - 1) / G) * ((d + 3) & ~3LL) * sizeof(S);
+}
 
 template <typename S>
 __device__ Smem<S> carve(const GmresArgs<S>& a, unsigned char* raw) {
   Smem<S> s;
-  const int m = a.m, M = a.g.M;
+  const int m = a.m;
   double* d = reinterpret_cast<double*>(raw);
-  s.mbar = reinterpret_cast<unsigned long long*>(d); d += kMaxStreamBufs;
   s.h1 = d; d += m + 3;
   s.h2 = d; d += m + 3;
   s.hs1 = d; d += m + 3;
   s.hs2 = d; d += m + 3;
-  s.gcs = d; d += m + 3;
-  s.gsn = d; d += m + 3;
+  s.z = d; d += m + 3;
+  s.xi = d; d += m + 3;
   s.gg = d; d += m + 3;
   s.col = d; d += m + 3;
   s.invb = d; d += m + 3;
   s.misc = d; d += 16;
-  s.cs = d; d += M;
   s.cst = d; d += a.g.d + 3;
-  s.cpv = d; d += 4 * (size_t)a.nown_w;
-  s.cpj = reinterpret_cast<int*>(d); d += 2 * (size_t)a.nown_w;
-  S* q = reinterpret_cast<S*>(d);
-  s.p = q; q += M;
-  s.r1 = q; q += M;
-  s.av = q; q += M;
-  s.z = q; q += M;
-  s.red = q; q += 256;
-  if (a.wscr) {
-    s.w = a.wscr + (size_t)team_rank(a) * 2 * (a.ES + 1);
-    s.w2 = s.w + a.ES + 1;
-  } else {
-    s.w = q; q += a.ES + 1;
-    s.w2 = q; q += a.ES + 1;
-  }
-  if (a.warp_elems) {  // 16-byte aligned base; each warp's 5M entries keep that alignment (M = 4n)
-    q = reinterpret_cast<S*>((reinterpret_cast<size_t>(q) + 15) & ~size_t(15));
-    s.wb = q;
-    q += (size_t)(blockDim.x / 32) * warp_scratch(M);
-  } else {
-    s.wb = nullptr;
-  }
-  s.V = q;
-  if (a.basis_smem) q += (size_t)(m + 1) * a.ES;
-  q = reinterpret_cast<S*>((reinterpret_cast<size_t>(q) + 15) & ~size_t(15));
-  s.mats = q;
+  auto align = [](void* p) { return reinterpret_cast<unsigned char*>((reinterpret_cast<size_t>(p) + 15) & ~size_t(15)); };
+  s.res = reinterpret_cast<Resident*>(align(d));
+  s.ob = reinterpret_cast<int4*>(align(s.res + 1));
+  s.ow = s.ob + a.nown_b;
+  s.wb = align(s.ow + a.nown_w);
+  S* q = reinterpret_cast<S*>(s.wb + (size_t)(kGmresThreads / 32 / a.W_item) * item_bytes<S>(a.g.M, a.g.n, a.blk));
+  if (a.wscr) s.w = a.wscr + (size_t)team_rank(a) * a.ES;
+  else { s.w = q; q += a.ES; }
+  if (a.basis_smem) { s.V = q; q += (size_t)(m + 1) * a.ES; }
+  else s.V = a.vown ? a.vown + (size_t)team_rank(a) * (m + 1) * a.ES : nullptr;
+  unsigned char* e = align(q);
+  s.tab = nullptr;
+  if (a.tab) { s.tab = reinterpret_cast<OwnedEntry*>(e); e += a.ES * sizeof(OwnedEntry); }
+  s.H = nullptr;
+  if (a.res_H) { s.H = reinterpret_cast<decltype(s.H)>(e); e += coarse_row_bytes<S>(a.g.d, a.G); }
+  s.end = e;  // resident matrices, or the scratch of the bodies around GMRES
   return s;
 }
 
 template <typename S>
-inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown_w, int basis_smem, int mats_smem,
-                               long long d, int stream_elems = 0, bool w_global = false, int nbuf = 2,
-                               bool warp_elems = false) {
-  size_t dbl = kMaxStreamBufs + 9 * (size_t)(m + 3) + 16 + M + (size_t)d + 3 + 6 * (size_t)nown_w;
-  size_t sel = 4 * (size_t)M + 256 + (w_global ? 0 : 2 * (size_t)(ES + 1));
-  if (warp_elems) sel += (size_t)(kGmresThreads / 32) * warp_scratch(M) + 16 / sizeof(S);
+inline size_t resident_bytes(int M, int n, int res_T, int res_G, int blk) {
+  return sizeof(uint4) * (res_T * digit_words<S>(M, M) +
+                          res_G * (blk ? digit_words<S>(2 * M, 2 * M) : digit_words<S>(M, M) + 4 * digit_words<S>(n, n)));
+}
+
+template <typename S>
+inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int W, int basis_smem, long long d, bool w_global = false,
+                               int res_T = 0, int res_G = 0, int blk = 0, int tab = 0, size_t H_bytes = 0) {
+  const size_t dbl = 9 * (size_t)(m + 3) + 16 + (size_t)d + 3;
+  size_t sel = w_global ? 0 : ES;
   if (basis_smem) sel += (size_t)(m + 1) * ES;
-  if (mats_smem) sel += (size_t)nown_b * (2 * (size_t)M * M + 4 * (size_t)n * n) + (size_t)nown_w * M * M;
-  sel += (size_t)nbuf * stream_elems;
-  return dbl * sizeof(double) + sel * sizeof(S) + 128;
+  return dbl * sizeof(double) + (size_t)(kGmresThreads / 32 / W) * item_bytes<S>(M, n, blk) + sel * sizeof(S) +
+         resident_bytes<S>(M, n, res_T, res_G, blk) + sizeof(Resident) +
+         (2 * (size_t)(ES / (2 * M)) + 4) * sizeof(int4) + (tab ? ES * sizeof(OwnedEntry) : 0) + H_bytes + 96;
 }
 
-// pointers to the owned matrices (shared-memory copies or global)
-template <typename S>
-__device__ __forceinline__ const S* mat_G(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib) {
-  const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) : a.Gc + (size_t)__ldg(a.gr + ib) * M * M;
-}
-template <typename S>
-__device__ __forceinline__ const S* mat_Tb(const GmresArgs<S>& a, const Smem<S>& s, int k, int e) {
-  const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + M * M : a.Tc + (size_t)__ldg(a.tr + e) * M * M;
-}
-template <typename S>
-__device__ __forceinline__ const S* mat_X(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib) {
-  const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)k * (2 * M * M + 4 * n * n) + 2 * M * M : a.Xc + (size_t)__ldg(a.gr + ib) * 4 * n * n;
-}
-template <typename S>
-__device__ __forceinline__ const S* mat_Tw(const GmresArgs<S>& a, const Smem<S>& s, int k, int e) {
-  const int M = a.g.M, n = a.g.n;
-  return a.mats_smem ? s.mats + (size_t)a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M
-                     : a.Tc + (size_t)__ldg(a.tr + e) * M * M;
-}
-
-template <typename S>
-__device__ __forceinline__ S* basis(const GmresArgs<S>& a, const Smem<S>& s, int l) {
-  return a.basis_smem ? s.V + (size_t)l * a.ES : a.vown + ((size_t)team_rank(a) * (a.m + 1) + l) * a.ES;
-}
-
-// ---- matrix stream: bulk copies into two shared-memory buffers ------------
-// Item sequence of a CTA (cyclic, the order in which the phases use them):
-// for each owned block k: [G_k | X_k], [T_e(k)]; then for each owned white
-// element: [T_e].  Item i lives in buffer i % nbuf; while it is used the next
-// nbuf - 1 items are in flight.  Thread 0 issues; waits are bounded.  Every
-// thread orders its earlier shared-memory accesses before the copy engine's
-// writes (fence.proxy.async) ahead of the barrier that precedes an issue.
-__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
-  for (long long spins = 0; spins < (1LL << 22); ++spins) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
+// The class most of cnt owned items have other than `skip` (-1: none): id[rank +
+// k G] for k < cnt, classes cls[id] (cls[ib] where id is null).  Warp 0; the
+// first 32 items stand for all.
+__device__ __forceinline__ int main_class(const int* cls, const int* id, int rank, int G, int cnt, int total, int skip) {
+  const int lane = threadIdx.x & 31;
+  int mine = -1;
+  if (lane < cnt && rank + lane * G < total) {
+    const int i = rank + lane * G;
+    mine = cls[id ? id[i] : i];
   }
-  return false;
+  int n = 0;
+  for (int k = 0; k < 32; ++k) n += __shfl_sync(0xffffffffu, mine, k) == mine;
+  const int best = __reduce_max_sync(0xffffffffu, mine >= 0 && mine != skip ? n * 32 + lane : -1);
+  return best < 0 ? -1 : __shfl_sync(0xffffffffu, mine, best & 31);
 }
 
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
+// The CTA's tables of owned blocks and white elements (all threads; the caller
+// synchronises): read in every phase, a dependent load from L2 each.
+template <typename S>
+__device__ __forceinline__ void load_owned(const GmresArgs<S>& a, const Smem<S>& s) {
+  const DigitMats& D = a.dm;
+  for (int k = threadIdx.x; k < a.nown_b + a.nown_w; k += blockDim.x) {
+    const bool b = k < a.nown_b;
+    const int i = team_rank(a) + (b ? k : k - a.nown_b) * a.G;
+    const int e = i < (b ? a.nblack : a.nwhite) ? __ldg((b ? a.black : a.white) + i) : -1;
+    const int ct = e >= 0 ? __ldg(D.tcls + e) : -1;
+    s.ob[k] = b ? make_int4(e, e >= 0 && D.bcls ? __ldg(D.bcls + i) : -1, ct, 0) : make_int4(e, ct, 0, 0);
+  }
 }
 
 template <typename S>
-struct MatStream {
-  int nb, nw, nitems;
-  long long issued, consumed;
-};
-
+__device__ __forceinline__ int4 owned_entry(const GmresArgs<S>& a, const Smem<S>& s, int i) {
+  return s.tab ? s.tab[i].en : owned_entry(a, i);
+}
 template <typename S>
-__device__ void ms_issue(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>& ms) {
-  if (ms.nitems == 0) return;
-  const long long i = ms.issued++;
-  if (threadIdx.x != 0) return;
-  const int M = a.g.M, n = a.g.n, G = a.G, rank = team_rank(a);
-  const int it = (int)(i % ms.nitems), b = (int)(i % a.nbuf);
-  S* dst = s.mats + (size_t)b * a.buf_elems;
-  unsigned long long* bar = s.mbar + b;
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  const unsigned mm = (unsigned)(M * M * sizeof(S)), xx = (unsigned)(4 * n * n * sizeof(S));
-  if (it < 2 * ms.nb) {
-    const int k = it >> 1, ib = rank + k * G;
-    if ((it & 1) == 0) {
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm + xx)
-                   : "memory");
-      const size_t ir = __ldg(a.gr + ib);
-      bulk_g2s(dst, a.Gc + ir * M * M, mm, bar);
-      bulk_g2s(dst + (size_t)M * M, a.Xc + ir * 4 * n * n, xx, bar);
-    } else {
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm) : "memory");
-      bulk_g2s(dst, a.Tc + (size_t)__ldg(a.tr + a.black[ib]) * M * M, mm, bar);
+__device__ __forceinline__ int entry_slot(const GmresArgs<S>& a, const Smem<S>& s, int i) {
+  return owned_entry(a, s, i).x;
+}
+
+// Loads the resident matrices and tables (all threads; ends with a barrier).
+template <typename S>
+__device__ SMPM_PHASE void load_resident(const GmresArgs<S>& a, const Smem<S>& s) {
+  const int M = a.g.M, n = a.g.n, rank = team_rank(a);
+  const size_t wM = digit_words<S>(M, M), wX = a.blk ? 0 : 4 * digit_words<S>(n, n);
+  const size_t wG = a.blk ? digit_words<S>(2 * M, 2 * M) : wM;
+  uint4* p = reinterpret_cast<uint4*>(s.end);
+  load_owned(a, s);
+  if (s.tab) {
+    for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
+      OwnedEntry o = {owned_entry(a, i), make_int4(0, 0, 0, 0), make_double2(0, 0), make_double2(0, 0)};
+      if (o.en.z >= 0) {
+        const double2* R = reinterpret_cast<const double2*>(a.Rd + 4 * (size_t)o.en.x);
+        o.J = __ldg(a.if4 + o.en.y);
+        o.r0 = __ldg(R);
+        o.r1 = __ldg(R + 1);
+      }
+      s.tab[i] = o;
     }
-  } else {
-    const int k = it - 2 * ms.nb, iw = rank + k * G;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(mm) : "memory");
-    bulk_g2s(dst, a.Tc + (size_t)__ldg(a.tr + a.white[iw]) * M * M, mm, bar);
   }
-}
-
-// wait for the next item; returns its buffer (null on timeout, err set)
-template <typename S>
-__device__ const S* ms_acquire(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>& ms) {
-  const long long i = ms.consumed;
-  const int b = (int)(i % a.nbuf);
-  const unsigned parity = (unsigned)((i / a.nbuf) & 1);
-  __shared__ int ok;
-  if (threadIdx.x == 0) ok = mbar_wait(s.mbar + b, parity) ? 1 : 0;
-  __syncthreads();
-  if (!ok) {
-    if (threadIdx.x == 0) atomicCAS(a.err, 0, 2);  // code 2: a matrix copy did not complete
-    return nullptr;
+  if (s.H && !a.use_strips && a.precond == 2) {
+    using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+    const int d = (int)a.g.d, ld = (d + 3) & ~3, per = (d + a.G - 1) / a.G;
+    const int r0 = min(d, rank * per), cnt = (min(d, r0 + per) - r0) * ld;
+    for (int i = threadIdx.x; i < cnt; i += blockDim.x) const_cast<T*>(s.H)[i] = __ldg(a.H + (size_t)r0 * ld + i);
   }
-  return s.mats + (size_t)b * a.buf_elems;
-}
-
-// done with the current item: the buffer is refilled with item consumed + nbuf
-template <typename S>
-__device__ void ms_release(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>& ms) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  __syncthreads();
-  ++ms.consumed;
-  ms_issue(a, s, ms);
-}
-
-// wait (bounded) for the copies still in flight before the body returns,
-// then invalidate the stream's mbarriers: the shared memory they occupy is
-// reused by the next body of a batched solve.  (A copy that never completed
-// leaves its mbarrier as it is: the caller is unwinding with the error flag
-// set and reuses nothing.)
-template <typename S>
-__device__ void ms_drain(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>& ms) {
-  if (!a.stream_mats) return;
-  bool all_done = true;
-  while (ms.consumed < ms.issued) {
-    const long long i = ms.consumed++;
-    if (threadIdx.x == 0 && !mbar_wait(s.mbar + (i % a.nbuf), (unsigned)((i / a.nbuf) & 1))) all_done = false;
+  if (threadIdx.x < 32) {
+    const DigitMats& D = a.dm;
+    const int t0 = a.res_T > 0 ? main_class(D.tcls, a.white, rank, a.G, a.nown_w, a.nwhite, -1) : -1;
+    int t1 = a.res_T > 1 ? main_class(D.tcls, a.black, rank, a.G, a.nown_b, a.nblack, t0) : -1;
+    const int g0 = a.res_G > 0 ? main_class(D.bcls, nullptr, rank, a.G, a.nown_b, a.nblack, -1) : -1;
+    if (threadIdx.x == 0) *s.res = {p, p + a.res_T * wM, p + (a.res_T + 1) * wM, {t0, t1}, g0};
   }
   __syncthreads();
-  if (threadIdx.x == 0 && all_done)
-    for (int b = 0; b < a.nbuf; ++b)
-      asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(s.mbar + b)) : "memory");
+  const Resident& R = *s.res;
+#pragma unroll 1
+  for (int k = 0; k < a.res_T; ++k)
+    if (R.clsT[k] >= 0)
+      for (size_t i = threadIdx.x; i < wM; i += blockDim.x) p[k * wM + i] = __ldg(a.dm.T + R.clsT[k] * wM + i);
+  if (R.clsG >= 0) {
+    uint4* q = p + a.res_T * wM;
+    for (size_t i = threadIdx.x; i < wG; i += blockDim.x) q[i] = __ldg((a.blk ? a.dm.B : a.dm.G) + R.clsG * wG + i);
+    for (size_t i = threadIdx.x; i < wX; i += blockDim.x) q[wM + i] = __ldg(a.dm.X + R.clsG * wX + i);
+  }
   __syncthreads();
+}
+// no resident matrices (the bodies around GMRES use their place)
+template <typename S>
+__device__ __forceinline__ void no_resident(const GmresArgs<S>& a, const Smem<S>& s) {
+  __syncthreads();
+  load_owned(a, s);
+  if (threadIdx.x == 0) *s.res = {nullptr, nullptr, nullptr, {-1, -1}, -1};
+  __syncthreads();
+}
+
+// packed matrices of a class: resident copy or global memory
+template <typename S>
+__device__ __forceinline__ const uint4* mat_T(const GmresArgs<S>& a, const Smem<S>& s, int cls) {
+  const size_t w = digit_words<S>(a.g.M, a.g.M);
+  const Resident& R = *s.res;
+  return cls == R.clsT[0] ? R.T : cls == R.clsT[1] ? R.T + w : a.dm.T + cls * w;
+}
+template <typename S>
+__device__ __forceinline__ const uint4* mat_G(const GmresArgs<S>& a, const Smem<S>& s, int cls) {
+  return cls == s.res->clsG ? s.res->G : a.dm.G + cls * digit_words<S>(a.g.M, a.g.M);
+}
+template <typename S>
+__device__ __forceinline__ const uint4* mat_B(const GmresArgs<S>& a, const Smem<S>& s, int cls) {
+  return cls == s.res->clsG ? s.res->G : a.dm.B + cls * digit_words<S>(2 * a.g.M, 2 * a.g.M);
+}
+template <typename S>
+__device__ __forceinline__ const uint4* mat_X(const GmresArgs<S>& a, const Smem<S>& s, int cls) {  // four of them
+  return cls == s.res->clsG ? s.res->X : a.dm.X + cls * 4 * digit_words<S>(a.g.n, a.g.n);
 }
 
 // ---- element phases ---------------------------------------------------------
-// Block solve of one black block from the block-slot values vb[0..2M)
-// (already scaled), t = M^-1 v on the block, in two halves around the
-// matrix stream: (1) r1 = p - X q, a = G r1; (2) z = T_e a, write t.
+// P = sc * (own slice, or the global src) of block ib, the k-th of this CTA: 2M
+// values by the W warps of a group (at: the thread's place in it)
 template <typename S>
-__device__ void block_solve_a(const GmresArgs<S>& a, const Smem<S>& s, const S* G, const S* X, const S* vb) {
-  const int M = a.g.M, n = a.g.n;
-  int P = 1;
-  while (P * 2 * M <= (int)blockDim.x && P < 8) P *= 2;
-  const int t = threadIdx.x, r = t % M, part = t / M;
-  if (part < P) {
-    const int F = r / n, tt = r % n;
-    const S* xf = X + (size_t)F * n * n;
-    const S* xq = vb + M + F * n;
-    S acc = 0;
-    for (int c = part; c < n; c += P) acc += xf[c * n + tt] * xq[c];
-    s.red[part * M + r] = acc;
+__device__ __forceinline__ void gather_block(const GmresArgs<S>& a, const S* src, double sc, const S* own, S* P, int ib,
+                                             int k, int at) {
+  const int M = a.g.M, W = a.W_item;
+#pragma unroll 1
+  for (int i0 = at; i0 < 2 * M; i0 += 128 * W) {  // four loads in flight per lane
+    S v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + 32 * W * u;
+      v[u] = S(0);
+      if (i >= 2 * M) continue;
+      if (own) {
+        v[u] = own[k * 2 * M + i];
+      } else {
+        const int sl = block_entry(a, ib, i).x;
+        if (sl >= 0) v[u] = ldcg(src + sl);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + 32 * W * u < 2 * M) P[i0 + 32 * W * u] = (S)(sc * (double)v[u]);
   }
-  __syncthreads();
-  for (int i = t; i < M; i += blockDim.x) {
-    S sum = s.red[i];
-    for (int p = 1; p < P; ++p) sum += s.red[p * M + i];
-    s.r1[i] = vb[i] - sum;
-  }
-  __syncthreads();
-  gemv_split(G, M, s.r1, s.av, M, M, s.red);
 }
 
+// Black block solves of this CTA: block values vb = sc * (own slice, or the
+// global src), r1 = p - X q, a = G r1, z = T_e a, t = [a; q - z], the products
+// in exact fixed point on the tensor cores.
 template <typename S>
-__device__ void block_solve_b(const GmresArgs<S>& a, const Smem<S>& s, int ib, const S* T, const S* vb) {
-  const int M = a.g.M;
-  gemv_split(T, M, s.av, s.z, M, M, s.red);
-  for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) {
-    const int sl = block_entry(a, ib, i).x;
-    if (sl < 0) continue;
-    a.t[sl] = i < M ? s.av[i] : (S)(vb[i] - s.z[i - M]);
+__device__ SMPM_PHASE void black_phase(const GmresArgs<S>& a, const Smem<S>& s, const S* src, double sc, const S* own) {
+  const DevGeo& g = a.g;
+  const DigitMats& D = a.dm;
+  const int M = g.M, n = g.n, W = a.W_item, ngrp = kGmresThreads / 32 / W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int kt_n = digit_tiles(M), kf_n = digit_tiles(n);
+  unsigned char* base = s.wb + (size_t)grp * item_bytes<S>(M, n, a.blk);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  S* P = reinterpret_cast<S*>(base + item_bf_bytes<S>(M, n, a.blk));
+  S* Rr = P + 2 * M;
+#pragma unroll 1
+  for (int k = grp; k < a.nown_b; k += ngrp) {
+    const int ib = team_rank(a) + k * a.G, e = s.ob[k].x, cb = s.ob[k].y, ct = s.ob[k].z;
+    if (e < 0) break;
+    gather_block(a, src, sc, own, P, ib, k, part * 32 + lane);
+    item_sync(grp, W);
+#pragma unroll 1
+    for (int F = part; F < 4; F += W) {  // r1 = p - X q, face by face
+      uint4* Bq = Bf + F * digit_bwords<S>(n);
+      const S* q = P + M + F * n;
+      const int E = pack_one<S>(Bq, q, n, lane, 0, 1);
+#pragma unroll 1
+      for (int mt = 0; mt < kf_n; ++mt) {
+        const S z = digits_tile1<S>(mat_X(a, s, cb) + F * digit_words<S>(n, n), D.Xe + ((size_t)cb * 4 + F) * n,
+                                    Bq, n, kf_n, mt, lane, E);
+        const int row = tile1_row(mt, lane, n);
+        if (row >= 0) Rr[F * n + row] = P[F * n + row] - z;
+      }
+    }
+    item_sync(grp, W);
+    for (int stage = 0; stage < 2; ++stage) {  // a = G r1, then z = T_e a and t = q - z on the facing slots
+      const int E = pack_one<S>(Bf, Rr, M, lane, part, W);
+      const uint4* A = stage == 0 ? mat_G(a, s, cb) : mat_T(a, s, ct);
+      const short* er = stage == 0 ? D.Ge + (size_t)cb * M : D.Te + (size_t)ct * M;
+      item_sync(grp, W);
+#pragma unroll 1
+      for (int mt = part; mt < kt_n; mt += W) {
+        const int row = tile1_row(mt, lane, M);
+        const int sl = row < 0 ? -1 : stage == 0 ? e * M + row : (s.tab ? s.tab[k * 2 * M + M + row].en.x : block_entry(a, ib, M + row).x);
+        const S z = digits_tile1<S>(A, er, Bf, M, kt_n, mt, lane, E);
+        if (stage == 0 && row >= 0) Rr[row] = z;
+        if (sl >= 0) a.t[sl] = stage == 0 ? z : P[M + row] - z;
+      }
+      item_sync(grp, W);
+    }
   }
   __syncthreads();
 }
 
+// The same with the whole inverse of a block, t = [G, -G X; -T G, I + T G X] [p; q]
+// in one product: twice the products and bytes of the three stages above, but
+// one gather, one packing and one product instead of a chain of four (14,000
+// SM cycles for one block of M = 64, the stages' latencies).  Taken where a CTA
+// owns so few blocks that the chain is what it waits for (see block_pays).
 template <typename S>
-__device__ void block_solve(const GmresArgs<S>& a, const Smem<S>& s, int k, int ib, int e, const S* vb) {
-  block_solve_a(a, s, mat_G(a, s, k, ib), mat_X(a, s, k, ib), vb);
-  block_solve_b(a, s, ib, mat_Tb(a, s, k, e), vb);
+__device__ SMPM_PHASE void black_block(const GmresArgs<S>& a, const Smem<S>& s, const S* src, double sc, const S* own) {
+  const DigitMats& D = a.dm;
+  const int M = a.g.M, n = a.g.n, W = a.W_item, ngrp = kGmresThreads / 32 / W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int kt_n = digit_tiles(2 * M);
+  unsigned char* base = s.wb + (size_t)grp * item_bytes<S>(M, n, a.blk);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  S* P = reinterpret_cast<S*>(base + item_bf_bytes<S>(M, n, a.blk));
+#pragma unroll 1
+  for (int k = grp; k < a.nown_b; k += ngrp) {
+    const int ib = team_rank(a) + k * a.G, e = s.ob[k].x, cb = s.ob[k].y;
+    if (e < 0) break;
+    gather_block(a, src, sc, own, P, ib, k, part * 32 + lane);
+    item_sync(grp, W);
+    const int E = pack_one<S>(Bf, P, 2 * M, lane, part, W);
+    item_sync(grp, W);
+#pragma unroll 1
+    for (int mt = part; mt < kt_n; mt += W) {
+      const int row = tile1_row(mt, lane, 2 * M);
+      const int sl = row < 0 ? -1 : row < M ? e * M + row : (s.tab ? s.tab[k * 2 * M + row].en.x : block_entry(a, ib, row).x);
+      const S z = digits_tile1<S>(mat_B(a, s, cb), D.Be + (size_t)cb * 2 * M, Bf, 2 * M, kt_n, mt, lane, E);
+      if (sl >= 0) a.t[sl] = z;
+    }
+    item_sync(grp, W);
+  }
+  __syncthreads();
 }
 
-// White element: y = S t on the black slots facing e, y = sc*v on e's slots,
+// What a white element's row needs besides its product: v on the own slot, t on
+// the facing slot sl (-1 on the physical boundary) and the weights of both in
+// the deflation vector.
+template <typename S>
+struct Facing {
+  int sl;
+  S v, t;
+  double w0, w1;
+};
+template <typename S>
+__device__ __forceinline__ Facing<S> facing_entry(const DevGeo& g, int e, int row, const S* v, const S* t) {
+  const int M = g.M, n = g.n, F = row / n, tt = row - F * n, e2 = dev_neighbour(g, e, F);
+  Facing<S> f;
+  f.sl = e2 >= 0 ? e2 * M + (F ^ 1) * n + tt : -1;
+  f.v = ldcg(v + (size_t)e * M + row);
+  f.t = e2 >= 0 ? ldcg(t + f.sl) : S(0);
+  f.w0 = g.zw && e2 >= 0 ? dev_zw(g, e, F) : 1.0;
+  f.w1 = g.zw && e2 >= 0 ? dev_zw(g, e2, F ^ 1) : 1.0;
+  return f;
+}
+// the row's share of c = Z^T y (uniform grids: weights 1, no multiplication)
+template <typename S>
+__device__ __forceinline__ double facing_c(const DevGeo& g, const Facing<S>& f, S vo, S ys) {
+  return g.zw ? f.w0 * (double)vo + f.w1 * (double)ys : (double)vo + (double)ys;
+}
+
+// White elements: y = S t on the black slots facing e, y = sc*v on e's slots,
 // c = Z^T y on e's interfaces (with_c).
 template <typename S>
-__device__ void white_step(const GmresArgs<S>& a, const Smem<S>& s, const S* Tw, int e, const S* v, double sc,
-                           bool with_c, int kstage = -1) {
+__device__ SMPM_PHASE void white_phase(const GmresArgs<S>& a, const Smem<S>& s, const S* v, double sc, bool with_c) {
   const DevGeo& g = a.g;
-  const int M = g.M, n = g.n;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) s.p[i] = ldcg(a.t + (size_t)e * M + i);
-  __syncthreads();
-  gemv_split(Tw, M, s.p, s.z, M, M, s.red);
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    int F = i / n, tt = i % n;
-    int e2 = dev_neighbour(g, e, F);
-    S vo = (S)(sc * (double)ldcg(v + (size_t)e * M + i));
-    a.y[(size_t)e * M + i] = vo;
-    double ci = 0;
-    if (e2 >= 0) {
-      size_t sl = (size_t)e2 * M + (F ^ 1) * n + tt;
-      S ys = ldcg(a.t + sl) + s.z[i];
-      a.y[sl] = ys;
-      ci = g.zw ? dev_zw(g, e, F) * (double)vo + dev_zw(g, e2, F ^ 1) * (double)ys : (double)vo + (double)ys;
+  const DigitMats& D = a.dm;
+  const int M = g.M, n = g.n, W = a.W_item, ngrp = kGmresThreads / 32 / W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int kt_n = digit_tiles(M);
+  unsigned char* base = s.wb + (size_t)grp * item_bytes<S>(M, n, a.blk);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  double* ci = reinterpret_cast<double*>(base + item_bf_bytes<S>(M, n, a.blk));  // contributions to c
+  S* te = reinterpret_cast<S*>(ci + M);                                   // t on e's slots
+#pragma unroll 1
+  for (int k = grp; k < a.nown_w; k += ngrp) {
+    const int e = s.ow[k].x, ct = s.ow[k].y;
+    if (e < 0) break;
+    Facing<S> f{};
+    if (part < kt_n && tile1_row(part, lane, M) >= 0) f = facing_entry(g, e, tile1_row(part, lane, M), v, a.t);
+    for (int i = part * 32 + lane; i < M; i += 32 * W) te[i] = ldcg(a.t + (size_t)e * M + i);
+    item_sync(grp, W);
+    const int E = pack_one<S>(Bf, te, M, lane, part, W);
+    item_sync(grp, W);
+#pragma unroll 1
+    for (int mt = part; mt < kt_n; mt += W) {
+      const int row = tile1_row(mt, lane, M);
+      if (row >= 0 && mt != part) f = facing_entry(g, e, row, v, a.t);
+      const S z = digits_tile1<S>(mat_T(a, s, ct), D.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E);
+      if (row < 0) continue;
+      const S vo = (S)(sc * (double)f.v);
+      a.y[(size_t)e * M + row] = vo;
+      double c1 = 0;
+      if (f.sl >= 0) {
+        const S ys = f.t + z;
+        a.y[f.sl] = ys;
+        c1 = facing_c(g, f, vo, ys);
+      }
+      ci[row] = c1;
     }
-    s.cs[i] = ci;
-  }
-  __syncthreads();
-  if (with_c && threadIdx.x < 128) {  // face F summed by warp F
-    const int F = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double sum = 0;
-    for (int tt = lane; tt < n; tt += 32) sum += s.cs[F * n + tt];
-    sum = warp_sum(sum);
-    const int j = dev_iface(g, e, F);
-    if (lane == 0 && j >= 0) a.c[j] = sum;
-    if (lane == 0 && kstage >= 0) {
-      s.cpv[kstage * 4 + F] = sum;
-      s.cpj[kstage * 4 + F] = j;
+    item_sync(grp, W);
+    if (with_c && part == 0) {  // face F summed by the eight lanes 8 F + r
+      const int F = lane >> 3, j = dev_iface(g, e, F);
+      double sum = 0;
+#pragma unroll 1
+      for (int tt = lane & 7; tt < n; tt += 8) sum += ci[F * n + tt];
+#pragma unroll 1
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if ((lane & 7) == 0 && j >= 0) a.c[j] = sum;
     }
+    item_sync(grp, W);
   }
   __syncthreads();
 }
 
-// Push form y = S (sc*v) for element e (Algorithm 1).
+// Push form y = S (sc*v) (Algorithm 1): elements rank, rank + G, ...
 template <typename S>
-__device__ void push_step(const GmresArgs<S>& a, const Smem<S>& s, int e, const S* v, double sc) {
+__device__ SMPM_PHASE void push_phase(const GmresArgs<S>& a, const Smem<S>& s, const S* v, double sc) {
   const DevGeo& g = a.g;
-  const int M = g.M, n = g.n;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) s.p[i] = (S)(sc * (double)ldcg(v + (size_t)e * M + i));
-  __syncthreads();
-  gemv_split(a.Tc + (size_t)__ldg(a.tr + e) * M * M, M, s.p, s.z, M, M, s.red);
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    int F = i / n, tt = i % n;
-    int e2 = dev_neighbour(g, e, F);
-    if (e2 >= 0) {
-      size_t sl = (size_t)e2 * M + (F ^ 1) * n + tt;
-      a.y[sl] = (S)(sc * (double)ldcg(v + sl)) + s.z[i];
-    } else {
-      a.y[(size_t)e * M + i] = s.p[i];
+  const DigitMats& D = a.dm;
+  const int M = g.M, n = g.n, W = a.W_item, ngrp = kGmresThreads / 32 / W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W;
+  const int kt_n = digit_tiles(M);
+  unsigned char* base = s.wb + (size_t)grp * item_bytes<S>(M, n, a.blk);
+  uint4* Bf = reinterpret_cast<uint4*>(base);
+  S* ve = reinterpret_cast<S*>(base + item_bf_bytes<S>(M, n, a.blk));
+#pragma unroll 1
+  for (long long el = team_rank(a) + (long long)grp * a.G; el < g.nel; el += (long long)ngrp * a.G) {
+    const int e = (int)el, ct = __ldg(D.tcls + e);
+    for (int i = part * 32 + lane; i < M; i += 32 * W) ve[i] = (S)(sc * (double)ldcg(v + (size_t)e * M + i));
+    item_sync(grp, W);
+    const int E = pack_one<S>(Bf, ve, M, lane, part, W);
+    item_sync(grp, W);
+#pragma unroll 1
+    for (int mt = part; mt < kt_n; mt += W) {
+      const int row = tile1_row(mt, lane, M);
+      Facing<S> f{};
+      if (row >= 0) f = facing_entry(g, e, row, v, v);
+      const S z = digits_tile1<S>(mat_T(a, s, ct), D.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E);
+      if (row < 0) continue;
+      if (f.sl >= 0) a.y[f.sl] = (S)(sc * (double)f.t) + z;
+      else a.y[(size_t)e * M + row] = ve[row];
     }
+    item_sync(grp, W);
   }
   __syncthreads();
-}
-
-// c_hat = H c: CTA c takes a contiguous range of rows; c is staged in shared
-// memory and P lanes split each row (H row-major: lanes read consecutive
-// columns), partial sums meet in warp shuffles.  Each lane keeps eight loads
-// in flight (16-byte loads when rows start 16-byte aligned, i.e. d even), so
-// that a matrix larger than L2 streams at HBM rate; such a matrix is read
-// with the evict-first hint, which keeps the Krylov basis resident in L2.
-__device__ __forceinline__ double2 ld_h2(const double* p, bool stream) {
-  return stream ? __ldcs(reinterpret_cast<const double2*>(p)) : __ldg(reinterpret_cast<const double2*>(p));
-}
-__device__ __forceinline__ double ld_h1(const double* p, bool stream) { return stream ? __ldcs(p) : __ldg(p); }
-
-// The FP32 inner solves of the mixed-precision path apply the coarse
-// inverse in FP32 (its FP32 copy, FP32 products and sums): an inner solve
-// needs only a relative 1e-4, and every refinement sweep recomputes the
-// residual in FP64.
-__device__ void coarse_rows32(const float* __restrict__ H32, const double* c, double* chat, int d, int r0, int r1,
-                              float* cf) {
-  for (int j = threadIdx.x; j < d; j += blockDim.x) cf[j] = (float)__ldcg(c + j);
-  __syncthreads();
-  const int rows = r1 - r0;
-  int P = 32;
-  while (P > 1 && P * rows > 2 * (int)blockDim.x) P >>= 1;
-  const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
-  const bool vec = (d & 3) == 0;  // rows start 16-byte aligned
-  for (int rb = 0; rb < rows; rb += ngrp) {
-    const int r = r0 + rb + grp;
-    float sum = 0.f;
-    if (r < r1) {
-      const float* hr = H32 + (size_t)r * d;
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-      int j = vec ? 4 * lane : lane;
-      if (vec) {
-        for (; j + 28 * P < d; j += 32 * P) {
-          float4 h[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) h[u] = __ldg(reinterpret_cast<const float4*>(hr + j + 4 * u * P));
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int jj = j + 4 * u * P;
-            acc[u & 3] += h[u].x * cf[jj] + h[u].y * cf[jj + 1] + h[u].z * cf[jj + 2] + h[u].w * cf[jj + 3];
-          }
-        }
-        for (; j < d; j += 4 * P) {
-          const float4 h = __ldg(reinterpret_cast<const float4*>(hr + j));
-          acc[0] += h.x * cf[j] + h.y * cf[j + 1] + h.z * cf[j + 2] + h.w * cf[j + 3];
-        }
-      } else {
-        for (; j + 7 * P < d; j += 8 * P) {
-          float h[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) h[u] = __ldg(hr + j + u * P);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u & 3] += h[u] * cf[j + u * P];
-        }
-        for (; j < d; j += P) acc[0] += __ldg(hr + j) * cf[j];
-      }
-      sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-    }
-    for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, P);
-    if (lane == 0 && r < r1) chat[r] = (double)sum;
-  }
-}
-
-template <typename S>
-__device__ void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s) {
-  const int d = (int)a.g.d;
-  const int per = (d + a.G - 1) / a.G;
-  const int r0 = team_rank(a) * per, r1 = min(d, r0 + per);
-  if (r0 >= r1) return;
-  if constexpr (sizeof(S) == 4) {
-    coarse_rows32(a.H, a.c, a.chat, d, r0, r1, reinterpret_cast<float*>(s.cst));
-    return;
-  } else {
-  for (int j = threadIdx.x; j < d; j += blockDim.x) s.cst[j] = __ldcg(a.c + j);
-  __syncthreads();
-  const bool stream = (size_t)d * d * sizeof(double) > ((size_t)48 << 20);
-  const bool vec = (d & 1) == 0;
-  const int rows = r1 - r0;
-  int P = 32;
-  while (P > 1 && P * rows > 2 * (int)blockDim.x) P >>= 1;
-  const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
-  const double* cs = s.cst;
-  for (int rb = 0; rb < rows; rb += ngrp) {  // uniform trip count per warp
-    const int r = r0 + rb + grp;
-    double sum = 0;
-    if (r < r1) {
-      const double* hr = a.H + (size_t)r * d;
-      double acc[4] = {0, 0, 0, 0};
-      if (vec) {
-        int j = 2 * lane;
-        for (; j + 30 * P < d; j += 32 * P) {
-          double2 h[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u) h[u] = ld_h2(hr + j + 2 * u * P, stream);
-#pragma unroll
-          for (int u = 0; u < 16; ++u) {
-            const int jj = j + 2 * u * P;
-            acc[u & 3] += h[u].x * cs[jj] + h[u].y * cs[jj + 1];
-          }
-        }
-        for (; j < d; j += 2 * P) {
-          const double2 h = ld_h2(hr + j, stream);
-          acc[0] += h.x * cs[j] + h.y * cs[j + 1];
-        }
-      } else {
-        int j = lane;
-        for (; j + 7 * P < d; j += 8 * P) {
-          double h[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) h[u] = ld_h1(hr + j + u * P, stream);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) acc[u & 3] += h[u] * cs[j + u * P];
-        }
-        for (; j < d; j += P) acc[0] += ld_h1(hr + j, stream) * cs[j];
-      }
-      sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-    }
-    for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, P);
-    if (lane == 0 && r < r1) a.chat[r] = sum;
-  }
-  }
 }
 
 // ---- C^+ by strips ----------------------------------------------------------
@@ -637,12 +660,14 @@ __device__ void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s) {
 // multiple of c0, which S Z maps to zero and the zero mean of u removes).
 // About d^2 / 7 products instead of d^2, in three phases of short dot
 // products with two more barriers (see strips_pay on when that is less).
+template <bool SM>  // SM: from shared memory
 __device__ __forceinline__ void ld_vec(const double* p, double (&v)[2]) {
-  const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+  const double2 t = SM ? *reinterpret_cast<const double2*>(p) : __ldg(reinterpret_cast<const double2*>(p));
   v[0] = t.x; v[1] = t.y;
 }
+template <bool SM>
 __device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
-  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  const float4 t = SM ? *reinterpret_cast<const float4*>(p) : __ldg(reinterpret_cast<const float4*>(p));
   v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
 }
 
@@ -651,13 +676,14 @@ __device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
 // padded length); put(r, sum) takes the dot product (len 0: no call).  P lanes
 // per row, P as large as the rows leave threads for, but 4 at least: each
 // halving step of the final sums costs as much FP64 time as a product.
-template <typename T, typename Get, typename Put>
+template <typename T, bool SM = false, typename Get, typename Put>
 __device__ __forceinline__ void row_dots(int r0, int r1, Get&& get, Put&& put) {
   constexpr int V = 16 / (int)sizeof(T), U = 4;
   const int rows = r1 - r0;
   int P = 32;
   while (P > 4 && P * rows > (int)blockDim.x) P >>= 1;
   const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
+#pragma unroll 1
   for (int rb = 0; rb < rows; rb += ngrp) {  // uniform trip count per warp
     const int r = r0 + rb + grp;
     const T* a = nullptr;
@@ -666,31 +692,34 @@ __device__ __forceinline__ void row_dots(int r0, int r1, Get&& get, Put&& put) {
     if (r < r1) get(r, a, x, len);
     T acc[4] = {T(0), T(0), T(0), T(0)};
     int j = V * lane;
+#pragma unroll 1
     for (; j + V * P * (U - 1) < len; j += V * P * U) {
       T h[U][V];
 #pragma unroll
-      for (int u = 0; u < U; ++u) ld_vec(a + j + u * V * P, h[u]);
+      for (int u = 0; u < U; ++u) ld_vec<SM>(a + j + u * V * P, h[u]);
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[u] += h[u][v] * x[j + u * V * P + v];
     }
+#pragma unroll 1
     for (; j < len; j += V * P) {
       T h[V];
-      ld_vec(a + j, h);
+      ld_vec<SM>(a + j, h);
 #pragma unroll
       for (int v = 0; v < V; ++v) acc[v & 3] += h[v] * x[j + v];
     }
     T sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll 1
     for (int o = P / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o, P);
     if (lane == 0 && len > 0) put(r, sum);
   }
 }
 
-// c_hat = C^+ c (a.c -> a.chat), complete after the final barrier; false when a
+// c_hat = C^+ c, complete after the final barrier; false when a
 // barrier timed out.  cst: staging for at least d + 1 entries.
 template <typename S>
-__device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsigned& epoch) {
+__device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsigned& epoch, const double* c, double* chat) {
   using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
   constexpr int V = 16 / (int)sizeof(T);
   T* xs = reinterpret_cast<T*>(cst);
@@ -702,7 +731,7 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
     const int n1 = k.p * RS, per = (n1 + G - 1) / G, r0 = min(n1, rank * per), r1 = min(n1, r0 + per);
     if (r0 < r1) {
       const int b0 = (r0 / RS) * srow, b1 = min(d, ((r1 - 1) / RS + 1) * srow);
-      for (int j = threadIdx.x; j < b1 - b0 + V; j += blockDim.x) xs[j] = b0 + j < b1 ? (T)__ldcg(a.c + b0 + j) : T(0);
+      for (int j = threadIdx.x; j < b1 - b0 + V; j += blockDim.x) xs[j] = b0 + j < b1 ? (T)__ldcg(c + b0 + j) : T(0);
       __syncthreads();
       row_dots<T>(
           r0, r1,
@@ -715,11 +744,11 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
           },
           [&](int r, T sum) {
             const int i = r / RS, l = r - i * RS;
-            if (l < k.m) a.chat[i * srow + l] = (double)sum;
+            if (l < k.m) chat[i * srow + l] = (double)sum;
             else a.gsep[2 * (size_t)i * k.mx + (l - k.m)] = (double)sum;
           });
     }
-    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+    if (!team_sync(a, epoch)) return false;
   }
   {  // P2: rows 0 .. ns-1 of H_ss, row ns: u_C on the separators
     const int n2 = k.ns + 1, per = (n2 + G - 1) / G, r0 = min(n2, rank * per), r1 = min(n2, r0 + per);
@@ -729,7 +758,7 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
         if (j < k.ns) {
           const int sp = j / k.mx, q = j - sp * k.mx;
           const double* up = a.gsep + (2 * (size_t)sp + 1) * k.mx + q;  // strip below; lower sums of the one above
-          v = (T)(__ldcg(a.c + (sp + 1) * srow - k.mx + q) - __ldcg(up) - __ldcg(up + k.mx));
+          v = (T)(__ldcg(c + (sp + 1) * srow - k.mx + q) - __ldcg(up) - __ldcg(up + k.mx));
         }
         xs[j] = v;
       }
@@ -743,10 +772,10 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
           },
           [&](int r, T sum) {
             if (r == k.ns) *alpha = (double)sum;
-            else a.chat[(r / k.mx + 1) * srow - k.mx + r % k.mx] = (double)sum;
+            else chat[(r / k.mx + 1) * srow - k.mx + r % k.mx] = (double)sum;
           });
     }
-    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+    if (!team_sync(a, epoch)) return false;
   }
   {  // P3: rows of W: 2 mx coefficients of the separators below and above, then C_ii^-1 u_C,i
     const int n3 = k.p * k.m, per = (n3 + G - 1) / G, r0 = min(n3, rank * per), r1 = min(n3, r0 + per);
@@ -754,7 +783,7 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
       const int i0 = r0 / k.m, i1 = (r1 - 1) / k.m;  // separators i0 - 1 .. i1
       for (int j = threadIdx.x; j < (i1 - i0 + 2) * k.mx + V; j += blockDim.x) {
         const int sp = i0 - 1 + j / k.mx;
-        xs[j] = (sp >= 0 && sp < k.p - 1 && sp <= i1) ? (T)__ldcg(a.chat + (sp + 1) * srow - k.mx + j % k.mx) : T(0);
+        xs[j] = (sp >= 0 && sp < k.p - 1 && sp <= i1) ? (T)__ldcg(chat + (sp + 1) * srow - k.mx + j % k.mx) : T(0);
       }
       const double al = __ldcg(alpha);
       __syncthreads();
@@ -768,21 +797,57 @@ __device__ SMPM_BODY bool coarse_strips(const GmresArgs<S>& a, void* cst, unsign
           },
           [&](int r, T sum) {
             const int i = r / k.m;
-            double* out = a.chat + i * srow + (r - i * k.m);
+            double* out = chat + i * srow + (r - i * k.m);
             *out = __ldcg(out) - al * (double)k.z[r] - (double)sum;
           });
     }
   }
-  return grid_sync(a.bar, a.err, epoch, G);
+  return team_sync(a, epoch);
+}
+
+// c_hat = H c by rows: the CTA takes a contiguous range of them, c staged in
+// shared memory.  The FP32 inner solves of the mixed-precision path use the
+// FP32 copy with FP32 products and sums: an inner solve needs only a relative
+// 1e-4, and every refinement sweep recomputes the residual in FP64.
+template <typename S>
+__device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, const double* c, double* chat) {
+  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+  T* xs = reinterpret_cast<T*>(s.cst);
+  const int d = (int)a.g.d, ld = (d + 3) & ~3, per = (d + a.G - 1) / a.G;
+  const int r0 = min(d, team_rank(a) * per), r1 = min(d, r0 + per);
+  if (r0 >= r1) return;
+  for (int j = threadIdx.x; j < d + 16 / (int)sizeof(T); j += blockDim.x) xs[j] = j < d ? (T)__ldcg(c + j) : T(0);
+  __syncthreads();
+  auto put = [&](int r, T sum) { chat[r] = (double)sum; };
+  if (s.H) {
+    row_dots<T, true>(
+        r0, r1,
+        [&](int r, const T*& row, const T*& x, int& len) {
+          row = s.H + (size_t)(r - r0) * ld;
+          x = xs;
+          len = d;
+        },
+        put);
+  } else {
+    row_dots<T>(
+        r0, r1,
+        [&](int r, const T*& row, const T*& x, int& len) {
+          row = a.H + (size_t)r * ld;
+          x = xs;
+          len = d;
+        },
+        put);
+  }
 }
 
 // c_hat = C^+ c by all CTAs of the team (strips or dense rows), complete after
 // its last barrier; false when a barrier timed out
 template <typename S>
-__device__ __forceinline__ bool coarse_solve(const GmresArgs<S>& a, const Smem<S>& s, unsigned& epoch) {
-  if (a.use_strips) return coarse_strips(a, s.cst, epoch);
-  coarse_rows(a, s);
-  return grid_sync(a.bar, a.err, epoch, a.G);
+__device__ __forceinline__ bool coarse_solve(const GmresArgs<S>& a, const Smem<S>& s, unsigned& epoch, const double* c,
+                                             double* chat) {
+  if (a.use_strips) return coarse_strips(a, s.cst, epoch, c, chat);
+  coarse_rows(a, s, c, chat);
+  return team_sync(a, epoch);
 }
 
 // ys - (S Z chat) at an entry (pull form); 0 on the physical boundary, ys
@@ -802,12 +867,13 @@ __device__ __forceinline__ double deflate_entry(const GmresArgs<A>& a, const S* 
   return deflate_value(a, en.x >= 0 ? (double)ldcg(y + en.x) : 0.0, chat, en);
 }
 
+// ---- Gram-Schmidt passes over the CTA's slice of the basis ---------------
 // Dot products of the owned basis slice with vec (ES entries) for l < nl,
 // l == nl - 1 giving vec.vec: P lanes per l (P a power of two <= 32, P*nl <=
 // blockDim when possible) read consecutive entries; partial sums meet in warp
 // shuffles and are added atomically to out[l] (FP64, in L2).
 template <typename S>
-__device__ void owned_dots(const GmresArgs<S>& a, const Smem<S>& s, const S* vec, int nl, double* out) {
+__device__ SMPM_PHASE void owned_dots(const GmresArgs<S>& a, const Smem<S>& s, const S* vec, int nl, double* out) {
   const int E = a.ES;
   int P = 32;
   while (P > 1 && P * nl > (int)blockDim.x) P >>= 1;
@@ -816,7 +882,7 @@ __device__ void owned_dots(const GmresArgs<S>& a, const Smem<S>& s, const S* vec
     const int l = lb + grp;
     double sum = 0;
     if (l < nl) {
-      const S* vl = (l == nl - 1) ? vec : basis(a, s, l);
+      const S* vl = (l == nl - 1) ? vec : (s.V + (size_t)l * a.ES);
       // eight entries per step, loaded before they are used: with the basis
       // in global memory each lane keeps eight independent loads in flight
       if constexpr (sizeof(S) == 4) {
@@ -870,330 +936,115 @@ __device__ __forceinline__ double basis_combo(const GmresArgs<S>& a, const Smem<
                                               int nl, int i) {
   if constexpr (sizeof(S) == 4) {
     float r = (float)base;
-    for (int l = 0; l < nl; ++l) r = fmaf(-(float)coef[l], (float)basis(a, s, l)[i], r);
+    for (int l = 0; l < nl; ++l) r = fmaf(-(float)coef[l], (float)(s.V + (size_t)l * a.ES)[i], r);
     return (double)r;
   } else {
     double r = base;
-    for (int l = 0; l < nl; ++l) r -= coef[l] * (double)basis(a, s, l)[i];
+    for (int l = 0; l < nl; ++l) r -= coef[l] * (double)(s.V + (size_t)l * a.ES)[i];
     return r;
   }
 }
 
-// owned entry i of the CTA: block rank + k G, entry i - 2M k of it
-template <typename S>
-__device__ __forceinline__ int4 owned_entry(const GmresArgs<S>& a, int i) {
-  const int M2 = 2 * a.g.M, k = i / M2, ib = team_rank(a) + k * a.G;
-  if (k >= a.nown_b || ib >= a.nblack) return make_int4(-1, 0, -1, 0);
-  return block_entry(a, ib, i - k * M2);
-}
-template <typename S>
-__device__ __forceinline__ int entry_slot(const GmresArgs<S>& a, int i) {
-  return owned_entry(a, i).x;
-}
-
-// ---- warp-per-element phases -------------------------------------------
-// z[r] = sum_c A[c*M + r] x[c] for r < M by one warp: lane l owns rows
-// l, l+32, ... (up to NR of them, M <= 32 NR); A column-major in shared or
-// global memory (read-only), U columns per step with all their loads issued
-// first (U NR independent loads per lane in flight: from global memory each
-// step is one round trip); x and z in the warp's shared scratch.  Ends with
-// __syncwarp.
-template <typename S, int U, int NR>
-__device__ __forceinline__ void warp_gemv_u(const S* A, const S* x, S* z, int M, int lane) {
-  S acc[NR];
-#pragma unroll
-  for (int j = 0; j < NR; ++j) acc[j] = S(0);
-  const int nr = (M - lane + 31) / 32;  // rows of this lane (0..NR)
-  int c = 0;
-  for (; c + U <= M; c += U) {
-    S av[U][NR];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int j = 0; j < NR; ++j) av[u][j] = j < nr ? A[(size_t)(c + u) * M + lane + 32 * j] : S(0);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const S xc = x[c + u];
-#pragma unroll
-      for (int j = 0; j < NR; ++j) acc[j] += av[u][j] * xc;
-    }
-  }
-  for (; c < M; ++c) {
-    const S xc = x[c];
-#pragma unroll
-    for (int j = 0; j < NR; ++j)
-      if (j < nr) acc[j] += A[(size_t)c * M + lane + 32 * j] * xc;
-  }
-#pragma unroll
-  for (int j = 0; j < NR; ++j)
-    if (j < nr) z[lane + 32 * j] = acc[j];
-  __syncwarp();
-}
-
-template <typename S>
-__device__ __forceinline__ void warp_gemv(const S* A, const S* x, S* z, int M, int lane) {
-  // lane owns rows lane + 32 j; U columns of loads are issued before their
-  // FMAs, so a warp keeps U * NR loads in flight (M <= 64: 16 columns x 2
-  // rows, else 8 x 4): matrices streamed from HBM need the bytes in flight
-  // more than the FP64 pipe needs short chains
-  if (M <= 64)
-    warp_gemv_u<S, 16, 2>(A, x, z, M, lane);
-  else
-    warp_gemv_u<S, 8, 4>(A, x, z, M, lane);
-}
-
-// Black block solves with one warp per owned block (blocks k = warp,
-// warp + nwarps, ...): vb = sc * (own slice or src), r1 = p - X q, a = G r1,
-// z = T_e a, t = [a; q - z] on the block's slots.
-template <typename S>
-__device__ void black_phase_warps(const GmresArgs<S>& a, const Smem<S>& s, const S* src, double sc, const S* own) {
-  const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  S* p = s.wb + (size_t)warp * warp_scratch(M);
-  S* q = p + M;
-  S* r1 = q + M;
-  S* av = r1 + M;
-  S* z = av + M;
-  for (int k = warp; k < a.nown_b; k += nwarps) {
-    const int ib = rank + k * G;
-    if (ib >= a.nblack) break;
-    const int e = a.black[ib];
-    for (int i = lane; i < 2 * M; i += 32) {
-      S v;
-      if (own) {
-        v = (S)(sc * (double)own[k * 2 * M + i]);
-      } else {
-        const int sl = block_entry(a, ib, i).x;
-        v = sl >= 0 ? (S)(sc * (double)ldcg(src + sl)) : S(0);
-      }
-      p[i] = v;  // p and q are contiguous: q = p + M
-    }
-    __syncwarp();
-    const S* X = mat_X(a, s, k, ib);
-    for (int i = lane; i < M; i += 32) {
-      const int F = i / n, t = i % n;
-      const S* xf = X + (size_t)F * n * n;
-      S acc = 0;
-      for (int c = 0; c < n; ++c) acc += xf[c * n + t] * q[F * n + c];
-      r1[i] = p[i] - acc;
-    }
-    __syncwarp();
-    warp_gemv(mat_G(a, s, k, ib), r1, av, M, lane);
-    warp_gemv(mat_Tb(a, s, k, e), av, z, M, lane);
-    for (int i = lane; i < 2 * M; i += 32) {
-      const int sl = block_entry(a, ib, i).x;
-      if (sl >= 0) a.t[sl] = i < M ? av[i] : (S)(q[i - M] - z[i - M]);
-    }
-    __syncwarp();
-  }
-  __syncthreads();
-}
-
-// White elements with one warp per element: y = S t on the black slots
-// facing e, y = sc*v on e's slots, c = Z^T y on e's interfaces (with_c).
-template <typename S>
-__device__ void white_phase_warps(const GmresArgs<S>& a, const Smem<S>& s, const S* v, double sc, bool with_c,
-                                  bool stage = false) {
-  const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, G = a.G, rank = team_rank(a);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  S* p = s.wb + (size_t)warp * warp_scratch(M);
-  S* z = p + M;
-  double* ci = reinterpret_cast<double*>(z + M + (M & 1));  // M doubles (within the 5M scratch for S = float
-                                                             // and for S = double)
-  for (int k = warp; k < a.nown_w; k += nwarps) {
-    const int iw = rank + k * G;
-    if (iw >= a.nwhite) break;
-    const int e = a.white[iw];
-    for (int i = lane; i < M; i += 32) p[i] = ldcg(a.t + (size_t)e * M + i);
-    __syncwarp();
-    warp_gemv(mat_Tw(a, s, k, e), p, z, M, lane);
-    for (int i = lane; i < M; i += 32) {
-      const int F = i / n, tt = i % n, e2 = dev_neighbour(g, e, F);
-      const S vo = (S)(sc * (double)ldcg(v + (size_t)e * M + i));
-      a.y[(size_t)e * M + i] = vo;
-      double c1 = 0;
-      if (e2 >= 0) {
-        const size_t sl = (size_t)e2 * M + (F ^ 1) * n + tt;
-        const S ys = ldcg(a.t + sl) + z[i];
-        a.y[sl] = ys;
-        c1 = g.zw ? dev_zw(g, e, F) * (double)vo + dev_zw(g, e2, F ^ 1) * (double)ys : (double)vo + (double)ys;
-      }
-      ci[i] = c1;
-    }
-    __syncwarp();
-    if (with_c && lane < 4) {  // face F summed by lane F
-      const int F = lane, j = dev_iface(g, e, F);
-      double sum = 0;
-      if (j >= 0) {
-        for (int tt = 0; tt < n; ++tt) sum += ci[F * n + tt];
-        a.c[j] = sum;
-      }
-      if (stage) {
-        s.cpv[k * 4 + F] = sum;
-        s.cpj[k * 4 + F] = j;
-      }
-    }
-    __syncwarp();
-  }
-  __syncthreads();
-}
-
-// black block solves of this CTA from the global vector sc * src
-template <typename S>
-__device__ bool black_phase(const GmresArgs<S>& a, const Smem<S>& s, MatStream<S>* ms, const S* src, double sc,
-                            const S* own) {
-  if (a.warp_elems) {
-    black_phase_warps(a, s, src, sc, own);
-    return true;
-  }
-  const DevGeo& g = a.g;
-  const int M = g.M, G = a.G;
-  for (int k = 0; k < a.nown_b; ++k) {
-    int ib = team_rank(a) + k * G;
-    if (ib >= a.nblack) break;
-    int e = a.black[ib];
-    for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) {
-      if (own) {
-        s.w[i] = (S)(sc * (double)own[k * 2 * M + i]);
-      } else {
-        const int sl = block_entry(a, ib, i).x;
-        s.w[i] = sl >= 0 ? (S)(sc * (double)ldcg(src + sl)) : S(0);
-      }
-    }
-    __syncthreads();
-    if (ms) {
-      const S* GX = ms_acquire(a, s, *ms);
-      if (!GX) return false;
-      block_solve_a(a, s, GX, GX + (size_t)M * M, s.w);
-      ms_release(a, s, *ms);
-      const S* T = ms_acquire(a, s, *ms);
-      if (!T) return false;
-      block_solve_b(a, s, ib, T, s.w);
-      ms_release(a, s, *ms);
-    } else {
-      block_solve(a, s, k, ib, e, s.w);
-    }
-  }
-  return true;
-}
-
 // op(sc * src) -> y (and c, chat).  With t_done the owners have already
-// written t = M^-1 v for their blocks.  With chat_acc (fused coarse solve,
-// Algorithm 3 only) the white phase also adds H[:, j] c_j for the interfaces
-// of the CTA's white elements into chat_acc (zero on entry), and there is no
-// separate coarse phase: c_hat is complete after the white phase's barrier.
+// written t = M^-1 v for their blocks.
 template <typename S>
-__device__ bool apply_op(const GmresArgs<S>& a, const Smem<S>& s, const S* src, double sc, bool t_done,
-                         int& trace_n, unsigned& epoch, MatStream<S>* ms = nullptr, double* chat_acc = nullptr) {
-  const DevGeo& g = a.g;
-  const int G = a.G;
+__device__ SMPM_PHASE bool apply_op(const GmresArgs<S>& a, const Smem<S>& s, const S* src, double sc, bool t_done,
+                         int& trace_n, unsigned& epoch) {
   if (a.precond == 0) {
-    for (long long e = team_rank(a); e < g.nel; e += G) push_step(a, s, (int)e, src, sc);
-    return grid_sync(a.bar, a.err, epoch, a.G);
+    push_phase(a, s, src, sc);
+    return team_sync(a, epoch);
   }
-  if (!t_done && !black_phase(a, s, ms, src, sc, (const S*)nullptr)) return false;
+  if (!t_done) {
+    if (a.blk) black_block(a, s, src, sc, (const S*)nullptr);
+    else black_phase(a, s, src, sc, (const S*)nullptr);
+  }
   GM_TRACE(20);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(21);
-  const bool fuse = chat_acc && a.precond == 2;
-  if (fuse)
-    for (int q = threadIdx.x; q < 4 * a.nown_w; q += blockDim.x) s.cpj[q] = -1;
-  __syncthreads();
-  if (a.warp_elems) white_phase_warps(a, s, src, sc, a.precond == 2, fuse);
-  for (int k = 0; k < (a.warp_elems ? 0 : a.nown_w); ++k) {
-    int iw = team_rank(a) + k * G;
-    if (iw >= a.nwhite) break;
-    if (ms) {
-      const S* T = ms_acquire(a, s, *ms);
-      if (!T) return false;
-      white_step(a, s, T, a.white[iw], src, sc, a.precond == 2, fuse ? k : -1);
-      ms_release(a, s, *ms);
-    } else {
-      white_step(a, s, mat_Tw(a, s, k, a.white[iw]), a.white[iw], src, sc, a.precond == 2, fuse ? k : -1);
-    }
-  }
-  if (fuse) {  // c_hat += sum over this CTA's interfaces j of H[:, j] c_j
-    __syncthreads();
-    const int d = (int)g.d, nq = 4 * a.nown_w;
-    for (int r = threadIdx.x; r < d; r += blockDim.x) {
-      double acc = 0;
-      for (int q = 0; q < nq; ++q) {
-        const int j = s.cpj[q];
-        if (j >= 0) acc += __ldg(a.HT + (size_t)j * d + r) * s.cpv[q];
-      }
-      if (acc != 0.0) atomicAdd(chat_acc + r, acc);
-    }
-  }
+  white_phase(a, s, src, sc, a.precond == 2);
   GM_TRACE(22);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(23);
-  if (a.precond == 2 && !fuse) {
-    if (!coarse_solve(a, s, epoch)) return false;
+  if (a.precond == 2) {
+    if (!coarse_solve(a, s, epoch, a.c, a.chat)) return false;
     GM_TRACE(25);
   }
   return true;
 }
 
-// Givens update of Hessenberg column j (thread 0; every CTA runs it on its
-// own copy): the j earlier rotations applied to s.col, the new rotation from
-// s.col[j] and the subdiagonal entry s.misc[4], the rotated right-hand side
-// gg and its last entry |gg[j+1]| (the residual estimate) in s.misc[2].
+// w = y - S Z chat on the owned entries (entries without a slot: 0)
 template <typename S>
-__device__ void givens_column(const GmresArgs<S>& a, const Smem<S>& s, int j, int rank) {
-  const double bnext = s.misc[4];
-  // the rotated entry is carried in a register: one dependent FMA per
-  // rotation (the products with the unrotated entries do not depend on the
-  // chain); the operands of eight rotations are loaded into registers ahead
-  // of them, so only the FMA chain is serial
-  double xi = s.col[0];
-  int i0 = 0;
-  for (; i0 + 8 <= j; i0 += 8) {
-    double x1[8], c[8], sn[8], out[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      x1[u] = s.col[i0 + u + 1];
-      c[u] = s.gcs[i0 + u];
-      sn[u] = s.gsn[i0 + u];
+__device__ SMPM_PHASE void deflate_pass(const GmresArgs<S>& a, const Smem<S>& s, const double* chat) {
+#pragma unroll 1
+  for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
+    double r;
+    if (s.tab) {
+      const OwnedEntry o = s.tab[i];
+      const bool on = o.en.z >= 0;
+      const double ys = on ? (double)ldcg(a.y + o.en.x) : 0.0;
+      double c0 = 0, c1 = 0, c2 = 0, c3 = 0;
+      if (on && chat) {
+        c0 = __ldcg(chat + o.J.x);
+        c1 = __ldcg(chat + o.J.y);
+        c2 = __ldcg(chat + o.J.z);
+        c3 = __ldcg(chat + o.J.w);
+      }
+      r = (ys - (o.r0.x * c0 + o.r0.y * c1)) - (o.r1.x * c2 + o.r1.y * c3);
+    } else {
+      r = deflate_entry(a, a.y, chat, owned_entry(a, i));
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const double cx1 = c[u] * x1[u], sx1 = sn[u] * x1[u];
-      out[u] = fma(c[u], xi, sx1);
-      xi = fma(-sn[u], xi, cx1);
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) s.col[i0 + u] = out[u];
-  }
-  for (int i = i0; i < j; ++i) {
-    const double x1 = s.col[i + 1], c = s.gcs[i], sn = s.gsn[i];
-    const double cx1 = c * x1, sx1 = sn * x1;
-    s.col[i] = fma(c, xi, sx1);
-    xi = fma(-sn, xi, cx1);
-  }
-  const double hh = xi * xi + bnext * bnext;
-  const double iden = hh > 0 ? rsqrt(hh) : 0.0;
-  const double cc = hh > 0 ? xi * iden : 1.0, ss = bnext * iden;
-  s.gcs[j] = cc;
-  s.gsn[j] = ss;
-  s.col[j] = hh * iden;
-  s.gg[j + 1] = -ss * s.gg[j];
-  s.gg[j] = cc * s.gg[j];
-  s.misc[2] = fabs(s.gg[j + 1]);
-  if (rank == 0) {
-    a.gs->g[j] = s.gg[j];
-    a.gs->g[j + 1] = s.gg[j + 1];
+    s.w[i] = (S)r;
   }
 }
 
-// column j of the triangular factor (rotated Hessenberg column), for the
-// end-of-cycle solve: all threads of CTA 0, after givens_column
-template <typename S>
-__device__ __forceinline__ void store_rcol(const GmresArgs<S>& a, const Smem<S>& s, int j, int rank) {
-  if (rank != 0) return;
-  double* Rc = a.gs->R + (size_t)j * (kMaxRestart + 1);
-  for (int l = threadIdx.x; l <= j; l += blockDim.x) Rc[l] = s.col[l];
+// End of a cycle: least squares min ||beta e_1 - H y|| over the j Hessenberg
+// columns that CTA 0 stored in gs->R, by Givens rotations, in one warp: each
+// rotation meets every later column at once, one column per lane (the loads of
+// the next row run ahead of the rotation's chain).  y -> gs->y; returns the
+// residual norm.  xi, gg: m + 3 entries of shared memory.
+__device__ __noinline__ double hessenberg_lsq(GState* gs, double* xi, double* gg, int j, double beta) {
+  const int lane = threadIdx.x & 31;
+  const size_t m1 = kMaxRestart + 1;
+  double* R = gs->R;
+#pragma unroll 1
+  for (int l = lane; l < j; l += 32) xi[l] = __ldcg(R + l * m1);
+  double gcur = beta;
+  int l0 = lane;
+  double nx = l0 < j ? __ldcg(R + l0 * m1 + 1) : 0.0;
+#pragma unroll 1
+  for (int i = 0; i < j; ++i) {
+    const int l1 = i + 1 + ((lane - i - 1) & 31);
+    const double ahead = l1 < j ? __ldcg(R + l1 * m1 + i + 2) : 0.0;
+    __syncwarp();
+    const double x = xi[i], b = __shfl_sync(0xffffffffu, nx, i & 31);  // h_ii rotated so far, h_i+1,i
+    const double hh = x * x + b * b;
+    const double iden = hh > 0 ? rsqrt(hh) : 0.0;
+    const double cc = hh > 0 ? x * iden : 1.0, ss = b * iden;
+#pragma unroll 1
+    for (int l = l0; l < j; l += 32) {
+      const double x1 = l == l0 ? nx : __ldcg(R + l * m1 + i + 1), xl = xi[l];
+      R[l * m1 + i] = l == i ? hh * iden : fma(cc, xl, ss * x1);
+      if (l > i) xi[l] = fma(-ss, xl, cc * x1);
+    }
+    if (lane == 0) gg[i] = cc * gcur;
+    gcur = -ss * gcur;
+    nx = ahead;
+    l0 = l1;
+  }
+  __syncwarp();
+  // y = R^-1 g column by column: y_k, then the entries above it lose R_ik y_k
+#pragma unroll 1
+  for (int k = j - 1; k >= 0; --k) {
+    const double* Rk = R + k * m1;
+    const double r0 = lane < k ? __ldcg(Rk + lane) : 0.0;
+    const double yk = gg[k] / __ldcg(Rk + k);
+    __syncwarp();
+#pragma unroll 1
+    for (int i = lane; i < k; i += 32) gg[i] = fma(-(i == lane ? r0 : __ldcg(Rk + i)), yk, gg[i]);
+    if (lane == 0) gs->y[k] = yk;
+    __syncwarp();
+  }
+  return fabs(gcur);
 }
 
 // One GMRES solve by the CTAs of a team (the whole grid for k_gmres).
@@ -1203,60 +1054,11 @@ template <typename S>
 __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw, unsigned& epoch) {
   const Smem<S> s = carve(a, smraw);
   const DevGeo& g = a.g;
-  const int M = g.M, n = g.n, m = a.m;
+  const int m = a.m;
   const int ES = a.ES, G = a.G, rank = team_rank(a);
   const int m3 = m + 3;
   int trace_n = 0;
-
-  // ---- matrix stream (owned matrices too large for shared memory)
-  MatStream<S> msd;
-  msd.nb = 0;
-  msd.nw = 0;
-  for (int k = 0; k < a.nown_b; ++k) msd.nb += (rank + k * G < a.nblack) ? 1 : 0;
-  for (int k = 0; k < a.nown_w; ++k) msd.nw += (rank + k * G < a.nwhite) ? 1 : 0;
-  msd.nitems = 2 * msd.nb + msd.nw;
-  msd.issued = msd.consumed = 0;
-  MatStream<S>* ms = a.stream_mats ? &msd : nullptr;
-  if (ms) {
-    // shared memory written by an earlier body (batched solves) before the
-    // copy engine writes it
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int b = 0; b < a.nbuf; ++b) mbar_init(s.mbar + b);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    for (int b = 0; b < a.nbuf; ++b) ms_issue(a, s, msd);
-  }
-#define GM_FAIL()           \
-  do {                      \
-    ms_drain(a, s, msd);    \
-    return false;           \
-  } while (0)
-
-  // ---- resident copies of the owned matrices
-  if (a.mats_smem) {
-    for (int k = 0; k < a.nown_b; ++k) {
-      int ib = rank + k * G;
-      if (ib >= a.nblack) break;
-      int e = a.black[ib];
-      S* dst = s.mats + (size_t)k * (2 * M * M + 4 * n * n);
-      for (int i = threadIdx.x; i < M * M; i += blockDim.x) {
-        dst[i] = a.Gc[(size_t)a.gr[ib] * M * M + i];
-        dst[M * M + i] = a.Tc[(size_t)a.tr[e] * M * M + i];
-      }
-      for (int i = threadIdx.x; i < 4 * n * n; i += blockDim.x)
-        dst[2 * M * M + i] = a.Xc[(size_t)a.gr[ib] * 4 * n * n + i];
-    }
-    for (int k = 0; k < a.nown_w; ++k) {
-      int iw = rank + k * G;
-      if (iw >= a.nwhite) break;
-      int e = a.white[iw];
-      S* dst = s.mats + (size_t)a.nown_b * (2 * M * M + 4 * n * n) + (size_t)k * M * M;
-      for (int i = threadIdx.x; i < M * M; i += blockDim.x) dst[i] = a.Tc[(size_t)a.tr[e] * M * M + i];
-    }
-  }
+  load_resident(a, s);
 
   int total = 0, cycle = 0, jlast = 0;
   bool converged = false, breakdown = false, nan = false;
@@ -1266,10 +1068,10 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
     double* accN = a.acc + (size_t)(2 * m) * m3;
     // ---- cycle start: V[0] = rhs - op(x)
     if (cycle > 0) {
-      if (!apply_op(a, s, a.x, 1.0, false, trace_n, epoch, ms)) GM_FAIL();
+      if (!apply_op(a, s, a.x, 1.0, false, trace_n, epoch)) return false;
     }
     {
-      S* v0 = basis(a, s, 0);
+      S* v0 = s.V;
       double nn = 0;
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
         const int4 en = owned_entry(a, i);
@@ -1287,11 +1089,7 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       nn = warp_sum(nn);
       if ((threadIdx.x & 31) == 0 && nn != 0.0) atomicAdd(accN, nn);
     }
-    const bool fused = a.fused && a.precond == 2;
-    if (fused)  // both c_hat buffers of the fused coarse solve start at zero
-      for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < 2 * g.d; i += (long long)G * blockDim.x)
-        a.chatd[i] = 0.0;
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) GM_FAIL();
+    if (!team_sync(a, epoch)) return false;
     const double beta = sqrt(__ldcg(accN));
     if (cycle == 0) {
       beta0 = beta;
@@ -1301,64 +1099,48 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
     if (!isfinite(beta)) { nan = true; break; }
     if (beta <= tolabs || beta == 0.0) { converged = true; break; }
     if (threadIdx.x == 0) {
-      s.gg[0] = beta;
+      s.z[0] = s.misc[6] = 1.0;
       s.invb[0] = 1.0 / beta;
     }
     __syncthreads();
-    int j = 0, pending = -1;  // pending: the step whose Givens rotation is deferred
+    int j = 0;
+    const double goal = (beta / tolabs) * (beta / tolabs);
+#pragma unroll 1
     for (; j < m && total < a.maxit; ++j) {
       double* accD = a.acc + (size_t)(2 * j) * m3;
       double* accE = a.acc + (size_t)(2 * j + 1) * m3;
       const double ivj = s.invb[j];
       GM_TRACE(1);
       // ---- A: finalize V[j] on the owned entries (j > 0), then block solves
-      S* vj = basis(a, s, j);
+      S* vj = s.V + (size_t)j * ES;
       if (j > 0) {
+#pragma unroll 1
         for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-          S rv = (S)basis_combo(a, s, (double)s.w2[i], s.hs2, j, i);
+          const S rv = (S)basis_combo(a, s, (double)s.w[i], s.hs2, j, i);
           vj[i] = rv;
-          const int sl = entry_slot(a, i);
+          const int sl = entry_slot(a, s, i);
           if (sl >= 0) a.vglob[sl] = rv;
         }
         __syncthreads();
       }
-      // fused coarse solve: this step accumulates c_hat into buffer j & 1; the
-      // other buffer was last read in the previous step's phase D (before its
-      // barrier) and is cleared here for the next step
-      double* chat_j = fused ? a.chatd + (size_t)(j & 1) * g.d : nullptr;
-      if (fused) {
-        double* nxt = a.chatd + (size_t)((j + 1) & 1) * g.d;
-        for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < g.d; i += (long long)G * blockDim.x)
-          nxt[i] = 0.0;
-      }
       if (a.precond == 0) {
-        if (!grid_sync(a.bar, a.err, epoch, a.G)) GM_FAIL();  // neighbours read v_j
-        if (!apply_op(a, s, a.vglob, ivj, false, trace_n, epoch, ms)) GM_FAIL();
+        if (!team_sync(a, epoch)) return false;  // neighbours read v_j
+        if (!apply_op(a, s, a.vglob, ivj, false, trace_n, epoch)) return false;
       } else {
-        if (!black_phase(a, s, ms, (const S*)nullptr, ivj, vj)) GM_FAIL();
-        if (!apply_op(a, s, a.vglob, ivj, true, trace_n, epoch, ms, chat_j)) GM_FAIL();
+        if (a.blk) black_block(a, s, (const S*)nullptr, ivj, vj);
+        else black_phase(a, s, (const S*)nullptr, ivj, vj);
+        if (!apply_op(a, s, a.vglob, ivj, true, trace_n, epoch)) return false;
       }
       GM_TRACE(4);
       // ---- D: w = y - S Z chat on owned entries; V^T w, ||w||^2
-      const double* chat_d = a.precond == 2 ? (fused ? chat_j : a.chat) : nullptr;
-      for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-        s.w[i] = (S)deflate_entry(a, a.y, chat_d, owned_entry(a, i));
-      }
+      const double* chat_d = a.precond == 2 ? a.chat : nullptr;
+      deflate_pass(a, s, chat_d);
       __syncthreads();
       owned_dots(a, s, s.w, j + 2, accD);
       GM_TRACE(5);
-      if (!grid_sync_with(a.bar, a.err, epoch, a.G, [&] {
-            if (pending >= 0) givens_column(a, s, pending, rank);
-          }))
-        GM_FAIL();
+      if (!team_sync(a, epoch)) return false;
       GM_TRACE(6);
-      if (pending >= 0) {  // the previous step's rotation and convergence test
-        store_rcol(a, s, pending, rank);
-        resid = s.misc[2];
-        pending = -1;
-        if (!isfinite(resid)) { nan = true; break; }
-        if (resid <= tolabs) { converged = true; break; }  // j columns: this step is dropped
-      }
+#pragma unroll 1
       for (int l = threadIdx.x; l < j + 2; l += blockDim.x) {
         double v = __ldcg(accD + l);
         if (l <= j) {
@@ -1371,12 +1153,14 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       }
       __syncthreads();
       // ---- E: w2 = w - V h1; V^T w2, ||w2||^2
-      for (int i = threadIdx.x; i < ES; i += blockDim.x) s.w2[i] = (S)basis_combo(a, s, (double)s.w[i], s.hs1, j + 1, i);
+#pragma unroll 1
+      for (int i = threadIdx.x; i < ES; i += blockDim.x) s.w[i] = (S)basis_combo(a, s, (double)s.w[i], s.hs1, j + 1, i);
       __syncthreads();
-      owned_dots(a, s, s.w2, j + 2, accE);
+      owned_dots(a, s, s.w, j + 2, accE);
       GM_TRACE(8);
-      if (!grid_sync(a.bar, a.err, epoch, a.G)) GM_FAIL();
+      if (!team_sync(a, epoch)) return false;
       GM_TRACE(9);
+#pragma unroll 1
       for (int l = threadIdx.x; l < j + 2; l += blockDim.x) {
         double v = __ldcg(accE + l);
         if (l <= j) {
@@ -1389,78 +1173,70 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       }
       __syncthreads();
       GM_TRACE(10);
-      if (threadIdx.x < 32) {  // ||h2||^2 and h1 + h2 in warp 0
-        double q = 0;
+      // ---- F: ||w2|| (Pythagorean), the breakdown test, and the residual norm
+      // from the left null vector z of the Hessenberg matrix, z^T H = 0, z_0 = 1:
+      // the least-squares residual is beta z / ||z||^2, so its norm is
+      // beta / ||z||, and a new column costs one dot product over the lanes and
+      // z_{j+1} = -(z . h_j) / h_{j+1,j}.  (Rotating the column instead is a
+      // serial chain of j FP64 steps in one thread: 4,000 cycles of a 57,000
+      // cycle step, and hidden behind the next step's barrier it cost a step
+      // more per solve.  The rotations are made once, at the end of the cycle.)
+      if (threadIdx.x < 32) {
+        double q = 0, zd = 0;
+        double* Rc = a.gs->R + (size_t)j * (kMaxRestart + 1);
+#pragma unroll 1
         for (int l = threadIdx.x; l <= j; l += 32) {
+          const double h = s.h1[l] + s.h2[l];
           q += s.h2[l] * s.h2[l];
-          s.col[l] = s.h1[l] + s.h2[l];
+          zd += s.z[l] * h;
+          if (rank == 0) Rc[l] = h;
         }
         q = warp_sum(q);
-        if (threadIdx.x == 0) s.misc[5] = q;
+        zd = warp_sum(zd);
+        if (threadIdx.x == 0) {
+          const double bsq = s.misc[1] - q;
+          const double ib = bsq > 0 ? rsqrt(bsq) : 0.0;
+          const double zn = -zd * ib, zz = s.misc[6] + zn * zn;
+          s.z[j + 1] = zn;
+          s.misc[6] = zz;
+          s.invb[j + 1] = ib;
+          s.misc[3] = (bsq <= 1e-28 * s.misc[0]) ? 1.0 : 0.0;
+          s.misc[4] = bsq > 0 ? bsq * ib : 0.0;  // the new subdiagonal entry
+          if (rank == 0) Rc[j + 1] = s.misc[4];
+        }
       }
       __syncthreads();
       GM_TRACE(11);
-      // ---- F: ||w2|| (Pythagorean) and the breakdown test now; the Givens
-      // rotation of column j -- a serial FP64 chain in thread 0, replicated in
-      // every CTA -- runs inside the next step's first grid barrier, while the
-      // other CTAs arrive, and its convergence test is read after it.  A step
-      // that converged thus costs one extra step of work, whose results
-      // (v_{j+1}, t, the dot products) are never used.
-      if (threadIdx.x == 0) {
-        const double bsq = s.misc[1] - s.misc[5];
-        const double ib = bsq > 0 ? rsqrt(bsq) : 0.0;
-        s.invb[j + 1] = ib;
-        s.misc[3] = (bsq <= 1e-28 * s.misc[0]) ? 1.0 : 0.0;
-        s.misc[4] = bsq > 0 ? bsq * ib : 0.0;  // the new subdiagonal entry
-      }
-      __syncthreads();
-      GM_TRACE(13);
       ++total;
-      if (!isfinite(s.misc[4]) || s.misc[3] != 0.0 || j + 1 >= m || total >= a.maxit) {
-        // last step of the cycle: rotate now
-        if (threadIdx.x == 0) givens_column(a, s, j, rank);
-        __syncthreads();
-        store_rcol(a, s, j, rank);
-        resid = s.misc[2];
-        if (!isfinite(resid) || !isfinite(s.misc[4])) { nan = true; ++j; break; }
-        if (resid <= tolabs) { converged = true; ++j; break; }
-        if (s.misc[3] != 0.0) { breakdown = true; ++j; break; }
-        continue;
-      }
-      pending = j;
+      // beta / ||z|| <= tolabs (an exact breakdown: residual 0)
+      const double zz = s.misc[6];
+      if (!isfinite(zz) || !isfinite(s.misc[4])) { nan = true; ++j; break; }
+      if (s.misc[4] == 0.0 || goal <= zz) { converged = true; ++j; break; }
+      if (s.misc[3] != 0.0) { breakdown = true; ++j; break; }
     }
     jlast = j;
     if (nan) break;
-    __syncthreads();  // the columns of R written by all threads of CTA 0
-    // ---- end of cycle: y = R^-1 g (warp 0 of CTA 0, column by column: y_k,
-    // then the entries above it lose R_ik y_k in parallel over the lanes),
-    // x += V diag(invb) y on owned entries
+    // ---- end of cycle: y by warp 0 of CTA 0, x += V diag(invb) y on owned entries
     if (rank == 0 && threadIdx.x < 32) {
-      const int m1 = kMaxRestart + 1, lane = threadIdx.x;
-      for (int l = lane; l < j; l += 32) s.col[l] = a.gs->g[l];
       __syncwarp();
-      for (int k = j - 1; k >= 0; --k) {
-        const double* Rk = a.gs->R + (size_t)k * m1;
-        const double yk = s.col[k] / Rk[k];
-        __syncwarp();
-        for (int i = lane; i < k; i += 32) s.col[i] = fma(-Rk[i], yk, s.col[i]);
-        if (lane == 0) a.gs->y[k] = yk;
-        __syncwarp();
-      }
+      resid = hessenberg_lsq(a.gs, s.xi, s.gg, j, beta);
     }
-    // the accumulators are consumed: zero them for the next cycle
+    if (!team_sync(a, epoch)) return false;
+    // the accumulators are consumed by all CTAs: zero them for the next cycle
+#pragma unroll 1
     for (size_t i = (size_t)rank * blockDim.x + threadIdx.x; i < (size_t)(2 * m + 1) * m3;
          i += (size_t)G * blockDim.x)
       a.acc[i] = 0.0;
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) GM_FAIL();
+#pragma unroll 1
     for (int l = threadIdx.x; l < j; l += blockDim.x) s.hs1[l] = -__ldcg(a.gs->y + l) * s.invb[l];
     __syncthreads();
+#pragma unroll 1
     for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-      const int sl = entry_slot(a, i);
+      const int sl = entry_slot(a, s, i);
       if (sl < 0) continue;
       a.x[sl] = (S)basis_combo(a, s, (double)ldcg(a.x + sl), s.hs1, j, i);
     }
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) GM_FAIL();
+    if (!team_sync(a, epoch)) return false;
     ++cycle;
     if (converged || breakdown || total >= a.maxit) break;
   }
@@ -1477,7 +1253,5 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
     a.gs->scal[5] += total;  // iterations over all launches of a solve
     if (a.its_out) *a.its_out = total;
   }
-  ms_drain(a, s, msd);
   return true;
-#undef GM_FAIL
 }

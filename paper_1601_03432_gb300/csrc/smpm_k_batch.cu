@@ -1,6 +1,5 @@
 // Kernel of a batched solve: teams of CTAs run the bodies of the single and
 // lockstep solves task by task.
-#define SMPM_BODY __noinline__
 #include "smpm_device.cuh"
 #include "smpm_digits.cuh"
 
@@ -55,7 +54,7 @@ __global__ void __launch_bounds__(256, 1) k_batch(const BatchTask* __restrict__ 
     auto failed = [&](int where) {
       if (threadIdx.x == 0 && atomicCAS(T.P.ga.err + 1, 0, t + 1) == 0) T.P.ga.err[2] = where;
     };
-    if (!grid_sync(T.P.ga.bar, T.P.ga.err, epoch, T.P.ga.G)) return failed(1);
+    if (!team_sync(T.P.ga, epoch)) return failed(1);
     if (!pre_body(T.P, body, epoch)) return failed(2);
     if (T.precision == 0) {
       if (!gmres_body<double>(T.a64, body, epoch)) return failed(3);
@@ -82,7 +81,7 @@ __global__ void __launch_bounds__(256, 1) k_batch(const BatchTask* __restrict__ 
     // control block (the zero-mean step reads its accumulator after the last
     // barrier of post_body) before rank 0 reads the report and the next task
     // clears the block
-    if (!grid_sync(T.P.ga.bar, T.P.ga.err, epoch, T.P.ga.G)) return failed(5);
+    if (!team_sync(T.P.ga, epoch)) return failed(5);
     if (rank == 0 && threadIdx.x == 0) {
       const GState* gs = T.P.ga.gs;
       const double* acc8 = T.P.acc;

@@ -10,10 +10,13 @@ namespace {
 #include "smpm_lockstep.cuh"
 
 template <typename S>
-__global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A) {
+__global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A0) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  if (lock_all_done(A)) return;
-  unsigned epoch = 0;
+  __shared__ LockArgs<S> A;  // the phases are calls: arguments from shared memory
+  if (lock_all_done(A0)) return;
+  if (threadIdx.x == 0) A = A0;
+  __syncthreads();
+  unsigned epoch = first_epoch(A.a.bar);
   lock_body(A, smraw, epoch);
 }
 
@@ -24,16 +27,26 @@ __global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A) {
 // the previous column.
 __global__ void __launch_bounds__(256, 1) k_pre_cols(const PrePostArgs* __restrict__ Ps, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  for (int c = 0; c < R; ++c)
-    if (!pre_body(Ps[c], smraw, epoch)) return;
+  unsigned epoch = first_epoch(Ps[0].ga.bar);
+  __shared__ PrePostArgs P;
+  for (int c = 0; c < R; ++c) {
+    __syncthreads();
+    stage16(&P, Ps + c, (int)sizeof(P));
+    __syncthreads();
+    if (!pre_body(P, smraw, epoch)) return;
+  }
 }
 
 __global__ void __launch_bounds__(256, 1) k_post_cols(const PrePostArgs* __restrict__ Ps, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
-  for (int c = 0; c < R; ++c)
-    if (!post_body(Ps[c], smraw, epoch)) return;
+  unsigned epoch = first_epoch(Ps[0].ga.bar);
+  __shared__ PrePostArgs P;
+  for (int c = 0; c < R; ++c) {
+    __syncthreads();
+    stage16(&P, Ps + c, (int)sizeof(P));
+    __syncthreads();
+    if (!post_body(P, smraw, epoch)) return;
+  }
 }
 
 // One refinement step (refine_body) for every column not yet done, one
@@ -41,10 +54,14 @@ __global__ void __launch_bounds__(256, 1) k_post_cols(const PrePostArgs* __restr
 // only its own body (rank 0, after a barrier every CTA passed) sets it.
 __global__ void __launch_bounds__(256, 1) k_refine_cols(const RefineArgs* __restrict__ Rs, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
+  unsigned epoch = first_epoch(Rs[0].ga.bar);
+  __shared__ RefineArgs A;
   for (int c = 0; c < R; ++c) {
     if (*((volatile const int*)Rs[c].done)) continue;
-    if (refine_body(Rs[c], smraw, epoch) < 0) return;
+    __syncthreads();
+    stage16(&A, Rs + c, (int)sizeof(A));
+    __syncthreads();
+    if (refine_body(A, smraw, epoch) < 0) return;
   }
 }
 

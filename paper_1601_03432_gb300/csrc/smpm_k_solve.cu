@@ -1,5 +1,6 @@
 // Kernels of a solve of one right-hand side (one team spanning the grid).
 #include "smpm_device.cuh"
+#include "smpm_digits.cuh"
 
 namespace {
 
@@ -8,29 +9,41 @@ namespace {
 #include "smpm_refine.cuh"
 
 template <typename S>
-__global__ void __launch_bounds__(256, 1) k_gmres(GmresArgs<S> a) {
+__global__ void __launch_bounds__(256, 1) k_gmres(GmresArgs<S> a0) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ GmresArgs<S> a;
+  if (threadIdx.x == 0) a = a0;
+  __syncthreads();
   if (a.skip && *((volatile const int*)a.skip)) return;
-  unsigned epoch = 0;
+  unsigned epoch = first_epoch(a.bar);
   gmres_body(a, smraw, epoch);
 }
 
-__global__ void __launch_bounds__(256, 1) k_pre(PrePostArgs P) {
+__global__ void __launch_bounds__(256, 1) k_pre(PrePostArgs P0) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
+  __shared__ PrePostArgs P;
+  if (threadIdx.x == 0) P = P0;
+  __syncthreads();
+  unsigned epoch = first_epoch(P.ga.bar);
   pre_body(P, smraw, epoch);
 }
 
-__global__ void __launch_bounds__(256, 1) k_post(PrePostArgs P) {
+__global__ void __launch_bounds__(256, 1) k_post(PrePostArgs P0) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = 0;
+  __shared__ PrePostArgs P;
+  if (threadIdx.x == 0) P = P0;
+  __syncthreads();
+  unsigned epoch = first_epoch(P.ga.bar);
   post_body(P, smraw, epoch);
 }
 
-__global__ void __launch_bounds__(256, 1) k_refine(RefineArgs R) {
+__global__ void __launch_bounds__(256, 1) k_refine(RefineArgs R0) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ RefineArgs R;
+  if (threadIdx.x == 0) R = R0;
+  __syncthreads();
   if (*((volatile const int*)R.done)) return;
-  unsigned epoch = 0;
+  unsigned epoch = first_epoch(R.ga.bar);
   refine_body(R, smraw, epoch);
 }
 

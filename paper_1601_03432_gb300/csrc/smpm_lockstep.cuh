@@ -19,7 +19,7 @@
 // Layouts: column rho of a kp-vector at base + rho * vs; of a d-vector at
 // base + rho * ds.  The basis lives in global memory (L2 / HBM): CTA rank's
 // slice of basis vector l, column rho at V + ((rank (m+1) + l) R + rho) ES;
-// w and w2 likewise (W + (rank 2R + rho) (ES+1), w2 at + R (ES+1)).
+// w likewise (see lk_w); ES is a multiple of 4 here.
 // Element work items are (owned element, eight columns); a group of W warps
 // takes items grp, grp + ngrp, ...; an item's tiles live in the group's
 // shared scratch.
@@ -42,14 +42,10 @@ struct LockArgs {
   int R;           // columns (<= kLockMaxCols)
   int W_item, ngrp;  // warps per element work item (eight columns of an element), groups of that many warps
   size_t wb_bytes;   // shared scratch of the groups
-  // packed matrices of the classes (smpm_digits.cuh) and the class of each
-  // block / element: G_b and X_b (4 per block class), T_e
-  const uint4 *Gd, *Xd, *Td;
-  const short *Ge, *Xe, *Te;
-  const int *bcls, *tcls;
   long long vs, ds;
   S* V;            // basis, G (m+1) R ES
-  S* W;            // w, w2: G 2R (ES+1)
+  S* W;            // w (w2 in its place): G R ES, unless w_smem
+  int w_smem;
   LockColState* cs;  // R
   double* Rh;        // R m (m+1): Hessenberg R factor per column (written by rank 0)
   double* yv;        // R m: least-squares solution per column
@@ -80,7 +76,7 @@ __host__ __device__ constexpr size_t lock_bf_bytes(int M, int n) {
 }
 template <typename S>
 __host__ __device__ constexpr size_t lock_group_bytes(int M, int n) {
-  const size_t black = 8 * sizeof(S) * (size_t)(lock_ld(2 * M) + lock_ld(M)), white = 8 * sizeof(double) * (size_t)lock_ld(M);
+  const size_t black = 8 * sizeof(S) * (size_t)(lock_ld(2 * M) + lock_ld(M)), white = 8 * (sizeof(double) + sizeof(S)) * (size_t)lock_ld(M);
   return lock_bf_bytes<S>(M, n) + (black > white ? black : white);
 }
 
@@ -132,19 +128,31 @@ template <typename S>
 __device__ __forceinline__ S* lk_basis(const LockArgs<S>& A, int l, int rho) {
   return A.V + (((size_t)team_rank(A.a) * (A.a.m + 1) + l) * A.R + rho) * A.a.ES;
 }
+// w of column rho, then w2 in its place: in the groups' scratch when it fits
+// (it lives from the deflation to the next step's v_j, while the element phases
+// do not run), else in global memory.
 template <typename S>
-__device__ __forceinline__ S* lk_w(const LockArgs<S>& A, int rho) {
-  return A.W + ((size_t)team_rank(A.a) * 2 * A.R + rho) * (A.a.ES + 1);
-}
-template <typename S>
-__device__ __forceinline__ S* lk_w2(const LockArgs<S>& A, int rho) {
-  return A.W + ((size_t)team_rank(A.a) * 2 * A.R + A.R + rho) * (A.a.ES + 1);
+__device__ __forceinline__ S* lk_w(const LockArgs<S>& A, const LockSmem<S>& s, int rho) {
+  return A.w_smem ? reinterpret_cast<S*>(s.wb) + (size_t)rho * A.a.ES
+                  : A.W + ((size_t)team_rank(A.a) * A.R + rho) * A.a.ES;
 }
 
-// The W warps of a group (named barrier of their own) work on one item.
-__device__ __forceinline__ void lk_group_sync(int grp, int W) {
-  if (W == 1) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * W) : "memory");
+// four consecutive entries (16-byte aligned; ES is a multiple of 4)
+template <typename S>
+struct alignas(16) Quad {
+  S v[4];
+};
+__device__ __forceinline__ Quad<double> ld_quad(const double* p) {  // basis: streamed past L1
+  const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+  return {a.x, a.y, b.x, b.y};
+}
+__device__ __forceinline__ Quad<float> ld_quad(const float* p) {
+  const float4 a = __ldcg(reinterpret_cast<const float4*>(p));
+  return {a.x, a.y, a.z, a.w};
+}
+template <typename S>
+__device__ __forceinline__ Quad<S> ld_quad_w(const S* p) {  // w: shared or global, written by this CTA
+  return *reinterpret_cast<const Quad<S>*>(p);
 }
 
 // Black block solves for all columns: items (owned block k, eight columns), a
@@ -153,7 +161,7 @@ __device__ __forceinline__ void lk_group_sync(int grp, int W) {
 // a = G r1, z = T_e a, t = [a; q - z]; the products run on the tensor cores
 // (smpm_digits.cuh), eight columns to a tile.
 template <typename S>
-__device__ void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int jbasis) {
+__device__ SMPM_PHASE void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int jbasis) {
   const GmresArgs<S>& a = A.a;
   const DevGeo& g = a.g;
   const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), R = A.R, Q = (R + 7) / 8, W = A.W_item;
@@ -167,49 +175,58 @@ __device__ void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* sr
     const int k = it / Q, c0 = (it % Q) * 8, nc = min(8, R - c0);
     const int ib = rank + k * G;
     if (ib >= a.nblack) continue;
-    const int e = a.black[ib], cb = A.bcls[ib], ct = A.tcls[e];
-    for (int idx = part * 32 + lane; idx < 2 * M * 8; idx += 32 * W) {
-      const int c = idx / (2 * M), i = idx % (2 * M), rho = c0 + c;
-      S v = S(0);
-      if (c < nc) {
-        if (jbasis >= 0) {
-          v = (S)(sc[rho] * (double)lk_basis(A, jbasis, rho)[k * 2 * M + i]);
-        } else {
-          const int sl = block_entry(a, ib, i).x;
-          if (sl >= 0) v = (S)(sc[rho] * (double)ldcg(src + rho * A.vs + sl));
-        }
+    const int e = a.black[ib], cb = a.dm.bcls[ib], ct = a.dm.tcls[e];
+    for (int i = part * 32 + lane; i < 2 * M; i += 32 * W) {  // an entry's eight columns together
+      S v[8];
+      const int sl = jbasis >= 0 ? 0 : block_entry(a, ib, i).x;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        const int rho = c0 + min(c, nc - 1);
+        v[c] = jbasis >= 0 ? lk_basis(A, jbasis, rho)[k * 2 * M + i] : sl >= 0 ? ldcg(src + rho * A.vs + sl) : S(0);
       }
-      P[c * ldp + i] = v;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) P[c * ldp + i] = c < nc ? (S)(sc[c0 + c] * (double)v[c]) : S(0);
     }
-    lk_group_sync(grp, W);
+    item_sync(grp, W);
     for (int F = part; F < 4; F += W) {  // r1 = p - X q, face by face
       uint4* Bq = Bf + F * digit_bwords<S>(n);
       const S* q = P + M + F * n;
-      const int E = pack_cols<S>(Bq, n, lane, [&](int kk, int c) { return q[c * ldp + kk]; });
-      __syncwarp();
-      for (int mt = 0; mt < kf_n; ++mt)
-        digits_tile8<S>(A.Xd + ((size_t)cb * 4 + F) * digit_words<S>(n, n), A.Xe + ((size_t)cb * 4 + F) * n, Bq, n, kf_n,
-                        mt, lane, E, [&](int row, int c, S v) { Rr[c * ldr + F * n + row] = P[c * ldp + F * n + row] - v; });
+      const int E = pack_cols<S>(Bq, q, 1, ldp, n, 8, lane, 0, 1);
+      for (int mt = 0; mt < kf_n; ++mt) {
+        const Tile8<S> t = digits_tile8<S>(a.dm.X + ((size_t)cb * 4 + F) * digit_words<S>(n, n),
+                                           a.dm.Xe + ((size_t)cb * 4 + F) * n, Bq, n, kf_n, mt, lane, E);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int r = mt * 16 + (lane >> 2) + 8 * (v >> 1), c = 2 * (lane & 3) + (v & 1);
+          if (r < n) Rr[c * ldr + F * n + r] = P[c * ldp + F * n + r] - t.z[v];
+        }
+      }
     }
-    lk_group_sync(grp, W);
-    int E = pack_cols<S>(Bf, M, lane, [&](int kk, int c) { return Rr[c * ldr + kk]; }, part, W);
-    lk_group_sync(grp, W);
-    for (int mt = part; mt < kt_n; mt += W)  // a = G r1
-      digits_tile8<S>(A.Gd + (size_t)cb * digit_words<S>(M, M), A.Ge + (size_t)cb * M, Bf, M, kt_n, mt, lane, E,
-                      [&](int row, int c, S v) {
-                        Rr[c * ldr + row] = v;
-                        if (c < nc) a.t[(c0 + c) * A.vs + (size_t)e * M + row] = v;
-                      });
-    lk_group_sync(grp, W);
-    E = pack_cols<S>(Bf, M, lane, [&](int kk, int c) { return Rr[c * ldr + kk]; }, part, W);
-    lk_group_sync(grp, W);
-    for (int mt = part; mt < kt_n; mt += W)  // z = T_e a, t = q - z on the facing slots
-      digits_tile8<S>(A.Td + (size_t)ct * digit_words<S>(M, M), A.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E,
-                      [&](int row, int c, S z) {
-                        const int sl = block_entry(a, ib, M + row).x;
-                        if (c < nc && sl >= 0) a.t[(c0 + c) * A.vs + sl] = P[c * ldp + M + row] - z;
-                      });
-    lk_group_sync(grp, W);
+    item_sync(grp, W);
+    for (int stage = 0; stage < 2; ++stage) {  // a = G r1, then z = T_e a and t = q - z on the facing slots
+      const int E = pack_cols<S>(Bf, Rr, 1, ldr, M, 8, lane, part, W);
+      const uint4* Am = stage == 0 ? a.dm.G + (size_t)cb * digit_words<S>(M, M) : a.dm.T + (size_t)ct * digit_words<S>(M, M);
+      const short* er = stage == 0 ? a.dm.Ge + (size_t)cb * M : a.dm.Te + (size_t)ct * M;
+      item_sync(grp, W);
+      for (int mt = part; mt < kt_n; mt += W) {
+        int sl[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = mt * 16 + (lane >> 2) + 8 * h;
+          sl[h] = r >= M ? -1 : stage == 0 ? e * M + r : block_entry(a, ib, M + r).x;
+        }
+        const Tile8<S> t = digits_tile8<S>(Am, er, Bf, M, kt_n, mt, lane, E);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int r = mt * 16 + (lane >> 2) + 8 * (v >> 1), c = 2 * (lane & 3) + (v & 1);
+          if (r >= M) continue;
+          if (stage == 0) Rr[c * ldr + r] = t.z[v];
+          if (c < nc && sl[v >> 1] >= 0)
+            a.t[(c0 + c) * A.vs + sl[v >> 1]] = stage == 0 ? t.z[v] : P[c * ldp + M + r] - t.z[v];
+        }
+      }
+      item_sync(grp, W);
+    }
   }
   __syncthreads();
 }
@@ -217,7 +234,7 @@ __device__ void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* sr
 // White elements for all columns: y = S t on the black slots facing e,
 // y = sc * v on e's own slots, c = Z^T y on e's interfaces (with_c).
 template <typename S>
-__device__ void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v, const double* sc, bool with_c) {
+__device__ SMPM_PHASE void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v0, const double* sc, bool with_c) {
   const GmresArgs<S>& a = A.a;
   const DevGeo& g = a.g;
   const int M = g.M, n = g.n, G = a.G, rank = team_rank(a), R = A.R, Q = (R + 7) / 8, W = A.W_item;
@@ -226,34 +243,47 @@ __device__ void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v,
   unsigned char* base = s.wb + (size_t)grp * lock_group_bytes<S>(M, n);
   uint4* Bf = reinterpret_cast<uint4*>(base);
   double* ci = reinterpret_cast<double*>(base + lock_bf_bytes<S>(M, n));  // contributions to c: column c at c ldc
+  S* Tt = reinterpret_cast<S*>(ci + 8 * ldc);                             // t on e's slots: column c at c ldc
   for (int it = grp; it < a.nown_w * Q; it += A.ngrp) {
     const int k = it / Q, c0 = (it % Q) * 8, nc = min(8, R - c0);
     const int iw = rank + k * G;
     if (iw >= a.nwhite) continue;
-    const int e = a.white[iw], ct = A.tcls[e];
-    const S* te = a.t + (size_t)e * M;
-    const int E = pack_cols<S>(
-        Bf, M, lane, [&](int kk, int c) { return c < nc ? ldcg(te + (c0 + c) * A.vs + kk) : S(0); }, part, W);
-    lk_group_sync(grp, W);
-    for (int mt = part; mt < kt_n; mt += W)
-      digits_tile8<S>(A.Td + (size_t)ct * digit_words<S>(M, M), A.Te + (size_t)ct * M, Bf, M, kt_n, mt, lane, E,
-                      [&](int row, int c, S z) {
-                        if (c >= nc) return;
-                        const int rho = c0 + c, F = row / n, tt = row - F * n, e2 = dev_neighbour(g, e, F);
-                        const size_t own = rho * A.vs + (size_t)e * M + row;
-                        const S vo = (S)(sc[rho] * (double)ldcg(v + own));
-                        a.y[own] = vo;
-                        double c1 = 0;
-                        if (e2 >= 0) {
-                          const size_t sl = rho * A.vs + (size_t)e2 * M + (F ^ 1) * n + tt;
-                          const S ys = ldcg(a.t + sl) + z;
-                          a.y[sl] = ys;
-                          c1 = g.zw ? dev_zw(g, e, F) * (double)vo + dev_zw(g, e2, F ^ 1) * (double)ys
-                                    : (double)vo + (double)ys;
-                        }
-                        ci[c * ldc + row] = c1;
-                      });
-    lk_group_sync(grp, W);
+    const int e = a.white[iw], ct = a.dm.tcls[e];
+    for (int i = part * 32 + lane; i < M; i += 32 * W) {
+      S v[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = ldcg(a.t + (c0 + min(c, nc - 1)) * A.vs + (size_t)e * M + i);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) Tt[c * ldc + i] = v[c];
+    }
+    item_sync(grp, W);
+    const int E = pack_cols<S>(Bf, Tt, 1, ldc, M, nc, lane, part, W);
+    item_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W) {
+      Facing<S> f[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int r = min(mt * 16 + (lane >> 2) + 8 * (v >> 1), M - 1), c = min(2 * (lane & 3) + (v & 1), nc - 1);
+        f[v] = facing_entry(g, e, r, v0 + (c0 + c) * A.vs, a.t + (c0 + c) * A.vs);
+      }
+      const Tile8<S> t = digits_tile8<S>(a.dm.T + (size_t)ct * digit_words<S>(M, M), a.dm.Te + (size_t)ct * M, Bf, M, kt_n,
+                                         mt, lane, E);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int r = mt * 16 + (lane >> 2) + 8 * (v >> 1), c = 2 * (lane & 3) + (v & 1), rho = c0 + c;
+        if (r >= M || c >= nc) continue;
+        const S vo = (S)(sc[rho] * (double)f[v].v);
+        a.y[rho * A.vs + (size_t)e * M + r] = vo;
+        double c1 = 0;
+        if (f[v].sl >= 0) {
+          const S ys = f[v].t + t.z[v];
+          a.y[rho * A.vs + f[v].sl] = ys;
+          c1 = facing_c(g, f[v], vo, ys);
+        }
+        ci[c * ldc + r] = c1;
+      }
+    }
+    item_sync(grp, W);
     if (with_c && part == 0 && lane < 4 * nc) {  // face F of column c summed by lane c * 4 + F
       const int c = lane / 4, F = lane % 4, j = dev_iface(g, e, F);
       if (j >= 0) {
@@ -262,7 +292,7 @@ __device__ void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v,
         a.c[(c0 + c) * A.ds + j] = sum;
       }
     }
-    lk_group_sync(grp, W);
+    item_sync(grp, W);
   }
   __syncthreads();
 }
@@ -273,7 +303,7 @@ __device__ void lk_white(const LockArgs<S>& A, const LockSmem<S>& s, const S* v,
 // next step are issued before the FMAs of this one (software pipelining); the
 // R partial sums meet in warp shuffles.
 template <typename S, typename HT>
-__device__ void lk_coarse_h(const LockArgs<S>& A, const HT* H) {
+__device__ SMPM_PHASE void lk_coarse_h(const LockArgs<S>& A, const HT* H) {
   const GmresArgs<S>& a = A.a;
   const int d = (int)a.g.d, R = A.R;
   const int per = (d + a.G - 1) / a.G;
@@ -282,7 +312,7 @@ __device__ void lk_coarse_h(const LockArgs<S>& A, const HT* H) {
   constexpr int U = 2, CG = 8;  // entries per lane and step; columns per pass over the row
   const int nfull = d / (32 * U);
   for (int r = r0 + warp; r < r1; r += nwarps) {
-    const HT* hr = H + (size_t)r * d;
+    const HT* hr = H + (size_t)r * ((d + 3) & ~3);
     for (int c0 = 0; c0 < R; c0 += CG) {
       const int nc = min(CG, R - c0);
       const double* cb = a.c + (size_t)c0 * A.ds;
@@ -339,7 +369,7 @@ __device__ void lk_coarse_h(const LockArgs<S>& A, const HT* H) {
 // row's pass costs as much as FP64 products); each warp keeps its rows'
 // partial sums in c_hat across the chunks.
 template <typename S>
-__device__ void lk_coarse32_staged(const LockArgs<S>& A, float* cf, int dc) {
+__device__ SMPM_PHASE void lk_coarse32_staged(const LockArgs<S>& A, float* cf, int dc) {
   const GmresArgs<S>& a = A.a;
   const int d = (int)a.g.d, R = A.R;
   const int per = (d + a.G - 1) / a.G;
@@ -354,7 +384,7 @@ __device__ void lk_coarse32_staged(const LockArgs<S>& A, float* cf, int dc) {
     }
     __syncthreads();
     for (int r = r0 + warp; r < r1; r += nwarps) {
-      const float* hr = a.H + (size_t)r * d + j0;
+      const float* hr = a.H + (size_t)r * ((d + 3) & ~3) + j0;
       for (int c0 = 0; c0 < R; c0 += CG) {
         const int nc = min(CG, R - c0);
         const float* cc = cf + (size_t)c0 * dc;
@@ -391,13 +421,15 @@ __device__ void lk_coarse32_staged(const LockArgs<S>& A, float* cf, int dc) {
   }
 }
 
-// As row_dots for NC columns at a time: eight lanes per row, lane l of the
-// group ends with column l's sum (the partial sums are exchanged halving the
-// columns each time: 7 adds per row and lane instead of 24).  x: column c of
-// the staged vectors at c * xld.
+// As row_dots for NC columns at a time: eight lanes per row or more, as far as
+// the rows leave threads; lane l < 8 of a group ends with column l's sum (the
+// partial sums are exchanged halving the columns each time: 7 adds per row and
+// lane of eight instead of 24).  x: column c of the staged vectors at c * xld.
 template <typename T, int NC, typename Get, typename Put>
 __device__ __forceinline__ void row_dots_cols(int r0, int r1, int xld, Get&& get, Put&& put) {
-  constexpr int V = 16 / (int)sizeof(T), P = 8;
+  constexpr int V = 16 / (int)sizeof(T);
+  int P = 8;
+  while (P < 32 && 2 * P * (r1 - r0) <= (int)blockDim.x) P *= 2;
   const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
   for (int rb = 0; rb < r1 - r0; rb += ngrp) {  // uniform trip count per warp
     const int r = r0 + rb + grp;
@@ -410,9 +442,9 @@ __device__ __forceinline__ void row_dots_cols(int r0, int r1, int xld, Get&& get
     for (int c = 0; c < NC; ++c) acc[c] = T(0);
     for (int j = V * lane; j < len; j += 2 * V * P) {
       T h[2][V];
-      ld_vec(a + j, h[0]);
+      ld_vec<false>(a + j, h[0]);
       const bool two = j + V * P < len;
-      if (two) ld_vec(a + j + V * P, h[1]);
+      if (two) ld_vec<false>(a + j + V * P, h[1]);
 #pragma unroll
       for (int c = 0; c < NC; ++c)
 #pragma unroll
@@ -427,6 +459,9 @@ __device__ __forceinline__ void row_dots_cols(int r0, int r1, int xld, Get&& get
     // lane keeps the half of the columns that its bit o selects; lanes beyond
     // the columns add the halves that are left
     int w = NC;
+    for (int o = P / 2; o >= 8; o >>= 1)  // lanes beyond eight first
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) {
       const int half = w > 1 ? w / 2 : 1;
@@ -436,21 +471,21 @@ __device__ __forceinline__ void row_dots_cols(int r0, int r1, int xld, Get&& get
         if (c >= half) break;
         const T keep = (w > 1 && up) ? acc[(c + half) % NC] : acc[c];
         const T give = (w > 1 && !up) ? acc[(c + half) % NC] : acc[c];
-        const T got = __shfl_xor_sync(0xffffffffu, give, o, P);
+        const T got = __shfl_xor_sync(0xffffffffu, give, o);
         acc[c] = keep + got;
       }
       if (w > 1) w = half;
     }
     // column of this lane: the top log2(NC) bits of lane
     constexpr int S3 = NC == 8 ? 0 : NC == 4 ? 1 : NC == 2 ? 2 : 3;
-    if (len > 0 && (lane & ((1 << S3) - 1)) == 0) put(r, lane >> S3, acc[0]);
+    if (len > 0 && lane < 8 && (lane & ((1 << S3) - 1)) == 0) put(r, lane >> S3, acc[0]);
   }
 }
 
 // C^+ by strips (coarse_strips) for all columns, NC of them at a time staged
 // in st (each phase's stretch of every column, xld entries apart).
 template <typename S, int NC>
-__device__ bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& epoch) {
+__device__ SMPM_PHASE bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& epoch) {
   using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
   constexpr int V = 16 / (int)sizeof(T);
   const GmresArgs<S>& a = A.a;
@@ -487,7 +522,7 @@ __device__ bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& ep
             });
       }
     }
-    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+    if (!team_sync(a, epoch)) return false;
   }
   {
     const int n2 = k.ns + 1, per = (n2 + G - 1) / G, r0 = min(n2, rank * per), r1 = min(n2, r0 + per);
@@ -520,7 +555,7 @@ __device__ bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& ep
             });
       }
     }
-    if (!grid_sync(a.bar, a.err, epoch, G)) return false;
+    if (!team_sync(a, epoch)) return false;
   }
   {
     const int n3 = k.p * k.m, per = (n3 + G - 1) / G, r0 = min(n3, rank * per), r1 = min(n3, r0 + per);
@@ -552,7 +587,7 @@ __device__ bool lk_coarse_strips_nc(const LockArgs<S>& A, void* st, unsigned& ep
       }
     }
   }
-  return grid_sync(a.bar, a.err, epoch, G);
+  return team_sync(a, epoch);
 }
 
 // longest stretch of a coarse vector that a CTA of a team of G stages
@@ -567,7 +602,7 @@ __host__ __device__ inline int strips_stage(const CoarseStrips<T>& k, int G) {
 
 // c_hat = C^+ c for all columns, complete after its last barrier.
 template <typename S>
-__device__ bool lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s, unsigned& epoch) {
+__device__ SMPM_PHASE bool lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s, unsigned& epoch) {
   const int room = (int)(A.wb_bytes / sizeof(S));  // the groups' scratch is idle here
   if (A.a.use_strips) {
     const int nc = room / strips_stage(A.a.strips, A.a.G);
@@ -584,22 +619,22 @@ __device__ bool lk_coarse(const LockArgs<S>& A, const LockSmem<S>& s, unsigned& 
     }
   }
   if (!done) lk_coarse_h(A, A.a.H);
-  return grid_sync(A.a.bar, A.a.err, epoch, A.a.G);
+  return team_sync(A.a, epoch);
 }
 
 // op(sc * src) -> y (and c, chat) for all columns; with own_j >= 0 the block
 // solves read basis vector own_j (owner slices), else the global src.
 template <typename S>
-__device__ bool lk_apply(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int own_j,
+__device__ SMPM_PHASE bool lk_apply(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int own_j,
                          unsigned& epoch, int& trace_n) {
   const GmresArgs<S>& a = A.a;
   lk_black(A, s, src, sc, own_j);
   GM_TRACE(31);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(32);
   lk_white(A, s, src, sc, a.precond == 2);
   GM_TRACE(33);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(34);
   if (a.precond == 2) {
     if (!lk_coarse(A, s, epoch)) return false;
@@ -608,114 +643,133 @@ __device__ bool lk_apply(const LockArgs<S>& A, const LockSmem<S>& s, const S* sr
   return true;
 }
 
-// Dot products of the owned basis slices with the columns' vectors: for each
-// pair (l, rho), l < nl, out[l * R + rho] += sum_i basis(l, rho)[i] vec(rho)[i],
-// with l == nl - 1 giving vec.vec.  Work items are (pair, chunk of the ES
-// entries), one warp per item: lanes read consecutive entries (coalesced),
-// eight entries per lane and step loaded ahead, and the partial sum meets in
-// warp shuffles before one FP64 atomic add.  FP32 products are summed in FP32
-// over chunks of 16 entries per lane, chunks in FP64.
+// Dot products of the owned basis slices with the columns' vectors w: for each
+// pair (l, rho), l < nl, out[l * R + rho] += sum_i basis(l, rho)[i] w(rho)[i],
+// with l == nl - 1 giving w.w.  A warp takes four l of a column at a time (over
+// all entries, or a chunk of them when there are few items): w is read once
+// for the four, lanes keep eight 16-byte loads in flight, and the four sums
+// meet in six shuffled additions instead of twenty (an FP64 addition costs as
+// much as a product here).  FP32 products are summed in FP32 over 16 entries
+// per lane, those in FP64.
 template <typename S>
-__device__ void lk_dots(const LockArgs<S>& A, bool second, int nl, double* out) {
-  const int E = A.a.ES, R = A.R, npairs = nl * R;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  int nch = 1;  // chunks per pair: at least two items per warp, chunks of 512 entries or more
-  while (npairs * nch < 2 * nwarps && E / (nch * 2) >= 512) nch *= 2;
-  const int clen = (E + nch - 1) / nch;
-  for (int it = warp; it < npairs * nch; it += nwarps) {
-    const int pr = it / nch, ch = it % nch;
-    const int l = pr / R, rho = pr % R;
-    const S* vec = second ? lk_w2(A, rho) : lk_w(A, rho);
-    const S* vl = (l == nl - 1) ? vec : lk_basis(A, l, rho);
+__device__ SMPM_PHASE void lk_dots(const LockArgs<S>& A, const LockSmem<S>& s, int nl, double* out) {
+  const int E = A.a.ES, R = A.R, ng = (nl + 3) / 4, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nwarps = blockDim.x >> 5;
+  int nch = 1;  // chunks of the entries: at least two items per warp, 256 entries or more each
+  while (ng * R * nch < 2 * nwarps && E / (nch * 2) >= 256) nch *= 2;
+  const int clen = (E / 4 + nch - 1) / nch * 4;
+  for (int it = warp; it < ng * R * nch; it += nwarps) {
+    const int ch = it % nch, pr = it / nch, rho = pr % R, l0 = (pr / R) * 4;
+    const S* w = lk_w(A, s, rho);
+    const S* v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = lk_basis(A, min(l0 + q, nl - 2), rho);
+    const int self = nl - 1 - l0;  // the q that is w itself (0 .. 3), if any
     const int i0 = ch * clen, i1 = min(E, i0 + clen);
-    double sum = 0;
-    if constexpr (sizeof(S) == 4) {
-      int i = i0 + lane, cnt = 0;
-      float f0 = 0.f;
-      for (; i + 7 * 32 < i1; i += 8 * 32) {
-        float bv[8], wv[8];
+    double sum[4] = {0, 0, 0, 0};
+    for (int i = i0 + 4 * lane; i < i1; i += 256) {
+      const bool two = i + 128 < i1;
+      Quad<S> b[2][4], ww[2];
+      ww[0] = ld_quad_w(w + i);
+      ww[1] = two ? ld_quad_w(w + i + 128) : Quad<S>{};
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          bv[u] = ldcg(vl + i + 32 * u);
-          wv[u] = ldcg(vec + i + 32 * u);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) f0 = fmaf(bv[u], wv[u], f0);
-        cnt += 8;
-        if (cnt == 16) {
-          sum += (double)f0;
-          f0 = 0.f;
-          cnt = 0;
+      for (int q = 0; q < 4; ++q) {
+        if (q == self) {
+          b[0][q] = ww[0];
+          b[1][q] = ww[1];
+        } else {
+          b[0][q] = ld_quad(v[q] + i);
+          b[1][q] = two ? ld_quad(v[q] + i + 128) : Quad<S>{};
         }
       }
-      for (; i < i1; i += 32) f0 = fmaf(ldcg(vl + i), ldcg(vec + i), f0);
-      sum += (double)f0;
-    } else {
-      double acc[4] = {0, 0, 0, 0};
-      int i = i0 + lane;
-      for (; i + 7 * 32 < i1; i += 8 * 32) {
-        double bv[8], wv[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          bv[u] = ldcg(vl + i + 32 * u);
-          wv[u] = ldcg(vec + i + 32 * u);
+      for (int q = 0; q < 4; ++q) {
+        if constexpr (sizeof(S) == 4) {
+          float f = 0.f;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) f = fmaf(b[k >> 2][q].v[k & 3], ww[k >> 2].v[k & 3], f);
+          sum[q] += (double)f;
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (k < 4 || two) sum[q] += b[k >> 2][q].v[k & 3] * ww[k >> 2].v[k & 3];
         }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) acc[u & 3] += bv[u] * wv[u];
       }
-      for (; i < i1; i += 32) acc[0] += ldcg(vl + i) * ldcg(vec + i);
-      sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     }
-    sum = warp_sum(sum);
-    if (lane == 0 && sum != 0.0) atomicAdd(out + pr, sum);
+    // lane bits 4 and 3 select the sum a lane keeps
+    const bool up = lane & 16, hi = lane & 8;
+    double a0 = (up ? sum[2] : sum[0]) + __shfl_xor_sync(0xffffffffu, up ? sum[0] : sum[2], 16);
+    double a1 = (up ? sum[3] : sum[1]) + __shfl_xor_sync(0xffffffffu, up ? sum[1] : sum[3], 16);
+    double a = (hi ? a1 : a0) + __shfl_xor_sync(0xffffffffu, hi ? a0 : a1, 8);
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const int l = l0 + (up ? 2 : 0) + (hi ? 1 : 0);
+    if ((lane & 7) == 0 && l < nl && a != 0.0) atomicAdd(out + l * R + rho, a);
   }
 }
 
-// dst(rho)[i] = base(rho)[i] - sum_{l < nl} coef[rho * m3 + l] basis(l, rho)[i]
-// for every column rho and owned entry i.  Each thread takes CH (column,
-// entry) pairs at a time and runs the l loop over all of them, so CH
-// independent loads are in flight per step (FP32 arithmetic for FP32 bases).
-// With vg, the result is also written to the column's global vector at the
-// entry's slot.
+// w(rho)[i] - sum_{l < nl} coef[rho * m3 + l] basis(l, rho)[i] for every column
+// rho and owned entry i, in place of w (to_basis: into basis vector jdst and the
+// column's global vector).  A thread takes U quads of entries at a time through
+// l, the next l's loads issued before this l's products (FP32 arithmetic for
+// FP32 bases).
 template <typename S>
-__device__ void lk_combo_pass(const LockArgs<S>& A, bool from_w2, const double* coef, int nl, bool to_basis, int jdst,
-                              bool to_vg) {
-  constexpr int CH = 16;
+__device__ SMPM_PHASE void lk_combo_pass(const LockArgs<S>& A, const LockSmem<S>& s, const double* coef, int nl, bool to_basis,
+                              int jdst) {
+  constexpr int U = sizeof(S) == 4 ? 4 : 2;
   const GmresArgs<S>& a = A.a;
-  const int E = a.ES, R = A.R, m3 = a.m + 3;
-  const int NP = R * E;
+  const int E = a.ES, R = A.R, m3 = a.m + 3, E4 = E / 4, NQ = R * E4;
+  const size_t lstep = (size_t)R * E;  // from basis vector l to l + 1
   using C = typename std::conditional<sizeof(S) == 4, float, double>::type;
-  for (int p0 = threadIdx.x; p0 < NP; p0 += CH * blockDim.x) {
-    C acc[CH];
-    int rho_[CH], i_[CH];
+  for (int p0 = threadIdx.x; p0 < NQ; p0 += U * blockDim.x) {
+    C acc[U][4];
+    const S* b[U];
+    const double* cf[U];
+    int rho_[U], i_[U];
+    Quad<S> cur[U];
 #pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int p = p0 + q * blockDim.x;
-      rho_[q] = p < NP ? p / E : 0;
-      i_[q] = p < NP ? p % E : 0;
-      const S* bsrc = from_w2 ? lk_w2(A, rho_[q]) : lk_w(A, rho_[q]);
-      acc[q] = p < NP ? (C)ldcg(bsrc + i_[q]) : C(0);
+    for (int q = 0; q < U; ++q) {
+      const int p = min(p0 + q * (int)blockDim.x, NQ - 1);
+      rho_[q] = p / E4;
+      i_[q] = 4 * (p - rho_[q] * E4);
+      cf[q] = coef + rho_[q] * m3;
+      b[q] = lk_basis(A, 0, rho_[q]) + i_[q];
+      if (nl > 0) cur[q] = ld_quad(b[q]);
+      const Quad<S> w = ld_quad_w(lk_w(A, s, rho_[q]) + i_[q]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[q][k] = (C)w.v[k];
     }
     for (int l = 0; l < nl; ++l) {
-      S v[CH];
+      Quad<S> nxt[U];
+      if (l + 1 < nl) {
 #pragma unroll
-      for (int q = 0; q < CH; ++q) v[q] = ldcg(lk_basis(A, l, rho_[q]) + i_[q]);
+        for (int q = 0; q < U; ++q) nxt[q] = ld_quad(b[q] + (l + 1) * lstep);
+      }
 #pragma unroll
-      for (int q = 0; q < CH; ++q) acc[q] -= (C)coef[rho_[q] * m3 + l] * (C)v[q];
+      for (int q = 0; q < U; ++q) {
+        const C c = (C)cf[q][l];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[q][k] -= c * (C)cur[q].v[k];
+      }
+      if (l + 1 < nl) {
+#pragma unroll
+        for (int q = 0; q < U; ++q) cur[q] = nxt[q];
+      }
     }
 #pragma unroll
-    for (int q = 0; q < CH; ++q) {
-      const int p = p0 + q * blockDim.x;
-      if (p >= NP) continue;
-      const S val = (S)acc[q];
-      if (to_basis) {
-        lk_basis(A, jdst, rho_[q])[i_[q]] = val;
+    for (int q = 0; q < U; ++q) {
+      if (p0 + q * (int)blockDim.x >= NQ) continue;
+      Quad<S> o;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) o.v[k] = (S)acc[q][k];
+      if (!to_basis) {
+        *reinterpret_cast<Quad<S>*>(lk_w(A, s, rho_[q]) + i_[q]) = o;
       } else {
-        lk_w2(A, rho_[q])[i_[q]] = val;
-      }
-      if (to_vg) {
-        const int sl = entry_slot(a, i_[q]);
-        if (sl >= 0) a.vglob[rho_[q] * A.vs + sl] = val;
+        *reinterpret_cast<Quad<S>*>(lk_basis(A, jdst, rho_[q]) + i_[q]) = o;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int sl = entry_slot(a, i_[q] + k);
+          if (sl >= 0) a.vglob[rho_[q] * A.vs + sl] = o.v[k];
+        }
       }
     }
   }
@@ -785,7 +839,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       nn = warp_sum(nn);
       if ((threadIdx.x & 31) == 0 && nn != 0.0) atomicAdd(accN + rho, nn);
     }
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!team_sync(a, epoch)) return false;
     if (threadIdx.x < R) {
       const int c = threadIdx.x;
       const double beta = sqrt(__ldcg(accN + c));
@@ -819,7 +873,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       // ---- A: v_j = w2 - V h2 (scaled later) on the owned entries, then block solves
       GM_TRACE(30);
       if (j > 0) {
-        lk_combo_pass(A, true, s.hs2, j, true, j, true);
+        lk_combo_pass(A, s, s.hs2, j, true, j);
         __syncthreads();
       }
       for (int c = threadIdx.x; c < R; c += blockDim.x) s.scl[c] = s.invb[c * m3 + j];
@@ -832,7 +886,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       for (int i = threadIdx.x; i < ES; i += blockDim.x) {
         const int4 en = owned_entry(a, i);
         if (en.z < 0 || a.precond != 2) {
-          for (int c = 0; c < R; ++c) lk_w(A, c)[i] = en.z < 0 ? S(0) : ldcg(a.y + c * A.vs + en.x);
+          for (int c = 0; c < R; ++c) lk_w(A, s, c)[i] = en.z < 0 ? S(0) : ldcg(a.y + c * A.vs + en.x);
           continue;
         }
         const int4 J = __ldg(a.if4 + en.y);
@@ -853,15 +907,15 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             if (c0 + q < R)
-              lk_w(A, c0 + q)[i] =
+              lk_w(A, s, c0 + q)[i] =
                   (S)((yv[q] - (r0.x * h[q][0] + r0.y * h[q][1])) - (r1.x * h[q][2] + r1.y * h[q][3]));
         }
       }
       __syncthreads();
       GM_TRACE(38);
-      lk_dots(A, false, j + 2, accD);
+      lk_dots(A, s, j + 2, accD);
       GM_TRACE(39);
-      if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+      if (!team_sync(a, epoch)) return false;
       GM_TRACE(40);
       for (int p = threadIdx.x; p < (j + 2) * R; p += blockDim.x) {
         const int l = p / R, c = p % R;
@@ -876,12 +930,12 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
       }
       __syncthreads();
       // ---- E: w2 = w - V h1; V^T w2, ||w2||^2
-      lk_combo_pass(A, false, s.hs1, j + 1, false, 0, false);
+      lk_combo_pass(A, s, s.hs1, j + 1, false, 0);
       __syncthreads();
       GM_TRACE(41);
-      lk_dots(A, true, j + 2, accE);
+      lk_dots(A, s, j + 2, accE);
       GM_TRACE(42);
-      if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+      if (!team_sync(a, epoch)) return false;
       GM_TRACE(43);
       for (int p = threadIdx.x; p < (j + 2) * R; p += blockDim.x) {
         const int l = p / R, c = p % R;
@@ -978,7 +1032,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
     for (size_t i = (size_t)rank * blockDim.x + threadIdx.x; i < (size_t)(2 * m + 1) * R * m3;
          i += (size_t)G * blockDim.x)
       a.acc[i] = 0.0;
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!team_sync(a, epoch)) return false;
     for (int p = threadIdx.x; p < R * m; p += blockDim.x) {
       const int c = p / m, l = p % m;
       s.hs1[c * m3 + l] = l < s.jc[c] ? -__ldcg(A.yv + (size_t)c * m + l) * s.invb[c * m3 + l] : 0.0;
@@ -994,7 +1048,7 @@ __device__ __noinline__ bool lock_body(const LockArgs<S>& A, unsigned char* smra
         *xp = (S)lk_combo(A, (double)ldcg(xp), s.hs1 + rho * m3, jj, rho, i);
       }
     }
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!team_sync(a, epoch)) return false;
     ++cycle;
     any_active = false;
     for (int c = 0; c < R; ++c) any_active |= s.active[c] != 0;

@@ -39,10 +39,20 @@
 #pragma once
 // Included inside the anonymous namespace of smpm_solver.cu.
 
+// Packed fast-diagonalisation factors (smpm_digits.cuh): per x entry (a
+// face-type class, or a column of a graded grid) the digits of V and V^-1 and
+// their row exponents, likewise per y entry, and 1 / (lx_i + ly_j) at
+// [j n + i] per pair of entries.
+struct FdMats {
+  const uint4 *x, *y;
+  const short *xe, *ye;
+  const double* rinv;
+  int nx, pad_;
+};
+
 struct alignas(16) PrePostArgs {  // 16-byte multiple: staged with 16-byte copies in batched solves
   GmresArgs<double> ga;  // geometry, ownership, operator matrices, t/y/c/chat buffers
-  const double* fdx;
-  const double* fdy;
+  FdMats fd;  // fast diagonalisation (packed)
   const double* D;
   const double* uL;
   const double* uS;
@@ -64,30 +74,118 @@ struct alignas(16) PrePostArgs {  // 16-byte multiple: staged with 16-byte copie
   float* zero32[4];  // kp-long FP32 buffers zeroed in P1 (mixed precision), or null
   double* cr;        // d, zeroed in P1 (mixed precision), or null
   float* rg32;       // kp, FP32 copy of the GMRES right-hand side (mixed precision), or null
+  int W_fd;          // warps per element in the element solves
   int assembled;     // k_post: x_S is given in xs (skip the assembly)
   int adjoint;       // transposed solve (see above)
   double* gg;        // adjoint: kp, dl/dg per padded slot, or null
 };
 
+// copy n bytes (a multiple of 16) from global memory into shared memory, all threads
+__device__ __forceinline__ void stage16(void* dst, const void* src, int n) {
+  const int4* s = reinterpret_cast<const int4*>(src);
+  int4* d = reinterpret_cast<int4*>(dst);
+  for (int i = threadIdx.x; i < n / 16; i += blockDim.x) d[i] = s[i];
+}
+
 // accumulator slots
 enum { ACC_ULB = 0, ACC_USBS = 1, ACC_MEAN = 2, ACC_RES = 3, ACC_BSN = 4, ACC_RGN = 5 };
 
-__device__ double* fd_scratch(const Smem<double>& s) { return s.mats; }
+// ---- element solves --------------------------------------------------------
+// A group of W warps solves U = A_e^-1 B by fast diagonalisation: U = Vy ((Vy^-1
+// B Vx^-T) .* rinv) Vx^T, four n x n products on the tensor cores, the columns
+// in tiles of eight shared out over the warps.  B, U, t1: n rows of fd_ld(n)
+// doubles; Bf: one packed tile per warp.
+__host__ __device__ constexpr int fd_ld(int n) { return (n + 3) / 8 * 8 + 4; }  // 4 modulo 8: rows spread over the banks
+// scratch of a group: three tiles, the slot values (two times 4n), packed tiles
+// (the element's residual product takes the first W of them for its vector)
+__host__ __device__ inline size_t fd_item_bytes(int n, int W) {
+  const size_t tile = sizeof(uint4) * (size_t)digit_bwords<double>(n), vec = sizeof(uint4) * (size_t)digit_bwords<double>(4 * n);
+  const size_t bf = W * tile > vec ? W * tile : vec;
+  return bf + sizeof(double) * (3 * (size_t)n * fd_ld(n) + 8 * (size_t)n);
+}
+struct FdItem {
+  uint4* Bf;
+  double *B, *U, *t1, *p, *q;  // p, q: 4n slot values each
+};
+__device__ __forceinline__ FdItem fd_item(unsigned char* base, int n, int W, int grp) {
+  FdItem f;
+  unsigned char* b = base + (size_t)grp * fd_item_bytes(n, W);
+  f.B = reinterpret_cast<double*>(b);
+  f.U = f.B + (size_t)n * fd_ld(n);
+  f.t1 = f.U + (size_t)n * fd_ld(n);
+  f.p = f.t1 + (size_t)n * fd_ld(n);
+  f.q = f.p + 4 * n;
+  f.Bf = reinterpret_cast<uint4*>(f.q + 4 * n);
+  return f;
+}
 
-// b_e (projected or not) is in B; solves U = A_e^-1 B.
-__device__ void elem_fd(const PrePostArgs& P, int e, double* B, double* U, double* t1) {
-  const DevGeo& g = P.ga.g;
-  elem_solve_dev(g.n, fd_x(g, P.fdx, e), fd_y(g, P.fdy, e), B, U, t1);
+// One product: row r, column c of A (packed, n x n) times the columns x[k ldk +
+// c ldc], times w[c n + r] where w is given, to out[r ldr + c ldo].
+__device__ __noinline__ void fd_pass(const uint4* A, const short* er, uint4* Bw, int n, int lane, int part, int W,
+                                     const double* x, int ldk, int ldc, double* out, int ldr, int ldo,
+                                     const double* __restrict__ w) {
+  const int kt_n = digit_tiles(n);
+  for (int c0 = 8 * part; c0 < n; c0 += 8 * W) {
+    const int nc = min(8, n - c0), E = pack_cols<double>(Bw, x + c0 * ldc, ldk, ldc, n, nc, lane, 0, 1);
+    for (int mt = 0; mt < kt_n; ++mt) {
+      const Tile8<double> t = digits_tile8<double>(A, er, Bw, n, kt_n, mt, lane, E);
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int r = mt * 16 + (lane >> 2) + 8 * (v >> 1), c = 2 * (lane & 3) + (v & 1);
+        if (r < n && c < nc) out[r * ldr + (c0 + c) * ldo] = w ? t.z[v] * __ldg(w + (c0 + c) * n + r) : t.z[v];
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// U = A_e^-1 B for element e, entered and left with the group in step
+__device__ __noinline__ void elem_fd(const FdMats& fd, const DevGeo& g, int e, const FdItem& f, int lane, int part,
+                                        int W, int grp) {
+  const int n = g.n, ld = fd_ld(n), ix = e % g.mx, iy = e / g.mx;
+  const int cx = g.graded ? ix : ((ix > 0 ? 1 : 0) | (ix < g.mx - 1 ? 2 : 0));
+  const int cy = g.graded ? iy : ((iy > 0 ? 1 : 0) | (iy < g.my - 1 ? 2 : 0));
+  const size_t nw = digit_words<double>(n, n);
+  const uint4 *Vx = fd.x + 2 * cx * nw, *Vxi = Vx + nw, *Vy = fd.y + 2 * cy * nw, *Vyi = Vy + nw;
+  const short *ex = fd.xe + 2 * cx * n, *exi = ex + n, *ey = fd.ye + 2 * cy * n, *eyi = ey + n;
+  const double* ri = fd.rinv + ((size_t)cy * fd.nx + cx) * n * n;
+  uint4* Bw = f.Bf + (size_t)part * digit_bwords<double>(n);
+  fd_pass(Vyi, eyi, Bw, n, lane, part, W, f.B, ld, 1, f.t1, ld, 1, nullptr);   // t1 = Vy^-1 B
+  item_sync(grp, W);
+  fd_pass(Vxi, exi, Bw, n, lane, part, W, f.t1, 1, ld, f.U, 1, ld, ri);         // U = (t1 Vx^-T) .* rinv
+  item_sync(grp, W);
+  fd_pass(Vx, ex, Bw, n, lane, part, W, f.U, 1, ld, f.t1, 1, ld, nullptr);      // t1 = U Vx^T
+  item_sync(grp, W);
+  fd_pass(Vy, ey, Bw, n, lane, part, W, f.t1, ld, 1, f.U, ld, 1, nullptr);      // U = Vy t1
+  item_sync(grp, W);
+}
+
+// n_F . grad U at face node t of face F (rows of ld doubles; sc = 2/h of the element across F)
+__device__ __forceinline__ double normal_deriv_ld(const DevGeo& g, const double* __restrict__ D, const double* U, int ld,
+                                                  int F, int t, double sc) {
+  const int n = g.n, st = F < 2 ? 1 : ld;
+  const double* u = F < 2 ? U + t * ld : U + t;
+  const double* d = D + ((F & 1) ? (n - 1) * n : 0);
+  double a0 = 0, a1 = 0;
+  int c = 0;
+  for (; c + 1 < n; c += 2) {
+    a0 += __ldg(d + c) * u[c * st];
+    a1 += __ldg(d + c + 1) * u[(c + 1) * st];
+  }
+  if (c < n) a0 += __ldg(d + c) * u[c * st];
+  return ((F & 1) ? sc : -sc) * (a0 + a1);
 }
 
 __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<double>& a = P.ga;
   const Smem<double> s = carve(a, smraw);
+  no_resident(a, s);
   const DevGeo& g = a.g;
   const int n = g.n, nn = n * n, M = g.M, G = a.G, rank = team_rank(a);
-  double* B = fd_scratch(s);
-  double* U = B + nn;
-  double* t1 = U + nn;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = P.W_fd, grp = warp / W, part = warp % W,
+            ngrp = kGmresThreads / 32 / W;
+  const FdItem f = fd_item(s.end, n, W, grp);
+  const int ld = fd_ld(n);
   int trace_n = 0;
   GM_TRACE(50);
   // ---- P1: zero the work vectors; b = f + tau g; u_L^T b
@@ -103,7 +201,7 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
     for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < g.kp; i += (long long)G * blockDim.x)
       for (int v = 0; v < 4; ++v) P.zero32[v][i] = 0.f;
   if (rank == 0 && threadIdx.x == 0) a.gs->scal[5] = 0.0;  // inner iterations of the solve
-  double part = 0;
+  double ulb = 0;
   for (long long e = rank; e < g.nel; e += G) {
     for (int q = threadIdx.x; q < nn; q += blockDim.x) {
       const int aa = q % n, bb = q / n;
@@ -118,60 +216,60 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
         if (bb == n - 1 && dev_neighbour(g, (int)e, 3) < 0) v += ty * P.gn[s0 + 3 * n + aa];
       }
       P.b[gq] = v;
-      part += P.adjoint ? v : P.uL[gq] * v;
+      ulb += P.adjoint ? v : P.uL[gq] * v;
     }
   }
-  part = warp_sum(part);
-  if ((threadIdx.x & 31) == 0 && part != 0.0) atomicAdd(P.acc + ACC_ULB, part);
+  ulb = warp_sum(ulb);
+  if ((threadIdx.x & 31) == 0 && ulb != 0.0) atomicAdd(P.acc + ACC_ULB, ulb);
   GM_TRACE(51);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(52);
   // ---- P2: project b; w = A_e^-1 b_e; push fluxes into b_S; u_S^T b_S; Z^T b_S
   const double alpha = __ldcg(P.acc + ACC_ULB);
   double pus = 0;
-  for (long long e = rank; e < g.nel; e += G) {
-    for (int q = threadIdx.x; q < nn; q += blockDim.x) {
-      const long long gq = e * nn + q;
-      double v = P.b[gq] - alpha * (P.adjoint ? P.what[gq] : P.uL[gq]);
+  for (long long el = rank + (long long)grp * G; el < g.nel; el += (long long)ngrp * G) {
+    const int e = (int)el;
+    for (int q = part * 32 + lane; q < nn; q += 32 * W) {
+      const long long gq = el * nn + q;
+      const double v = P.b[gq] - alpha * (P.adjoint ? P.what[gq] : P.uL[gq]);
       P.b[gq] = v;
-      B[q] = v;
+      f.B[(q / n) * ld + q % n] = v;
     }
-    __syncthreads();
-    elem_fd(P, (int)e, B, U, t1);
+    item_sync(grp, W);
+    elem_fd(P.fd, g, e, f, lane, part, W, grp);
     // flux of w into the slot (nbr, opp F, t): -tau' (p' w - n_F . grad w) with
     // tau', p' of the neighbour's face opp F and the gradient in e's own size
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-      const int F = i / n, t = i % n;
-      const int e2 = dev_neighbour(g, (int)e, F);
+    for (int i = part * 32 + lane; i < M; i += 32 * W) {
+      const int F = i / n, t = i - F * n, e2 = dev_neighbour(g, e, F);
       double val = 0;
       if (e2 >= 0) {
         int aa, bb;
         face_node(n, F, t, &aa, &bb);
         const double* fn = face_geo(g, e2, F ^ 1);
-        val = P.adjoint ? U[bb * n + aa]
-                        : -fn[0] * (fn[1] * U[bb * n + aa] - normal_deriv(g, P.D, U, F, t, face_geo(g, (int)e, F)[2]));
+        val = P.adjoint ? f.U[bb * ld + aa]
+                        : -fn[0] * (fn[1] * f.U[bb * ld + aa] -
+                                    normal_deriv_ld(g, P.D, f.U, ld, F, t, face_geo(g, e, F)[2]));
         const size_t sl = (size_t)e2 * M + (F ^ 1) * n + t;
         P.bS[sl] = val;
         pus += P.uS[sl] * val;
         val *= dev_zw(g, e2, F ^ 1);  // its weight in Z^T b_S
       }
-      s.cs[i] = val;
+      f.p[i] = val;
     }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-      const int F = threadIdx.x, j = dev_iface(g, (int)e, F);
-      if (j >= 0) {
-        double sum = 0;
-        for (int t = 0; t < n; ++t) sum += s.cs[F * n + t];
-        atomicAdd(P.cb + j, sum);
-      }
+    item_sync(grp, W);
+    if (part == 0) {  // face F summed by the eight lanes 8 F + r
+      const int F = lane >> 3, j = dev_iface(g, e, F);
+      double sum = 0;
+      for (int t = lane & 7; t < n; t += 8) sum += f.p[F * n + t];
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if ((lane & 7) == 0 && j >= 0) atomicAdd(P.cb + j, sum);
     }
-    __syncthreads();
+    item_sync(grp, W);
   }
   pus = warp_sum(pus);
   if ((threadIdx.x & 31) == 0 && pus != 0.0) atomicAdd(P.acc + ACC_USBS, pus);
   GM_TRACE(53);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(54);
   // ---- P3: c_hat_b = C^+ Z^T (b_S - beta u_S)
   const double beta = __ldcg(P.acc + ACC_USBS);
@@ -179,9 +277,9 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
     for (int j = rank * blockDim.x + threadIdx.x; j < (int)g.d; j += G * blockDim.x)
       a.c[j] = __ldcg(P.cb + j) - beta * P.ZtuS[j];
     GM_TRACE(55);
-    if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+    if (!team_sync(a, epoch)) return false;
     GM_TRACE(56);
-    if (!coarse_solve(a, s, epoch)) return false;  // a.c -> a.chat
+    if (!coarse_solve(a, s, epoch, a.c, a.chat)) return false;  // a.c -> a.chat
     GM_TRACE(58);
     for (int j = rank * blockDim.x + threadIdx.x; j < (int)g.d; j += G * blockDim.x)
       P.chatb[j] = __ldcg(a.chat + j);
@@ -218,11 +316,13 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
 __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<double>& a = P.ga;
   const Smem<double> s = carve(a, smraw);
+  no_resident(a, s);
   const DevGeo& g = a.g;
   const int n = g.n, nn = n * n, M = g.M, G = a.G, rank = team_rank(a);
-  double* B = fd_scratch(s);
-  double* U = B + nn;
-  double* t1 = U + nn;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = P.W_fd, grp = warp / W, part = warp % W,
+            ngrp = kGmresThreads / 32 / W;
+  const FdItem f = fd_item(s.end, n, W, grp);
+  const int ld = fd_ld(n), kt_n = digit_tiles(M);
   int trace_n = 0;
   // ---- Q1-Q4: x_S
   if (P.assembled) {
@@ -233,20 +333,10 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
       if (sl >= 0) P.xs[sl] = __ldcg(a.x + sl);
     }
   } else {
-    for (int k = 0; k < a.nown_b; ++k) {
-      const int ib = rank + k * G;
-      if (ib >= a.nblack) break;
-      const int e = a.black[ib];
-      for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) {
-        const int sl = block_entry(a, ib, i).x;
-        s.w[i] = sl >= 0 ? __ldcg(a.x + sl) : 0.0;
-      }
-      __syncthreads();
-      block_solve(a, s, k, ib, e, s.w);
-    }
+    black_phase(a, s, (const double*)a.x, 1.0, (const double*)nullptr);
     if (a.precond == 1) {
       GM_TRACE(61);
-      if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+      if (!team_sync(a, epoch)) return false;
       GM_TRACE(62);
       for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
         const int sl = entry_slot(a, i);
@@ -263,59 +353,65 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
     }
   }
   GM_TRACE(63);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(64);
   // ---- Q5: recovery u_e = A_e^-1 (b_e - E_e x_S), residual b_S - S x_S, mean
   double pm = 0, pr = 0;
-  for (long long e = rank; e < g.nel; e += G) {
-    for (int q = threadIdx.x; q < nn; q += blockDim.x) B[q] = P.b[e * nn + q];
-    for (int i = threadIdx.x; i < M; i += blockDim.x) s.p[i] = __ldcg(P.xs + e * M + i);
-    __syncthreads();
+  for (long long el = rank + (long long)grp * G; el < g.nel; el += (long long)ngrp * G) {
+    const int e = (int)el, ct = __ldg(a.dm.tcls + e);
+    for (int q = part * 32 + lane; q < nn; q += 32 * W) f.B[(q / n) * ld + q % n] = P.b[el * nn + q];
+    for (int i = part * 32 + lane; i < M; i += 32 * W) f.p[i] = __ldcg(P.xs + el * M + i);
+    item_sync(grp, W);
     for (int F = 0; F < 4; ++F) {  // faces in turn: a corner node takes both slots
-      if (dev_neighbour(g, (int)e, F) >= 0) {
+      if (dev_neighbour(g, e, F) >= 0) {
         if (!P.adjoint) {
-          for (int t = threadIdx.x; t < n; t += blockDim.x) {
+          for (int t = part * 32 + lane; t < n; t += 32 * W) {
             int aa, bb;
             face_node(n, F, t, &aa, &bb);
-            B[bb * n + aa] -= s.p[F * n + t];
+            f.B[bb * ld + aa] -= f.p[F * n + t];
           }
         } else {
           // - B_e^T mu: the slot (F, t) feeds, through B, the flux
           // -tau' (p' u(q) - n_F.grad u(q)) at face node q = (F, t), tau' and p'
           // of the neighbour's face opp F; its transpose touches the n nodes
           // on the normal line through q
-          const double* fn = face_geo(g, dev_neighbour(g, (int)e, F), F ^ 1);
+          const double* fn = face_geo(g, dev_neighbour(g, e, F), F ^ 1);
           const double tau = fn[0], pw = fn[1];
-          const double sc = face_geo(g, (int)e, F)[2];
+          const double sc = face_geo(g, e, F)[2];
           const int drow = (F & 1) ? n - 1 : 0;   // D row of the face end
           const double sgn = (F & 1) ? 1.0 : -1.0;  // outward normal along the axis
-          for (int idx = threadIdx.x; idx < nn; idx += blockDim.x) {
+          for (int idx = part * 32 + lane; idx < nn; idx += 32 * W) {
             const int t = idx / n, k = idx % n;
-            const double v = s.p[F * n + t];
+            const double v = f.p[F * n + t];
             const double dn = sgn * sc * __ldg(P.D + drow * n + k);
             const double coef = -tau * ((k == drow ? pw : 0.0) - dn);
-            const int q = F < 2 ? t * n + k : k * n + t;
-            B[q] -= coef * v;
+            f.B[F < 2 ? t * ld + k : k * ld + t] -= coef * v;
           }
         }
       }
-      __syncthreads();
+      item_sync(grp, W);
     }
-    elem_fd(P, (int)e, B, U, t1);
-    for (int q = threadIdx.x; q < nn; q += blockDim.x) {
-      P.u[e * nn + q] = U[q];
-      pm += (P.adjoint ? P.uL[e * nn + q] : P.what[e * nn + q]) * U[q];
+    elem_fd(P.fd, g, e, f, lane, part, W, grp);
+    for (int q = part * 32 + lane; q < nn; q += 32 * W) {
+      const double u = f.U[(q / n) * ld + q % n];
+      P.u[el * nn + q] = u;
+      pm += (P.adjoint ? P.uL[el * nn + q] : P.what[el * nn + q]) * u;
     }
     // (S x_S) on the slots facing e: x_S + T_e x_S,e
-    gemv_split(a.Tc + (size_t)__ldg(a.tr + e) * M * M, M, s.p, s.z, M, M, s.red);
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-      const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
-      if (e2 < 0) continue;
-      const size_t sl = (size_t)e2 * M + (F ^ 1) * n + t;
-      const double rr = P.bS[sl] - (__ldcg(P.xs + sl) + s.z[i]);
+    const int E = pack_one<double>(f.Bf, f.p, M, lane, part, W);
+    item_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W) {
+      const int row = tile1_row(mt, lane, M);
+      Facing<double> fc{};
+      fc.sl = -1;
+      if (row >= 0) fc = facing_entry(g, e, row, P.xs, P.xs);
+      const double z = digits_tile1<double>(a.dm.T + (size_t)ct * digit_words<double>(M, M), a.dm.Te + (size_t)ct * M, f.Bf,
+                                            M, kt_n, mt, lane, E);
+      if (fc.sl < 0) continue;
+      const double rr = P.bS[fc.sl] - (fc.t + z);
       pr += rr * rr;
     }
-    __syncthreads();
+    item_sync(grp, W);
   }
   pm = warp_sum(pm);
   pr = warp_sum(pr);
@@ -324,7 +420,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
     if (pr != 0.0) atomicAdd(P.acc + ACC_RES, pr);
   }
   GM_TRACE(65);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return false;
+  if (!team_sync(a, epoch)) return false;
   GM_TRACE(66);
   // ---- Q6: zero GLL-weighted mean (adjoint: projection out of u_L, dl/dg)
   const double mean = __ldcg(P.acc + ACC_MEAN);
@@ -352,8 +448,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
   return true;
 }
 
-inline size_t prepost_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown_w, long long d,
-                                 bool w_global = false) {
-  return gmres_smem_bytes<double>(m, M, n, ES, nown_b, nown_w, 0, 0, d, 0, w_global) +
-         (3 * (size_t)n * n + 64) * sizeof(double);
+inline size_t prepost_smem_bytes(int m, int M, int n, int ES, int W, int W_fd, long long d, bool w_global = false) {
+  return gmres_smem_bytes<double>(m, M, n, ES, W, 0, d, w_global) +
+         (size_t)(kGmresThreads / 32 / W_fd) * fd_item_bytes(n, W_fd);
 }

@@ -17,7 +17,8 @@
 
 struct alignas(16) RefineArgs {  // 16-byte multiple: staged with 16-byte copies in batched solves
   GmresArgs<float> ga;   // FP32 operator and vectors: x = inner y, t, y, c, chat, rhs (next inner rhs)
-  const double* Tc64;    // nel * M*M, FP64 T_e (column-major)
+  const uint4* T64;      // FP64 T_e per class, packed, and the row exponents (smpm_digits.cuh)
+  const short* Te64;
   double* xS;            // kp, FP64 Schur iterate
   const double* bS;      // kp, projected b_S
   double* r;             // kp, FP64 residual
@@ -31,10 +32,9 @@ struct alignas(16) RefineArgs {  // 16-byte multiple: staged with 16-byte copies
   double tol;
 };
 
-inline size_t refine_smem_bytes(int m, int M, int n, int ES, int nown_b, int nown_w, long long d,
-                                bool w_global = false, bool warp_elems = false) {
-  return gmres_smem_bytes<float>(m, M, n, ES, nown_b, nown_w, 0, 0, d, 0, w_global, 2, warp_elems) +
-         (2 * (size_t)M + 256 + 16) * sizeof(double);
+inline size_t refine_smem_bytes(int m, int M, int n, int ES, int W, long long d, bool w_global = false) {
+  return gmres_smem_bytes<float>(m, M, n, ES, W, 0, d, w_global) +
+         (size_t)(kGmresThreads / 32 / W) * (sizeof(uint4) * (size_t)digit_bwords<double>(M) + M * sizeof(double));
 }
 
 // One refinement step by the CTAs of a team; returns 1 when converged (done
@@ -42,14 +42,17 @@ inline size_t refine_smem_bytes(int m, int M, int n, int ES, int nown_b, int now
 __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, unsigned& epoch) {
   const GmresArgs<float>& a = R.ga;
   const Smem<float> s = carve(a, smraw);
-  double* p64 = reinterpret_cast<double*>(s.mats);
-  double* z64 = p64 + a.g.M;
-  double* red64 = z64 + a.g.M;
+  no_resident(a, s);
   const DevGeo& g = a.g;
-  const int n = g.n, M = g.M, G = a.G, rank = team_rank(a);
+  const int n = g.n, M = g.M, G = a.G, rank = team_rank(a), W = a.W_item, kt_n = digit_tiles(M);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = warp / W, part = warp % W,
+            ngrp = kGmresThreads / 32 / W;
+  uint4* Bf = reinterpret_cast<uint4*>(s.end + (size_t)grp * (sizeof(uint4) * (size_t)digit_bwords<double>(M) +
+                                                              M * sizeof(double)));
+  double* rw = reinterpret_cast<double*>(Bf + digit_bwords<double>(M));  // x_S on the element's slots, then its weighted residual entries
   int trace_n = 0;
   // ---- R1-R3: t = M^-1 y, S t, c_hat
-  if (!black_phase(a, s, (MatStream<float>*)nullptr, a.x, 1.0, (const float*)nullptr)) return -1;
+  black_phase(a, s, (const float*)a.x, 1.0, (const float*)nullptr);
   if (!apply_op(a, s, a.x, 1.0, true, trace_n, epoch)) return -1;
   // ---- R4: x_S += t - Z (c_hat - c_hat_r); y <- 0 for the next inner solve
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
@@ -59,69 +62,44 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
       R.xS[en.x] += (double)__ldcg(a.t + en.x) - entry_zw(g, en) * (__ldcg(a.chat + en.z) - R.chat_r[en.z]);
     a.x[en.x] = 0.f;
   }
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return -1;
+  if (!team_sync(a, epoch)) return -1;
   // ---- R5: r = b_S - S x_S (FP64), ||r||^2, Z^T r
   double pr = 0;
-  if (a.warp_elems) {  // one warp per element (elements rank + k G, k = warp, warp + nwarps, ...)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    double* pw = reinterpret_cast<double*>(s.wb + (size_t)warp * warp_scratch(M));  // 2M doubles fit in 5M floats
-    double* zw = pw + M;
-    for (long long e = rank + (long long)warp * G; e < g.nel; e += (long long)nwarps * G) {
-      for (int i = lane; i < M; i += 32) pw[i] = __ldcg(R.xS + e * M + i);
-      __syncwarp();
-      warp_gemv(R.Tc64 + (size_t)__ldg(a.tr + e) * M * M, pw, zw, M, lane);
-      for (int i = lane; i < M; i += 32) {  // pw is free again: it takes the residual entries
-        const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
-        double rr = 0;
-        if (e2 >= 0) {
-          const size_t sl = (size_t)e2 * M + (F ^ 1) * n + t;
-          rr = R.bS[sl] - (__ldcg(R.xS + sl) + zw[i]);
-          R.r[sl] = rr;
-          pr += rr * rr;
-          rr *= dev_zw(g, e2, F ^ 1);  // its weight in Z^T r
-        }
-        pw[i] = rr;
-      }
-      __syncwarp();
-      if (lane < 4) {  // face F summed by lane F
-        const int F = lane, j = dev_iface(g, (int)e, F);
-        double sum = 0;
-        for (int t = 0; t < n; ++t) sum += pw[F * n + t];
-        if (j >= 0 && sum != 0.0) atomicAdd(R.cr + j, sum);
-      }
-      __syncwarp();
-    }
-  }
-  for (long long e = rank; e < (a.warp_elems ? 0 : g.nel); e += G) {
-    for (int i = threadIdx.x; i < M; i += blockDim.x) p64[i] = __ldcg(R.xS + e * M + i);
-    __syncthreads();
-    gemv_split(R.Tc64 + (size_t)__ldg(a.tr + e) * M * M, M, p64, z64, M, M, red64);
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-      const int F = i / n, t = i % n, e2 = dev_neighbour(g, (int)e, F);
+  for (long long el = rank + (long long)grp * G; el < g.nel; el += (long long)ngrp * G) {
+    const int e = (int)el, ct = __ldg(a.dm.tcls + e);
+    for (int i = part * 32 + lane; i < M; i += 32 * W) rw[i] = __ldcg(R.xS + el * M + i);
+    item_sync(grp, W);
+    const int E = pack_one<double>(Bf, rw, M, lane, part, W);
+    item_sync(grp, W);
+    for (int mt = part; mt < kt_n; mt += W) {
+      const int row = tile1_row(mt, lane, M);
+      Facing<double> f{};
+      if (row >= 0) f = facing_entry(g, e, row, R.xS, R.xS);
+      const double z = digits_tile1<double>(R.T64 + (size_t)ct * digit_words<double>(M, M), R.Te64 + (size_t)ct * M, Bf, M,
+                                            kt_n, mt, lane, E);
+      if (row < 0) continue;
       double rr = 0;
-      if (e2 >= 0) {
-        const size_t sl = (size_t)e2 * M + (F ^ 1) * n + t;
-        rr = R.bS[sl] - (__ldcg(R.xS + sl) + z64[i]);
-        R.r[sl] = rr;
+      if (f.sl >= 0) {
+        rr = R.bS[f.sl] - (f.t + z);
+        R.r[f.sl] = rr;
         pr += rr * rr;
-        rr *= dev_zw(g, e2, F ^ 1);  // its weight in Z^T r
+        if (g.zw) rr *= f.w1;  // its weight in Z^T r
       }
-      red64[i] = rr;
+      rw[row] = rr;  // (x_S is packed: its place is free)
     }
-    __syncthreads();
-    if (threadIdx.x < 128) {  // face F summed by warp F
-      const int F = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    item_sync(grp, W);
+    if (part == 0) {  // face F summed by the eight lanes 8 F + r
+      const int F = lane >> 3, j = dev_iface(g, e, F);
       double sum = 0;
-      for (int t = lane; t < n; t += 32) sum += red64[F * n + t];
-      sum = warp_sum(sum);
-      const int j = dev_iface(g, (int)e, F);
-      if (lane == 0 && j >= 0 && sum != 0.0) atomicAdd(R.cr + j, sum);
+      for (int t = lane & 7; t < n; t += 8) sum += rw[F * n + t];
+      for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if ((lane & 7) == 0 && j >= 0 && sum != 0.0) atomicAdd(R.cr + j, sum);
     }
-    __syncthreads();
+    item_sync(grp, W);
   }
   pr = warp_sum(pr);
   if ((threadIdx.x & 31) == 0 && pr != 0.0) atomicAdd(R.rn, pr);
-  if (!grid_sync(a.bar, a.err, epoch, a.G)) return -1;
+  if (!team_sync(a, epoch)) return -1;
   // ---- R6: convergence test (uniform), else c_hat_r = C^+ Z^T r
   const double rho = sqrt(__ldcg(R.rn)), target = R.tol * sqrt(__ldcg(R.rgn));
   if (rank == 0 && threadIdx.x == 0) *R.nref += 1;
@@ -129,12 +107,7 @@ __device__ SMPM_BODY int refine_body(const RefineArgs& R, unsigned char* smraw, 
     if (rank == 0 && threadIdx.x == 0) *R.done = 1;
     return 1;
   }
-  {
-    GmresArgs<float> b = a;
-    b.c = R.cr;
-    b.chat = R.chat_r;
-    if (!coarse_solve(b, s, epoch)) return -1;
-  }
+  if (!coarse_solve(a, s, epoch, R.cr, R.chat_r)) return -1;
   // ---- R7: next inner right-hand side P r (FP32); Z^T r back to zero
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
     const int4 en = owned_entry(a, i);

@@ -20,9 +20,11 @@
 // (smpm_batch.cuh): teams of CTAs run the same bodies with team barriers.
 //
 // The single-operator entry points use small one-pass kernels:
-//   y = S v          k_schur_warpk (several warps per element, M <= 96),
-//                    k_schur_stream (bulk-copy ring, larger M), k_schur
-//                    (from global memory when one matrix exceeds the ring);
+//   y = S v          k_schur_class (class-shared digits, eight elements per
+//                    CTA; what AUTO takes where the tiles fill), k_schur_warpk
+//                    (several warps per element, M <= 96), k_schur_stream
+//                    (bulk-copy ring, larger M), k_schur (from global memory
+//                    when one matrix exceeds the ring);
 //                    batched: k_schur_warp_batch, k_schur_stream_batch;
 //   S M^-1 and M^-1  k_black (block solves a = G (p - X q), b = q - T_e a),
 //                    k_white (white elements' T_e products, c = Z^T y);
@@ -350,6 +352,33 @@ __global__ void k_assemble(DevGeo g, const double* __restrict__ t, const double*
   if (j < 0) { x[s] = 0.0; return; }
   double cb = chat_b ? chat_b[j] : 0.0;
   x[s] = t[s] - dev_zw(g, e, F) * ((chat ? chat[j] : 0.0) - cb);
+}
+
+// ---- bulk copies into shared memory (apply kernels) ----
+__device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
+  for (long long spins = 0; spins < (1LL << 22); ++spins) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
 }
 
 #include "smpm_gmres.cuh"
@@ -796,41 +825,62 @@ cudaError_t launch_schur_warp(const ElemMeta<S>* tab, long long nelem, const S* 
 // 9 classes: interior, 4 edges, 4 corners), so y = v + scatter(T_c X_c) with
 // X_c the M x n_c matrix of the own slots of all elements of class c: a dense
 // contraction on the tensor cores (smpm_digits.cuh), with the vectors as the
-// only traffic from HBM.  One CTA per tile of up to kClassTile elements of one
-// class, one warp per eight of them: the warp cuts their slot vectors into
-// digits (in its shared scratch) and walks the row tiles of T_c, whose packed
-// digits all warps of the CTA read from L1.
-constexpr int kClassTile = 32, kClassThreads = 32 * (kClassTile / 8);
-template <typename S>
-inline size_t class_smem(int M) {
-  return (size_t)(kClassTile / 8) * digit_bwords<S>(M) * sizeof(uint4);
-}
+// only traffic from HBM.  One CTA per eight elements of one class, one warp per
+// 16 rows of T_c: the warps cut the slot vectors into digits together (shared
+// memory), each then runs its row tile; T_c's digits come from L1.  Many small
+// CTAs per SM: a row tile is a chain of loads and dependent products.
+constexpr int kClassTile = 8;
 
 template <typename S>
-__global__ void __launch_bounds__(kClassThreads) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
-                                                               const short* __restrict__ Texp,
-                                                               const int* __restrict__ tiles,
-                                                               const int* __restrict__ elems, const S* v, S* y) {
+__global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
+                                                     const short* __restrict__ Texp, const int* __restrict__ tiles,
+                                                     const int* __restrict__ elems, const S* v, S* y) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const int M = g.M, n = g.n, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int M = g.M, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cls = tiles[3 * blockIdx.x], start = tiles[3 * blockIdx.x + 1], cnt = tiles[3 * blockIdx.x + 2];
-  if (warp * 8 >= cnt) return;
-  uint4* Bf = reinterpret_cast<uint4*>(raw) + (size_t)warp * digit_bwords<S>(M);
-  const int left = cnt - warp * 8;  // elements of this warp (of 8)
-  const int* el = elems + start + warp * 8;
-  const int mine = __ldg(el + min(lane >> 2, left - 1));
-  const S* vm = v + (size_t)mine * M;
-  const bool live = (lane >> 2) < left;
-  const int E = pack_cols<S>(Bf, M, lane, [&](int k, int) { return live ? __ldg(vm + k) : S(0); });
-  const uint4* A = Tdig + (size_t)cls * digit_words<S>(M, M);
-  const short* er = Texp + (size_t)cls * M;
-  for (int mt = 0; mt < kt_n; ++mt)
-    digits_tile8<S>(A, er, Bf, M, kt_n, mt, lane, E, [&](int row, int col, S z) {
-      if (col >= left) return;
-      const int e = __ldg(el + col), F = row / n, tt = row - F * n, e2 = dev_neighbour(g, e, F);
-      const size_t sl = e2 >= 0 ? (size_t)e2 * M + (F ^ 1) * n + tt : (size_t)e * M + row;
-      y[sl] = e2 >= 0 ? v[sl] + z : v[sl];
-    });
+  uint4* Bf = reinterpret_cast<uint4*>(raw);
+  __shared__ int Emax[8];  // largest exponent field per column
+  if (threadIdx.x < 8) Emax[threadIdx.x] = 1;
+  // this warp's 16 slots of the eight elements, loaded once
+  const int* el = elems + start;
+  const int gc = lane >> 2, q = lane & 3;
+  const S* vm = v + (size_t)__ldg(el + min(gc, cnt - 1)) * M;
+  S x[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int k = warp * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
+    x[u] = (gc < cnt && k < M) ? __ldg(vm + k) : S(0);
+  }
+  // outputs of the warp's row tile: facing slots and what they hold
+  long long sl[4];
+  bool push[4];
+  S vf[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = warp * 16 + gc + 8 * (u >> 1), c = 2 * q + (u & 1);
+    sl[u] = -1;
+    push[u] = false;
+    vf[u] = S(0);
+    if (r >= M || c >= cnt) continue;
+    const int e = __ldg(el + c), F = r / g.n, e2 = dev_neighbour(g, e, F);
+    push[u] = e2 >= 0;
+    sl[u] = e2 >= 0 ? (long long)e2 * M + (F ^ 1) * g.n + r - F * g.n : (long long)e * M + r;
+    vf[u] = __ldg(v + sl[u]);
+  }
+  __syncthreads();
+  int E = max(max(exp_field(x[0]), exp_field(x[1])), max(exp_field(x[2]), exp_field(x[3])));
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+  if (q == 0) atomicMax(Emax + gc, E);
+  __syncthreads();
+  E = Emax[gc];
+  pack_tile<S>(Bf, warp, lane, x, E);
+  __syncthreads();
+  const Tile8<S> t = tile8_products<S>(Tdig + (size_t)cls * digit_words<S>(M, M), Texp + (size_t)cls * M, Bf, M, kt_n,
+                                       warp, lane, E);
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    if (sl[u] >= 0) y[sl[u]] = push[u] ? vf[u] + t.z[u] : vf[u];
 }
 
 template <typename S>
@@ -854,20 +904,20 @@ struct smpm_handle_s {
   bool factored = false;
   bool op_factored = false;  // operator-only factor step (SMPM_FLAG_OPERATOR_ONLY): S can be applied
   // element classes (face-type masks) for the class-shared apply
-  int ncls = 0, ntiles = 0, cls_ok = 0;  // cls_ok: packed, and the kernel's shared-memory limit is set
+  int ncls = 0, ntiles = 0, cls_ok = 0;  // cls_ok: the class matrices are packed
   int apply_kind = 0;                     // kernel of smpm_apply_schur(32): SMPM_APPLY_*
   // packed digits (smpm_digits.cuh) of one T_e per class, G_b and the four X_F
   // per block class, their row exponents, and the class of each element / block
   struct DigitSet {
-    uint4 *T = nullptr, *G = nullptr, *X = nullptr;
-    short *Te = nullptr, *Ge = nullptr, *Xe = nullptr;
-  } dig, dig32;
+    uint4 *T = nullptr, *G = nullptr, *X = nullptr, *B = nullptr;
+    short *Te = nullptr, *Ge = nullptr, *Xe = nullptr, *Be = nullptr;
+  } dig, dig32, diga;  // forward FP64 / FP32, adjoint
+  FdMats fd{}, fda{};  // packed fast-diagonalisation factors, forward / adjoint
   int *dtcls = nullptr, *dbcls = nullptr;
   int* dtiles = nullptr;     // ntiles * (class, first, count) into dclsel
   int* dclsel = nullptr;     // nel: elements sorted by class
-  // tables of the solve kernels (GmresArgs): class representatives, block
-  // entries, interfaces per element, S Z per slot (forward, adjoint)
-  int *dtr = nullptr, *dgr = nullptr;
+  // tables of the solve kernels (GmresArgs): block entries, interfaces per
+  // element, S Z per slot (forward, adjoint)
   int4 *dbt = nullptr, *dif4 = nullptr;
   double *dRd = nullptr, *dRda = nullptr;
   // C^+ by strips (StripFactors) on the device, forward and adjoint, and the
@@ -876,8 +926,6 @@ struct smpm_handle_s {
   CoarseStrips<float> st32{};
   double st_products = 0, sta_products = 0;
   double* wgsep = nullptr;
-  double* dHT = nullptr;     // H column-major, for the fused coarse solve of the Arnoldi steps
-  double* wchatd = nullptr;  // 2 d: its two c_hat buffers
   Factors f;
   DevGeo dg{};
   // device factors
@@ -897,29 +945,30 @@ struct smpm_handle_s {
   int* werr = nullptr;
   GState* wgs = nullptr;
   struct {
-    int grid = 0, nown_b = 0, nown_w = 0, ES = 0, mats_smem = 0, basis_smem = 0, stream_mats = 0, buf_elems = 0,
-        nbuf = 2, warp_elems = 0;
+    int grid = 0, nown_b = 0, nown_w = 0, ES = 0, basis_smem = 0, W = 1, res_T = 0, res_G = 0, blk = 0, tab = 0, res_H = 0, W_pp = 1, W_fd = 1;
+    bool wg = false;  // w, w2 in global memory
     size_t smem = 0, smem_pp = 0;
   } gm;  // launch shape of the persistent GMRES kernel
-  double* wvown = nullptr;
+  double *wvown = nullptr, *wscr = nullptr;
+  float* wscr32 = nullptr;
   double* wacc = nullptr;
   // mixed precision: FP32 operator copies and work vectors, FP64 residual
-  float *dT32 = nullptr, *dG32 = nullptr, *dX32 = nullptr;
+  float* dT32 = nullptr;
   float* dH32 = nullptr;  // FP32 copy of the coarse inverse, for the FP32 inner solves
   float *wx32 = nullptr, *wt32 = nullptr, *wy32 = nullptr, *wV32 = nullptr, *wrg32 = nullptr, *wvown32 = nullptr;
   double *wr = nullptr, *wcr = nullptr, *wrn = nullptr;
   int *wdone = nullptr, *wnref = nullptr;
   struct {
-    int basis_smem = 0, mats_smem = 0, stream_mats = 0, buf_elems = 0, nbuf = 2, warp_elems = 0;
+    int basis_smem = 0, W = 1, res_T = 0, res_G = 0, blk = 0, tab = 0, res_H = 0, W_ref = 1;
     size_t smem = 0, smem_ref = 0;
   } gm32;
   double *wacc8 = nullptr, *wxs = nullptr, *dZtuS = nullptr;
   // transposed system for the adjoint solve (SMPM_FLAG_ADJOINT)
-  double *dTa = nullptr, *dGa = nullptr, *dXa = nullptr, *dHa = nullptr;
+  double *dHa = nullptr, *dHp = nullptr;  // coarse inverses with padded rows: adjoint, forward
   // element tables of the register-streamed apply (k_schur_warp_batch / k_schur_warpk)
   ElemMeta<double>* dtab64 = nullptr;
   ElemMeta<float>* dtab32 = nullptr;
-  double *dfdxT = nullptr, *dfdyT = nullptr, *duSa = nullptr, *dZtuSa = nullptr;
+  double *duSa = nullptr, *dZtuSa = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // bracket the GMRES kernel of each solve
   cudaEvent_t evp = nullptr, evq = nullptr;  // start of k_pre, end of k_post
   unsigned char* wctl = nullptr;              // [bar x4 | err | pad | acc8] zeroed per solve
@@ -1122,14 +1171,23 @@ bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
   }
 }
 
-// y = S v with the handle's apply kernel (SMPM_APPLY_AUTO: one warp per
-// element, register-streamed from global memory, for M <= 96 -- 1, 2 or 4
-// elements per warp by the element count -- else the shared-memory stream).
+// y = S v with the handle's apply kernel.  SMPM_APPLY_AUTO: the class-shared
+// products where the elements fall into few enough classes that the tiles of
+// eight are filled to a fifth on average (any uniform grid from 4x4 on;
+// measured, FP64 / FP32 in us, best per-element kernel against the class
+// kernel: 4x59, n = 21 14.0 / 9.3 against 10.8 / 8.4; 32x32, n = 24 26.8 / 12.1
+// against 11.6 / 8.3; 96x96, n = 24 162 / 76 against 35 / 20; 128x128, n = 16
+// 184 / 61 against 28 / 18).  Graded grids, mostly one element to a class: one
+// warp per element, register-streamed from global memory, for M <= 96 -- 1, 2
+// or 4 warps per element by the element count -- else the shared-memory stream.
 template <typename S>
 smpm_status launch_schur_kind(smpm_handle h, int kind, const S* v, S* y, cudaStream_t st) {
   const bool fp32 = sizeof(S) == 4;
   const ElemMeta<S>* tab = reinterpret_cast<const ElemMeta<S>*>(fp32 ? (const void*)h->dtab32 : (const void*)h->dtab64);
   const S* T = reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT);
+  if (kind == SMPM_APPLY_AUTO && apply_kind_ok(h, SMPM_APPLY_CLASS, fp32) &&
+      (long long)h->ntiles * kClassTile <= 5 * h->g.nel)
+    kind = SMPM_APPLY_CLASS;
   if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
   if (kind == SMPM_APPLY_STREAM) return launch_schur_stream<S>(h, T, v, y, st);
   if (kind == SMPM_APPLY_CLASS) {
@@ -1224,46 +1282,59 @@ smpm_status print_trace(smpm_handle h, cudaStream_t st) {
   return SMPM_OK;
 }
 
-// Shared-memory layout of the owned data of the GMRES kernel, in order of
-// preference: resident matrices + basis; streamed matrices (two bulk-copy
-// buffers) + basis; streamed matrices with the basis in global memory; all
-// global.
+// Shared memory of the GMRES body: warps per item (more of them when the
+// groups' scratch would not fit) and the Krylov basis resident when it fits.
+// smem above the budget: nothing fits.
 struct Layout {
-  int basis_smem, mats_smem, stream_mats, buf_elems, nbuf, warp_elems;
+  int basis_smem, W, res_T, res_G, blk, tab, res_H;
   size_t smem;
 };
 
 template <typename S>
-Layout choose_layout(const Geometry& g, int m, int ES, int nown_b, int nown_w, int precond, bool no_smem,
-                     bool force_stream, int smem_optin, bool w_global = false, bool warp = false) {
+Layout choose_layout(const Geometry& g, int m, int ES, int items, bool no_smem, size_t budget, bool w_global, int blk, int G, bool rows_H) {
   Layout L;
-  L.warp_elems = warp ? 1 : 0;  // warps read their matrices resident or from global memory: no stream
-  L.buf_elems = g.M * g.M + 4 * g.n * g.n;
-  L.basis_smem = no_smem ? 0 : 1;
-  L.mats_smem = (no_smem || force_stream) ? 0 : 1;
-  L.stream_mats = 0;
-  L.nbuf = 2;
-  auto need = [&]() {
-    return gmres_smem_bytes<S>(m, g.M, g.n, ES, nown_b, nown_w, L.basis_smem, L.mats_smem, g.d,
-                               L.stream_mats ? L.buf_elems : 0, w_global, L.nbuf, warp);
+  L.blk = blk;
+  L.W = item_warps(items);
+  L.basis_smem = L.res_T = L.res_G = L.tab = L.res_H = 0;
+  auto need = [&] {
+    return gmres_smem_bytes<S>(m, g.M, g.n, ES, L.W, L.basis_smem, g.d, w_global, L.res_T, L.res_G, blk,
+                               L.tab, L.res_H ? coarse_row_bytes<S>(g.d, G) : 0);
   };
-  if (need() > (size_t)smem_optin) L.mats_smem = 0;
-  if (!L.mats_smem && !no_smem && precond > 0 && !warp) {
-    L.stream_mats = 1;
-    if (need() > (size_t)smem_optin) L.basis_smem = 0;
-    if (need() > (size_t)smem_optin) L.stream_mats = 0;
+  while (L.W < kGmresThreads / 32 && need() > budget) L.W *= 2;
+  if (!no_smem) {  // in order of use per step: T_e of the main class, G_b, the entries' table, the basis, rows of H, a second T_e
+    auto take = [&](int& v, int to) {
+      const int old = v;
+      v = to;
+      if (need() > budget) v = old;
+    };
+    take(L.res_T, 1);
+    take(L.res_G, 1);
+    take(L.tab, 1);
+    take(L.basis_smem, 1);
+    if (rows_H) take(L.res_H, 1);
+    if (L.res_T == 1) take(L.res_T, 2);
   }
-  if (need() > (size_t)smem_optin) L.basis_smem = 0;
-  if (L.stream_mats)  // deepest stream that fits: nbuf - 1 copies in flight during each item
-    while (L.nbuf < kMaxStreamBufs) {
-      ++L.nbuf;
-      if (need() > (size_t)smem_optin) {
-        --L.nbuf;
-        break;
-      }
-    }
   L.smem = need();
   return L;
+}
+
+// The same for the pre/post bodies (warps per item and per element solve) and
+// for the refinement body.
+size_t prepost_shape(const Geometry& g, int m, int ES, int items, int G, size_t budget, bool w_global, int* W, int* W_fd) {
+  *W = item_warps(items);
+  *W_fd = std::min(item_warps((g.nel + G - 1) / G), std::max(1, (g.n + 7) / 8 > 2 ? 4 : (g.n + 7) / 8));
+  auto need = [&] { return prepost_smem_bytes(m, g.M, g.n, ES, *W, *W_fd, g.d, w_global); };
+  while (need() > budget && (*W < kGmresThreads / 32 || *W_fd < kGmresThreads / 32)) {
+    if (*W_fd < kGmresThreads / 32) *W_fd *= 2;
+    if (need() > budget && *W < kGmresThreads / 32) *W *= 2;
+  }
+  return need();
+}
+size_t refine_shape(const Geometry& g, int m, int ES, int items, size_t budget, bool w_global, int* W) {
+  *W = item_warps(items);
+  auto need = [&] { return refine_smem_bytes(m, g.M, g.n, ES, *W, g.d, w_global); };
+  while (need() > budget && *W < kGmresThreads / 32) *W *= 2;
+  return need();
 }
 
 // Whether C^+ by strips is the cheaper form for R columns on a team of G CTAs:
@@ -1274,11 +1345,25 @@ bool strips_pay(long long d, double products, int G, int R, bool fp32) {
   return R * ((double)d * d - products) / G >= (fp32 ? 24000.0 : 9000.0);
 }
 
+// Whether black blocks are solved with their whole inverse (black_block): a
+// CTA's blocks then read 7/4 M^2 more entries each, at about 64 bytes per SM
+// cycle, and save three of four dependent stages (about 8,000 cycles at
+// M = 64, 5,000 at M = 20).
+template <typename S>
+int block_pays(smpm_handle h) {
+  const double bytes = 1.75 * h->g.M * h->g.M * sizeof(S) * h->gm.nown_b;
+  const bool have = sizeof(S) == 4 ? h->dig32.B != nullptr : h->dig.B != nullptr;
+  return have && h->opts.precond != 0 && bytes <= 256e3;
+}
+
 // Form of the coarse solve for a solve of R columns by a.G CTAs.
 template <typename S>
 void choose_coarse(GmresArgs<S>& a, double products, int R) {
   a.use_strips = a.precond == 2 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4);
-  a.fused = a.HT && !a.use_strips;
+}
+
+DigitMats digit_mats(smpm_handle h, const smpm_handle_s::DigitSet& d) {
+  return {d.G, d.X, d.T, d.Ge, d.Xe, d.Te, h->dbcls, h->dtcls, d.B, d.Be};
 }
 
 // Kernel arguments shared by the three cooperative kernels of a solve
@@ -1290,24 +1375,28 @@ GmresArgs<double> gmres_args(smpm_handle h, double tol, bool adj = false) {
   a.white = h->dwhite;
   a.nblack = (int)h->f.black.size();
   a.nwhite = (int)h->f.white.size();
-  a.Tc = h->dT; a.Gc = h->dG; a.Xc = h->dX; a.Rd = h->dRd; a.H = h->dH;
-  if (adj) { a.Tc = h->dTa; a.Gc = h->dGa; a.Xc = h->dXa; a.Rd = h->dRda; a.H = h->dHa; a.g.zw = h->dzwa; }
-  a.tr = h->dtr; a.gr = h->dgr; a.bt = h->dbt; a.if4 = h->dif4;
+  a.dm = digit_mats(h, adj ? h->diga : h->dig);
+  a.Rd = h->dRd; a.H = h->dHp;
+  if (adj) { a.Rd = h->dRda; a.H = h->dHa; a.g.zw = h->dzwa; }
+  a.bt = h->dbt; a.if4 = h->dif4;
   a.vglob = h->wV; a.vown = h->wvown; a.t = h->wt; a.y = h->wy;
   a.c = h->wc; a.chat = h->wchat; a.rhs = h->wrg; a.x = h->wx;
   a.acc = h->wacc; a.gs = h->wgs; a.bar = h->wbar; a.err = h->werr;
   a.precond = h->opts.precond; a.m = h->opts.restart; a.maxit = h->opts.maxit; a.tol = tol;
   a.nown_b = h->gm.nown_b; a.nown_w = h->gm.nown_w; a.ES = h->gm.ES;
-  a.mats_smem = h->gm.mats_smem; a.basis_smem = h->gm.basis_smem;
-  a.stream_mats = h->gm.stream_mats; a.buf_elems = h->gm.buf_elems; a.nbuf = h->gm.nbuf;
-  a.warp_elems = h->gm.warp_elems;
+  a.basis_smem = h->gm.basis_smem;
+  a.W_item = h->gm.W;
+  a.res_T = h->gm.res_T;
+  a.res_G = h->gm.res_G;
+  a.blk = h->gm.blk && a.dm.B;
+  a.tab = h->gm.tab;
+  a.res_H = h->gm.res_H;
+  a.wscr = h->wscr;
   a.trace = h->wtrace;
   a.trace_cap = h->wtrace ? kTraceCap / 2 : 0;
   a.skip = nullptr;
   a.G = h->gm.grid;
   a.base = 0;
-  a.HT = adj ? nullptr : h->dHT;
-  a.chatd = h->wchatd;
   a.strips = adj ? h->sta : h->st;
   a.gsep = h->wgsep;
   choose_coarse(a, adj ? h->sta_products : h->st_products, 1);
@@ -1321,23 +1410,27 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.white = h->dwhite;
   a.nblack = (int)h->f.black.size();
   a.nwhite = (int)h->f.white.size();
-  a.Tc = h->dT32; a.Gc = h->dG32; a.Xc = h->dX32; a.Rd = h->dRd; a.H = h->dH32;
-  a.tr = h->dtr; a.gr = h->dgr; a.bt = h->dbt; a.if4 = h->dif4;
+  a.dm = digit_mats(h, h->dig32);
+  a.Rd = h->dRd; a.H = h->dH32;
+  a.bt = h->dbt; a.if4 = h->dif4;
   a.vglob = h->wV32; a.vown = h->wvown32; a.t = h->wt32; a.y = h->wy32;
   a.c = h->wc; a.chat = h->wchat; a.rhs = h->wrg32; a.x = h->wx32;
   a.acc = h->wacc; a.gs = h->wgs; a.bar = h->wbar; a.err = h->werr;
   a.precond = h->opts.precond; a.m = h->opts.restart; a.maxit = h->opts.restart; a.tol = tol;
   a.nown_b = h->gm.nown_b; a.nown_w = h->gm.nown_w; a.ES = h->gm.ES;
-  a.mats_smem = h->gm32.mats_smem; a.basis_smem = h->gm32.basis_smem;
-  a.stream_mats = h->gm32.stream_mats; a.buf_elems = h->gm32.buf_elems; a.nbuf = h->gm32.nbuf;
-  a.warp_elems = h->gm32.warp_elems;
+  a.basis_smem = h->gm32.basis_smem;
+  a.W_item = h->gm32.W;
+  a.res_T = h->gm32.res_T;
+  a.res_G = h->gm32.res_G;
+  a.blk = h->gm32.blk;
+  a.tab = h->gm32.tab;
+  a.res_H = h->gm32.res_H;
+  a.wscr = h->wscr32;
   a.trace = nullptr;
   a.trace_cap = 0;
   a.skip = h->wdone;
   a.G = h->gm.grid;
   a.base = 0;
-  a.HT = h->dHT;
-  a.chatd = h->wchatd;
   a.strips = h->st32;
   a.gsep = h->wgsep;
   choose_coarse(a, h->st_products, 1);
@@ -1351,12 +1444,12 @@ PrePostArgs prepost_args(smpm_handle h, double tol, const double* f, const doubl
   const int m = h->opts.restart;
   PrePostArgs P{};
   P.ga = gmres_args(h, tol, adj);
-  P.ga.mats_smem = 0;
   P.ga.basis_smem = 0;
-  P.ga.stream_mats = 0;
-  P.ga.warp_elems = 0;  // the pre/post kernels' shared memory has no per-warp scratch
+  P.ga.W_item = h->gm.W_pp;
+  P.ga.blk = P.ga.tab = P.ga.res_H = 0;
+  P.W_fd = h->gm.W_fd;
   P.ga.trace = nullptr;
-  P.fdx = h->dfdx; P.fdy = h->dfdy; P.D = h->dD; P.uL = h->duL; P.uS = h->duS; P.what = h->dwhat;
+  P.fd = h->fd; P.D = h->dD; P.uL = h->duL; P.uS = h->duS; P.what = h->dwhat;
   P.ZtuS = h->dZtuS; P.f = f; P.gn = gn; P.b = h->wb; P.bS = h->wbS; P.rg = h->wrg; P.cb = h->wcb;
   P.chatb = h->wchatb; P.xs = h->wxs; P.u = u; P.acc = h->wacc8;
   double* zs[7] = {h->wx, h->wt, h->wy, h->wV, h->wbS, h->wrg, h->wxs};
@@ -1373,7 +1466,7 @@ PrePostArgs prepost_args(smpm_handle h, double tol, const double* f, const doubl
     P.adjoint = 1;
     P.gg = gg;
     P.gn = nullptr;
-    P.fdx = h->dfdxT; P.fdy = h->dfdyT; P.uS = h->duSa; P.ZtuS = h->dZtuSa;
+    P.fd = h->fda; P.uS = h->duSa; P.ZtuS = h->dZtuSa;
   }
   return P;
 }
@@ -1382,11 +1475,12 @@ PrePostArgs prepost_args(smpm_handle h, double tol, const double* f, const doubl
 RefineArgs refine_args(smpm_handle h, const GmresArgs<float>& a, double tol) {
   RefineArgs RA{};
   RA.ga = a;
-  RA.ga.mats_smem = 0;
   RA.ga.basis_smem = 0;
-  RA.ga.stream_mats = 0;
+  RA.ga.W_item = h->gm32.W_ref;
+  RA.ga.blk = RA.ga.tab = RA.ga.res_H = 0;
   RA.ga.rhs = h->wrg32;
-  RA.Tc64 = h->dT;
+  RA.T64 = h->dig.T;
+  RA.Te64 = h->dig.Te;
   RA.xS = h->wxs;
   RA.bS = h->wbS;
   RA.r = h->wr;
@@ -1413,7 +1507,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   PrePostArgs P = prepost_args(h, tol, f, gn, u, true);
   CU(cudaEventRecord(h->evp, st));
   {
-    P.ga.bar = h->wbar + 0;
+    P.ga.bar = h->wbar;
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_pre(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
@@ -1422,7 +1516,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   CU(cudaEventRecord(h->ev0, st));
   for (int ref = 0; ref < kMaxRefine; ++ref) {
     GmresArgs<float> a = gmres_args32(h, kInnerTol);
-    a.bar = h->wbar + 2 + 2 * ref;
+    a.bar = h->wbar;
     a.its_out = reinterpret_cast<int*>(h->wctl + 592) + ref;
     if (ref == 0 && h->wtrace) {
       a.trace = h->wtrace;
@@ -1435,7 +1529,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
       CHECK_LAUNCH();
     }
     RefineArgs RA = refine_args(h, a, tol);
-    RA.ga.bar = h->wbar + 3 + 2 * ref;
+    RA.ga.bar = h->wbar;
     RA.rn = h->wrn + ref;
     void* args[] = {&RA};
     CU(cudaLaunchCooperativeKernel(fn_refine(), dim3(h->gm.grid), dim3(kGmresThreads), args,
@@ -1444,7 +1538,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   }
   CU(cudaEventRecord(h->ev1, st));
   {
-    P.ga.bar = h->wbar + 1;
+    P.ga.bar = h->wbar;
     P.assembled = 1;
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
@@ -1509,7 +1603,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   // pre/post accumulators (contiguous); everything else is zeroed in k_pre
   CU(cudaMemsetAsync(h->wctl, 0, kCtlBytes, st));
   PrePostArgs P = prepost_args(h, tol, f, gn, u, false, adj, gg);
-  P.ga.bar = h->wbar + 0;
+  P.ga.bar = h->wbar;
   if (h->wtrace) {  // pre and post trace into the upper halves of the buffer
     P.ga.trace = h->wtrace + kTraceCap / 2;
     P.ga.trace_cap = kTraceCap / 4;
@@ -1524,7 +1618,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   CU(cudaEventRecord(h->ev0, st));
   {
     GmresArgs<double> a = gmres_args(h, tol, adj);
-    a.bar = h->wbar + 1;
+    a.bar = h->wbar;
     void* args[] = {&a};
     CU(cudaLaunchCooperativeKernel(fn_gmres64(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm.smem, st));
@@ -1532,7 +1626,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   }
   CU(cudaEventRecord(h->ev1, st));
   {
-    P.ga.bar = h->wbar + 2;
+    P.ga.bar = h->wbar;
     if (h->wtrace) P.ga.trace = h->wtrace + 3 * (kTraceCap / 4);
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
@@ -1589,11 +1683,14 @@ smpm_status lalloc(smpm_handle h, P** p, size_t count) {
   return SMPM_OK;
 }
 
-// control block of a lockstep solve: 32 barrier counters (pre 0, post 1,
-// inner GMRES 2 + 2 ref, refinement 3 + 2 ref), err at 128; column k's block
+// control block of a lockstep solve: barrier counter (shared by the solve's
+// kernels in turn) at 0, err at 128; column k's block
 // at kLockCtlBytes + k kLockColBytes: acc8 (8 doubles) | done, nref (ints at
 // +64) | rn[kMaxRefine] at +128
 constexpr size_t kLockCtlBytes = 256;  // (kLockColBytes, the column block size, is shared with the batch)
+
+// Entries per CTA and column in a basis slice (whole 16-byte groups).
+int basis_entries(int M, int nown_b) { return (2 * M * nown_b + 3) & ~3; }
 
 // Workspace of the lockstep kernels for up to R columns (FP32 inner buffers
 // too when the handle is factored for mixed precision).
@@ -1605,7 +1702,7 @@ smpm_status lock_prepare(smpm_handle h, int R) {
   int cap = 2;
   while (cap < R) cap *= 2;
   const Geometry& g = h->g;
-  const size_t kp = g.kp, r = g.r, d = g.d, m = h->opts.restart, G = h->gm.grid, ES = h->gm.ES;
+  const size_t kp = g.kp, r = g.r, d = g.d, m = h->opts.restart, G = h->gm.grid, ES = basis_entries(g.M, h->gm.nown_b);
   smpm_status s;
   if ((s = lalloc(h, &L.b, cap * r)) || (s = lalloc(h, &L.bS, cap * kp)) || (s = lalloc(h, &L.rg, cap * kp)) ||
       (s = lalloc(h, &L.cb, cap * d)) || (s = lalloc(h, &L.chatb, cap * d)) || (s = lalloc(h, &L.xs, cap * kp)) ||
@@ -1619,12 +1716,12 @@ smpm_status lock_prepare(smpm_handle h, int R) {
   if (!mixed) {
     if ((s = lalloc(h, &L.x, cap * kp)) || (s = lalloc(h, &L.t, cap * kp)) || (s = lalloc(h, &L.y, cap * kp)) ||
         (s = lalloc(h, &L.vg, cap * kp)) || (s = lalloc(h, &L.V, G * (m + 1) * cap * ES)) ||
-        (s = lalloc(h, &L.W, G * 2 * cap * (ES + 1))))
+        (s = lalloc(h, &L.W, G * cap * ES)))
       return s;
   } else {
     if ((s = lalloc(h, &L.x32, cap * kp)) || (s = lalloc(h, &L.t32, cap * kp)) || (s = lalloc(h, &L.y32, cap * kp)) ||
         (s = lalloc(h, &L.vg32, cap * kp)) || (s = lalloc(h, &L.rg32, cap * kp)) ||
-        (s = lalloc(h, &L.V32, G * (m + 1) * cap * ES)) || (s = lalloc(h, &L.W32, G * 2 * cap * (ES + 1))) ||
+        (s = lalloc(h, &L.V32, G * (m + 1) * cap * ES)) || (s = lalloc(h, &L.W32, G * cap * ES)) ||
         (s = lalloc(h, &L.cr, cap * d)) || (s = lalloc(h, &L.dR, (size_t)kMaxRefine * cap)))
       return s;
     L.has32 = true;
@@ -1643,15 +1740,11 @@ smpm_status lock_prepare(smpm_handle h, int R) {
 // does not fit).
 template <typename S>
 size_t lock_shape(smpm_handle h, LockArgs<S>& A, int R, int nown_b, size_t budget) {
-  const auto& D = sizeof(S) == 8 ? h->dig : h->dig32;
-  A.Gd = D.G; A.Xd = D.X; A.Td = D.T;
-  A.Ge = D.Ge; A.Xe = D.Xe; A.Te = D.Te;
-  A.bcls = h->dbcls;
-  A.tcls = h->dtcls;
   A.R = R;
   const size_t fixed = lock_fixed_bytes(h->opts.restart, R);
   if (fixed >= budget) return 0;
   A.wb_bytes = lock_groups<S>(h->g.M, h->g.n, (long long)nown_b * ((R + 7) / 8), budget - fixed, &A.W_item, &A.ngrp);
+  A.w_smem = (size_t)R * basis_entries(h->g.M, nown_b) * sizeof(S) <= A.wb_bytes;
   return A.wb_bytes ? fixed + A.wb_bytes : 0;
 }
 
@@ -1673,7 +1766,9 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   LockArgs<double> A64{};
   LockArgs<float> A32{};
-  const size_t smem = mixed ? lock_shape(h, A32, R, h->gm.nown_b, optin) : lock_shape(h, A64, R, h->gm.nown_b, optin);
+  const size_t budget = (size_t)optin - 2048;  // the kernel stages its arguments in static shared memory
+  const size_t smem =
+      mixed ? lock_shape(h, A32, R, h->gm.nown_b, budget) : lock_shape(h, A64, R, h->gm.nown_b, budget);
   if (!smem) return fail(SMPM_EINVAL, "lockstep layout does not fit in shared memory");
   CU(set_smem_limit(mixed ? fn_lock32() : fn_lock64(), optin));
   CU(set_smem_limit(fn_pre_cols(), optin));
@@ -1722,9 +1817,9 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       P.cr = L.cr + (size_t)k * g.d;
       P.rg32 = L.rg32 + (size_t)k * g.kp;
     }
-    P.ga.bar = bar + 0;
+    P.ga.bar = bar;
     L.hP[k] = P;
-    P.ga.bar = bar + 1;
+    P.ga.bar = bar;
     P.assembled = mixed ? 1 : 0;
     L.hP[R + k] = P;
   }
@@ -1741,7 +1836,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
         a.err = err;
         a.skip = nullptr;
         RefineArgs RA = refine_args(h, a, tol);
-        RA.ga.bar = bar + 3 + 2 * ref;
+        RA.ga.bar = bar;
         RA.xS = L.xs + (size_t)k * g.kp;
         RA.bS = L.bS + (size_t)k * g.kp;
         RA.cr = L.cr + (size_t)k * g.d;
@@ -1767,7 +1862,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   CU(cudaEventRecord(h->ev0, st));
   auto lock_fields = [&](auto& A) {
     A.a.err = err;
-    A.a.mats_smem = 0; A.a.basis_smem = 0; A.a.stream_mats = 0; A.a.warp_elems = 1;
+    A.a.basis_smem = 0; A.a.ES = basis_entries(g.M, h->gm.nown_b);
     A.a.trace = nullptr; A.a.trace_cap = 0; A.a.skip = nullptr; A.a.its_out = nullptr; A.a.wscr = nullptr;
     A.a.c = L.c; A.a.chat = L.chat; A.a.acc = L.acc; A.a.gsep = L.gsep;
     choose_coarse(A.a, h->st_products, R);
@@ -1779,7 +1874,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     A.a = gmres_args(h, tol);
     lock_fields(A);
     A.a.rhs = L.rg; A.a.x = L.x; A.a.t = L.t; A.a.y = L.y; A.a.vglob = L.vg;
-    A.a.bar = bar + 2;
+    A.a.bar = bar;
     A.V = L.V; A.W = L.W;
     A.done = nullptr; A.done_stride = 0;
     if (h->wtrace) {
@@ -1797,7 +1892,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       A.a = gmres_args32(h, kInnerTol);
       lock_fields(A);
       A.a.rhs = L.rg32; A.a.x = L.x32; A.a.t = L.t32; A.a.y = L.y32; A.a.vglob = L.vg32;
-      A.a.bar = bar + 2 + 2 * ref;
+      A.a.bar = bar;
       A.V = L.V32; A.W = L.W32;
       A.done = reinterpret_cast<const int*>(colblk(0) + 64);
       A.done_stride = (int)(kLockColBytes / sizeof(int));
@@ -1942,39 +2037,187 @@ smpm_status balloc(smpm_batch b, P** p, size_t count) {
   return SMPM_OK;
 }
 
-// Lay the batch out for teams of T CTAs: longest-processing-time assignment
-// of whole problems to teams, per-problem scratch for that team size, the
-// task table (one task per right-hand side) and the launch's shared memory.
-smpm_status batch_layout(smpm_batch b, int T) {
+// Teams of a batch: CTAs of each, and the problems it works through.
+struct TeamPlan {
+  std::vector<int> size;
+  std::vector<std::vector<int>> problems;
+};
+
+bool batch_mixed(smpm_batch b, int p) {
+  return (b->precision < 0 ? b->hs[p]->opts.precision : b->precision) == 1;
+}
+
+// Estimated time (us) of problem p's right-hand sides on a team of T CTAs:
+// Arnoldi steps, each a fixed cost (barriers, phase starts) and the work of the
+// CTA with the most elements: per element, per 16 x 16 tile of its matrices, per
+// slot, and the CTA's share of the coarse products.  Constants: least squares
+// over the task times of 560 runs (80 problems of 28 to 1024 elements, n 8 to
+// 24, up to 16 columns, on teams of 4 to 152 CTAs), which they give back within
+// 10 % (one standard deviation; 30 % at worst).  The number of steps grows with
+// n and the elements' aspect ratio (within 7 % on the same problems).
+double batch_cost(smpm_batch b, int p, int T) {
+  smpm_handle h = b->hs[p];
+  const Geometry& g = h->g;
+  const bool mixed = batch_mixed(b, p);
+  const double hr = (g.Lx / g.mx) / (g.Ly / g.my);
+  const double steps = (mixed ? 37 : 29) * std::pow(g.n / 15.0, 0.55) * std::pow(std::max(hr, 1 / hr), 0.35);
+  const double kt = digit_tiles(g.M), d = (double)g.d;
+  const double prods = (h->st.p > 0 ? std::min(d * d, h->st_products) : d * d) / T;
+  const double ne = 2 * std::ceil(((g.nel + 1) / 2) / (double)T), tiles = ne * kt * kt, slots = ne * g.M;
+  double total = 0;
+  for (int k = 0; k < b->nrhs[p]; k += kLockMaxCols) {
+    const int R = std::min(kLockMaxCols, b->nrhs[p] - k);
+    const double fp = mixed ? 1 : 2;  // lockstep columns in FP64: twice the work
+    if (R > 1) total += steps * (49 + 3.9 * R + fp * (0.27 * tiles + R * (0.36 * ne + 0.003 * tiles + 0.028 * slots + 0.00034 * prods)));
+    else if (mixed) total += steps * (24 + 0.41 * ne + 0.081 * tiles + 0.047 * slots + 0.0035 * prods);
+    else total += steps * (24 + 1.95 * ne + 0.38 * tiles + 0.022 * slots + 0.0004 * prods);
+  }
+  return total;
+}
+
+// Uniform teams of T CTAs, whole problems to teams, longest first onto the
+// least-loaded one.
+TeamPlan uniform_plan(smpm_batch b, int T, int sms) {
+  const int np = (int)b->hs.size(), nt = sms / T;
+  std::vector<double> cost(np), load(nt, 0.0);
+  std::vector<int> order(np);
+  for (int p = 0; p < np; ++p) {
+    cost[p] = batch_cost(b, p, T);
+    order[p] = p;
+  }
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+  TeamPlan plan;
+  plan.size.assign(nt, T);
+  plan.problems.resize(nt);
+  for (int p : order) {
+    const int t = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+    load[t] += cost[p];
+    plan.problems[t].push_back(p);
+  }
+  return plan;
+}
+
+// The estimated time of the longest team of a plan.
+double plan_span(smpm_batch b, const TeamPlan& plan) {
+  double span = 0;
+  for (size_t t = 0; t < plan.size.size(); ++t) {
+    double load = 0;
+    for (int p : plan.problems[t]) load += batch_cost(b, p, plan.size[t]);
+    span = std::max(span, load);
+  }
+  return span;
+}
+
+// Teams of different sizes: the smallest deadline for which every problem gets
+// a team large enough to meet it and the teams fit the SMs (problems in order
+// of the team size they need; each goes to the fullest team that can still
+// finish it in time, else opens a team).  A batch whose largest problem takes
+// longer on a small team than all the others together is bound by that
+// problem; on large teams the many small ones lose their time to barriers.
+TeamPlan mixed_plan(smpm_batch b, int sms) {
+  const int np = (int)b->hs.size();
+  std::vector<int> sizes;
+  for (int c : {2, 4, 6, 8, 10, 12, 16, 19, 22, 25, 30, 38, 50, 76, 100, 152})
+    if (c < sms) sizes.push_back(c);
+  sizes.push_back(sms);
+  const int ns = (int)sizes.size();
+  std::vector<double> cost((size_t)np * ns);
+  double lo = 0, hi = 0;
+  for (int p = 0; p < np; ++p) {
+    double best = 1e300;
+    for (int k = 0; k < ns; ++k) {
+      const double c = batch_cost(b, p, sizes[k]);
+      cost[(size_t)p * ns + k] = c;
+      best = std::min(best, c);
+    }
+    lo = std::max(lo, best);
+    hi += cost[(size_t)p * ns + ns - 1];
+  }
+  auto build = [&](double D, TeamPlan* plan) {
+    std::vector<int> need(np), order(np);
+    for (int p = 0; p < np; ++p) {
+      order[p] = p;
+      need[p] = -1;
+      for (int k = 0; k < ns && need[p] < 0; ++k)
+        if (cost[(size_t)p * ns + k] <= D) need[p] = k;
+      if (need[p] < 0) return false;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+      return need[x] != need[y] ? need[x] > need[y]
+                                : cost[(size_t)x * ns + need[x]] > cost[(size_t)y * ns + need[y]];
+    });
+    TeamPlan t;
+    std::vector<int> kind;
+    std::vector<double> load;
+    int used = 0;
+    for (int p : order) {
+      int best = -1;
+      for (int q = 0; q < (int)kind.size(); ++q)
+        if (load[q] + cost[(size_t)p * ns + kind[q]] <= D && (best < 0 || load[q] > load[best])) best = q;
+      if (best < 0) {
+        if (used + sizes[need[p]] > sms) return false;
+        used += sizes[need[p]];
+        best = (int)kind.size();
+        kind.push_back(need[p]);
+        load.push_back(0);
+        t.size.push_back(sizes[need[p]]);
+        t.problems.emplace_back();
+      }
+      load[best] += cost[(size_t)p * ns + kind[best]];
+      t.problems[best].push_back(p);
+    }
+    *plan = t;
+    return true;
+  };
+  TeamPlan plan;
+  hi = std::max(hi, lo) * 1.01;
+  if (!build(hi, &plan)) return uniform_plan(b, sms, sms);
+  for (int it = 0; it < 30; ++it) {
+    const double mid = 0.5 * (lo + hi);
+    TeamPlan t;
+    if (build(mid, &t)) {
+      plan = t;
+      hi = mid;
+    } else {
+      lo = mid;
+    }
+  }
+  // equal teams where the estimate prefers them
+  double best = plan_span(b, plan);
+  for (int T : sizes) {
+    const TeamPlan u = uniform_plan(b, T, sms);
+    const double span = plan_span(b, u);
+    if (span < best) {
+      best = span;
+      plan = u;
+    }
+  }
+  return plan;
+}
+
+// Lay the batch out for a plan's teams: per-problem scratch for its team's
+// size, the task table (one task per right-hand side or lockstep group) and
+// the launch's shared memory.
+smpm_status batch_layout(smpm_batch b, const TeamPlan& plan) {
   batch_free_layout(b);
   int dev = 0, sms = 0, optin = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (T < 1 || T > sms) return fail(SMPM_EINVAL, "team size must be in [1, number of SMs]");
   const int np = (int)b->hs.size();
   b->grid = sms;
-  b->team_size = T;
-  b->nteams = sms / T;
-  // cost estimate of a problem: right-hand sides x operator entries
-  std::vector<double> cost(np);
-  std::vector<int> order(np);
-  for (int p = 0; p < np; ++p) {
-    const Geometry& g = b->hs[p]->g;
-    cost[p] = (double)b->nrhs[p] * ((double)g.nel * g.M * g.M + 2e4 * T);
-    order[p] = p;
+  b->team_size = *std::max_element(plan.size.begin(), plan.size.end());
+  b->nteams = (int)plan.size.size();
+  const std::vector<std::vector<int>>& plist = plan.problems;
+  std::vector<int> team_base(b->nteams + 1, 0), pteam(np, 0);
+  for (int t = 0; t < b->nteams; ++t) {
+    team_base[t + 1] = team_base[t] + plan.size[t];
+    for (int p : plist[t]) pteam[p] = t;
   }
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
-  std::vector<double> load(b->nteams, 0.0);
-  std::vector<std::vector<int>> plist(b->nteams);
-  for (int p : order) {
-    int t = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-    load[t] += cost[p];
-    plist[t].push_back(p);
-  }
-  // per-problem layout for G = T (all-global operator and basis)
+  if (team_base[b->nteams] > sms) return fail(SMPM_EINVAL, "the teams do not fit the SMs");
+  // per-problem layout for its team's size T (all-global operator and basis)
   struct PL {
-    int nown_b, nown_w, ES;
+    int nown_b, nown_w, ES, W_pp, W_fd, W_ref;
     bool wg;
     Layout lay;  // layout of the GMRES body (FP64, or the FP32 inner solve)
     double* vown64;
@@ -1992,40 +2235,36 @@ smpm_status batch_layout(smpm_batch b, int T) {
     smpm_handle h = b->hs[p];
     const Geometry& g = h->g;
     const int nb = (int)h->f.black.size(), nw = (int)h->f.white.size(), m = h->opts.restart;
+    const int T = plan.size[pteam[p]];
     PL& L = pl[p];
     L.nown_b = (nb + T - 1) / T;
     L.nown_w = (nw + T - 1) / T;
-    L.ES = 2 * g.M * L.nown_b;
-    if (L.ES % 2 == 0) L.ES += 1;
-    const bool mixed = (b->precision < 0 ? h->opts.precision : b->precision) == 1;
+    L.ES = basis_entries(g.M, L.nown_b);
+    const bool mixed = batch_mixed(b, p);
     // the all-global needs of pre/post and refinement, then the richest
     // GMRES layout that fits beside the argument header (resident or
     // streamed operator matrices, resident basis)
-    const int budget = budget_all;
+    const size_t budget = budget_all;
+    const int items = std::max(L.nown_b, L.nown_w);
     auto need_fixed = [&](bool wg) {
-      size_t a = prepost_smem_bytes(m, g.M, g.n, L.ES, L.nown_b, L.nown_w, g.d, wg);
-      if (mixed) a = std::max(a, refine_smem_bytes(m, g.M, g.n, L.ES, L.nown_b, L.nown_w, g.d, wg));
+      size_t a = prepost_shape(g, m, L.ES, items, T, budget, wg, &L.W_pp, &L.W_fd);
+      if (mixed) a = std::max(a, refine_shape(g, m, L.ES, items, budget, wg, &L.W_ref));
       return a;
     };
     const int precond = h->opts.precond;
-    const bool warp = precond > 0 && L.nown_b >= kWarpElemsMin;
     auto lay_for = [&](bool wg) {
-      return mixed ? choose_layout<float>(g, m, L.ES, L.nown_b, L.nown_w, precond, false, false, budget, wg, warp)
-                   : choose_layout<double>(g, m, L.ES, L.nown_b, L.nown_w, precond, false, false, budget, wg, warp);
+      return mixed ? choose_layout<float>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2)
+                   : choose_layout<double>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2);
     };
     // w, w2 move to global scratch when either the pre/post bodies or the
     // GMRES body (with its per-warp scratch) would not fit beside them
-    L.wg = need_fixed(false) > (size_t)budget || lay_for(false).smem > (size_t)budget;
+    L.wg = need_fixed(false) > budget || lay_for(false).smem > budget;
     L.lay = lay_for(L.wg);
-    if (mixed && warp)  // the refinement body runs the warp phases too
-      L.lay.smem = std::max(L.lay.smem, refine_smem_bytes(m, g.M, g.n, L.ES, L.nown_b, L.nown_w, g.d, L.wg, true));
     // several right-hand sides of a block-Jacobi problem: lockstep groups of
     // up to kLockMaxCols columns when their body fits (bound: the widest tile)
     L.lock = 0;
     L.lsmem = 0;
     if (b->nrhs[p] >= 2 && precond > 0 && !(h->opts.flags & SMPM_FLAG_NO_LOCKSTEP)) {
-      const int Rg = std::min(b->nrhs[p], kLockMaxCols);
-      L.lsmem = 0;
       bool fits = true;
       for (int k0 = 0; k0 < b->nrhs[p]; k0 += kLockMaxCols) {
         const int Rg = std::min(kLockMaxCols, b->nrhs[p] - k0);
@@ -2038,7 +2277,10 @@ smpm_status batch_layout(smpm_batch b, int T) {
       }
       if (fits && need_fixed(L.wg) <= (size_t)budget) L.lock = 1;
     }
-    const size_t nd = kBatchHdr + std::max(need_fixed(L.wg), L.lock ? L.lsmem : L.lay.smem);
+    // the one-column body runs too: every right-hand side of a problem without
+    // groups, or one left over by the groups
+    const bool singles = !L.lock || b->nrhs[p] % kLockMaxCols == 1;
+    const size_t nd = kBatchHdr + std::max(need_fixed(L.wg), std::max(L.lock ? L.lsmem : 0, singles ? L.lay.smem : 0));
     if (nd > (size_t)optin - 1024)
       return fail(SMPM_EINVAL, "a problem of the batch is too large for teams of this size");
     smem = std::max(smem, nd);
@@ -2047,11 +2289,11 @@ smpm_status batch_layout(smpm_batch b, int T) {
     L.wscr64 = nullptr;
     L.wscr32 = nullptr;
     const size_t vn = (size_t)T * (m + 1) * L.ES;
-    if (!L.lock && !L.lay.basis_smem && !mixed && (st = balloc(b, &L.vown64, vn))) return st;
-    if (!L.lock && !L.lay.basis_smem && mixed && (st = balloc(b, &L.vown32, vn))) return st;
+    if (singles && !L.lay.basis_smem && !mixed && (st = balloc(b, &L.vown64, vn))) return st;
+    if (singles && !L.lay.basis_smem && mixed && (st = balloc(b, &L.vown32, vn))) return st;
     if (L.wg) {
-      if ((st = balloc(b, &L.wscr64, (size_t)T * 2 * (L.ES + 1)))) return st;
-      if (mixed && (st = balloc(b, &L.wscr32, (size_t)T * 2 * (L.ES + 1)))) return st;
+      if ((st = balloc(b, &L.wscr64, (size_t)T * L.ES))) return st;
+      if (mixed && (st = balloc(b, &L.wscr32, (size_t)T * L.ES))) return st;
     }
   }
   // task table: one task per right-hand side, or one per lockstep group of
@@ -2079,6 +2321,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
   }
   for (int t = 0; t < b->nteams; ++t) {
     begin[t] = (int)tasks.size();
+    const int T = plan.size[t];
     // ---- the team's lockstep workspace: the largest group it runs
     struct {
       size_t R = 0, r = 0, kp = 0, d = 0, gs = 0, acc = 0, Rh = 0, yv = 0, V64 = 0, W64 = 0, V32 = 0, W32 = 0;
@@ -2088,8 +2331,9 @@ smpm_status batch_layout(smpm_batch b, int T) {
       if (!pl[p].lock) continue;
       smpm_handle h = b->hs[p];
       const Geometry& g = h->g;
-      const size_t R = (size_t)std::min(b->nrhs[p], kLockMaxCols), m = h->opts.restart, ES = pl[p].ES;
-      const bool mixed = (b->precision < 0 ? h->opts.precision : b->precision) == 1;
+      const size_t R = (size_t)std::min(b->nrhs[p], kLockMaxCols), m = h->opts.restart,
+                   ES = basis_entries(g.M, pl[p].nown_b);
+      const bool mixed = batch_mixed(b, p);
       need.R = std::max(need.R, R);
       need.r = std::max(need.r, (size_t)g.r);
       need.kp = std::max(need.kp, (size_t)g.kp);
@@ -2101,11 +2345,11 @@ smpm_status batch_layout(smpm_batch b, int T) {
       if (mixed) {
         need.f32 = true;
         need.V32 = std::max(need.V32, (size_t)T * (m + 1) * R * ES);
-        need.W32 = std::max(need.W32, (size_t)T * 2 * R * (ES + 1));
+        need.W32 = std::max(need.W32, (size_t)T * R * ES);
       } else {
         need.f64 = true;
         need.V64 = std::max(need.V64, (size_t)T * (m + 1) * R * ES);
-        need.W64 = std::max(need.W64, (size_t)T * 2 * R * (ES + 1));
+        need.W64 = std::max(need.W64, (size_t)T * R * ES);
       }
     }
     double *wb = nullptr, *wbS = nullptr, *wrg = nullptr, *wcb = nullptr, *wchatb = nullptr, *wxs = nullptr;
@@ -2143,17 +2387,15 @@ smpm_status batch_layout(smpm_batch b, int T) {
     for (int p : plist[t]) {
       smpm_handle h = b->hs[p];
       const PL& L = pl[p];
-      const bool mixed = (b->precision < 0 ? h->opts.precision : b->precision) == 1;
+      const bool mixed = batch_mixed(b, p);
       const double tol = h->opts.tol;
       auto team_fields = [&](auto& a) {
         a.G = T;
-        a.base = t * T;
+        a.base = team_base[t];
         a.nown_b = L.nown_b;
         a.nown_w = L.nown_w;
         a.ES = L.ES;
-        a.mats_smem = 0;
         a.basis_smem = 0;
-        a.stream_mats = 0;
         a.bar = b->dbars + t;
         a.err = b->derr;
         a.trace = nullptr;
@@ -2163,17 +2405,20 @@ smpm_status batch_layout(smpm_batch b, int T) {
         choose_coarse(a, h->st_products, 1);
       };
       auto layout_fields = [&](auto& a) {
-        a.mats_smem = L.lay.mats_smem;
         a.basis_smem = L.lay.basis_smem;
-        a.stream_mats = L.lay.stream_mats;
-        a.buf_elems = L.lay.buf_elems;
-        a.nbuf = L.lay.nbuf;
-        a.warp_elems = L.lay.warp_elems;
+        a.W_item = L.lay.W;
+        a.res_T = L.lay.res_T;
+        a.res_G = L.lay.res_G;
+        a.blk = 0;
+        a.tab = L.lay.tab;
+        a.res_H = L.lay.res_H;
       };
       auto single_task = [&](int k) {
         BatchTask bt{};
         bt.P = prepost_args(h, tol, nullptr, nullptr, nullptr, mixed);
         team_fields(bt.P.ga);
+        bt.P.ga.W_item = L.W_pp;
+        bt.P.W_fd = L.W_fd;
         bt.P.ga.vown = nullptr;
         bt.P.ga.wscr = L.wscr64;
         if (mixed) {
@@ -2182,7 +2427,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
           bt.a32.vown = L.vown32;
           bt.a32.wscr = L.wscr32;
           bt.R = refine_args(h, bt.a32, tol);  // all-global (refine_args clears the layout)
-          bt.R.ga.warp_elems = L.lay.warp_elems;
+          bt.R.ga.W_item = L.W_ref;
           layout_fields(bt.a32);
         } else {
           bt.a64 = gmres_args(h, tol);
@@ -2214,6 +2459,8 @@ smpm_status batch_layout(smpm_batch b, int T) {
         BatchTask bt{};
         bt.P = prepost_args(h, tol, nullptr, nullptr, nullptr, mixed);
         team_fields(bt.P.ga);
+        bt.P.ga.W_item = L.W_pp;
+        bt.P.W_fd = L.W_fd;
         bt.P.ga.vown = nullptr;
         bt.P.ga.wscr = L.wscr64;
         bt.precision = mixed ? 1 : 0;
@@ -2263,13 +2510,10 @@ smpm_status batch_layout(smpm_batch b, int T) {
         hRc.resize(hRc.size() + (size_t)kMaxRefine * R);
         auto lock_fields = [&](auto& A) {
           team_fields(A.a);
-          A.a.mats_smem = 0;
           A.a.basis_smem = 0;
-          A.a.stream_mats = 0;
-          A.a.warp_elems = 1;
+          A.a.ES = basis_entries(g.M, L.nown_b);
           A.a.wscr = nullptr;
           A.a.vown = nullptr;
-          A.a.fused = 0;
           A.a.c = wc;
           A.a.chat = wchat;
           A.a.acc = wacc;
@@ -2310,7 +2554,6 @@ smpm_status batch_layout(smpm_batch b, int T) {
             for (int c = 0; c < R; ++c) {
               GmresArgs<float> a = gmres_args32(h, kInnerTol);
               team_fields(a);
-              a.warp_elems = L.lay.warp_elems;
               a.wscr = L.wscr32;
               a.x = wx32 + (size_t)c * g.kp;
               a.t = wt32;
@@ -2318,7 +2561,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
               a.vglob = wvg32;
               a.rhs = wrg32 + (size_t)c * g.kp;
               RefineArgs RA = refine_args(h, a, tol);
-              RA.ga.warp_elems = L.lay.warp_elems;
+              RA.ga.W_item = L.W_ref;
               RA.xS = wxs + (size_t)c * g.kp;
               RA.bS = wbS + (size_t)c * g.kp;
               RA.cr = wcr + (size_t)c * g.d;
@@ -2344,7 +2587,7 @@ smpm_status batch_layout(smpm_batch b, int T) {
   }
   begin[b->nteams] = (int)tasks.size();
   std::vector<int> team_of(sms, -1);
-  for (int c = 0; c < b->nteams * T; ++c) team_of[c] = c / T;
+  for (int t = 0; t < b->nteams; ++t) std::fill(team_of.begin() + team_base[t], team_of.begin() + team_base[t + 1], t);
   if ((st = balloc(b, &b->dtasks, tasks.size())) || (st = balloc(b, &b->dbegin, begin.size())) ||
       (st = balloc(b, &b->dteam, team_of.size())))
     return st;
@@ -2357,6 +2600,15 @@ smpm_status batch_layout(smpm_batch b, int T) {
   CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn_batch(), kGmresThreads, smem));
   if (per < 1) return fail(SMPM_ECUDA, "the batch kernel does not fit on an SM");
   return SMPM_OK;
+}
+
+// Uniform teams of T CTAs.
+smpm_status batch_uniform(smpm_batch b, int T) {
+  int dev = 0, sms = 0;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (T < 1 || T > sms) return fail(SMPM_EINVAL, "team size must be in [1, number of SMs]");
+  return batch_layout(b, uniform_plan(b, T, sms));
 }
 
 // y_p = S_p v_p for all problems: stages as in launch_schur_stream, sized
@@ -2667,29 +2919,138 @@ smpm_status upload_digits(smpm_handle h, const std::vector<double>& A, int b, ui
   return SMPM_OK;
 }
 
-// Packed digits of the block classes' G_b and X_F, for the lockstep solves.
-smpm_status upload_block_digits(smpm_handle h, cudaStream_t st) {
-  const Geometry& g = h->g;
-  const size_t MM = (size_t)g.M * g.M, XX = 4 * (size_t)g.n * g.n, nb = h->f.black.size();
-  std::vector<int> idx(nb), of(nb, -1);
-  std::vector<double> Gc, Xc;
+// The distinct blocks among equal-sized consecutive ones (rep[i]: the first
+// block equal to block i), in order of appearance; cls: their index per block.
+std::vector<double> distinct_blocks(const std::vector<double>& A, size_t len, const std::vector<int>& rep,
+                                    std::vector<int>* cls) {
+  std::vector<int> of(rep.size(), -1);
+  std::vector<double> out;
   int n = 0;
-  for (size_t ib = 0; ib < nb; ++ib) {
-    const int r = h->f.grep[ib];
+  cls->resize(rep.size());
+  for (size_t i = 0; i < rep.size(); ++i) {
+    const int r = rep[i];
     if (of[r] < 0) {
       of[r] = n++;
-      Gc.insert(Gc.end(), h->f.G.begin() + r * MM, h->f.G.begin() + (r + 1) * MM);
-      Xc.insert(Xc.end(), h->f.X.begin() + r * XX, h->f.X.begin() + (r + 1) * XX);
+      out.insert(out.end(), A.begin() + r * len, A.begin() + (r + 1) * len);
     }
-    idx[ib] = of[r];
+    (*cls)[i] = of[r];
   }
+  return out;
+}
+
+// Whole inverses of the distinct blocks, [G, -G X; -T G, I + T G X] (2M x 2M
+// row-major; T: the block's own T_e).  Empty when a class mixes T classes.
+std::vector<double> block_inverses(const Geometry& g, const Factors& f, const std::vector<double>& G,
+                                   const std::vector<double>& X, const std::vector<double>& T) {
+  const int M = g.M, n = g.n, M2 = 2 * M;
+  const size_t MM = (size_t)M * M, nn = (size_t)n * n;
+  std::vector<int> reps;
+  std::vector<char> seen(f.grep.size(), 0);
+  for (size_t i = 0; i < f.grep.size(); ++i) {  // in the order of distinct_blocks
+    const int r = f.grep[i];
+    if (f.tcls[f.black[i]] != f.tcls[f.black[r]]) return {};
+    if (!seen[r]) reps.push_back(r);
+    seen[r] = 1;
+  }
+  std::vector<double> out(reps.size() * 4 * MM);
+#pragma omp parallel for schedule(static)
+  for (long long c = 0; c < (long long)reps.size(); ++c) {
+    const double *Gb = G.data() + reps[c] * MM, *Xb = X.data() + reps[c] * 4 * nn;
+    const double* Te = T.data() + (size_t)f.black[reps[c]] * MM;
+    double* B = out.data() + c * 4 * MM;
+    for (int i = 0; i < M; ++i) {
+      for (int k = 0; k < M; ++k) B[(size_t)i * M2 + k] = Gb[(size_t)i * M + k];
+      for (int F = 0; F < 4; ++F)
+        for (int k = 0; k < n; ++k) {
+          double v = 0;
+          for (int l = 0; l < n; ++l) v += Gb[(size_t)i * M + F * n + l] * Xb[F * nn + (size_t)l * n + k];
+          B[(size_t)i * M2 + M + F * n + k] = -v;
+        }
+    }
+    for (int i = 0; i < M; ++i) {
+      double* b = B + (size_t)(M + i) * M2;
+      for (int l = 0; l < M; ++l)
+        for (int k = 0; k < M2; ++k) b[k] -= Te[(size_t)i * M + l] * B[(size_t)l * M2 + k];
+      b[M + i] += 1.0;
+    }
+  }
+  return out;
+}
+
+// Packed digits of the block classes' G_b and X_F (forward FP64 and FP32, and
+// the adjoint's, with its T_e^T), the class indices and the element solves'
+// factors: everything the solve kernels multiply by.
+smpm_status upload_solve_digits(smpm_handle h, cudaStream_t st) {
+  const Geometry& g = h->g;
+  const Factors& f = h->f;
+  const size_t MM = (size_t)g.M * g.M, XX = 4 * (size_t)g.n * g.n;
   smpm_status s;
-  if ((s = upload(h, &h->dbcls, idx, st)) || (s = upload_digits<double>(h, Gc, g.M, &h->dig.G, &h->dig.Ge, st)) ||
-      (s = upload_digits<double>(h, Xc, g.n, &h->dig.X, &h->dig.Xe, st)))
-    return s;
-  if (h->opts.precision == 1 && ((s = upload_digits<float>(h, Gc, g.M, &h->dig32.G, &h->dig32.Ge, st)) ||
-                                 (s = upload_digits<float>(h, Xc, g.n, &h->dig32.X, &h->dig32.Xe, st))))
-    return s;
+  std::vector<int> idx;
+  if (!f.G.empty()) {
+    const std::vector<double> Gc = distinct_blocks(f.G, MM, f.grep, &idx), Xc = distinct_blocks(f.X, XX, f.grep, &idx);
+    if ((s = upload(h, &h->dbcls, idx, st)) || (s = upload_digits<double>(h, Gc, g.M, &h->dig.G, &h->dig.Ge, st)) ||
+        (s = upload_digits<double>(h, Xc, g.n, &h->dig.X, &h->dig.Xe, st)))
+      return s;
+    if (h->opts.precision == 1 && ((s = upload_digits<float>(h, Gc, g.M, &h->dig32.G, &h->dig32.Ge, st)) ||
+                                   (s = upload_digits<float>(h, Xc, g.n, &h->dig32.X, &h->dig32.Xe, st))))
+      return s;
+  }
+  // for a single solve's CTAs that own few blocks (block_pays); the limit
+  // keeps the tables of many distinct blocks small
+  const double blk_bytes = 1.75 * MM * ((f.black.size() + 151) / 152) * (h->opts.precision == 1 ? 4 : 8);
+  const bool blk = !f.G.empty() && blk_bytes <= 256e3;
+  if (blk) {
+    const std::vector<double> B = block_inverses(g, f, f.G, f.X, f.T);
+    if (!B.empty() && B.size() <= (size_t(16) << 20)) {
+      if ((s = upload_digits<double>(h, B, 2 * g.M, &h->dig.B, &h->dig.Be, st))) return s;
+      if (h->opts.precision == 1 && (s = upload_digits<float>(h, B, 2 * g.M, &h->dig32.B, &h->dig32.Be, st))) return s;
+      if (!f.Ga.empty() && f.has_adjoint &&
+          (s = upload_digits<double>(h, block_inverses(g, f, f.Ga, f.Xa, f.Ta), 2 * g.M, &h->diga.B, &h->diga.Be, st)))
+        return s;
+    }
+  }
+  if (f.has_adjoint) {
+    std::vector<int> rep(g.nel), first(g.nel, -1), cls;
+    for (long long e = 0; e < g.nel; ++e) {
+      if (first[f.tcls[e]] < 0) first[f.tcls[e]] = (int)e;
+      rep[e] = first[f.tcls[e]];
+    }
+    if ((s = upload_digits<double>(h, distinct_blocks(f.Ta, MM, rep, &cls), g.M, &h->diga.T, &h->diga.Te, st)))
+      return s;
+    if (!f.Ga.empty() &&
+        ((s = upload_digits<double>(h, distinct_blocks(f.Ga, MM, f.grep, &idx), g.M, &h->diga.G, &h->diga.Ge, st)) ||
+         (s = upload_digits<double>(h, distinct_blocks(f.Xa, XX, f.grep, &idx), g.n, &h->diga.X, &h->diga.Xe, st))))
+      return s;
+  }
+  // fast diagonalisation: per entry [V | V^-1 | lam]
+  const size_t nn = (size_t)g.n * g.n, ent = 2 * nn + g.n;
+  auto pack_fd = [&](const std::vector<double>& fx, const std::vector<double>& fy, FdMats* out) -> smpm_status {
+    auto mats = [&](const std::vector<double>& v) {
+      std::vector<double> o;
+      for (size_t i = 0; i + ent <= v.size(); i += ent) o.insert(o.end(), v.begin() + i, v.begin() + i + 2 * nn);
+      return o;
+    };
+    const size_t nx = fx.size() / ent, ny = fy.size() / ent;
+    std::vector<double> ri(nx * ny * nn);
+    for (size_t cy = 0; cy < ny; ++cy)
+      for (size_t cx = 0; cx < nx; ++cx)
+        for (int j = 0; j < g.n; ++j)
+          for (int i = 0; i < g.n; ++i)
+            ri[(cy * nx + cx) * nn + j * g.n + i] = 1.0 / (fx[cx * ent + 2 * nn + i] + fy[cy * ent + 2 * nn + j]);
+    uint4 *X = nullptr, *Y = nullptr;
+    short *xe = nullptr, *ye = nullptr;
+    double* r = nullptr;
+    smpm_status q;
+    if ((q = upload_digits<double>(h, mats(fx), g.n, &X, &xe, st)) ||
+        (q = upload_digits<double>(h, mats(fy), g.n, &Y, &ye, st)) || (q = upload(h, &r, ri, st)))
+      return q;
+    CU(cudaStreamSynchronize(st));  // ri goes out of scope
+    *out = {X, Y, xe, ye, r, (int)nx, 0};
+    return SMPM_OK;
+  };
+  if ((s = pack_fd(f.fdx, f.fdy, &h->fd))) return s;
+  if (f.has_adjoint && (s = pack_fd(f.fdxT, f.fdyT, &h->fda))) return s;
+  CU(cudaStreamSynchronize(st));
   return SMPM_OK;
 }
 
@@ -2734,14 +3095,7 @@ smpm_status upload_classes(smpm_handle h, cudaStream_t st) {
   if (h->opts.precision == 1 && (s = upload_digits<float>(h, Tcls, g.M, &h->dig32.T, &h->dig32.Te, st))) return s;
   h->ncls = (int)members.size();
   h->ntiles = (int)(tiles.size() / 3);
-  int dev = 0, optin = 0;
-  CU(cudaGetDevice(&dev));
-  CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  if (class_smem<double>(g.M) <= (size_t)optin) {
-    CU(set_smem_limit(k_schur_class<double>, optin));
-    CU(set_smem_limit(k_schur_class<float>, optin));
-    h->cls_ok = 1;
-  }
+  h->cls_ok = 1;
   return SMPM_OK;
 }
 
@@ -2781,6 +3135,15 @@ smpm_status factor_device_operator(smpm_handle h, cudaStream_t st) {
   return SMPM_OK;
 }
 
+// d x d row-major -> rows of d rounded up to a multiple of 4, zero padded
+std::vector<double> padded_rows(const std::vector<double>& H, long long d) {
+  const long long ld = (d + 3) & ~3LL;
+  if (ld == d) return H;
+  std::vector<double> out(d * ld, 0.0);
+  for (long long r = 0; r < d; ++r) std::copy(H.begin() + r * d, H.begin() + (r + 1) * d, out.begin() + r * ld);
+  return out;
+}
+
 // S Z at every slot from the row sums of the pushed products: slot (e, F, t)
 // takes row (opp F, t) of the neighbour's Rs, and its own weight in z_j as
 // the identity's share (zw: weights of the 4 faces of each element).
@@ -2804,13 +3167,6 @@ std::vector<double> pulled_row_sums(const Geometry& g, const std::vector<double>
 // Tables of the solve kernels (see GmresArgs).
 smpm_status upload_tables(smpm_handle h, cudaStream_t st) {
   const Geometry& g = h->g;
-  std::vector<int> tr(g.nel), first;
-  for (long long e = 0; e < g.nel; ++e) {
-    const size_t c = h->f.tcls[e];
-    if (first.size() <= c) first.resize(c + 1, -1);
-    if (first[c] < 0) first[c] = (int)e;
-    tr[e] = first[c];
-  }
   std::vector<int4> if4(g.nel), bt(h->f.black.size() * 2 * (size_t)g.M);
   for (long long e = 0; e < g.nel; ++e) {
     int j[4];
@@ -2830,8 +3186,7 @@ smpm_status upload_tables(smpm_handle h, cudaStream_t st) {
     }
   }
   smpm_status s;
-  if ((s = upload(h, &h->dtr, tr, st)) || (s = upload(h, &h->dgr, h->f.grep, st)) || (s = upload(h, &h->dif4, if4, st)) ||
-      (s = upload(h, &h->dbt, bt, st)) || (s = upload(h, &h->dRd, pulled_row_sums(g, h->f.Rs, h->f.zw), st)))
+  if ((s = upload(h, &h->dif4, if4, st)) || (s = upload(h, &h->dbt, bt, st)) || (s = upload(h, &h->dRd, pulled_row_sums(g, h->f.Rs, h->f.zw), st)))
     return s;
   if (h->f.has_adjoint && (s = upload(h, &h->dRda, pulled_row_sums(g, h->f.Rsa, h->f.zwa), st))) return s;
   return SMPM_OK;
@@ -2865,6 +3220,8 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
   }
   dg.zw = h->dzw;
   if ((s = upload_tables(h, st))) return s;
+  h->dHp = h->dH;
+  if (g.d % 4 != 0 && (s = upload(h, &h->dHp, padded_rows(h->f.H, g.d), st))) return s;
   const size_t kp = g.kp, r = g.r, d = g.d, m = opts.restart;
   const size_t nbs = blocks_for(g.kp, kSlotsPerBlock);
   if ((s = dalloc(h, &h->wb, r)) || (s = dalloc(h, &h->wbS, kp)) || (s = dalloc(h, &h->wV, (m + 1) * kp)) ||
@@ -2884,6 +3241,8 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     if ((s = dalloc(h, &h->wtrace, kTraceCap))) return s;
     CU(cudaMemsetAsync(h->wtrace, 0, kTraceCap * sizeof(long long), st));
   }
+  if ((s = upload_classes(h, st))) return s;
+  if ((s = upload_solve_digits(h, st))) return s;
   {
     // persistent GMRES kernel: one CTA per SM at most (all CTAs co-resident);
     // CTA c owns blocks c, c+G, ... and keeps their matrices and its basis
@@ -2897,25 +3256,33 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     gm.grid = std::max(1, std::min(sms, std::max(nb, nw)));
     gm.nown_b = (nb + gm.grid - 1) / gm.grid;
     gm.nown_w = (nw + gm.grid - 1) / gm.grid;
-    gm.ES = 2 * g.M * gm.nown_b;
-    if (gm.ES % 2 == 0) gm.ES += 1;
+    gm.ES = basis_entries(g.M, gm.nown_b);
     const int m = opts.restart;
     const bool no_smem = (opts.flags & SMPM_FLAG_NO_SMEM_RESIDENCY) != 0;
-    const bool force_stream = (opts.flags & SMPM_FLAG_STREAM_MATRICES) != 0;
-    // one warp per element when every CTA owns several blocks (or on request)
-    const bool warp = opts.precond > 0 && !force_stream &&
-                      (gm.nown_b >= kWarpElemsMin || (opts.flags & SMPM_FLAG_WARP_ELEMS) != 0);
+    const int items = std::max(gm.nown_b, gm.nown_w);
+    const size_t budget = (size_t)smem_optin - 2048;  // static shared memory: staged arguments
+    // w and w2 of the bodies move to global memory on grids so large that the
+    // coarse vector leaves no room for them
+    gm.smem_pp = prepost_shape(g, m, gm.ES, items, gm.grid, budget, false, &gm.W_pp, &gm.W_fd);
+    gm.wg = gm.smem_pp > budget || choose_layout<double>(g, m, gm.ES, items, true, budget, false, 0, gm.grid, false).smem > budget;
+    if (gm.wg) {
+      gm.smem_pp = prepost_shape(g, m, gm.ES, items, gm.grid, budget, true, &gm.W_pp, &gm.W_fd);
+      if ((s = dalloc(h, &h->wscr, (size_t)gm.grid * gm.ES))) return s;
+      if (opts.precision == 1 && (s = dalloc(h, &h->wscr32, (size_t)gm.grid * gm.ES))) return s;
+    }
     {
-      Layout L = choose_layout<double>(g, m, gm.ES, gm.nown_b, gm.nown_w, opts.precond, no_smem, force_stream,
-                                       smem_optin, false, warp);
+      Layout L = choose_layout<double>(g, m, gm.ES, items, no_smem, budget, gm.wg, block_pays<double>(h), gm.grid,
+                                       opts.precond == 2);
       gm.basis_smem = L.basis_smem;
-      gm.mats_smem = L.mats_smem;
-      gm.stream_mats = L.stream_mats;
-      gm.buf_elems = L.buf_elems;
-      gm.nbuf = L.nbuf;
-      gm.warp_elems = L.warp_elems;
+      gm.W = L.W;
+      gm.res_T = L.res_T;
+      gm.res_G = L.res_G;
+      gm.blk = L.blk;
+      gm.tab = L.tab;
+      gm.res_H = L.res_H;
       gm.smem = L.smem;
     }
+    if (gm.smem_pp > budget || gm.smem > budget) return fail(SMPM_EINVAL, "grid too large for the solve kernels");
     CU(set_smem_limit(fn_gmres64(), smem_optin));
     int per_sm = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_gmres64(), kGmresThreads, gm.smem));
@@ -2923,28 +3290,28 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     if (opts.precision == 1) {
       // FP32 inner GMRES: FP32 copies of the operator, its own layout, the
       // refinement kernel, FP32 work vectors and the FP64 residual
-      Layout L = choose_layout<float>(g, m, gm.ES, gm.nown_b, gm.nown_w, opts.precond, no_smem, force_stream,
-                                      smem_optin, false, warp);
       auto& g32 = h->gm32;
+      Layout L = choose_layout<float>(g, m, gm.ES, items, no_smem, budget, gm.wg, block_pays<float>(h), gm.grid,
+                                      opts.precond == 2);
       g32.basis_smem = L.basis_smem;
-      g32.mats_smem = L.mats_smem;
-      g32.stream_mats = L.stream_mats;
-      g32.buf_elems = L.buf_elems;
-      g32.nbuf = L.nbuf;
-      g32.warp_elems = L.warp_elems;
+      g32.W = L.W;
+      g32.res_T = L.res_T;
+      g32.res_G = L.res_G;
+      g32.blk = L.blk;
+      g32.tab = L.tab;
+      g32.res_H = L.res_H;
       g32.smem = L.smem;
       CU(set_smem_limit(fn_gmres32(), smem_optin));
       CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_gmres32(), kGmresThreads, g32.smem));
       if (per_sm < 1) return fail(SMPM_ECUDA, "the FP32 GMRES kernel does not fit on an SM");
-      g32.smem_ref = refine_smem_bytes(m, g.M, g.n, gm.ES, gm.nown_b, gm.nown_w, g.d, false, g32.warp_elems != 0);
+      g32.smem_ref = refine_shape(g, m, gm.ES, items, budget, gm.wg, &g32.W_ref);
       if (g32.smem_ref > (size_t)smem_optin) return fail(SMPM_EINVAL, "grid too large for the refinement kernel");
       CU(set_smem_limit(fn_refine(), smem_optin));
       CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn_refine(), kGmresThreads, g32.smem_ref));
       if (per_sm < 1) return fail(SMPM_ECUDA, "the refinement kernel does not fit on an SM");
       auto to32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
-      if ((s = upload(h, &h->dT32, to32(Tc), st)) || (s = upload(h, &h->dG32, to32(Gc), st)) ||
-          (s = upload(h, &h->dX32, to32(Xc), st)) ||
-          (s = upload(h, &h->dH32, to32(h->f.H), st)))
+      if ((s = upload(h, &h->dT32, to32(Tc), st)) ||
+          (s = upload(h, &h->dH32, to32(padded_rows(h->f.H, g.d)), st)))
         return s;
       if ((s = dalloc(h, &h->wx32, g.kp)) || (s = dalloc(h, &h->wt32, g.kp)) || (s = dalloc(h, &h->wy32, g.kp)) ||
           (s = dalloc(h, &h->wV32, g.kp)) || (s = dalloc(h, &h->wrg32, g.kp)) || (s = dalloc(h, &h->wr, g.kp)) ||
@@ -2952,8 +3319,6 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
         return s;
       if (!g32.basis_smem && (s = dalloc(h, &h->wvown32, (size_t)gm.grid * (m + 1) * gm.ES))) return s;
     }
-    gm.smem_pp = prepost_smem_bytes(m, g.M, g.n, gm.ES, gm.nown_b, gm.nown_w, g.d);
-    if (gm.smem_pp > (size_t)smem_optin) return fail(SMPM_EINVAL, "grid too large for the solve kernels");
     CU(set_smem_limit(fn_pre(), smem_optin));
     CU(set_smem_limit(fn_post(), smem_optin));
     for (const void* fn : {fn_pre(), fn_post()}) {
@@ -2994,13 +3359,8 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       }
       if ((s = upload(h, &h->dtab64, t64, st))) return s;
       if (h->dT32 && (s = upload(h, &h->dtab32, t32, st))) return s;
-      if ((s = upload_classes(h, st))) return s;
-      if (opts.precond > 0 && (s = upload_block_digits(h, st))) return s;
     }
     if (h->f.has_adjoint) {
-      // T~_e = T_e^T: its column-major device copy is T_e row-major
-      std::vector<double> Gca = transpose_blocks(h->f.Ga, g.M, h->f.black.size()),
-                          Xca = transpose_blocks(h->f.Xa, g.n, 4 * h->f.black.size());
       std::vector<double> ztusa(g.d, 0.0);
       for (long long e = 0; e < g.nel; ++e)
         for (int F = 0; F < 4; ++F) {
@@ -3008,10 +3368,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
           if (j < 0) continue;
           for (int t = 0; t < g.n; ++t) ztusa[j] += h->f.zwa[4 * e + F] * h->f.uSa[e * g.M + F * g.n + t];
         }
-      if ((s = upload(h, &h->dTa, h->f.T, st)) ||
-          (s = upload(h, &h->dGa, Gca, st)) || (s = upload(h, &h->dXa, Xca, st)) ||
-          (s = upload(h, &h->dHa, h->f.Ha, st)) || (s = upload(h, &h->dfdxT, h->f.fdxT, st)) ||
-          (s = upload(h, &h->dfdyT, h->f.fdyT, st)) || (s = upload(h, &h->duSa, h->f.uSa, st)) ||
+      if ((s = upload(h, &h->dHa, padded_rows(h->f.Ha, g.d), st)) || (s = upload(h, &h->duSa, h->f.uSa, st)) ||
           (s = upload(h, &h->dZtuSa, ztusa, st)))
         return s;
     }
@@ -3035,12 +3392,6 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     h->wrn = reinterpret_cast<double*>(h->wctl + 336);
     if ((s = dalloc(h, &h->wacc, (size_t)(2 * m + 1) * (m + 3)))) return s;
     if (!gm.basis_smem && (s = dalloc(h, &h->wvown, (size_t)gm.grid * (m + 1) * gm.ES))) return s;
-    if (opts.precond == 2 && g.d * (long long)gm.grid <= kFusedCoarseMaxAdds) {
-      std::vector<double> HT((size_t)g.d * g.d);
-      for (long long r = 0; r < g.d; ++r)
-        for (long long j = 0; j < g.d; ++j) HT[(size_t)j * g.d + r] = h->f.H[(size_t)r * g.d + j];
-      if ((s = upload(h, &h->dHT, HT, st)) || (s = dalloc(h, &h->wchatd, 2 * (size_t)g.d))) return s;
-    }
   }
   CU(cudaStreamSynchronize(st));
   h->factored = true;
@@ -3060,8 +3411,7 @@ smpm_status schur_solve(smpm_handle h, const double* f, const double* gn, double
   smpm_status worst = SMPM_OK;
   // several right-hand sides of an FP64 solve with block-Jacobi: lockstep
   // groups of up to kLockMaxCols columns
-  const bool lock = nrhs > 1 && h->opts.precond > 0 && !(h->opts.flags & SMPM_FLAG_NO_LOCKSTEP) &&
-                    h->gm.stream_mats == 0 && (h->opts.precision == 0 || h->gm32.stream_mats == 0);
+  const bool lock = nrhs > 1 && h->opts.precond > 0 && !(h->opts.flags & SMPM_FLAG_NO_LOCKSTEP);
   for (int k = 0; lock && k < nrhs; k += kLockMaxCols) {
     const int R = std::min(kLockMaxCols, nrhs - k);
     smpm_status s = R == 1 ? solve_one(h, f + (size_t)k * h->g.r, gn ? gn + (size_t)k * h->g.kp : nullptr,
@@ -3239,7 +3589,7 @@ template <typename S>
 smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st) {
   if (!h->cls_ok) return fail(SMPM_EINVAL, "the class-shared apply needs its packed matrices and tile in shared memory");
   const bool fp32 = sizeof(S) == 4;
-  k_schur_class<S><<<(unsigned)h->ntiles, kClassThreads, class_smem<S>(h->g.M), st>>>(
+  k_schur_class<S><<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), digit_bwords<S>(h->g.M) * sizeof(uint4), st>>>(
       h->dg, fp32 ? h->dig32.T : h->dig.T, fp32 ? h->dig32.Te : h->dig.Te, h->dtiles, h->dclsel, v, y);
   CHECK_LAUNCH();
   return SMPM_OK;
@@ -3475,19 +3825,14 @@ smpm_status smpm_batch_create(const smpm_handle* hs, int count, const int* nrhs,
       cudaMallocHost(&b->herr, 4 * sizeof(int)) || cudaStreamCreateWithFlags(&b->bs, cudaStreamNonBlocking) ||
       cudaEventCreate(&b->ein) || cudaEventCreate(&b->eout))
     return bad(fail(SMPM_ENOMEM, "batch allocation failed"));
-  int T = team_size;
-  if (T <= 0) {  // default: the smallest team size of the candidate list that fits
-    T = sms;
-    for (int c : {8, 16, 19, 38, 76})
-      if (c <= sms) {
-        smpm_status st = batch_layout(b, c);
-        if (st == SMPM_OK) {
-          T = c;
-          break;
-        }
-      }
+  smpm_status st = SMPM_EINVAL;
+  if (team_size > 0) {
+    st = batch_uniform(b, team_size);
+  } else {  // default: teams of different sizes, else the smallest uniform size that fits
+    st = batch_layout(b, mixed_plan(b, sms));
+    for (int c : {8, 16, 19, 38, 76, sms})
+      if (st != SMPM_OK && c <= sms) st = batch_uniform(b, c);
   }
-  smpm_status st = batch_layout(b, T);
   if (st != SMPM_OK) return bad(st);
   {
     // per-element tables of the batched apply
@@ -3632,7 +3977,7 @@ smpm_status smpm_batch_autotune(smpm_batch b, const double* f, const double* g, 
   double best_ms = 1e300;
   for (int i = 0; i < ncand; ++i) {
     if (ms_out) ms_out[i] = -1.0;
-    if (batch_layout(b, candidates[i]) != SMPM_OK) continue;
+    if (batch_uniform(b, candidates[i]) != SMPM_OK) continue;
     smpm_status st = smpm_batch_solve(b, f, g, u, nullptr, stream);  // warm-up (and graph capture)
     if (st != SMPM_OK && st != SMPM_ENOTCONV) return st;
     st = smpm_batch_solve(b, f, g, u, nullptr, stream);
@@ -3644,7 +3989,7 @@ smpm_status smpm_batch_autotune(smpm_batch b, const double* f, const double* g, 
     }
   }
   if (best < 0) return fail(SMPM_EINVAL, "no candidate team size fits the batch");
-  smpm_status st = batch_layout(b, best);
+  smpm_status st = batch_uniform(b, best);
   if (st != SMPM_OK) return st;
   if (chosen) *chosen = best;
   return SMPM_OK;
@@ -3742,6 +4087,25 @@ static __device__ __align__(256) double g_noalloc_scratch[2 * kNoAllocMaxInterfa
 // cudaDeviceReset, after which the module is loaded again).
 std::mutex g_noalloc_mu;
 double* g_noalloc_ptr[256] = {nullptr};
+
+// Grid barrier on one monotonic counter (zero on entry), bounded spin.
+__device__ bool grid_sync(unsigned* bar, int* err, unsigned& epoch, int G) {
+  ++epoch;
+  __syncthreads();
+  bool ok = true;
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(1u) : "memory");
+    long long spins = 0;
+    const long long limit = g_barrier_spin_limit;
+    while ((int)(ld_acquire(bar) - epoch * (unsigned)G) < 0)
+      if (++spins > limit || ((spins & 4095) == 0 && *((volatile int*)err))) {
+        atomicCAS(err, 0, 1);
+        ok = false;
+        break;
+      }
+  }
+  return __syncthreads_and(ok);
+}
 
 // One cooperative launch: c = Z^T v | c_hat = C^+ c | y = v - S Z c_hat.
 // On a barrier timeout (not expected: all CTAs are co-resident) y is NaN.
