@@ -237,8 +237,8 @@ smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, vo
 
 /* Kernels of y = S v (smpm_apply_schur, smpm_apply_schur32 and the S apply
  * inside the deflation entry points): AUTO takes CLASS where the elements
- * fall into few enough classes that its tiles of eight elements are at least 5/8
- * full on average, else by thresholds one warp per element for 4n <= 96 (1, 2 or
+ * fall into few enough classes that its tiles of eight elements are at least a
+ * fifth full on average, else by thresholds one warp per element for 4n <= 96 (1, 2 or
  * 4 warps by the element count) or the shared-memory stream; WARP: persistent CTAs, one warp per element,
  * T_e read column by column from global memory; WARP2 / WARP4: 2 or 4 warps
  * per element; STREAM: bulk copies of T_e into a shared-memory ring; CLASS:
