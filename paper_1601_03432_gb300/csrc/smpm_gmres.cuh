@@ -13,8 +13,7 @@
 // packed in digits (smpm_digits.cuh); the class a CTA uses most, its slice of
 // the Krylov basis, its entries' table and its rows of C^+ stay in shared
 // memory as far as they fit.  One step:
-//   A  owner: v_j = w2 - V h2 on its block slots (lazy, see E), then the
-//      block solve t = M^-1 v_j: a = G (p - X q), b = q - T_e a, in stages
+//   A  owner: block solves t = M^-1 v_j on its block slots: a = G (p - X q), b = q - T_e a, in stages
 //      (black_phase) or with the whole inverse (black_block)
 //   B  white elements: y = S t (y = v on white-owned slots), c = Z^T y
 //   C  c_hat = C^+ c (rows over all CTAs, or by element-row strips; Algorithm 3)
@@ -22,7 +21,8 @@
 //      atomics in L2
 //   E  owner: w2 = w - V h1; V^T w2 and ||w2||^2 likewise; every CTA forms
 //      ||v_{j+1}||^2 = ||w2||^2 - ||h2||^2 and the residual norm from its own
-//      copy of the Hessenberg column, so all CTAs take the same decision.
+//      copy of the Hessenberg column (warp 0), so all CTAs take the same
+//      decision, while the other warps form v_{j+1} = w2 - V h2
 // Phases are separated by a team barrier (5 per step for Algorithm 3, 7 with
 // strips).  The basis is kept unnormalised with the inverse norms replicated
 // in every CTA.
@@ -674,14 +674,15 @@ __device__ __forceinline__ void ld_vec(const float* p, float (&v)[4]) {
 // For rows r0 <= r < r1: get(r, &row, &x, &len) names a row (16-byte aligned,
 // zero-padded to whole 16-byte groups) and the staged vector (readable to the
 // padded length); put(r, sum) takes the dot product (len 0: no call).  P lanes
-// per row, P as large as the rows leave threads for, but 4 at least: each
+// per row, P as large as the rows (longest: their greatest length) leave threads
+// and entries for, but 4 at least: each
 // halving step of the final sums costs as much FP64 time as a product.
 template <typename T, bool SM = false, typename Get, typename Put>
-__device__ __forceinline__ void row_dots(int r0, int r1, Get&& get, Put&& put) {
+__device__ __forceinline__ void row_dots(int r0, int r1, int longest, Get&& get, Put&& put) {
   constexpr int V = 16 / (int)sizeof(T), U = 4;
   const int rows = r1 - r0;
   int P = 32;
-  while (P > 4 && P * rows > (int)blockDim.x) P >>= 1;
+  while (P > 4 && (P * rows > (int)blockDim.x || V * P >= 2 * longest)) P >>= 1;
   const int lane = threadIdx.x % P, grp = threadIdx.x / P, ngrp = blockDim.x / P;
 #pragma unroll 1
   for (int rb = 0; rb < rows; rb += ngrp) {  // uniform trip count per warp
@@ -734,7 +735,7 @@ __device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsig
       for (int j = threadIdx.x; j < b1 - b0 + V; j += blockDim.x) xs[j] = b0 + j < b1 ? (T)__ldcg(c + b0 + j) : T(0);
       __syncthreads();
       row_dots<T>(
-          r0, r1,
+          r0, r1, k.m,
           [&](int r, const T*& row, const T*& x, int& len) {
             const int i = r / RS, l = r - i * RS, mi = min(k.m, d - i * srow);
             const bool on = l < k.m ? l < mi : (l < k.m + k.mx ? i > 0 : i < k.p - 1);
@@ -764,7 +765,7 @@ __device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsig
       }
       __syncthreads();
       row_dots<T>(
-          r0, r1,
+          r0, r1, k.ns,
           [&](int r, const T*& row, const T*& x, int& len) {
             row = k.Hs + (size_t)r * k.lds;
             x = xs;
@@ -788,7 +789,7 @@ __device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsig
       const double al = __ldcg(alpha);
       __syncthreads();
       row_dots<T>(
-          r0, r1,
+          r0, r1, 2 * k.mx,
           [&](int r, const T*& row, const T*& x, int& len) {
             const int i = r / k.m;
             row = k.W + (size_t)r * k.ldw;
@@ -821,7 +822,7 @@ __device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, 
   auto put = [&](int r, T sum) { chat[r] = (double)sum; };
   if (s.H) {
     row_dots<T, true>(
-        r0, r1,
+        r0, r1, d,
         [&](int r, const T*& row, const T*& x, int& len) {
           row = s.H + (size_t)(r - r0) * ld;
           x = xs;
@@ -830,7 +831,7 @@ __device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, 
         put);
   } else {
     row_dots<T>(
-        r0, r1,
+        r0, r1, d,
         [&](int r, const T*& row, const T*& x, int& len) {
           row = a.H + (size_t)r * ld;
           x = xs;
@@ -1001,8 +1002,8 @@ __device__ SMPM_PHASE void deflate_pass(const GmresArgs<S>& a, const Smem<S>& s,
 // columns that CTA 0 stored in gs->R, by Givens rotations, in one warp: each
 // rotation meets every later column at once, one column per lane (the loads of
 // the next row run ahead of the rotation's chain).  y -> gs->y; returns the
-// residual norm.  xi, gg: m + 3 entries of shared memory.
-__device__ __noinline__ double hessenberg_lsq(GState* gs, double* xi, double* gg, int j, double beta) {
+// residual norm.  xi, gg, inv: m + 3 entries of shared memory.
+__device__ __noinline__ double hessenberg_lsq(GState* gs, double* xi, double* gg, double* inv, int j, double beta) {
   const int lane = threadIdx.x & 31;
   const size_t m1 = kMaxRestart + 1;
   double* R = gs->R;
@@ -1026,23 +1027,26 @@ __device__ __noinline__ double hessenberg_lsq(GState* gs, double* xi, double* gg
       R[l * m1 + i] = l == i ? hh * iden : fma(cc, xl, ss * x1);
       if (l > i) xi[l] = fma(-ss, xl, cc * x1);
     }
-    if (lane == 0) gg[i] = cc * gcur;
+    if (lane == 0) {
+      gg[i] = cc * gcur;
+      inv[i] = hh > 0 ? iden : __longlong_as_double(0x7ff0000000000000LL);
+    }
     gcur = -ss * gcur;
     nx = ahead;
     l0 = l1;
   }
   __syncwarp();
-  // y = R^-1 g column by column: y_k, then the entries above it lose R_ik y_k
-#pragma unroll 1
+  // y = R^-1 g column by column: y_k (1 / R_kk is the rotation's 1 / norm, in inv), then the entries above it lose R_ik y_k; two columns ahead in flight
+  auto column = [&](int k) { return k >= 0 && lane < k ? __ldcg(R + k * m1 + lane) : 0.0; };
+  double r0 = column(j - 1), r1 = column(j - 2);
   for (int k = j - 1; k >= 0; --k) {
-    const double* Rk = R + k * m1;
-    const double r0 = lane < k ? __ldcg(Rk + lane) : 0.0;
-    const double yk = gg[k] / __ldcg(Rk + k);
+    const double r2 = column(k - 2), yk = gg[k] * inv[k];
     __syncwarp();
-#pragma unroll 1
-    for (int i = lane; i < k; i += 32) gg[i] = fma(-(i == lane ? r0 : __ldcg(Rk + i)), yk, gg[i]);
+    for (int i = lane; i < k; i += 32) gg[i] = fma(-(i == lane ? r0 : __ldcg(R + k * m1 + i)), yk, gg[i]);
     if (lane == 0) gs->y[k] = yk;
     __syncwarp();
+    r0 = r1;
+    r1 = r2;
   }
   return fabs(gcur);
 }
@@ -1060,6 +1064,22 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
   int trace_n = 0;
   load_resident(a, s);
 
+  // v_{j+1} = w2 - V h2 by the threads `at` of n: on few entries by the warps
+  // that have nothing else to do while warp 0 forms the residual norm (never
+  // read when the step turns out to be the last), on many (more than about
+  // two per thread, where the missing warp would cost more) by all, afterwards
+  constexpr int kOverlapEntries = 512;
+  auto form_next = [&](int at, int n, int j) {
+    if (j + 1 >= m ) return;
+    S* vn = s.V + (size_t)(j + 1) * ES;
+#pragma unroll 1
+    for (int i = at; i < ES; i += n) {
+      const S rv = (S)basis_combo(a, s, (double)s.w[i], s.hs2, j + 1, i);
+      vn[i] = rv;
+      const int sl = entry_slot(a, s, i);
+      if (sl >= 0) a.vglob[sl] = rv;
+    }
+  };
   int total = 0, cycle = 0, jlast = 0;
   bool converged = false, breakdown = false, nan = false;
   double tolabs = 0, beta0 = 0, resid = 0;
@@ -1111,18 +1131,8 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       double* accE = a.acc + (size_t)(2 * j + 1) * m3;
       const double ivj = s.invb[j];
       GM_TRACE(1);
-      // ---- A: finalize V[j] on the owned entries (j > 0), then block solves
+      // ---- A: block solves with v_j
       S* vj = s.V + (size_t)j * ES;
-      if (j > 0) {
-#pragma unroll 1
-        for (int i = threadIdx.x; i < ES; i += blockDim.x) {
-          const S rv = (S)basis_combo(a, s, (double)s.w[i], s.hs2, j, i);
-          vj[i] = rv;
-          const int sl = entry_slot(a, s, i);
-          if (sl >= 0) a.vglob[sl] = rv;
-        }
-        __syncthreads();
-      }
       if (a.precond == 0) {
         if (!team_sync(a, epoch)) return false;  // neighbours read v_j
         if (!apply_op(a, s, a.vglob, ivj, false, trace_n, epoch)) return false;
@@ -1204,6 +1214,8 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
           s.misc[4] = bsq > 0 ? bsq * ib : 0.0;  // the new subdiagonal entry
           if (rank == 0) Rc[j + 1] = s.misc[4];
         }
+      } else if (ES <= kOverlapEntries) {
+        form_next(threadIdx.x - 32, blockDim.x - 32, j);
       }
       __syncthreads();
       GM_TRACE(11);
@@ -1213,13 +1225,17 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       if (!isfinite(zz) || !isfinite(s.misc[4])) { nan = true; ++j; break; }
       if (s.misc[4] == 0.0 || goal <= zz) { converged = true; ++j; break; }
       if (s.misc[3] != 0.0) { breakdown = true; ++j; break; }
+      if (ES > kOverlapEntries) {
+        form_next(threadIdx.x, blockDim.x, j);
+        __syncthreads();
+      }
     }
     jlast = j;
     if (nan) break;
     // ---- end of cycle: y by warp 0 of CTA 0, x += V diag(invb) y on owned entries
     if (rank == 0 && threadIdx.x < 32) {
       __syncwarp();
-      resid = hessenberg_lsq(a.gs, s.xi, s.gg, j, beta);
+      resid = hessenberg_lsq(a.gs, s.xi, s.gg, s.hs1, j, beta);
     }
     if (!team_sync(a, epoch)) return false;
     // the accumulators are consumed by all CTAs: zero them for the next cycle

@@ -47,6 +47,7 @@ struct FdMats {
   const uint4 *x, *y;
   const short *xe, *ye;
   const double* rinv;
+  const double *fx, *fy;  // V and V^-1 in FP64, two per class (fd_thread_pass)
   int nx, pad_;
 };
 
@@ -139,6 +140,29 @@ __device__ __noinline__ void fd_pass(const uint4* A, const short* er, uint4* Bw,
   }
 }
 
+// The same by plain FP64 products, a thread per entry of out, for a CTA that has
+// one element of n <= kFdThreadN nodes a side: its 256 threads form an 8 x 8
+// product in about 900 SM cycles, the packing and the tile of eight columns
+// take 3,500 in the one warp they occupy.  From n = 16 on (2,048 cycles of
+// FP64 products alone, two warps of tiles) the digits are not slower.
+constexpr int kFdThreadN = 12;
+__device__ __noinline__ void fd_thread_pass(const double* __restrict__ A, int n, int tid, int nthr, const double* x, int ldk,
+                                            int ldc, double* out, int ldr, int ldo, const double* __restrict__ w) {
+  for (int q = tid; q < n * n; q += nthr) {
+    const int c = q / n, r = q - c * n;
+    double s0 = 0, s1 = 0;
+    int k = 0;
+#pragma unroll 4
+    for (; k + 1 < n; k += 2) {
+      s0 += __ldg(A + r * n + k) * x[k * ldk + c * ldc];
+      s1 += __ldg(A + r * n + k + 1) * x[(k + 1) * ldk + c * ldc];
+    }
+    if (k < n) s0 += __ldg(A + r * n + k) * x[k * ldk + c * ldc];
+    const double z = s0 + s1;
+    out[r * ldr + c * ldo] = w ? z * __ldg(w + q) : z;
+  }
+}
+
 // U = A_e^-1 B for element e, entered and left with the group in step
 __device__ __noinline__ void elem_fd(const FdMats& fd, const DevGeo& g, int e, const FdItem& f, int lane, int part,
                                         int W, int grp) {
@@ -149,6 +173,19 @@ __device__ __noinline__ void elem_fd(const FdMats& fd, const DevGeo& g, int e, c
   const uint4 *Vx = fd.x + 2 * cx * nw, *Vxi = Vx + nw, *Vy = fd.y + 2 * cy * nw, *Vyi = Vy + nw;
   const short *ex = fd.xe + 2 * cx * n, *exi = ex + n, *ey = fd.ye + 2 * cy * n, *eyi = ey + n;
   const double* ri = fd.rinv + ((size_t)cy * fd.nx + cx) * n * n;
+  if (W == kGmresThreads / 32 && n <= kFdThreadN) {
+    const size_t nn = (size_t)n * n;
+    const double *X = fd.fx + 2 * cx * nn, *Y = fd.fy + 2 * cy * nn;
+    fd_thread_pass(Y + nn, n, 32 * part + lane, 32 * W, f.B, ld, 1, f.t1, ld, 1, nullptr);
+    item_sync(grp, W);
+    fd_thread_pass(X + nn, n, 32 * part + lane, 32 * W, f.t1, 1, ld, f.U, 1, ld, ri);
+    item_sync(grp, W);
+    fd_thread_pass(X, n, 32 * part + lane, 32 * W, f.U, 1, ld, f.t1, 1, ld, nullptr);
+    item_sync(grp, W);
+    fd_thread_pass(Y, n, 32 * part + lane, 32 * W, f.t1, ld, 1, f.U, ld, 1, nullptr);
+    item_sync(grp, W);
+    return;
+  }
   uint4* Bw = f.Bf + (size_t)part * digit_bwords<double>(n);
   fd_pass(Vyi, eyi, Bw, n, lane, part, W, f.B, ld, 1, f.t1, ld, 1, nullptr);   // t1 = Vy^-1 B
   item_sync(grp, W);

@@ -1323,6 +1323,7 @@ Layout choose_layout(const Geometry& g, int m, int ES, int items, bool no_smem, 
 size_t prepost_shape(const Geometry& g, int m, int ES, int items, int G, size_t budget, bool w_global, int* W, int* W_fd) {
   *W = item_warps(items);
   *W_fd = std::min(item_warps((g.nel + G - 1) / G), std::max(1, (g.n + 7) / 8 > 2 ? 4 : (g.n + 7) / 8));
+  if (g.nel <= G && g.n <= kFdThreadN) *W_fd = kGmresThreads / 32;
   auto need = [&] { return prepost_smem_bytes(m, g.M, g.n, ES, *W, *W_fd, g.d, w_global); };
   while (need() > budget && (*W < kGmresThreads / 32 || *W_fd < kGmresThreads / 32)) {
     if (*W_fd < kGmresThreads / 32) *W_fd *= 2;
@@ -1347,13 +1348,18 @@ bool strips_pay(long long d, double products, int G, int R, bool fp32) {
 
 // Whether black blocks are solved with their whole inverse (black_block): a
 // CTA's blocks then read 7/4 M^2 more entries each, at about 64 bytes per SM
-// cycle, and save three of four dependent stages (about 8,000 cycles at
-// M = 64, 5,000 at M = 20).
+// cycle, and save three of four dependent stages (about 8,000 cycles at M = 64,
+// 5,000 at M = 20).  Up to 4,000 cycles of reading.  In lockstep, where eight
+// columns share a matrix and the products count, it gave nothing (M = 96, four
+// blocks: 113,000 cycles instead of 121,000, and less even CTAs).
+template <typename S>
+bool block_fits(smpm_handle h, int nown_b) {
+  return 1.75 * h->g.M * h->g.M * sizeof(S) * nown_b <= 256e3;
+}
 template <typename S>
 int block_pays(smpm_handle h) {
-  const double bytes = 1.75 * h->g.M * h->g.M * sizeof(S) * h->gm.nown_b;
   const bool have = sizeof(S) == 4 ? h->dig32.B != nullptr : h->dig.B != nullptr;
-  return have && h->opts.precond != 0 && bytes <= 256e3;
+  return have && h->opts.precond != 0 && block_fits<S>(h, h->gm.nown_b);
 }
 
 // Form of the coarse solve for a solve of R columns by a.G CTAs.
@@ -2939,7 +2945,8 @@ std::vector<double> distinct_blocks(const std::vector<double>& A, size_t len, co
 }
 
 // Whole inverses of the distinct blocks, [G, -G X; -T G, I + T G X] (2M x 2M
-// row-major; T: the block's own T_e).  Empty when a class mixes T classes.
+// row-major; T: the block's own T_e).  Empty when a class mixes T classes
+// or the blocks are too many.
 std::vector<double> block_inverses(const Geometry& g, const Factors& f, const std::vector<double>& G,
                                    const std::vector<double>& X, const std::vector<double>& T) {
   const int M = g.M, n = g.n, M2 = 2 * M;
@@ -2952,6 +2959,7 @@ std::vector<double> block_inverses(const Geometry& g, const Factors& f, const st
     if (!seen[r]) reps.push_back(r);
     seen[r] = 1;
   }
+  if (reps.size() * 4 * MM > (size_t(4) << 20)) return {};  // many distinct blocks: 32 MB at most
   std::vector<double> out(reps.size() * 4 * MM);
 #pragma omp parallel for schedule(static)
   for (long long c = 0; c < (long long)reps.size(); ++c) {
@@ -2995,13 +3003,15 @@ smpm_status upload_solve_digits(smpm_handle h, cudaStream_t st) {
                                    (s = upload_digits<float>(h, Xc, g.n, &h->dig32.X, &h->dig32.Xe, st))))
       return s;
   }
-  // for a single solve's CTAs that own few blocks (block_pays); the limit
-  // keeps the tables of many distinct blocks small
-  const double blk_bytes = 1.75 * MM * ((f.black.size() + 151) / 152) * (h->opts.precision == 1 ? 4 : 8);
-  const bool blk = !f.G.empty() && blk_bytes <= 256e3;
-  if (blk) {
+  // whole block inverses, where a solve could take them
+  int dev = 0, sms = 0;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int nown_b = ((int)f.black.size() + sms - 1) / sms;
+  const bool mixed = h->opts.precision == 1;
+  if (!f.G.empty() && (mixed ? block_fits<float>(h, nown_b) : block_fits<double>(h, nown_b))) {
     const std::vector<double> B = block_inverses(g, f, f.G, f.X, f.T);
-    if (!B.empty() && B.size() <= (size_t(16) << 20)) {
+    if (!B.empty()) {
       if ((s = upload_digits<double>(h, B, 2 * g.M, &h->dig.B, &h->dig.Be, st))) return s;
       if (h->opts.precision == 1 && (s = upload_digits<float>(h, B, 2 * g.M, &h->dig32.B, &h->dig32.Be, st))) return s;
       if (!f.Ga.empty() && f.has_adjoint &&
@@ -3041,11 +3051,14 @@ smpm_status upload_solve_digits(smpm_handle h, cudaStream_t st) {
     short *xe = nullptr, *ye = nullptr;
     double* r = nullptr;
     smpm_status q;
-    if ((q = upload_digits<double>(h, mats(fx), g.n, &X, &xe, st)) ||
-        (q = upload_digits<double>(h, mats(fy), g.n, &Y, &ye, st)) || (q = upload(h, &r, ri, st)))
+    double *vx = nullptr, *vy = nullptr;
+    const std::vector<double> mx = mats(fx), my = mats(fy);
+    if ((q = upload(h, &vx, mx, st)) || (q = upload(h, &vy, my, st)) ||
+        (q = upload_digits<double>(h, mx, g.n, &X, &xe, st)) ||
+        (q = upload_digits<double>(h, my, g.n, &Y, &ye, st)) || (q = upload(h, &r, ri, st)))
       return q;
     CU(cudaStreamSynchronize(st));  // ri goes out of scope
-    *out = {X, Y, xe, ye, r, (int)nx, 0};
+    *out = {X, Y, xe, ye, r, vx, vy, (int)nx, 0};
     return SMPM_OK;
   };
   if ((s = pack_fd(f.fdx, f.fdy, &h->fd))) return s;
