@@ -831,10 +831,20 @@ cudaError_t launch_schur_warp(const ElemMeta<S>* tab, long long nelem, const S* 
 // CTAs per SM: a row tile is a chain of loads and dependent products.
 constexpr int kClassTile = 8;
 
+// one entry of T_e v on an element whose v has an Inf or NaN, which have no
+// digits: the plain sum, as the per-element kernels form it (row: T_e's row,
+// column-major)
+template <typename S>
+__device__ __noinline__ S plain_row(const S* __restrict__ row, const S* v, int M) {
+  S z = S(0);
+  for (int k = 0; k < M; ++k) z += __ldg(row + (size_t)k * M) * __ldg(v + k);
+  return z;
+}
+
 template <typename S>
 __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
                                                      const short* __restrict__ Texp, const int* __restrict__ tiles,
-                                                     const int* __restrict__ elems, const S* v, S* y) {
+                                                     const int* __restrict__ elems, const S* __restrict__ T, const S* v, S* y) {
   extern __shared__ __align__(16) unsigned char raw[];
   const int M = g.M, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cls = tiles[3 * blockIdx.x], start = tiles[3 * blockIdx.x + 1], cnt = tiles[3 * blockIdx.x + 2];
@@ -879,8 +889,14 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
   const Tile8<S> t = tile8_products<S>(Tdig + (size_t)cls * digit_words<S>(M, M), Texp + (size_t)cls * M, Bf, M, kt_n,
                                        warp, lane, E);
 #pragma unroll
-  for (int u = 0; u < 4; ++u)
-    if (sl[u] >= 0) y[sl[u]] = push[u] ? vf[u] + t.z[u] : vf[u];
+  for (int u = 0; u < 4; ++u) {
+    if (sl[u] < 0) continue;
+    const int r = warp * 16 + gc + 8 * (u >> 1), c = 2 * q + (u & 1);
+    S z = t.z[u];
+    if (Emax[c] == (sizeof(S) == 4 ? 0xff : 0x7ff) && push[u])
+      z = plain_row(T + (size_t)__ldg(el + c) * M * M + r, v + (size_t)__ldg(el + c) * M, M);
+    y[sl[u]] = push[u] ? vf[u] + z : vf[u];
+  }
 }
 
 template <typename S>
@@ -3603,7 +3619,8 @@ smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st)
   if (!h->cls_ok) return fail(SMPM_EINVAL, "the class-shared apply needs its packed matrices and tile in shared memory");
   const bool fp32 = sizeof(S) == 4;
   k_schur_class<S><<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), digit_bwords<S>(h->g.M) * sizeof(uint4), st>>>(
-      h->dg, fp32 ? h->dig32.T : h->dig.T, fp32 ? h->dig32.Te : h->dig.Te, h->dtiles, h->dclsel, v, y);
+      h->dg, fp32 ? h->dig32.T : h->dig.T, fp32 ? h->dig32.Te : h->dig.Te, h->dtiles, h->dclsel,
+      reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT), v, y);
   CHECK_LAUNCH();
   return SMPM_OK;
 }
