@@ -140,10 +140,12 @@ __device__ long long g_barrier_spin_limit = 1LL << 28;
 // the CTA's next epoch (the counter's value on entry to a kernel, which all
 // CTAs share, plus the team size G per barrier).  One flag per CTA, polled by
 // a thread each, was four times slower at 152 CTAs (10 k against 2.6 k cycles:
-// the polls of all CTAs crowd the flags' L2 slice).  Bounded spin; err is set
+// the polls of all CTAs crowd the flags' L2 slice).  A team of one CTA needs no
+// counter.  Bounded spin; err is set
 // on timeout and the caller unwinds.
-__device__ __noinline__ bool team_sync_call(unsigned* bar, int* err, unsigned epoch) {
+__device__ __noinline__ bool team_sync_call(unsigned* bar, int* err, unsigned epoch, int G) {
   __syncthreads();
+  if (G == 1) return true;
   bool ok = true;
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(1u) : "memory");
@@ -165,8 +167,8 @@ __device__ __noinline__ bool team_sync_call(unsigned* bar, int* err, unsigned ep
 }
 template <typename S>
 __device__ __forceinline__ bool team_sync(const GmresArgs<S>& a, unsigned& epoch) {
-  epoch += (unsigned)a.G;
-  return team_sync_call(a.bar, a.err, epoch);
+  if (a.G > 1) epoch += (unsigned)a.G;  // the counter stays where it is for a team of one
+  return team_sync_call(a.bar, a.err, epoch, a.G);
 }
 // the epoch on entry to a kernel
 __device__ __forceinline__ unsigned first_epoch(const unsigned* bar) { return __ldcg(bar); }

@@ -128,6 +128,7 @@ __device__ __noinline__ void fd_pass(const uint4* A, const short* er, uint4* Bw,
   const int kt_n = digit_tiles(n);
   for (int c0 = 8 * part; c0 < n; c0 += 8 * W) {
     const int nc = min(8, n - c0), E = pack_cols<double>(Bw, x + c0 * ldc, ldk, ldc, n, nc, lane, 0, 1);
+#pragma unroll 1
     for (int mt = 0; mt < kt_n; ++mt) {
       const Tile8<double> t = digits_tile8<double>(A, er, Bw, n, kt_n, mt, lane, E);
 #pragma unroll
@@ -140,19 +141,20 @@ __device__ __noinline__ void fd_pass(const uint4* A, const short* er, uint4* Bw,
   }
 }
 
-// The same by plain FP64 products, a thread per entry of out, for a CTA that has
-// one element of n <= kFdThreadN nodes a side: its 256 threads form an 8 x 8
-// product in about 900 SM cycles, the packing and the tile of eight columns
-// take 3,500 in the one warp they occupy.  From n = 16 on (2,048 cycles of
-// FP64 products alone, two warps of tiles) the digits are not slower.
-constexpr int kFdThreadN = 12;
+// The same by plain FP64 products, a thread per entry of out.  An 8 x 8 product
+// takes a warp about 1,500 SM cycles, 256 of them FP64 issue; its packing and
+// tile of eight columns (half of it padding) 3,500.  At n = 12 the FP64 products
+// alone cost what the tiles do, so there only where the group has a thread for
+// every other entry; from n = 16 on the digits win.
+__host__ __device__ constexpr bool fd_by_threads(int n, int W) { return n <= 8 || (n <= 12 && n * n <= 64 * W); }
 __device__ __noinline__ void fd_thread_pass(const double* __restrict__ A, int n, int tid, int nthr, const double* x, int ldk,
                                             int ldc, double* out, int ldr, int ldo, const double* __restrict__ w) {
+#pragma unroll 1
   for (int q = tid; q < n * n; q += nthr) {
     const int c = q / n, r = q - c * n;
     double s0 = 0, s1 = 0;
     int k = 0;
-#pragma unroll 4
+#pragma unroll 2
     for (; k + 1 < n; k += 2) {
       s0 += __ldg(A + r * n + k) * x[k * ldk + c * ldc];
       s1 += __ldg(A + r * n + k + 1) * x[(k + 1) * ldk + c * ldc];
@@ -173,7 +175,7 @@ __device__ __noinline__ void elem_fd(const FdMats& fd, const DevGeo& g, int e, c
   const uint4 *Vx = fd.x + 2 * cx * nw, *Vxi = Vx + nw, *Vy = fd.y + 2 * cy * nw, *Vyi = Vy + nw;
   const short *ex = fd.xe + 2 * cx * n, *exi = ex + n, *ey = fd.ye + 2 * cy * n, *eyi = ey + n;
   const double* ri = fd.rinv + ((size_t)cy * fd.nx + cx) * n * n;
-  if (W == kGmresThreads / 32 && n <= kFdThreadN) {
+  if (fd_by_threads(n, W)) {
     const size_t nn = (size_t)n * n;
     const double *X = fd.fx + 2 * cx * nn, *Y = fd.fy + 2 * cy * nn;
     fd_thread_pass(Y + nn, n, 32 * part + lane, 32 * W, f.B, ld, 1, f.t1, ld, 1, nullptr);
@@ -205,6 +207,7 @@ __device__ __forceinline__ double normal_deriv_ld(const DevGeo& g, const double*
   const double* d = D + ((F & 1) ? (n - 1) * n : 0);
   double a0 = 0, a1 = 0;
   int c = 0;
+#pragma unroll 2
   for (; c + 1 < n; c += 2) {
     a0 += __ldg(d + c) * u[c * st];
     a1 += __ldg(d + c + 1) * u[(c + 1) * st];
@@ -226,19 +229,24 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
   int trace_n = 0;
   GM_TRACE(50);
   // ---- P1: zero the work vectors; b = f + tau g; u_L^T b
+#pragma unroll 1
   for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < g.kp; i += (long long)G * blockDim.x)
     for (int v = 0; v < 7; ++v) P.zero[v][i] = 0.0;
+#pragma unroll 1
   for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < P.gacc_n; i += (long long)G * blockDim.x)
     P.gacc[i] = 0.0;
+#pragma unroll 1
   for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < g.d; i += (long long)G * blockDim.x) {
     P.cb[i] = 0.0;
     if (P.cr) P.cr[i] = 0.0;
   }
   if (P.zero32[0])
+#pragma unroll 1
     for (long long i = (long long)rank * blockDim.x + threadIdx.x; i < g.kp; i += (long long)G * blockDim.x)
       for (int v = 0; v < 4; ++v) P.zero32[v][i] = 0.f;
   if (rank == 0 && threadIdx.x == 0) a.gs->scal[5] = 0.0;  // inner iterations of the solve
   double ulb = 0;
+#pragma unroll 1
   for (long long e = rank; e < g.nel; e += G) {
     for (int q = threadIdx.x; q < nn; q += blockDim.x) {
       const int aa = q % n, bb = q / n;
@@ -264,6 +272,7 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
   // ---- P2: project b; w = A_e^-1 b_e; push fluxes into b_S; u_S^T b_S; Z^T b_S
   const double alpha = __ldcg(P.acc + ACC_ULB);
   double pus = 0;
+#pragma unroll 1
   for (long long el = rank + (long long)grp * G; el < g.nel; el += (long long)ngrp * G) {
     const int e = (int)el;
     for (int q = part * 32 + lane; q < nn; q += 32 * W) {
@@ -276,6 +285,7 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
     elem_fd(P.fd, g, e, f, lane, part, W, grp);
     // flux of w into the slot (nbr, opp F, t): -tau' (p' w - n_F . grad w) with
     // tau', p' of the neighbour's face opp F and the gradient in e's own size
+#pragma unroll 1
     for (int i = part * 32 + lane; i < M; i += 32 * W) {
       const int F = i / n, t = i - F * n, e2 = dev_neighbour(g, e, F);
       double val = 0;
@@ -297,6 +307,7 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
     if (part == 0) {  // face F summed by the eight lanes 8 F + r
       const int F = lane >> 3, j = dev_iface(g, e, F);
       double sum = 0;
+#pragma unroll 1
       for (int t = lane & 7; t < n; t += 8) sum += f.p[F * n + t];
       for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       if ((lane & 7) == 0 && j >= 0) atomicAdd(P.cb + j, sum);
@@ -311,6 +322,7 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
   // ---- P3: c_hat_b = C^+ Z^T (b_S - beta u_S)
   const double beta = __ldcg(P.acc + ACC_USBS);
   if (a.precond == 2) {
+#pragma unroll 1
     for (int j = rank * blockDim.x + threadIdx.x; j < (int)g.d; j += G * blockDim.x)
       a.c[j] = __ldcg(P.cb + j) - beta * P.ZtuS[j];
     GM_TRACE(55);
@@ -318,11 +330,13 @@ __device__ SMPM_BODY bool pre_body(const PrePostArgs& P, unsigned char* smraw, u
     GM_TRACE(56);
     if (!coarse_solve(a, s, epoch, a.c, a.chat)) return false;  // a.c -> a.chat
     GM_TRACE(58);
+#pragma unroll 1
     for (int j = rank * blockDim.x + threadIdx.x; j < (int)g.d; j += G * blockDim.x)
       P.chatb[j] = __ldcg(a.chat + j);
   }
   // ---- P4: owner entries: project b_S, rhs = P b_S
   double bsn = 0, rgn = 0;
+#pragma unroll 1
   for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
     const int4 en = owned_entry(a, i);
     const int sl = en.x;
@@ -365,6 +379,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
   if (P.assembled) {
     // x_S given (iterative refinement)
   } else if (a.precond == 0) {
+#pragma unroll 1
     for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
       const int sl = entry_slot(a, i);
       if (sl >= 0) P.xs[sl] = __ldcg(a.x + sl);
@@ -375,6 +390,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
       GM_TRACE(61);
       if (!team_sync(a, epoch)) return false;
       GM_TRACE(62);
+#pragma unroll 1
       for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
         const int sl = entry_slot(a, i);
         if (sl >= 0) P.xs[sl] = __ldcg(a.t + sl);
@@ -382,6 +398,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
     } else {
       // white step and coarse solve of y = S t, then x_S = t - Z (c_hat - c_hat_b)
       if (!apply_op(a, s, a.x, 1.0, true, trace_n, epoch)) return false;
+#pragma unroll 1
       for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
         const int4 en = owned_entry(a, i);
         if (en.x < 0) continue;
@@ -394,14 +411,17 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
   GM_TRACE(64);
   // ---- Q5: recovery u_e = A_e^-1 (b_e - E_e x_S), residual b_S - S x_S, mean
   double pm = 0, pr = 0;
+#pragma unroll 1
   for (long long el = rank + (long long)grp * G; el < g.nel; el += (long long)ngrp * G) {
     const int e = (int)el, ct = __ldg(a.dm.tcls + e);
     for (int q = part * 32 + lane; q < nn; q += 32 * W) f.B[(q / n) * ld + q % n] = P.b[el * nn + q];
     for (int i = part * 32 + lane; i < M; i += 32 * W) f.p[i] = __ldcg(P.xs + el * M + i);
     item_sync(grp, W);
+#pragma unroll 1
     for (int F = 0; F < 4; ++F) {  // faces in turn: a corner node takes both slots
       if (dev_neighbour(g, e, F) >= 0) {
         if (!P.adjoint) {
+#pragma unroll 1
           for (int t = part * 32 + lane; t < n; t += 32 * W) {
             int aa, bb;
             face_node(n, F, t, &aa, &bb);
@@ -417,6 +437,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
           const double sc = face_geo(g, e, F)[2];
           const int drow = (F & 1) ? n - 1 : 0;   // D row of the face end
           const double sgn = (F & 1) ? 1.0 : -1.0;  // outward normal along the axis
+#pragma unroll 1
           for (int idx = part * 32 + lane; idx < nn; idx += 32 * W) {
             const int t = idx / n, k = idx % n;
             const double v = f.p[F * n + t];
@@ -437,6 +458,7 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
     // (S x_S) on the slots facing e: x_S + T_e x_S,e
     const int E = pack_one<double>(f.Bf, f.p, M, lane, part, W);
     item_sync(grp, W);
+#pragma unroll 1
     for (int mt = part; mt < kt_n; mt += W) {
       const int row = tile1_row(mt, lane, M);
       Facing<double> fc{};
@@ -462,10 +484,12 @@ __device__ SMPM_BODY bool post_body(const PrePostArgs& P, unsigned char* smraw, 
   // ---- Q6: zero GLL-weighted mean (adjoint: projection out of u_L, dl/dg)
   const double mean = __ldcg(P.acc + ACC_MEAN);
   if (!P.adjoint) {
+#pragma unroll 1
     for (long long e = rank; e < g.nel; e += G)
       for (int q = threadIdx.x; q < nn; q += blockDim.x) P.u[e * nn + q] -= mean;
     return true;
   }
+#pragma unroll 1
   for (long long e = rank; e < g.nel; e += G) {
     if (P.gg)
       for (int i = threadIdx.x; i < M; i += blockDim.x) {

@@ -1339,7 +1339,8 @@ Layout choose_layout(const Geometry& g, int m, int ES, int items, bool no_smem, 
 size_t prepost_shape(const Geometry& g, int m, int ES, int items, int G, size_t budget, bool w_global, int* W, int* W_fd) {
   *W = item_warps(items);
   *W_fd = std::min(item_warps((g.nel + G - 1) / G), std::max(1, (g.n + 7) / 8 > 2 ? 4 : (g.n + 7) / 8));
-  if (g.nel <= G && g.n <= kFdThreadN) *W_fd = kGmresThreads / 32;
+  const int W_all = item_warps((g.nel + G - 1) / G);
+  if (fd_by_threads(g.n, W_all)) *W_fd = W_all;
   auto need = [&] { return prepost_smem_bytes(m, g.M, g.n, ES, *W, *W_fd, g.d, w_global); };
   while (need() > budget && (*W < kGmresThreads / 32 || *W_fd < kGmresThreads / 32)) {
     if (*W_fd < kGmresThreads / 32) *W_fd *= 2;
@@ -3282,7 +3283,12 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     CU(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int nb = (int)h->f.black.size(), nw = (int)h->f.white.size();
     auto& gm = h->gm;
+    // A handful of blocks goes to one CTA: its phases then meet at CTA barriers
+    // (five team barriers, 2,400 cycles each, of a 37,000 cycle step at 2 x 2, n = 8).
+    // With more than about an entry per thread the FP64 Gram-Schmidt sums of one SM
+    // would cost as much.
     gm.grid = std::max(1, std::min(sms, std::max(nb, nw)));
+    if (2 * g.M * nb <= kGmresThreads) gm.grid = 1;
     gm.nown_b = (nb + gm.grid - 1) / gm.grid;
     gm.nown_w = (nw + gm.grid - 1) / gm.grid;
     gm.ES = basis_entries(g.M, gm.nown_b);
