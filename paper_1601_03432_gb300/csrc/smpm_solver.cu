@@ -3283,12 +3283,12 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     CU(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const int nb = (int)h->f.black.size(), nw = (int)h->f.white.size();
     auto& gm = h->gm;
-    // A handful of blocks goes to one CTA: its phases then meet at CTA barriers
-    // (five team barriers, 2,400 cycles each, of a 37,000 cycle step at 2 x 2, n = 8).
-    // With more than about an entry per thread the FP64 Gram-Schmidt sums of one SM
-    // would cost as much.
+    // Two small blocks go to one CTA: its phases then meet at CTA barriers (five
+    // team barriers, 2,400 cycles each, of a 37,000 cycle step at 2 x 2, n = 8:
+    // 386 against 325 us).  Beyond that the FP64 Gram-Schmidt sums of one SM cost
+    // as much (2 x 2, n = 12: 445 us either way; 3 x 2, n = 10: 490 against 599).
     gm.grid = std::max(1, std::min(sms, std::max(nb, nw)));
-    if (2 * g.M * nb <= kGmresThreads) gm.grid = 1;
+    if (nb <= 2 && 2 * g.M * nb <= 128) gm.grid = 1;
     gm.nown_b = (nb + gm.grid - 1) / gm.grid;
     gm.nown_w = (nw + gm.grid - 1) / gm.grid;
     gm.ES = basis_entries(g.M, gm.nown_b);
