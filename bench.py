@@ -35,7 +35,7 @@ WORKLOAD_NAME = "SMPM Poisson-Neumann, 16x16 elements, n=16 (r=65536), FP64, 1 F
 L2_FLUSH_BYTES = 512 << 20          # written between timed steps: 3.9x the 135.5 MB L2 of a GB300
 CONFIG = {"workload": WORKLOAD_NAME, **WORKLOAD, "precision": "fp64", "precond": "block-Jacobi + deflation"}
 GMRES_PROFILE = os.path.join(ROOT, "profiles", "k_gmres_16x16_n16_fp64.md")
-GMRES_SOURCES = [os.path.join(ROOT, "paper_1601_03432_gb300", "csrc", f) for f in ("smpm_gmres.cuh", "smpm_kernels.cuh")]
+GMRES_SOURCES = [os.path.join(ROOT, "paper_1601_03432_gb300", "csrc", f) for f in ("smpm_gmres.cuh", "smpm_digits.cuh")]
 
 
 def kernel_traffic():
@@ -330,7 +330,7 @@ def run_ours(args):
     mixed = {"value": mix_rate, "unit": "solves/s",
              "ms_per_step": mix_max / args.steps, "inner_iterations": mix_rep["iterations"],
              "refinements": mix_rep["refinements"], "schur_relres": mix_rep["schur_relres"],
-             "precision": "FP32 inner GMRES (FP32 operator; FP32 coarse product, or the FP64 fused coarse update on small grids; FP64 Givens and dot accumulation) + FP64 refinement"}
+             "precision": "FP32 inner GMRES (30-bit digit operator products, FP32 coarse product; FP64 Hessenberg least squares and dot accumulation) + FP64 refinement"}
 
     # ---- Schur apply y = S v on single grids of growing size (operator-only
     # factor step: T_e only), L2 flushed before each launch (write + read
@@ -342,6 +342,8 @@ def run_ours(args):
         ga.factor(precision=1, flags=_B.FLAG_OPERATOR_ONLY)
         Ma, nela = 4 * an, amx * amy
         pt = {"grid": "%dx%d, n=%d" % (amx, amy, an)}
+        # per-element matrices (left to itself the apply takes the class-shared product here)
+        ga.set_apply_kernel(_B.APPLY_WARP4 if nela < 2048 else _B.APPLY_WARP)
         for name, dt, fn, sz in (("fp64", torch.float64, ga.apply_schur, 8),
                                  ("fp32", torch.float32, ga.apply_schur32, 4)):
             va = torch.randn(ga.kp, dtype=dt, device="cuda")

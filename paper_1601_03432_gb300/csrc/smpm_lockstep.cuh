@@ -160,6 +160,10 @@ __device__ __forceinline__ Quad<S> ld_quad_w(const S* p) {  // w: shared or glob
 // own, else the global vector src).  t = M^-1 v on the block: r1 = p - X q,
 // a = G r1, z = T_e a, t = [a; q - z]; the products run on the tensor cores
 // (smpm_digits.cuh), eight columns to a tile.
+// Bound by the row tiles' chains (first digits from L2, unpacking, 36 products of
+// 8 cycles per k tile in FP64): at M = 96, four blocks and eight columns 116,000 SM
+// cycles -- gather 14, X 27, packing 10, G and T 25 each per group of two warps --
+// against 492,000 with FP64 FMA.
 template <typename S>
 __device__ SMPM_PHASE void lk_black(const LockArgs<S>& A, const LockSmem<S>& s, const S* src, const double* sc, int jbasis) {
   const GmresArgs<S>& a = A.a;

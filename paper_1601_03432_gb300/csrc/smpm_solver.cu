@@ -829,6 +829,9 @@ cudaError_t launch_schur_warp(const ElemMeta<S>* tab, long long nelem, const S* 
 // 16 rows of T_c: the warps cut the slot vectors into digits together (shared
 // memory), each then runs its row tile; T_c's digits come from L1.  Many small
 // CTAs per SM: a row tile is a chain of loads and dependent products.
+// Bound by that chain, not by HBM: 96 x 96 elements, n = 24, FP64 34.8 us (14.8 MB
+// of vectors are 2.2 us; 222 us with FP64 FMA on 64 elements per CTA, 160 us by
+// per-element matrices from HBM); 128 x 128, n = 16, FP32 18.3 us (24.6 and 59.4).
 constexpr int kClassTile = 8;
 
 // one entry of T_e v on an element whose v has an Inf or NaN, which have no
