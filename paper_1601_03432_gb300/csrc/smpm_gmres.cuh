@@ -307,16 +307,13 @@ inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int W, int basis_sme
          (2 * (size_t)(ES / (2 * M)) + 4) * sizeof(int4) + (tab ? ES * sizeof(OwnedEntry) : 0) + H_bytes + 96;
 }
 
-// The class most of cnt owned items have other than `skip` (-1: none): id[rank +
-// k G] for k < cnt, classes cls[id] (cls[ib] where id is null).  Warp 0; the
-// first 32 items stand for all.
-__device__ __forceinline__ int main_class(const int* cls, const int* id, int rank, int G, int cnt, int total, int skip) {
+// The class that most of the CTA's cnt owned items have other than `skip` (-1:
+// none): field f of their tables' entries.  Warp 0; the first 32 items stand for
+// all.
+__device__ __forceinline__ int main_class(const int4* own, int cnt, int f, int skip) {
   const int lane = threadIdx.x & 31;
   int mine = -1;
-  if (lane < cnt && rank + lane * G < total) {
-    const int i = rank + lane * G;
-    mine = cls[id ? id[i] : i];
-  }
+  if (lane < cnt && own[lane].x >= 0) mine = f == 1 ? own[lane].y : own[lane].z;
   int n = 0;
   for (int k = 0; k < 32; ++k) n += __shfl_sync(0xffffffffu, mine, k) == mine;
   const int best = __reduce_max_sync(0xffffffffu, mine >= 0 && mine != skip ? n * 32 + lane : -1);
@@ -354,6 +351,13 @@ __device__ SMPM_PHASE void load_resident(const GmresArgs<S>& a, const Smem<S>& s
   const size_t wG = a.blk ? digit_words<S>(2 * M, 2 * M) : wM;
   uint4* p = reinterpret_cast<uint4*>(s.end);
   load_owned(a, s);
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int t0 = a.res_T > 0 ? main_class(s.ow, a.nown_w, 1, -1) : -1;
+    const int t1 = a.res_T > 1 ? main_class(s.ob, a.nown_b, 2, t0) : -1;
+    const int g0 = a.res_G > 0 ? main_class(s.ob, a.nown_b, 1, -1) : -1;
+    if (threadIdx.x == 0) *s.res = {p, p + a.res_T * wM, p + (a.res_T + 1) * wM, {t0, t1}, g0};
+  }
   if (s.tab) {
     for (int i = threadIdx.x; i < a.ES; i += blockDim.x) {
       OwnedEntry o = {owned_entry(a, i), make_int4(0, 0, 0, 0), make_double2(0, 0), make_double2(0, 0)};
@@ -371,13 +375,6 @@ __device__ SMPM_PHASE void load_resident(const GmresArgs<S>& a, const Smem<S>& s
     const int d = (int)a.g.d, ld = (d + 3) & ~3, per = (d + a.G - 1) / a.G;
     const int r0 = min(d, rank * per), cnt = (min(d, r0 + per) - r0) * ld;
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) const_cast<T*>(s.H)[i] = __ldg(a.H + (size_t)r0 * ld + i);
-  }
-  if (threadIdx.x < 32) {
-    const DigitMats& D = a.dm;
-    const int t0 = a.res_T > 0 ? main_class(D.tcls, a.white, rank, a.G, a.nown_w, a.nwhite, -1) : -1;
-    int t1 = a.res_T > 1 ? main_class(D.tcls, a.black, rank, a.G, a.nown_b, a.nblack, t0) : -1;
-    const int g0 = a.res_G > 0 ? main_class(D.bcls, nullptr, rank, a.G, a.nown_b, a.nblack, -1) : -1;
-    if (threadIdx.x == 0) *s.res = {p, p + a.res_T * wM, p + (a.res_T + 1) * wM, {t0, t1}, g0};
   }
   __syncthreads();
   const Resident& R = *s.res;
