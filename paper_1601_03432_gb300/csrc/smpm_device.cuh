@@ -49,8 +49,9 @@ constexpr int kSlotsPerBlock = 256;   // slots per CTA in the vector kernels
 constexpr int kElemThreads = 256;     // threads per element CTA
 constexpr int kTraceCap = 1 << 16;    // entries of the optional phase trace
 constexpr int kGmresThreads = 256;    // threads per CTA of the persistent GMRES kernel
-// per-solve control block (zeroed by one memset): barrier counter | (at 256)
-// err, done, nref | 8 accumulators | 32 refinement residual norms
+// per-solve control block (zeroed by one memset): 64 barrier counters, one per
+// launch of the solve | (at 256) err, done, nref | 8 accumulators | 32
+// refinement residual norms
 constexpr size_t kCtlBytes = 720;  // + 32 inner iteration counts
 constexpr int kMaxRefine = 8;        // FP64 refinement steps of the mixed-precision path
 constexpr double kInnerTol = 1e-4;   // relative tolerance of each FP32 inner GMRES

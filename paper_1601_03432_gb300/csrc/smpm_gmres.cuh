@@ -137,12 +137,14 @@ __device__ long long g_barrier_spin_limit = 1LL << 28;
 
 // Team barrier on a monotonic counter: thread 0 of each CTA adds one with
 // release semantics and polls with acquire loads until the counter reaches
-// the CTA's next epoch (the counter's value on entry to a kernel, which all
-// CTAs share, plus the team size G per barrier).  One flag per CTA, polled by
-// a thread each, was four times slower at 152 CTAs (10 k against 2.6 k cycles:
-// the polls of all CTAs crowd the flags' L2 slice).  A team of one CTA needs no
-// counter.  Bounded spin; err is set
-// on timeout and the caller unwinds.
+// the CTA's next epoch: zero on entry to a kernel, plus the team size G per
+// barrier.  Every launch has a counter of its own, zeroed on its stream before
+// it.  A cooperative launch does not make its CTAs start together (work on
+// another stream can hold an SM back), so the epoch on entry cannot be read from
+// a counter that CTAs already running may have advanced.  One flag per CTA,
+// polled by a thread each, was four times slower at 152 CTAs (10 k against 2.6 k
+// cycles: the polls of all CTAs crowd the flags' L2 slice).  A team of one CTA
+// needs no counter.  Bounded spin; err is set on timeout and the caller unwinds.
 __device__ __noinline__ bool team_sync_call(unsigned* bar, int* err, unsigned epoch, int G) {
   __syncthreads();
   if (G == 1) return true;
@@ -170,8 +172,6 @@ __device__ __forceinline__ bool team_sync(const GmresArgs<S>& a, unsigned& epoch
   if (a.G > 1) epoch += (unsigned)a.G;  // the counter stays where it is for a team of one
   return team_sync_call(a.bar, a.err, epoch, a.G);
 }
-// the epoch on entry to a kernel
-__device__ __forceinline__ unsigned first_epoch(const unsigned* bar) { return __ldcg(bar); }
 
 // entry i (< 2M) of black block ib
 template <typename S>

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A0) {
   if (lock_all_done(A0)) return;
   if (threadIdx.x == 0) A = A0;
   __syncthreads();
-  unsigned epoch = first_epoch(A.a.bar);
+  unsigned epoch = 0;
   lock_body(A, smraw, epoch);
 }
 
@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(256, 1) k_gmres_lock(LockArgs<S> A0) {
 // the previous column.
 __global__ void __launch_bounds__(256, 1) k_pre_cols(const PrePostArgs* __restrict__ Ps, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = first_epoch(Ps[0].ga.bar);
+  unsigned epoch = 0;
   __shared__ PrePostArgs P;
   for (int c = 0; c < R; ++c) {
     __syncthreads();
@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256, 1) k_pre_cols(const PrePostArgs* __restri
 
 __global__ void __launch_bounds__(256, 1) k_post_cols(const PrePostArgs* __restrict__ Ps, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = first_epoch(Ps[0].ga.bar);
+  unsigned epoch = 0;
   __shared__ PrePostArgs P;
   for (int c = 0; c < R; ++c) {
     __syncthreads();
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256, 1) k_post_cols(const PrePostArgs* __restr
 // only its own body (rank 0, after a barrier every CTA passed) sets it.
 __global__ void __launch_bounds__(256, 1) k_refine_cols(const RefineArgs* __restrict__ Rs, int R) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  unsigned epoch = first_epoch(Rs[0].ga.bar);
+  unsigned epoch = 0;
   __shared__ RefineArgs A;
   for (int c = 0; c < R; ++c) {
     if (*((volatile const int*)Rs[c].done)) continue;

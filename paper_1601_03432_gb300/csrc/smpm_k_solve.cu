@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(256, 1) k_gmres(GmresArgs<S> a0) {
   if (threadIdx.x == 0) a = a0;
   __syncthreads();
   if (a.skip && *((volatile const int*)a.skip)) return;
-  unsigned epoch = first_epoch(a.bar);
+  unsigned epoch = 0;
   gmres_body(a, smraw, epoch);
 }
 
@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256, 1) k_pre(PrePostArgs P0) {
   __shared__ PrePostArgs P;
   if (threadIdx.x == 0) P = P0;
   __syncthreads();
-  unsigned epoch = first_epoch(P.ga.bar);
+  unsigned epoch = 0;
   pre_body(P, smraw, epoch);
 }
 
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256, 1) k_post(PrePostArgs P0) {
   __shared__ PrePostArgs P;
   if (threadIdx.x == 0) P = P0;
   __syncthreads();
-  unsigned epoch = first_epoch(P.ga.bar);
+  unsigned epoch = 0;
   post_body(P, smraw, epoch);
 }
 
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256, 1) k_refine(RefineArgs R0) {
   if (threadIdx.x == 0) R = R0;
   __syncthreads();
   if (*((volatile const int*)R.done)) return;
-  unsigned epoch = first_epoch(R.ga.bar);
+  unsigned epoch = 0;
   refine_body(R, smraw, epoch);
 }
 

@@ -1533,7 +1533,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   PrePostArgs P = prepost_args(h, tol, f, gn, u, true);
   CU(cudaEventRecord(h->evp, st));
   {
-    P.ga.bar = h->wbar;
+    P.ga.bar = h->wbar + 0;
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_pre(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
                                    st));
@@ -1542,7 +1542,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   CU(cudaEventRecord(h->ev0, st));
   for (int ref = 0; ref < kMaxRefine; ++ref) {
     GmresArgs<float> a = gmres_args32(h, kInnerTol);
-    a.bar = h->wbar;
+    a.bar = h->wbar + 2 + 2 * ref;
     a.its_out = reinterpret_cast<int*>(h->wctl + 592) + ref;
     if (ref == 0 && h->wtrace) {
       a.trace = h->wtrace;
@@ -1555,7 +1555,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
       CHECK_LAUNCH();
     }
     RefineArgs RA = refine_args(h, a, tol);
-    RA.ga.bar = h->wbar;
+    RA.ga.bar = h->wbar + 3 + 2 * ref;
     RA.rn = h->wrn + ref;
     void* args[] = {&RA};
     CU(cudaLaunchCooperativeKernel(fn_refine(), dim3(h->gm.grid), dim3(kGmresThreads), args,
@@ -1564,7 +1564,7 @@ smpm_status solve_one_mixed(smpm_handle h, const double* f, const double* gn, do
   }
   CU(cudaEventRecord(h->ev1, st));
   {
-    P.ga.bar = h->wbar;
+    P.ga.bar = h->wbar + 1;
     P.assembled = 1;
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
@@ -1629,7 +1629,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   // pre/post accumulators (contiguous); everything else is zeroed in k_pre
   CU(cudaMemsetAsync(h->wctl, 0, kCtlBytes, st));
   PrePostArgs P = prepost_args(h, tol, f, gn, u, false, adj, gg);
-  P.ga.bar = h->wbar;
+  P.ga.bar = h->wbar + 0;
   if (h->wtrace) {  // pre and post trace into the upper halves of the buffer
     P.ga.trace = h->wtrace + kTraceCap / 2;
     P.ga.trace_cap = kTraceCap / 4;
@@ -1644,7 +1644,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   CU(cudaEventRecord(h->ev0, st));
   {
     GmresArgs<double> a = gmres_args(h, tol, adj);
-    a.bar = h->wbar;
+    a.bar = h->wbar + 1;
     void* args[] = {&a};
     CU(cudaLaunchCooperativeKernel(fn_gmres64(), dim3(h->gm.grid), dim3(kGmresThreads), args,
                                    h->gm.smem, st));
@@ -1652,7 +1652,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   }
   CU(cudaEventRecord(h->ev1, st));
   {
-    P.ga.bar = h->wbar;
+    P.ga.bar = h->wbar + 2;
     if (h->wtrace) P.ga.trace = h->wtrace + 3 * (kTraceCap / 4);
     void* args[] = {&P};
     CU(cudaLaunchCooperativeKernel(fn_post(), dim3(h->gm.grid), dim3(kGmresThreads), args, h->gm.smem_pp,
@@ -1709,11 +1709,12 @@ smpm_status lalloc(smpm_handle h, P** p, size_t count) {
   return SMPM_OK;
 }
 
-// control block of a lockstep solve: barrier counter (shared by the solve's
-// kernels in turn) at 0, err at 128; column k's block
+// control block of a lockstep solve: 32 barrier counters, one per launch (pre 0,
+// post 1, GMRES 2 + 2 ref, refinement 3 + 2 ref), err at 128; column k's block
 // at kLockCtlBytes + k kLockColBytes: acc8 (8 doubles) | done, nref (ints at
 // +64) | rn[kMaxRefine] at +128
 constexpr size_t kLockCtlBytes = 256;  // (kLockColBytes, the column block size, is shared with the batch)
+static_assert(2 + 2 * kMaxRefine <= 32, "a barrier counter per launch before err");
 
 // Entries per CTA and column in a basis slice (whole 16-byte groups).
 int basis_entries(int M, int nown_b) { return (2 * M * nown_b + 3) & ~3; }
@@ -1843,9 +1844,9 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       P.cr = L.cr + (size_t)k * g.d;
       P.rg32 = L.rg32 + (size_t)k * g.kp;
     }
-    P.ga.bar = bar;
+    P.ga.bar = bar + 0;
     L.hP[k] = P;
-    P.ga.bar = bar;
+    P.ga.bar = bar + 1;
     P.assembled = mixed ? 1 : 0;
     L.hP[R + k] = P;
   }
@@ -1862,7 +1863,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
         a.err = err;
         a.skip = nullptr;
         RefineArgs RA = refine_args(h, a, tol);
-        RA.ga.bar = bar;
+        RA.ga.bar = bar + 3 + 2 * ref;
         RA.xS = L.xs + (size_t)k * g.kp;
         RA.bS = L.bS + (size_t)k * g.kp;
         RA.cr = L.cr + (size_t)k * g.d;
@@ -1900,7 +1901,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     A.a = gmres_args(h, tol);
     lock_fields(A);
     A.a.rhs = L.rg; A.a.x = L.x; A.a.t = L.t; A.a.y = L.y; A.a.vglob = L.vg;
-    A.a.bar = bar;
+    A.a.bar = bar + 2;
     A.V = L.V; A.W = L.W;
     A.done = nullptr; A.done_stride = 0;
     if (h->wtrace) {
@@ -1918,7 +1919,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
       A.a = gmres_args32(h, kInnerTol);
       lock_fields(A);
       A.a.rhs = L.rg32; A.a.x = L.x32; A.a.t = L.t32; A.a.y = L.y32; A.a.vglob = L.vg32;
-      A.a.bar = bar;
+      A.a.bar = bar + 2 + 2 * ref;
       A.V = L.V32; A.W = L.W32;
       A.done = reinterpret_cast<const int*>(colblk(0) + 64);
       A.done_stride = (int)(kLockColBytes / sizeof(int));
