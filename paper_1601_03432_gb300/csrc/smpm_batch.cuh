@@ -95,6 +95,14 @@ __device__ __noinline__ int batch_group(BatchTask& T, unsigned char* smraw, unsi
     const size_t nacc = (size_t)(2 * a.m + 1) * R * (a.m + 3);
     double* acc = T.precision == 0 ? T.L64.a.acc : T.L32.a.acc;
     for (size_t i = (size_t)rank * blockDim.x + threadIdx.x; i < nacc; i += (size_t)a.G * blockDim.x) acc[i] = 0.0;
+    // t starts at zero: the phases never write its physical-boundary slots, which
+    // an earlier group of another shape may have used.  They meet zero columns
+    // of T_e, but set the scale of the digits that the other slots are cut to.
+    const size_t nt = (size_t)R * T.kp_len, i0 = (size_t)rank * blockDim.x + threadIdx.x, di = (size_t)a.G * blockDim.x;
+    if (T.precision == 0)
+      for (size_t i = i0; i < nt; i += di) T.L64.a.t[i] = 0.0;
+    else
+      for (size_t i = i0; i < nt; i += di) T.L32.a.t[i] = 0.f;
   }
   if (!team_sync(ga, epoch)) return 1;
   for (int c = 0; c < R; ++c) {
