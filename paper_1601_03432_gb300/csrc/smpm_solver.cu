@@ -857,12 +857,20 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
   // this warp's 16 slots of the eight elements, loaded once
   const int* el = elems + start;
   const int gc = lane >> 2, q = lane & 3;
-  const S* vm = v + (size_t)__ldg(el + min(gc, cnt - 1)) * M;
+  const int ec = __ldg(el + min(gc, cnt - 1));
+  const S* vm = v + (size_t)ec * M;
+  constexpr int kNonFinite = sizeof(S) == 4 ? 0xff : 0x7ff;  // exponent field of Inf and NaN
   S x[4];
+  int E = 1;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int k = warp * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
-    x[u] = (gc < cnt && k < M) ? __ldg(vm + k) : S(0);
+    const S r = (gc < cnt && k < M) ? __ldg(vm + k) : S(0);
+    const int Er = exp_field(r);
+    // slots on the physical boundary meet zero columns: they must not set the scale
+    const bool on = k < M && dev_neighbour(g, ec, k / g.n) >= 0;
+    x[u] = on ? r : S(0);
+    if (on || Er == kNonFinite) E = max(E, Er);
   }
   // outputs of the warp's row tile: facing slots and what they hold
   long long sl[4];
@@ -881,7 +889,6 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
     vf[u] = __ldg(v + sl[u]);
   }
   __syncthreads();
-  int E = max(max(exp_field(x[0]), exp_field(x[1])), max(exp_field(x[2]), exp_field(x[3])));
   E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
   E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
   if (q == 0) atomicMax(Emax + gc, E);
@@ -896,7 +903,7 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
     if (sl[u] < 0) continue;
     const int r = warp * 16 + gc + 8 * (u >> 1), c = 2 * q + (u & 1);
     S z = t.z[u];
-    if (Emax[c] == (sizeof(S) == 4 ? 0xff : 0x7ff) && push[u])
+    if (Emax[c] == kNonFinite && push[u])
       z = plain_row(T + (size_t)__ldg(el + c) * M * M + r, v + (size_t)__ldg(el + c) * M, M);
     y[sl[u]] = push[u] ? vf[u] + z : vf[u];
   }

@@ -8,6 +8,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 from paper_1601_03432_gb300 import Batch, Grid, inputs
+from paper_1601_03432_gb300 import _binding as B
 
 
 @pytest.fixture(scope="module")
@@ -50,3 +51,32 @@ def test_batch_groups_are_independent_of_what_ran_before(built, precision):
                 assert abs(reps[i * R + k]["iterations"] - ref["iterations"]) <= (1 + ref["iterations"] // 7
                                                                                    if precision == 0 else 12)
     b.close()
+
+
+def applied(g, kind, v):
+    g.set_apply_kernel(kind)
+    y = torch.full_like(v, -7.0)
+    (g.apply_schur if v.dtype == torch.float64 else g.apply_schur32)(v, y)
+    torch.cuda.synchronize()
+    return y.double().cpu().numpy()
+
+
+# n: part of a tile, a tile and a remainder, whole tiles
+@pytest.mark.parametrize("mx,my,n", [(7, 5, 3), (5, 6, 9), (6, 6, 16)])
+@pytest.mark.parametrize("big", [1e12, 1e100])
+def test_apply_is_blind_to_boundary_slots(built, mx, my, n, big):
+    """Large values on physical-boundary slots (T_e's columns there are zero) leave
+    every other entry of S v as it is, and stay where they are themselves."""
+    g = Grid(mx, my, n)
+    g.factor(precision=1)
+    face = np.ones((my, mx, 4, n), bool)
+    face[:, 0, 0], face[:, -1, 1], face[0, :, 2], face[-1, :, 3] = False, False, False, False
+    face = face.ravel()
+    v = np.random.default_rng(n).standard_normal(face.size)
+    for dtype in (torch.float64, torch.float32):
+        b = min(big, 1e30) if dtype == torch.float32 else big
+        for kind in (B.APPLY_AUTO, B.APPLY_CLASS, B.APPLY_WARP):
+            plain = applied(g, kind, dev(np.where(face, v, 0.0), dtype))
+            got = applied(g, kind, dev(np.where(face, v, b * v), dtype))
+            assert np.array_equal(got[face], plain[face]), kind
+            assert np.array_equal(got[~face], dev(b * v, dtype).double().cpu().numpy()[~face])
