@@ -224,31 +224,33 @@ smpm_status smpm_apply_schur_precond(smpm_handle h, const double* v, double* y, 
 smpm_status smpm_apply_deflation(smpm_handle h, const double* v, double* y, void* stream);
 /* y = Q v, Q = I - Z C^-1 Z^T S (Eq. projection2). */
 smpm_status smpm_apply_deflation_q(smpm_handle h, const double* v, double* y, void* stream);
-/* y = S v as smpm_apply_schur / smpm_apply_schur32, by the element-class-
- * shared path: on the axis-aligned uniform grids of this library T_e depends
+/* y = S v as smpm_apply_schur / smpm_apply_schur32 (every entry within the
+ * rounding error of a chain of FMAs in the vector's precision), by the
+ * element-class-shared path: on the axis-aligned uniform grids of this library T_e depends
  * only on which faces of the element are interfaces (at most 9 classes), so
  * the apply is one dense product T_c X_c per class (X_c: the own slots of the
  * class's elements side by side) and only the vectors stream from HBM.  The
  * paper's method keeps per-element factors (mapped elements, Sec. 1.2); this
- * is a property of uniform grids.  Needs n <= 32.  Errors as
- * smpm_apply_schur. */
+ * is a property of uniform grids.  Where the elements fall into many small
+ * classes, or a row of T_e spans more than 2^35 (FP32: 2^33) in magnitude, the
+ * per-element kernels run in its place.  Errors as smpm_apply_schur. */
 smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, void* stream);
 smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, void* stream);
 
 /* Kernels of y = S v (smpm_apply_schur, smpm_apply_schur32 and the S apply
  * inside the deflation entry points): AUTO takes CLASS where the elements
  * fall into few enough classes that its tiles of eight elements are at least a
- * fifth full on average, else by thresholds one warp per element for 4n <= 96 (1, 2 or
- * 4 warps by the element count) or the shared-memory stream; WARP: persistent CTAs, one warp per element,
- * T_e read column by column from global memory; WARP2 / WARP4: 2 or 4 warps
- * per element; STREAM: bulk copies of T_e into a shared-memory ring; CLASS:
- * the element-class-shared product (smpm_apply_schur_class). */
+ * fifth full on average and the grid is large enough for it to be the faster
+ * one, else by thresholds one warp per element for 4n <= 96 (1, 2 or 4 warps by
+ * the element count) or the shared-memory stream; WARP: persistent CTAs, one
+ * warp per element, T_e read column by column from global memory; WARP2 / WARP4:
+ * 2 or 4 warps per element; STREAM: bulk copies of T_e into a shared-memory
+ * ring; CLASS: the element-class-shared product (smpm_apply_schur_class). */
 enum { SMPM_APPLY_AUTO = 0, SMPM_APPLY_WARP = 1, SMPM_APPLY_WARP2 = 2, SMPM_APPLY_WARP4 = 3,
        SMPM_APPLY_STREAM = 4, SMPM_APPLY_CLASS = 5 };
 
 /* Fix the apply kernel of h.  Errors: ESTATE (not factored), EINVAL (kind
- * not available on this grid: WARP* need 4n <= 96, CLASS its tile in shared
- * memory). */
+ * not available on this grid: WARP* need 4n <= 96). */
 smpm_status smpm_set_apply_kernel(smpm_handle h, int kind);
 
 /* Time every available apply kernel on h's grid in precision 0 (FP64) or 1

@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 namespace {
@@ -42,6 +43,12 @@ struct Digits<double> {
 template <>
 struct Digits<float> {
   static constexpr int ND = 4, GMIN = 2, NG = 5, B = 30;
+};
+
+struct Wide {};  // FP64 operands of 94 bits: the class apply (tile8_wide)
+template <>
+struct Digits<Wide> {
+  static constexpr int ND = 12, GMIN = 11, NG = 12, B = 94;
 };
 
 constexpr short kBadRow = 32767;  // row exponent of a matrix row with an Inf or NaN
@@ -107,6 +114,33 @@ __device__ __forceinline__ uint32_t to_digits(float v, int E) {
   else x = -sh < 28 ? (m + (1 << (-sh - 1))) >> -sh : 0;
   x = bits < 0 ? -x : x;
   return (uint32_t)x + 0x80808080u;
+}
+
+// the same to 94 bits, as three words
+struct Bits96 {
+  uint32_t w[3];
+};
+__device__ __forceinline__ Bits96 to_digits96(double v, int E) {
+  const long long bits = __double_as_longlong(v);
+  const int ev = (int)((bits >> 52) & 0x7ff);
+  unsigned long long m = bits & 0xfffffffffffffLL;
+  if (ev) m |= 1ULL << 52;
+  const int sh = 41 - (E - (ev ? ev : 1));  // m < 2^53 -> below 2^94
+  unsigned long long lo;
+  uint32_t hi = 0;
+  if (sh >= 0) {
+    lo = m << sh;
+    if (sh > 0) hi = (uint32_t)(m >> (64 - sh));
+  } else {
+    lo = -sh < 60 ? (m + (1ULL << (-sh - 1))) >> -sh : 0;
+  }
+  if (bits < 0) {
+    lo = 0 - lo;
+    hi = ~hi + (lo == 0);
+  }
+  const unsigned long long b = lo + 0x8080808080808080ull;
+  hi += 0x80808080u + (b < lo);
+  return {{(uint32_t)b, (uint32_t)(b >> 32), hi}};
 }
 
 // byte j of a and b as the two low halves' digits
@@ -327,6 +361,101 @@ __device__ __noinline__ Tile8<S> digits_tile8(const uint4* Af, const short* __re
   return tile8_products<S>(Af, er, Bf, rows, kt_n, mt, lane, E);
 }
 
+// ---- eight columns, 94-bit operands ---------------------------------------------
+// For the single products y = S v, whose every entry is a result of its own: T_e's
+// rows span up to 2^30 and more (slots of the far face against the near ones), so
+// an entry can be that much smaller than row maximum times column maximum, and
+// 62 bits relative to those left it 25 bits or fewer.  With rows that span at most
+// 2^R the error of an entry is below that of a chain of K FMAs, K 2^-53 of its sum of
+// magnitudes, as far as R <= 35: that sum is at least 2^-R of row maximum times
+// column maximum, of which the operands lose K 2^-92 and the left-out weights, at
+// most (11 K 2^14 256^10) 2^-188, four times K 2^-90.5.
+//
+// A weight takes up to 12 products per column: K <= 80 columns add exactly in an
+// accumulator (12 * 80 * 2^14 < 2^24), so the sums of more than five k tiles are
+// taken out halfway.
+
+// value of hi 2^64 + mid 2^32 + lo (each below 2^52), times 2^s
+__device__ __forceinline__ double wide_value(long long hi, long long mid, long long lo, int s) {
+  mid += lo >> 32;
+  hi += mid >> 32;
+  unsigned long long t = ((unsigned long long)(uint32_t)mid << 32) | (uint32_t)lo;
+  const bool neg = hi < 0;
+  if (neg) {
+    t = 0 - t;
+    hi = ~hi + (t == 0);
+  }
+  double v = fma((double)hi, 0x1p64, (double)t);
+  v = neg ? -v : v;
+  return s > -1000 && s < 850 ? v * __longlong_as_double((long long)(1023 + s) << 52) : scale2(v, s);
+}
+
+__device__ __forceinline__ void pack_tile_wide(uint4* Bf, int lane, const double (&v)[4], int E) {
+  Bits96 Y[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) Y[u] = to_digits96(v[u], E);
+#pragma unroll
+  for (int j = 0; j < 12; j += 2)
+    Bf[j / 2 * 32 + lane] = make_uint4(digit_pair(Y[0].w[j / 4], Y[1].w[j / 4], j & 3), digit_pair(Y[2].w[j / 4], Y[3].w[j / 4], j & 3),
+                                       digit_pair(Y[0].w[j / 4], Y[1].w[j / 4], (j & 3) + 1),
+                                       digit_pair(Y[2].w[j / 4], Y[3].w[j / 4], (j & 3) + 1));
+}
+
+// Row tile mt of A times the packed columns, as tile8_products.
+__device__ __forceinline__ Tile8<double> tile8_wide(const uint4* Af, const short* __restrict__ er, const uint4* Bf, int rows,
+                                                    int kt_n, int mt, int lane, int E) {
+  constexpr int ND = Digits<Wide>::ND, GMIN = Digits<Wide>::GMIN, NG = Digits<Wide>::NG, H = ND / 2;
+  const int g = lane >> 2, q = lane & 3, row0 = mt * 16 + g;
+  const uint4* A = Af + (size_t)mt * kt_n * H * 32 + lane;
+  uint4 nx[H];
+  ld_frag<Wide>(nx, A, 0);
+  const int er0 = row0 < rows ? __ldg(er + row0) : 0, er1 = row0 + 8 < rows ? __ldg(er + row0 + 8) : 0;
+  long long sum[4][3] = {};  // per value: weights 0-3, 4-7, 8-11 (units of 256^GMIN, 256^4, 256^8 of it)
+  const int half = kt_n > 5 ? (kt_n + 1) / 2 : kt_n;
+#pragma unroll 1
+  for (int k0 = 0; k0 < kt_n; k0 += half) {
+    float acc[NG][4];
+#pragma unroll
+    for (int c = 0; c < NG; ++c)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) acc[c][v] = 0.f;
+#pragma unroll 1
+    for (int kt = k0; kt < min(k0 + half, kt_n); ++kt) {
+      uint4 av[H], bv[H];
+#pragma unroll
+      for (int p = 0; p < H; ++p) {
+        av[p] = nx[p];
+        bv[p] = Bf[(kt * H + p) * 32 + lane];
+      }
+      if (kt + 1 < kt_n) ld_frag<Wide>(nx, A, kt + 1);
+#pragma unroll
+      for (int i = 0; i < ND; ++i) {
+        uint32_t a[4];
+        const uint4 w = av[i / 2];
+        digit_a((i & 1) ? w.z : w.x, (i & 1) ? w.w : w.y, a);
+#pragma unroll
+        for (int j = 0; j < ND; ++j) {
+          if (i + j < GMIN) continue;
+          const uint4 b = bv[j / 2];
+          mma_16816(acc[i + j - GMIN], a, (j & 1) ? b.z : b.x, (j & 1) ? b.w : b.y);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+      for (int c = 0; c < NG; ++c) sum[v][c / 4] += (long long)__float2int_rn(acc[c][v]) << (8 * (c & 3));
+  }
+  Tile8<double> o;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const int Ec = __shfl_sync(0xffffffffu, E, 4 * (2 * q + (v & 1)));
+    // 256^11 2^(er - 94) 2^(E - 1022 - 94)
+    o.z[v] = wide_value(sum[v][2], sum[v][1], sum[v][0], (v < 2 ? er0 : er1) + Ec - 1022 + 88 - 188);
+  }
+  return o;
+}
+
 // ---- one column --------------------------------------------------------------
 // The eight mma columns are the weights: digit i of A meets digit n + GMIN - i
 // of x in column n, so the digits of A share one accumulator tile (two, by
@@ -426,6 +555,20 @@ __device__ __noinline__ S digits_tile1(const uint4* Af, const short* __restrict_
   return digits_short(q < 2 ? got : w[1], q < 2 ? w[0] : got, err, E, S(0));
 }
 
+// v 2^sh rounded to an integer (below 2^62, or 2^94 in 128 bits)
+template <typename U>
+inline U to_fixed(double v, int sh) {
+  if constexpr (sizeof(U) == 8) {
+    return (U)std::llrint(std::ldexp(v, sh));
+  } else {
+    int e = 0;
+    const double m = std::frexp(v, &e);  // |v| 2^sh = |m| 2^(e + sh)
+    const int up = e + sh - 53;          // places that 53 bits of m move up
+    if (up <= 0) return (U)(__int128)std::llrint(std::ldexp(m, e + sh));
+    return (U)((__int128)std::llrint(std::ldexp(m, 53)) << up);
+  }
+}
+
 // Packs count row-major rows x cols matrices: fragments (digit_words each) and
 // row exponents (rows each, within +-400: the results' exponents are formed
 // without checks).  A row with an Inf or NaN, or above 2^400, is marked.
@@ -435,11 +578,13 @@ void pack_digits(const double* A, int rows, int cols, size_t count, std::vector<
   const int mt_n = digit_tiles(rows), kt_n = digit_tiles(cols);
   frag->assign(count * digit_words<S>(rows, cols), make_uint4(0, 0, 0, 0));
   er->assign(count * rows, 0);
-  constexpr uint64_t kBias = ND == 8 ? 0x8080808080808080ull : 0x80808080ull;
+  using U = typename std::conditional<(ND > 8), unsigned __int128, uint64_t>::type;
+  U kBias = 0;
+  for (int i = 0; i < ND; ++i) kBias |= (U)0x80 << (8 * i);
 #pragma omp parallel for schedule(static) if (count > 16)
   for (long long c = 0; c < (long long)count; ++c) {
     const double* a = A + c * rows * cols;
-    std::vector<uint64_t> Y((size_t)mt_n * 16 * kt_n * 16, kBias);
+    std::vector<U> Y((size_t)mt_n * 16 * kt_n * 16, kBias);
     for (int r = 0; r < rows; ++r) {
       double mx = 0;
       bool ok = true;
@@ -454,7 +599,7 @@ void pack_digits(const double* A, int rows, int cols, size_t count, std::vector<
       (*er)[c * rows + r] = ok ? (short)e : kBadRow;
       if (!ok) continue;
       for (int k = 0; k < cols; ++k)
-        Y[(size_t)r * kt_n * 16 + k] = kBias + (uint64_t)std::llrint(std::ldexp(a[(size_t)r * cols + k], B - e));
+        Y[(size_t)r * kt_n * 16 + k] = kBias + to_fixed<U>(a[(size_t)r * cols + k], B - e);
     }
     uint4* f = frag->data() + c * digit_words<S>(rows, cols);
     for (int mt = 0; mt < mt_n; ++mt)
@@ -467,7 +612,7 @@ void pack_digits(const double* A, int rows, int cols, size_t count, std::vector<
               w[h] = 0;
               for (int b = 0; b < 4; ++b) {
                 const int row = mt * 16 + g + 8 * (b / 2), col = kt * 16 + 2 * q + (b % 2) + 8 * (h % 2);
-                const uint64_t y = Y[(size_t)row * kt_n * 16 + col];
+                const U y = Y[(size_t)row * kt_n * 16 + col];
                 w[h] |= (uint32_t)((y >> (8 * (2 * p + h / 2))) & 0xff) << (8 * b);
               }
             }

@@ -829,9 +829,11 @@ cudaError_t launch_schur_warp(const ElemMeta<S>* tab, long long nelem, const S* 
 // 16 rows of T_c: the warps cut the slot vectors into digits together (shared
 // memory), each then runs its row tile; T_c's digits come from L1.  Many small
 // CTAs per SM: a row tile is a chain of loads and dependent products.
-// Bound by that chain, not by HBM: 96 x 96 elements, n = 24, FP64 34.8 us (14.8 MB
-// of vectors are 2.2 us; 222 us with FP64 FMA on 64 elements per CTA, 160 us by
-// per-element matrices from HBM); 128 x 128, n = 16, FP32 18.3 us (24.6 and 59.4).
+// Bound by that chain, not by HBM: 96 x 96 elements, n = 24, FP64 54 us back to back
+// (14.8 MB of vectors are 2.2 us; 222 us with FP64 FMA on 64 elements per CTA,
+// 160 us by per-element matrices from HBM; 35 us with the solves' eight digits, whose
+// small entries lose accuracy); 128 x 128, n = 16, FP32 33 us (24.6 and 59.4; 18 in
+// four digits).
 constexpr int kClassTile = 8;
 
 // one entry of T_e v on an element whose v has an Inf or NaN, which have no
@@ -844,10 +846,20 @@ __device__ __noinline__ S plain_row(const S* __restrict__ row, const S* v, int M
   return z;
 }
 
+// Digits of the class apply: FP64 vectors in twelve (tile8_wide), FP32 vectors in
+// the eight of FP64 operands: an FP32 entry then keeps its accuracy as far as
+// T_e's rows span at most 2^33 (the left-out weights are K 2^-57 of row maximum
+// times column maximum, an FP32 chain K 2^-24 of its sum of magnitudes).
 template <typename S>
-__global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
+using ClassDigits = typename std::conditional<sizeof(S) == 4, double, Wide>::type;
+template <typename S>
+constexpr double kClassSpan = sizeof(S) == 4 ? 0x1p33 : 0x1p35;
+
+template <typename S, int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads <= 192 ? 2 : 1) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
                                                      const short* __restrict__ Texp, const int* __restrict__ tiles,
                                                      const int* __restrict__ elems, const S* __restrict__ T, const S* v, S* y) {
+  using D = ClassDigits<S>;
   extern __shared__ __align__(16) unsigned char raw[];
   const int M = g.M, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cls = tiles[3 * blockIdx.x], start = tiles[3 * blockIdx.x + 1], cnt = tiles[3 * blockIdx.x + 2];
@@ -859,17 +871,17 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
   const int gc = lane >> 2, q = lane & 3;
   const int ec = __ldg(el + min(gc, cnt - 1));
   const S* vm = v + (size_t)ec * M;
-  constexpr int kNonFinite = sizeof(S) == 4 ? 0xff : 0x7ff;  // exponent field of Inf and NaN
-  S x[4];
+  constexpr int kNonFinite = 0x7ff;  // exponent field of Inf and NaN
+  double x[4];
   int E = 1;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int k = warp * 16 + 2 * q + (u & 1) + 8 * (u >> 1);
-    const S r = (gc < cnt && k < M) ? __ldg(vm + k) : S(0);
+    const double r = (gc < cnt && k < M) ? (double)__ldg(vm + k) : 0.0;
     const int Er = exp_field(r);
     // slots on the physical boundary meet zero columns: they must not set the scale
     const bool on = k < M && dev_neighbour(g, ec, k / g.n) >= 0;
-    x[u] = on ? r : S(0);
+    x[u] = on ? r : 0.0;
     if (on || Er == kNonFinite) E = max(E, Er);
   }
   // outputs of the warp's row tile: facing slots and what they hold
@@ -894,18 +906,26 @@ __global__ void __launch_bounds__(256, 2) k_schur_class(DevGeo g, const uint4* _
   if (q == 0) atomicMax(Emax + gc, E);
   __syncthreads();
   E = Emax[gc];
-  pack_tile<S>(Bf, warp, lane, x, E);
-  __syncthreads();
-  const Tile8<S> t = tile8_products<S>(Tdig + (size_t)cls * digit_words<S>(M, M), Texp + (size_t)cls * M, Bf, M, kt_n,
-                                       warp, lane, E);
+  const uint4* A = Tdig + (size_t)cls * digit_words<D>(M, M);
+  const short* er = Texp + (size_t)cls * M;
+  Tile8<double> t;
+  if constexpr (sizeof(S) == 4) {
+    pack_tile<double>(Bf, warp, lane, x, E);
+    __syncthreads();
+    t = tile8_products<double>(A, er, Bf, M, kt_n, warp, lane, E);
+  } else {
+    pack_tile_wide(Bf + warp * (Digits<Wide>::ND / 2) * 32, lane, x, E);
+    __syncthreads();
+    t = tile8_wide(A, er, Bf, M, kt_n, warp, lane, E);
+  }
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     if (sl[u] < 0) continue;
     const int r = warp * 16 + gc + 8 * (u >> 1), c = 2 * q + (u & 1);
-    S z = t.z[u];
+    double z = t.z[u];
     if (Emax[c] == kNonFinite && push[u])
-      z = plain_row(T + (size_t)__ldg(el + c) * M * M + r, v + (size_t)__ldg(el + c) * M, M);
-    y[sl[u]] = push[u] ? vf[u] + z : vf[u];
+      z = (double)plain_row(T + (size_t)__ldg(el + c) * M * M + r, v + (size_t)__ldg(el + c) * M, M);
+    y[sl[u]] = push[u] ? (S)((double)vf[u] + z) : vf[u];
   }
 }
 
@@ -930,7 +950,11 @@ struct smpm_handle_s {
   bool factored = false;
   bool op_factored = false;  // operator-only factor step (SMPM_FLAG_OPERATOR_ONLY): S can be applied
   // element classes (face-type masks) for the class-shared apply
-  int ncls = 0, ntiles = 0, cls_ok = 0;  // cls_ok: the class matrices are packed
+  int ncls = 0, ntiles = 0;
+  // T_e per class in the digits of the class apply (null: not packed, see
+  // class_digits) and its row exponents; the FP32 one may be dig.T
+  uint4 *clsT64 = nullptr, *clsT32 = nullptr;
+  short *clsTe64 = nullptr, *clsTe32 = nullptr;
   int apply_kind = 0;                     // kernel of smpm_apply_schur(32): SMPM_APPLY_*
   // packed digits (smpm_digits.cuh) of one T_e per class, G_b and the four X_F
   // per block class, their row exponents, and the class of each element / block
@@ -1192,36 +1216,53 @@ bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
     case SMPM_APPLY_AUTO: case SMPM_APPLY_STREAM: return true;
     case SMPM_APPLY_WARP: case SMPM_APPLY_WARP2: case SMPM_APPLY_WARP4:
       return h->g.M <= 96 && (fp32 ? h->dtab32 != nullptr : h->dtab64 != nullptr);
-    case SMPM_APPLY_CLASS: return h->cls_ok && (fp32 ? h->dig32.T != nullptr : h->dig.T != nullptr);
+    case SMPM_APPLY_CLASS: return fp32 ? h->dT32 != nullptr : h->dT != nullptr;
     default: return false;
   }
 }
 
+// Whether the class apply's tiles of eight elements are filled to a fifth on average.
+bool class_tiles_pay(smpm_handle h) { return (long long)h->ntiles * kClassTile <= 5 * h->g.nel; }
+
+// Whether SMPM_APPLY_AUTO takes the class apply: its matrices are packed
+// (class_span), its tiles fill, and it is the faster one.  Measured, back to back,
+// FP64 / FP32 in us, best per-element kernel (T_e in L2 where it fits) against the
+// class kernel, which takes 9.5 us for M <= 64 and 14.5 / 12.3 beyond until its CTAs
+// fill the SMs several times:
+//   FP64: 16x16, n = 24 12.7 / 14.5; 20x24, n = 24 14.5 / 14.5; 32x32, n = 5 9.5 / 9.7,
+//     n = 16 16.8 / 9.8, n = 24 24.8 / 14.5; 96x96, n = 24 160 / 54; 128x128, n = 16 183 / 46:
+//     from four elements per SM on.
+//   FP32: 32x32, n = 24 9.6 / 12.4, n = 32 22.8 / 12.7; 48x48, n = 24 14.7 / 14.5; 96x96,
+//     n = 11 14.8 / 18.8, n = 24 74 / 39; 128x128, n = 8 17.6 / 18.8, n = 11 39 / 27, n = 16 60 / 33:
+//     where the matrices leave L2 (three quarters of it), or M > 96, whose
+//     per-element kernel stages them in shared memory.
+template <typename S>
+bool class_pays(smpm_handle h, int sms, int l2) {
+  if (!class_tiles_pay(h)) return false;
+  if (sizeof(S) == 8) return h->g.nel >= 4LL * sms;
+  return (double)h->g.nel * h->g.M * h->g.M * sizeof(S) >= 0.75 * l2 || (h->g.M > 96 && h->g.nel >= 4LL * sms);
+}
+
 // y = S v with the handle's apply kernel.  SMPM_APPLY_AUTO: the class-shared
-// products where the elements fall into few enough classes that the tiles of
-// eight are filled to a fifth on average (any uniform grid from 4x4 on;
-// measured, FP64 / FP32 in us, best per-element kernel against the class
-// kernel: 4x59, n = 21 14.0 / 9.3 against 10.8 / 8.4; 32x32, n = 24 26.8 / 12.1
-// against 11.6 / 8.3; 96x96, n = 24 162 / 76 against 35 / 20; 128x128, n = 16
-// 184 / 61 against 28 / 18).  Graded grids, mostly one element to a class: one
-// warp per element, register-streamed from global memory, for M <= 96 -- 1, 2
-// or 4 warps per element by the element count -- else the shared-memory stream.
+// products where they pay (class_pays), else one warp per element, register-streamed
+// from global memory, for M <= 96 -- 1, 2 or 4 warps per element by the element
+// count -- and the shared-memory stream beyond.  SMPM_APPLY_CLASS without packed
+// matrices runs as AUTO.
 template <typename S>
 smpm_status launch_schur_kind(smpm_handle h, int kind, const S* v, S* y, cudaStream_t st) {
   const bool fp32 = sizeof(S) == 4;
   const ElemMeta<S>* tab = reinterpret_cast<const ElemMeta<S>*>(fp32 ? (const void*)h->dtab32 : (const void*)h->dtab64);
   const S* T = reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT);
-  if (kind == SMPM_APPLY_AUTO && apply_kind_ok(h, SMPM_APPLY_CLASS, fp32) &&
-      (long long)h->ntiles * kClassTile <= 5 * h->g.nel)
-    kind = SMPM_APPLY_CLASS;
-  if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
-  if (kind == SMPM_APPLY_STREAM) return launch_schur_stream<S>(h, T, v, y, st);
-  if (kind == SMPM_APPLY_CLASS) {
-    return launch_schur_class<S>(h, v, y, st);
-  }
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, l2 = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  CU(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+  const bool packed = fp32 ? h->clsT32 != nullptr : h->clsT64 != nullptr;
+  if (kind == SMPM_APPLY_AUTO && packed && class_pays<S>(h, sms, l2)) kind = SMPM_APPLY_CLASS;
+  if (kind == SMPM_APPLY_CLASS && !packed) kind = SMPM_APPLY_AUTO;
+  if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
+  if (kind == SMPM_APPLY_STREAM) return launch_schur_stream<S>(h, T, v, y, st);
+  if (kind == SMPM_APPLY_CLASS) return launch_schur_class<S>(h, v, y, st);
   const long long ne = h->g.nel;
   if (kind == -1) {
     CU(launch_schur_warp<S>(tab, ne, v, y, sms, st));
@@ -3095,6 +3136,33 @@ smpm_status upload_solve_digits(smpm_handle h, cudaStream_t st) {
   return SMPM_OK;
 }
 
+// Largest ratio of two magnitudes within a row of the classes' T_e, physical-boundary
+// rows and columns (zero) left out; infinite with a zero or a non-finite entry among
+// them, or one beyond the exponents of pack_digits.  first: an element of each class.
+double class_span(const Geometry& g, const std::vector<double>& Tcls, const std::vector<int>& first) {
+  const int n = g.n, M = g.M;
+  double span = 1;
+  for (size_t c = 0; c < first.size(); ++c)
+    for (int r = 0; r < M; ++r) {
+      if (g.neighbour(first[c], r / n) < 0) continue;
+      const double* row = Tcls.data() + (c * M + r) * M;
+      double lo = INFINITY, hi = 0;
+      for (int k = 0; k < M; ++k) {
+        if (g.neighbour(first[c], k / n) < 0) continue;
+        const double a = std::fabs(row[k]);
+        if (!(a > 0x1p-400 && a < 0x1p400)) return INFINITY;
+        lo = std::min(lo, a);
+        hi = std::max(hi, a);
+      }
+      span = std::max(span, hi / lo);
+    }
+  return span;
+}
+
+// The class apply can be asked for on grids of few classes (any uniform grid)
+// even where its tiles don't fill.
+constexpr int kClassFew = 16;
+
 // Class tables of the class-shared apply: one T per T class of the factor
 // step (face types, and on a graded grid the sizes; the copies of T_e within
 // a class are identical), tiles of kClassTile elements.
@@ -3132,11 +3200,22 @@ smpm_status upload_classes(smpm_handle h, cudaStream_t st) {
   if ((s = upload(h, &h->dtiles, tiles, st)) || (s = upload(h, &h->dclsel, sel, st)) ||
       (s = upload(h, &h->dtcls, cidx, st)))
     return s;
-  if ((s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
-  if (h->opts.precision == 1 && (s = upload_digits<float>(h, Tcls, g.M, &h->dig32.T, &h->dig32.Te, st))) return s;
   h->ncls = (int)members.size();
   h->ntiles = (int)(tiles.size() / 3);
-  h->cls_ok = 1;
+  const bool mixed = h->opts.precision == 1;
+  if (!h->f.operator_only) {  // the solve kernels' copies
+    if ((s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
+    if (mixed && (s = upload_digits<float>(h, Tcls, g.M, &h->dig32.T, &h->dig32.Te, st))) return s;
+  }
+  // the class apply's: where it can be taken, and the digits hold the rows' span
+  if (!class_tiles_pay(h) && h->ncls > kClassFew) return SMPM_OK;
+  const double span = class_span(g, Tcls, first);
+  if (span <= kClassSpan<double> && (s = upload_digits<Wide>(h, Tcls, g.M, &h->clsT64, &h->clsTe64, st))) return s;
+  if (mixed && span <= kClassSpan<float>) {
+    if (!h->dig.T && (s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
+    h->clsT32 = h->dig.T;
+    h->clsTe32 = h->dig.Te;
+  }
   return SMPM_OK;
 }
 
@@ -3633,10 +3712,11 @@ namespace {
 
 template <typename S>
 smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st) {
-  if (!h->cls_ok) return fail(SMPM_EINVAL, "the class-shared apply needs its packed matrices and tile in shared memory");
   const bool fp32 = sizeof(S) == 4;
-  k_schur_class<S><<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), digit_bwords<S>(h->g.M) * sizeof(uint4), st>>>(
-      h->dg, fp32 ? h->dig32.T : h->dig.T, fp32 ? h->dig32.Te : h->dig.Te, h->dtiles, h->dclsel,
+  // two CTAs per SM need at most 168 registers a thread, which M <= 96 leaves
+  const auto k = h->g.M <= 96 ? k_schur_class<S, 192> : k_schur_class<S, 256>;
+  k<<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), digit_bwords<ClassDigits<S>>(h->g.M) * sizeof(uint4), st>>>(
+      h->dg, fp32 ? h->clsT32 : h->clsT64, fp32 ? h->clsTe32 : h->clsTe64, h->dtiles, h->dclsel,
       reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT), v, y);
   CHECK_LAUNCH();
   return SMPM_OK;
@@ -3649,7 +3729,7 @@ extern "C" {
 smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, void* stream) try {
   NEED_OPERATOR();
   if (!v || !y) return fail(SMPM_EINVAL, "null vector");
-  return launch_schur_class<double>(h, v, y, as_stream(stream));
+  return launch_schur_kind<double>(h, SMPM_APPLY_CLASS, v, y, as_stream(stream));
 } catch (...) {
   return host_exception();
 }
@@ -3658,7 +3738,7 @@ smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, vo
   NEED_OPERATOR();
   if (!v || !y) return fail(SMPM_EINVAL, "null vector");
   if (!h->dT32) return fail(SMPM_ESTATE, "FP32 factors exist only after schur_factor with precision = 1");
-  return launch_schur_class<float>(h, v, y, as_stream(stream));
+  return launch_schur_kind<float>(h, SMPM_APPLY_CLASS, v, y, as_stream(stream));
 } catch (...) {
   return host_exception();
 }

@@ -80,3 +80,63 @@ def test_apply_is_blind_to_boundary_slots(built, mx, my, n, big):
             got = applied(g, kind, dev(np.where(face, v, b * v), dtype))
             assert np.array_equal(got[face], plain[face]), kind
             assert np.array_equal(got[~face], dev(b * v, dtype).double().cpu().numpy()[~face])
+
+
+def own_bound(T, v, mx, my, n, u):
+    """(M + 2) u sum |T_e||v_e|, the error of a chain of M FMAs and the addition to
+    v, at the facing slots that the products are pushed to."""
+    M, e = 4 * n, np.arange(mx * my)
+    own = (M + 2) * u * np.einsum("erk,ek->er", np.abs(T), np.abs(v))
+    out = np.zeros_like(own)
+    ix, iy = e % mx, e // mx
+    for F, (dx, dy) in enumerate(((-1, 0), (1, 0), (0, -1), (0, 1))):
+        ok = (0 <= ix + dx) & (ix + dx < mx) & (0 <= iy + dy) & (iy + dy < my)
+        f2 = (F ^ 1) * n
+        out[(e + dx + mx * dy)[ok], f2:f2 + n] = own[e[ok], F * n:(F + 1) * n]
+    return out
+
+
+def exact_apply(T, v, mx, my, n):
+    """S v in extended precision (np.longdouble where it is longer than a double)."""
+    L = np.longdouble
+    M, e = 4 * n, np.arange(mx * my)
+    z = np.einsum("erk,ek->er", T.astype(L), v.astype(L))
+    y = v.astype(L).copy()
+    ix, iy = e % mx, e // mx
+    for F, (dx, dy) in enumerate(((-1, 0), (1, 0), (0, -1), (0, 1))):
+        ok = (0 <= ix + dx) & (ix + dx < mx) & (0 <= iy + dy) & (iy + dy < my)
+        f2 = (F ^ 1) * n
+        y[(e + dx + mx * dy)[ok], f2:f2 + n] += z[e[ok], F * n:(F + 1) * n]
+    return y
+
+
+# square and stretched elements (rows of T_e spanning up to 2^38, where the digits
+# no longer hold it), n up to the largest, three k tiles and six and eight
+@pytest.mark.parametrize("mx,my,n,Lx", [(4, 5, 5, 1.0), (4, 4, 11, 1.0), (5, 4, 16, 1.0), (4, 4, 24, 1.0), (3, 4, 32, 1.0),
+                                        (4, 4, 16, 8.0), (4, 4, 24, 8.0)])
+def test_apply_keeps_every_entry(built, mx, my, n, Lx):
+    """Every entry of S v within the rounding error of a chain of FMAs, relative to its
+    own sum of magnitudes: for a unit value on one slot of each element, and for
+    entries that span 2^40."""
+    g = Grid(mx, my, n, Lx, 1.0)
+    g.factor(precision=1)
+    M, nel = 4 * n, mx * my
+    T = g.host_factor("T").reshape(nel, M, M)
+    rng = np.random.default_rng(n)
+    vs = []
+    for k in range(0, M, 1 if n <= 16 else 5):
+        v = np.zeros((nel, M))
+        v[:, k] = 1.0
+        vs.append(v)
+    for _ in range(8):
+        vs.append(rng.choice([-1.0, 1.0], (nel, M)) * np.exp2(rng.uniform(-40, 0, (nel, M))))
+    for dtype, u in ((torch.float64, 2.0 ** -53), (torch.float32, 2.0 ** -24)):
+        for kind in (B.APPLY_AUTO, B.APPLY_CLASS):
+            for v in vs:
+                vt = dev(v.ravel(), dtype)
+                vr = vt.double().cpu().numpy().reshape(nel, M)
+                got = applied(g, kind, vt).reshape(nel, M)
+                ref = exact_apply(T, vr, mx, my, n)
+                bound = own_bound(T, vr, mx, my, n, u) + u * np.abs(ref).astype(float) + 1e-44 * (u > 1e-10)
+                err = np.abs(got - ref).astype(float)
+                assert np.all(err <= bound), (kind, dtype, float(np.max(err / np.maximum(bound, 1e-300))))
