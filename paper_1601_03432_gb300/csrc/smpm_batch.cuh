@@ -49,6 +49,7 @@ struct TaskReport {
   double res2, bsn2;            // ||b_S - S x_S||^2, ||b_S||^2
   unsigned long long t_begin, t_end;  // global timer (ns) at the task's start and end on its team's first CTA
   int team, breakdown;  // breakdown: an FP64 solve ended on an Arnoldi breakdown before tol
+  int nan, pad_;        // nan: an FP64 solve met a NaN or Inf
 };
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -147,6 +148,7 @@ __device__ __noinline__ int batch_group(BatchTask& T, unsigned char* smraw, unsi
       r.restarts = cs.cycles > 1 ? cs.cycles - 1 : 0;
       r.converged = cs.converged;
       r.breakdown = cs.breakdown;
+      r.nan = cs.nan;
       r.gmres_num = cs.resid;
       r.gmres_den = cs.beta0;
     } else {

@@ -1223,9 +1223,15 @@ __device__ SMPM_BODY bool gmres_body(const GmresArgs<S>& a, unsigned char* smraw
       __syncthreads();
       GM_TRACE(11);
       ++total;
-      // beta / ||z|| <= tolabs (an exact breakdown: residual 0)
+      // beta / ||z|| <= tolabs (an exact breakdown: residual 0; ||z||^2 beyond the
+      // range: below any tolerance).  After a NaN there is no residual to report.
       const double zz = s.misc[6];
-      if (!isfinite(zz) || !isfinite(s.misc[4])) { nan = true; ++j; break; }
+      if (isnan(zz) || !isfinite(s.misc[4])) {
+        nan = true;
+        resid = __longlong_as_double(0x7ff8000000000000LL);
+        ++j;
+        break;
+      }
       if (s.misc[4] == 0.0 || goal <= zz) { converged = true; ++j; break; }
       if (s.misc[3] != 0.0) { breakdown = true; ++j; break; }
       if (ES > kOverlapEntries) {

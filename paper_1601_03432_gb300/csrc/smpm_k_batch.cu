@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(256, 1) k_batch(const BatchTask* __restrict__ 
         r.restarts = gs->scal[7] > 1 ? (int)gs->scal[7] - 1 : 0;
         r.converged = (gs->converged || gs->beta0 == 0.0) ? 1 : 0;
         r.breakdown = gs->breakdown;
+        r.nan = gs->nan;
         r.gmres_num = gs->resid;
         r.gmres_den = gs->beta0;
       } else {

@@ -4084,7 +4084,10 @@ smpm_status smpm_batch_solve(smpm_batch b, const double* f, const double* g, dou
       R.schur_relres = t.bsn2 > 0 ? std::sqrt(t.res2 / t.bsn2) : 0.0;
       R.launches = 1;
       R.gmres_ms = b->last_ms;
-      if (!std::isfinite(R.gmres_relres) || !std::isfinite(R.schur_relres))
+      // (a norm that is NaN itself leaves its ratio above at 0)
+      const bool finite = std::isfinite(t.gmres_num) && std::isfinite(t.gmres_den) && std::isfinite(t.res2) &&
+                          std::isfinite(t.bsn2) && std::isfinite(R.gmres_relres) && std::isfinite(R.schur_relres);
+      if (t.nan || !finite)
         return fail(SMPM_ENAN, "non-finite residual in a batched solve");
       if (!t.converged && worst == SMPM_OK) worst = t.breakdown ? SMPM_EBREAKDOWN : SMPM_ENOTCONV;
       if (rep) rep[i] = R;
