@@ -286,7 +286,11 @@ smpm_status smpm_factor_host_only(smpm_handle h, const smpm_opts* o);
  * "null_iterations" (1 value), and the strips of the coarse inverse:
  * "strips_shape" (h, p, m, ns, ldn, lds, ldw; all 0 when not built),
  * "strips_N", "strips_Hs", "strips_W", "strips_z", for the adjoint system
- * "stripsa_...". */
+ * "stripsa_...".  After schur_factor also the launch shape of the one-column
+ * solve kernel, "solve_layout" (FP64) and "solve_layout32" (the FP32 inner solve
+ * of precision 1): CTAs, warps per block or element, classes of T_e and of block
+ * matrices in shared memory, entry table and basis there (0 or 1), whole block
+ * inverses, C^+ by strips, C^+ in FP64 (0 or 1); else ESTATE. */
 smpm_status smpm_host_factor(smpm_handle h, const char* name, double* out, long long count, long long* len);
 
 /* y = P v exactly as smpm_apply_deflation, for callers that cannot allocate

@@ -68,6 +68,7 @@ struct GmresArgs {
   // coarse inverse, d rows of (d rounded up to a multiple of 4) entries: FP64, or
   // its FP32 copy for the FP32 inner solves of the mixed-precision path
   const typename std::conditional<sizeof(S) == 4, float, double>::type* H;
+  const double* H64;  // FP32 solves of small grids: the FP64 inverse, used instead; else null
   S* vglob;         // kp : current basis vector (raw), exchanged between CTAs
   S* vown;          // G * (m+1) * ES : basis slices when not resident in smem
   S* t;             // kp
@@ -809,25 +810,22 @@ __device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsig
   return team_sync(a, epoch);
 }
 
-// c_hat = H c by rows: the CTA takes a contiguous range of them, c staged in
-// shared memory.  The FP32 inner solves of the mixed-precision path use the
-// FP32 copy with FP32 products and sums: an inner solve needs only a relative
-// 1e-4, and every refinement sweep recomputes the residual in FP64.
-template <typename S>
-__device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, const double* c, double* chat) {
-  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
-  T* xs = reinterpret_cast<T*>(s.cst);
+// c_hat = H c by rows: the CTA takes a contiguous range of them (own: its rows in
+// shared memory, or null), c staged in shared memory, sums in T.
+template <typename T, typename S>
+__device__ __forceinline__ void coarse_rows_in(const GmresArgs<S>& a, const T* H, const T* own, T* xs, const double* c,
+                                               double* chat) {
   const int d = (int)a.g.d, ld = (d + 3) & ~3, per = (d + a.G - 1) / a.G;
   const int r0 = min(d, team_rank(a) * per), r1 = min(d, r0 + per);
   if (r0 >= r1) return;
   for (int j = threadIdx.x; j < d + 16 / (int)sizeof(T); j += blockDim.x) xs[j] = j < d ? (T)__ldcg(c + j) : T(0);
   __syncthreads();
   auto put = [&](int r, T sum) { chat[r] = (double)sum; };
-  if (s.H) {
+  if (own) {
     row_dots<T, true>(
         r0, r1, d,
         [&](int r, const T*& row, const T*& x, int& len) {
-          row = s.H + (size_t)(r - r0) * ld;
+          row = own + (size_t)(r - r0) * ld;
           x = xs;
           len = d;
         },
@@ -836,12 +834,22 @@ __device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, 
     row_dots<T>(
         r0, r1, d,
         [&](int r, const T*& row, const T*& x, int& len) {
-          row = a.H + (size_t)r * ld;
+          row = H + (size_t)r * ld;
           x = xs;
           len = d;
         },
         put);
   }
+}
+// The FP32 inner solves of the mixed-precision path take the FP64 inverse on small
+// grids (H64), where its products are a small part of a step, and else its FP32
+// copy with FP32 products and sums: an inner solve needs only a relative 1e-4, and
+// every refinement sweep recomputes the residual in FP64.
+template <typename S>
+__device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, const double* c, double* chat) {
+  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+  if (sizeof(S) == 4 && a.H64) coarse_rows_in<double>(a, a.H64, (const double*)nullptr, s.cst, c, chat);
+  else coarse_rows_in<T>(a, a.H, s.H, reinterpret_cast<T*>(s.cst), c, chat);
 }
 
 // c_hat = C^+ c by all CTAs of the team (strips or dense rows), complete after

@@ -1430,10 +1430,18 @@ int block_pays(smpm_handle h) {
   return have && h->opts.precond != 0 && block_fits<S>(h, h->gm.nown_b);
 }
 
+// Whether the one-column FP32 inner solves of a mixed-precision handle apply the
+// coarse inverse in FP64: where its products per step and CTA are few.  At the limit,
+// d = 862 on 152 CTAs, 4,900 FP64 products a CTA; 16 x 16 elements (d = 480): 1,500.
+constexpr long long kCoarse64Max = 1LL << 17;
+bool coarse_in_fp64(smpm_handle h) {
+  return h->opts.precision == 1 && h->opts.precond == 2 && h->g.d * h->gm.grid <= kCoarse64Max;
+}
+
 // Form of the coarse solve for a solve of R columns by a.G CTAs.
 template <typename S>
 void choose_coarse(GmresArgs<S>& a, double products, int R) {
-  a.use_strips = a.precond == 2 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4);
+  a.use_strips = a.precond == 2 && !a.H64 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4);
 }
 
 DigitMats digit_mats(smpm_handle h, const smpm_handle_s::DigitSet& d) {
@@ -1505,6 +1513,7 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.skip = h->wdone;
   a.G = h->gm.grid;
   a.base = 0;
+  a.H64 = coarse_in_fp64(h) ? h->dHp : nullptr;
   a.strips = h->st32;
   a.gsep = h->wgsep;
   choose_coarse(a, h->st_products, 1);
@@ -1940,6 +1949,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
     A.a.basis_smem = 0; A.a.ES = basis_entries(g.M, h->gm.nown_b);
     A.a.trace = nullptr; A.a.trace_cap = 0; A.a.skip = nullptr; A.a.its_out = nullptr; A.a.wscr = nullptr;
     A.a.c = L.c; A.a.chat = L.chat; A.a.acc = L.acc; A.a.gsep = L.gsep;
+    A.a.H64 = nullptr;  // the lockstep kernel's coarse product is FP32's own
     choose_coarse(A.a, h->st_products, R);
     A.vs = g.kp; A.ds = g.d;
     A.cs = L.cs; A.Rh = L.Rh; A.yv = L.yv;
@@ -2328,7 +2338,7 @@ smpm_status batch_layout(smpm_batch b, const TeamPlan& plan) {
     };
     const int precond = h->opts.precond;
     auto lay_for = [&](bool wg) {
-      return mixed ? choose_layout<float>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2)
+      return mixed ? choose_layout<float>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2 && !coarse_in_fp64(h))
                    : choose_layout<double>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2);
     };
     // w, w2 move to global scratch when either the pre/post bodies or the
@@ -2593,6 +2603,7 @@ smpm_status batch_layout(smpm_batch b, const TeamPlan& plan) {
           A.a.chat = wchat;
           A.a.acc = wacc;
           A.a.gsep = wgs;
+          A.a.H64 = nullptr;  // the lockstep kernel's coarse product is FP32's own
           choose_coarse(A.a, h->st_products, R);
           lock_shape(h, A, R, L.nown_b, (size_t)budget_all);
           A.vs = g.kp;
@@ -3417,7 +3428,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       // refinement kernel, FP32 work vectors and the FP64 residual
       auto& g32 = h->gm32;
       Layout L = choose_layout<float>(g, m, gm.ES, items, no_smem, budget, gm.wg, block_pays<float>(h), gm.grid,
-                                      opts.precond == 2);
+                                      opts.precond == 2 && !coarse_in_fp64(h));
       g32.basis_smem = L.basis_smem;
       g32.W = L.W;
       g32.res_T = L.res_T;
@@ -3889,6 +3900,17 @@ smpm_status smpm_host_factor(smpm_handle h, const char* name, double* out, long 
       tmp = {(double)k.h, (double)k.p, (double)k.m, (double)k.ns, (double)k.ldn, (double)k.lds, (double)k.ldw};
       src = &tmp;
     } else return fail(SMPM_EINVAL, "unknown factor name " + nm);
+  }
+  else if (nm == "solve_layout" || nm == "solve_layout32") {  // launch shape of the one-column solve kernel
+    if (!h->factored || (nm.back() == '2' && h->opts.precision != 1))
+      return fail(SMPM_ESTATE, "no factored solve of this precision");
+    auto shape = [&](const auto& a) {
+      tmp = {(double)a.G, (double)a.W_item, (double)a.res_T, (double)a.res_G, (double)a.tab, (double)a.basis_smem,
+             (double)a.blk, (double)a.use_strips, a.H64 || sizeof(*a.H) == 8 ? 1.0 : 0.0};
+    };
+    if (nm.back() == '2') shape(gmres_args32(h, h->opts.tol));
+    else shape(gmres_args(h, h->opts.tol));
+    src = &tmp;
   }
   else if (nm == "black") { tmp.assign(f.black.begin(), f.black.end()); src = &tmp; }
   else if (nm == "null_iterations") { tmp.assign(1, (double)f.null_iterations); src = &tmp; }

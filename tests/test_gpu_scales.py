@@ -140,3 +140,19 @@ def test_apply_keeps_every_entry(built, mx, my, n, Lx):
                 bound = own_bound(T, vr, mx, my, n, u) + u * np.abs(ref).astype(float) + 1e-44 * (u > 1e-10)
                 err = np.abs(got - ref).astype(float)
                 assert np.all(err <= bound), (kind, dtype, float(np.max(err / np.maximum(bound, 1e-300))))
+
+
+@pytest.mark.parametrize("mx,my,n,fp64", [(4, 3, 6, 1), (16, 16, 5, 1), (24, 20, 4, 0)])
+def test_mixed_solves_of_small_grids_keep_the_fp64_coarse_inverse(built, mx, my, n, fp64):
+    """Up to 2^17 entries of c_hat times CTAs the FP32 inner solves apply C^+ in FP64,
+    beyond it its FP32 copy; the solution is the FP64 solve's."""
+    g = Grid(mx, my, n)
+    g.factor(tol=1e-11)
+    f = dev(inputs.white_noise(g.r, 3))
+    u, um = torch.empty_like(f), torch.empty_like(f)
+    g.solve(f, u)
+    g.factor(tol=1e-11, precision=1)
+    ctas, coarse64 = (int(g.host_factor("solve_layout32")[i]) for i in (0, 8))
+    assert coarse64 == fp64 == int(g.d * ctas <= 1 << 17)
+    assert g.solve(f, um)[0]["converged"] == 1
+    assert (u - um).norm() <= 1e-8 * u.norm()
