@@ -73,14 +73,13 @@ typedef struct {
 
 /* flags: keep the GMRES kernel's matrices, tables and Krylov basis in global
  * memory even when they fit in shared memory (the large-grid layout, selectable
- * for testing).  STREAM_MATRICES and WARP_ELEMS are accepted and change
- * nothing: the matrices are packed once per element or block class and read
- * from L1 and L2, and a group of warps per block or element is sized by the
- * number a CTA owns. */
+ * for testing); read the operator matrices from L2 in every phase even when the
+ * most used ones would fit in shared memory (likewise). */
 #define SMPM_FLAG_NO_SMEM_RESIDENCY 1
 #define SMPM_FLAG_STREAM_MATRICES 2
 #define SMPM_FLAG_ADJOINT 4        /* also build the transposed system for schur_solve_adjoint */
-#define SMPM_FLAG_WARP_ELEMS 8
+#define SMPM_FLAG_WARP_ELEMS 8     /* one warp per block / element in the GMRES phases even when few
+                                      are owned per CTA (as far as their scratch fits; for testing) */
 #define SMPM_FLAG_ROBIN_LITERAL 16 /* Robin flux R = I + n.grad with identity weight p_F = 1 on every face
                                       (the literal form of Sec. 1.2); robin_scale is then unused */
 #define SMPM_FLAG_NO_LOCKSTEP 32    /* solve several right-hand sides one after another instead of in

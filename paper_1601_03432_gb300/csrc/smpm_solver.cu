@@ -1357,14 +1357,18 @@ struct Layout {
   size_t smem;
 };
 
+// flags: SMPM_FLAG_NO_SMEM_RESIDENCY (nothing resident), STREAM_MATRICES (no
+// matrices resident), WARP_ELEMS (one warp per item, blocks in stages: eight whole
+// inverses' vectors would not fit at n = 32).
 template <typename S>
-Layout choose_layout(const Geometry& g, int m, int ES, int items, bool no_smem, size_t budget, bool w_global, int blk, int G, bool rows_H) {
+Layout choose_layout(const Geometry& g, int m, int ES, int items, int flags, size_t budget, bool w_global, int blk, int G, bool rows_H) {
   Layout L;
-  L.blk = blk;
-  L.W = item_warps(items);
+  L.blk = (flags & SMPM_FLAG_WARP_ELEMS) ? 0 : blk;
+  L.W = (flags & SMPM_FLAG_WARP_ELEMS) ? 1 : item_warps(items);
+  const bool no_smem = flags & SMPM_FLAG_NO_SMEM_RESIDENCY, mats = !(flags & SMPM_FLAG_STREAM_MATRICES);
   L.basis_smem = L.res_T = L.res_G = L.tab = L.res_H = 0;
   auto need = [&] {
-    return gmres_smem_bytes<S>(m, g.M, g.n, ES, L.W, L.basis_smem, g.d, w_global, L.res_T, L.res_G, blk,
+    return gmres_smem_bytes<S>(m, g.M, g.n, ES, L.W, L.basis_smem, g.d, w_global, L.res_T, L.res_G, L.blk,
                                L.tab, L.res_H ? coarse_row_bytes<S>(g.d, G) : 0);
   };
   while (L.W < kGmresThreads / 32 && need() > budget) L.W *= 2;
@@ -1374,8 +1378,8 @@ Layout choose_layout(const Geometry& g, int m, int ES, int items, bool no_smem, 
       v = to;
       if (need() > budget) v = old;
     };
-    take(L.res_T, 1);
-    take(L.res_G, 1);
+    if (mats) take(L.res_T, 1);
+    if (mats) take(L.res_G, 1);
     take(L.tab, 1);
     take(L.basis_smem, 1);
     if (rows_H) take(L.res_H, 1);
@@ -2338,8 +2342,8 @@ smpm_status batch_layout(smpm_batch b, const TeamPlan& plan) {
     };
     const int precond = h->opts.precond;
     auto lay_for = [&](bool wg) {
-      return mixed ? choose_layout<float>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2 && !coarse_in_fp64(h))
-                   : choose_layout<double>(g, m, L.ES, items, false, budget, wg, 0, T, precond == 2);
+      return mixed ? choose_layout<float>(g, m, L.ES, items, 0, budget, wg, 0, T, precond == 2 && !coarse_in_fp64(h))
+                   : choose_layout<double>(g, m, L.ES, items, 0, budget, wg, 0, T, precond == 2);
     };
     // w, w2 move to global scratch when either the pre/post bodies or the
     // GMRES body (with its per-warp scratch) would not fit beside them
@@ -3394,20 +3398,19 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
     gm.nown_w = (nw + gm.grid - 1) / gm.grid;
     gm.ES = basis_entries(g.M, gm.nown_b);
     const int m = opts.restart;
-    const bool no_smem = (opts.flags & SMPM_FLAG_NO_SMEM_RESIDENCY) != 0;
     const int items = std::max(gm.nown_b, gm.nown_w);
     const size_t budget = (size_t)smem_optin - 2048;  // static shared memory: staged arguments
     // w and w2 of the bodies move to global memory on grids so large that the
     // coarse vector leaves no room for them
     gm.smem_pp = prepost_shape(g, m, gm.ES, items, gm.grid, budget, false, &gm.W_pp, &gm.W_fd);
-    gm.wg = gm.smem_pp > budget || choose_layout<double>(g, m, gm.ES, items, true, budget, false, 0, gm.grid, false).smem > budget;
+    gm.wg = gm.smem_pp > budget || choose_layout<double>(g, m, gm.ES, items, SMPM_FLAG_NO_SMEM_RESIDENCY, budget, false, 0, gm.grid, false).smem > budget;
     if (gm.wg) {
       gm.smem_pp = prepost_shape(g, m, gm.ES, items, gm.grid, budget, true, &gm.W_pp, &gm.W_fd);
       if ((s = dalloc(h, &h->wscr, (size_t)gm.grid * gm.ES))) return s;
       if (opts.precision == 1 && (s = dalloc(h, &h->wscr32, (size_t)gm.grid * gm.ES))) return s;
     }
     {
-      Layout L = choose_layout<double>(g, m, gm.ES, items, no_smem, budget, gm.wg, block_pays<double>(h), gm.grid,
+      Layout L = choose_layout<double>(g, m, gm.ES, items, opts.flags, budget, gm.wg, block_pays<double>(h), gm.grid,
                                        opts.precond == 2);
       gm.basis_smem = L.basis_smem;
       gm.W = L.W;
@@ -3427,7 +3430,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       // FP32 inner GMRES: FP32 copies of the operator, its own layout, the
       // refinement kernel, FP32 work vectors and the FP64 residual
       auto& g32 = h->gm32;
-      Layout L = choose_layout<float>(g, m, gm.ES, items, no_smem, budget, gm.wg, block_pays<float>(h), gm.grid,
+      Layout L = choose_layout<float>(g, m, gm.ES, items, opts.flags, budget, gm.wg, block_pays<float>(h), gm.grid,
                                       opts.precond == 2 && !coarse_in_fp64(h));
       g32.basis_smem = L.basis_smem;
       g32.W = L.W;
