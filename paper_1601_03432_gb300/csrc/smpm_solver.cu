@@ -272,12 +272,21 @@ __global__ void k_zt(DevGeo g, const S* __restrict__ v, double* c) {
   c[j] = s;
 }
 
-// out = H c (FP64, d x d, warp per row).
+// entries per row of the coarse inverses on the device: d rounded up to whole
+// groups of four, zeros behind (16-byte loads of the solve kernels)
+__host__ __device__ __forceinline__ long long coarse_ld(long long d) { return (d + 3) & ~3LL; }
+
+__global__ void k_round32(const double* __restrict__ src, float* __restrict__ dst, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    dst[i] = (float)src[i];
+}
+
+// out = H c (FP64, d rows, warp per row).
 __global__ void k_coarse(const double* __restrict__ H, const double* __restrict__ c, double* out, int d) {
   const int lane = threadIdx.x & 31;
   const long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
   if (row >= d) return;
-  const double* h = H + row * (long long)d;
+  const double* h = H + row * coarse_ld(d);
   double acc = 0;
   for (int j = lane; j < d; j += 32) acc += __ldg(h + j) * __ldg(c + j);
   acc = warp_sum(acc);
@@ -1014,7 +1023,7 @@ struct smpm_handle_s {
   } gm32;
   double *wacc8 = nullptr, *wxs = nullptr, *dZtuS = nullptr;
   // transposed system for the adjoint solve (SMPM_FLAG_ADJOINT)
-  double *dHa = nullptr, *dHp = nullptr;  // coarse inverses with padded rows: adjoint, forward
+  double* dHa = nullptr;
   // element tables of the register-streamed apply (k_schur_warp_batch / k_schur_warpk)
   ElemMeta<double>* dtab64 = nullptr;
   ElemMeta<float>* dtab32 = nullptr;
@@ -1462,7 +1471,7 @@ GmresArgs<double> gmres_args(smpm_handle h, double tol, bool adj = false) {
   a.nblack = (int)h->f.black.size();
   a.nwhite = (int)h->f.white.size();
   a.dm = digit_mats(h, adj ? h->diga : h->dig);
-  a.Rd = h->dRd; a.H = h->dHp;
+  a.Rd = h->dRd; a.H = h->dH;
   if (adj) { a.Rd = h->dRda; a.H = h->dHa; a.g.zw = h->dzwa; }
   a.bt = h->dbt; a.if4 = h->dif4;
   a.vglob = h->wV; a.vown = h->wvown; a.t = h->wt; a.y = h->wy;
@@ -1517,7 +1526,7 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.skip = h->wdone;
   a.G = h->gm.grid;
   a.base = 0;
-  a.H64 = coarse_in_fp64(h) ? h->dHp : nullptr;
+  a.H64 = coarse_in_fp64(h) ? h->dH : nullptr;
   a.strips = h->st32;
   a.gsep = h->wgsep;
   choose_coarse(a, h->st_products, 1);
@@ -3270,13 +3279,14 @@ smpm_status factor_device_operator(smpm_handle h, cudaStream_t st) {
   return SMPM_OK;
 }
 
-// d x d row-major -> rows of d rounded up to a multiple of 4, zero padded
-std::vector<double> padded_rows(const std::vector<double>& H, long long d) {
-  const long long ld = (d + 3) & ~3LL;
-  if (ld == d) return H;
-  std::vector<double> out(d * ld, 0.0);
-  for (long long r = 0; r < d; ++r) std::copy(H.begin() + r * d, H.begin() + (r + 1) * d, out.begin() + r * ld);
-  return out;
+// d x d row-major into rows of coarse_ld(d) on the device
+smpm_status upload_rows(smpm_handle h, double** p, const std::vector<double>& H, long long d, cudaStream_t st) {
+  const size_t ld = coarse_ld(d), row = d * sizeof(double);
+  smpm_status s = dalloc(h, p, d * ld);
+  if (s != SMPM_OK || H.empty()) return s;
+  CU(cudaMemsetAsync(*p, 0, d * ld * sizeof(double), st));
+  CU(cudaMemcpy2DAsync(*p, ld * sizeof(double), H.data(), row, row, d, cudaMemcpyHostToDevice, st));
+  return SMPM_OK;
 }
 
 // S Z at every slot from the row sums of the pushed products: slot (e, F, t)
@@ -3340,7 +3350,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
                       Xc = transpose_blocks(h->f.X, g.n, 4 * h->f.black.size());
   if ((s = upload(h, &h->dT, Tc, st)) || (s = upload(h, &h->dRs, h->f.Rs, st)) ||
       (s = upload(h, &h->dG, Gc, st)) || (s = upload(h, &h->dX, Xc, st)) ||
-      (s = upload(h, &h->dH, h->f.H, st)) || (s = upload(h, &h->dfdx, h->f.fdx, st)) ||
+      (s = upload_rows(h, &h->dH, h->f.H, g.d, st)) || (s = upload(h, &h->dfdx, h->f.fdx, st)) ||
       (s = upload(h, &h->dfdy, h->f.fdy, st)) || (s = upload(h, &h->dD, h->f.D, st)) ||
       (s = upload(h, &h->duL, h->f.uL, st)) || (s = upload(h, &h->duS, h->f.uS, st)) ||
       (s = upload(h, &h->duC, h->f.uC, st)) || (s = upload(h, &h->dwhat, h->f.what, st)) ||
@@ -3355,8 +3365,6 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
   }
   dg.zw = h->dzw;
   if ((s = upload_tables(h, st))) return s;
-  h->dHp = h->dH;
-  if (g.d % 4 != 0 && (s = upload(h, &h->dHp, padded_rows(h->f.H, g.d), st))) return s;
   const size_t kp = g.kp, r = g.r, d = g.d, m = opts.restart;
   const size_t nbs = blocks_for(g.kp, kSlotsPerBlock);
   if ((s = dalloc(h, &h->wb, r)) || (s = dalloc(h, &h->wbS, kp)) || (s = dalloc(h, &h->wV, (m + 1) * kp)) ||
@@ -3450,8 +3458,10 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
       if (per_sm < 1) return fail(SMPM_ECUDA, "the refinement kernel does not fit on an SM");
       auto to32 = [](const std::vector<double>& v) { return std::vector<float>(v.begin(), v.end()); };
       if ((s = upload(h, &h->dT32, to32(Tc), st)) ||
-          (s = upload(h, &h->dH32, to32(padded_rows(h->f.H, g.d)), st)))
+          (s = dalloc(h, &h->dH32, (size_t)g.d * coarse_ld(g.d))))
         return s;
+      k_round32<<<1024, 256, 0, st>>>(h->dH, h->dH32, (size_t)g.d * coarse_ld(g.d));
+      CU(cudaGetLastError());
       if ((s = dalloc(h, &h->wx32, g.kp)) || (s = dalloc(h, &h->wt32, g.kp)) || (s = dalloc(h, &h->wy32, g.kp)) ||
           (s = dalloc(h, &h->wV32, g.kp)) || (s = dalloc(h, &h->wrg32, g.kp)) || (s = dalloc(h, &h->wr, g.kp)) ||
           (s = dalloc(h, &h->wcr, g.d)))
@@ -3507,7 +3517,7 @@ smpm_status factor_device(smpm_handle h, cudaStream_t st) {
           if (j < 0) continue;
           for (int t = 0; t < g.n; ++t) ztusa[j] += h->f.zwa[4 * e + F] * h->f.uSa[e * g.M + F * g.n + t];
         }
-      if ((s = upload(h, &h->dHa, padded_rows(h->f.Ha, g.d), st)) || (s = upload(h, &h->duSa, h->f.uSa, st)) ||
+      if ((s = upload_rows(h, &h->dHa, h->f.Ha, g.d, st)) || (s = upload(h, &h->duSa, h->f.uSa, st)) ||
           (s = upload(h, &h->dZtuSa, ztusa, st)))
         return s;
     }
@@ -4289,7 +4299,7 @@ __global__ void __launch_bounds__(256) k_deflate_noalloc(DevGeo g, const double*
     const int lane = threadIdx.x & 31;
     const long long nw = nthr >> 5;
     for (long long r = tid >> 5; r < g.d; r += nw) {
-      const double* h = H + r * g.d;
+      const double* h = H + r * coarse_ld(g.d);
       double acc = 0;
       for (long long j = lane; j < g.d; j += 32) acc += __ldg(h + j) * __ldcg(c + j);
       acc = warp_sum(acc);
