@@ -798,6 +798,32 @@ void diff_matrix(const std::vector<double>& x, std::vector<double>* D) {
   }
 }
 
+// Strip height of strip_factors with the fewest multiplications of one C^+ c (0:
+// the strips would not save half of the dense products), and their number.
+static int strip_height(const Geometry& g, double* products) {
+  const int mx = g.mx, row = 2 * mx - 1;
+  *products = 0;
+  if (g.d < 128) return 0;
+  int hbest = 0;
+  double best = 0.5 * static_cast<double>(g.d) * static_cast<double>(g.d);
+  auto count = [&](int h) {
+    const double p = (g.my + h - 1) / h, m = static_cast<double>(h) * row - mx, ns = (p - 1) * mx;
+    return p * (m + 2.0 * mx) * m + (ns + 1) * ns + p * m * 2.0 * mx;
+  };
+  for (int h = 1; 2 * h <= g.my; ++h) {
+    const int p = (g.my + h - 1) / h;
+    if (static_cast<long long>(p + 1) * mx > g.d + 1) continue;  // the staging buffer holds d + 1 entries
+    if (count(h) < best) { best = count(h); hbest = h; }
+  }
+  if (hbest) *products = best;
+  return hbest;
+}
+
+static double host_bytes() {  // physical memory, or 0 when unknown
+  const long pages = sysconf(_SC_PHYS_PAGES), page = sysconf(_SC_PAGE_SIZE);
+  return pages > 0 && page > 0 ? static_cast<double>(pages) * static_cast<double>(page) : 0.0;
+}
+
 // The coarse solve is dense (Sec. 2): C, the LU of the bordered K (factored
 // in place) and the leading block of K^-1, which becomes H = C^+ in place,
 // hold 3 (d+1)^2 doubles on the host at once; with the adjoint, H and the
@@ -805,16 +831,25 @@ void diff_matrix(const std::vector<double>& x, std::vector<double>* D) {
 // when that exceeds the machine's physical memory.
 static int coarse_memory_check(const Geometry& g, bool adjoint, std::string* err) {
   const double dd = static_cast<double>(g.d + 1);
-  const double need = (adjoint ? 5.0 : 3.0) * dd * dd * sizeof(double);
-  const long pages = sysconf(_SC_PHYS_PAGES), page = sysconf(_SC_PAGE_SIZE);
-  const double have = static_cast<double>(pages) * static_cast<double>(page);
-  if (pages <= 0 || page <= 0 || need <= have) return SMPM_OK;
+  const double need = (adjoint ? 5.0 : 3.0) * dd * dd * sizeof(double), have = host_bytes();
+  if (have == 0 || need <= have) return SMPM_OK;
   char msg[200];
   std::snprintf(msg, sizeof msg,
                 "the dense coarse matrices (d = %lld interfaces) need %.3g GB of host memory, more than this "
                 "machine has (%.3g GB)", g.d, need * 1e-9, have * 1e-9);
   *err = msg;
   return SMPM_ENOMEM;
+}
+
+// Whether the strips' factors fit beside them (else C^+ stays dense): about one
+// double per product, their interiors' LU and right-hand sides twice that while
+// they are formed, beside C, H and Ha; and the forward strips beside the
+// adjoint's inversion.
+static bool strips_fit(const Geometry& g, bool adjoint) {
+  const double dd = static_cast<double>(g.d + 1), D = dd * dd, have = host_bytes();
+  double q = 0;
+  if (!strip_height(g, &q)) return false;
+  return have == 0 || (adjoint ? std::max(5 * D + q, 3 * D + 4 * q) : 2 * D + 3 * q) * sizeof(double) <= have;
 }
 
 // Strip height with the fewest products, and its factors, for the coarse
@@ -826,25 +861,13 @@ static void strip_factors(const Geometry& g, const std::vector<double>& C, const
                           const double* u, bool transpose, StripFactors* out) {
   *out = StripFactors();
   const int d = static_cast<int>(g.d), mx = g.mx, row = 2 * mx - 1;
-  if (d < 128) return;
-  int hbest = 0;
-  double best = 0.5 * static_cast<double>(d) * d;  // at least half of the dense products saved
-  auto count = [&](int h) {
-    const double p = (g.my + h - 1) / h, m = static_cast<double>(h) * row - mx, ns = (p - 1) * mx;
-    return p * (m + 2.0 * mx) * m + (ns + 1) * ns + p * m * 2.0 * mx;
-  };
-  for (int h = 1; 2 * h <= g.my; ++h) {
-    const int p = (g.my + h - 1) / h;
-    if ((p + 1) * mx > d + 1) continue;  // the staging buffer holds d + 1 entries
-    if (count(h) < best) { best = count(h); hbest = h; }
-  }
-  if (!hbest) return;
   StripFactors& f = *out;
-  const int h = hbest, p = (g.my + h - 1) / h, m = h * row - mx, srow = h * row;
+  const int h = strip_height(g, &f.products);
+  if (!h) return;
+  const int p = (g.my + h - 1) / h, m = h * row - mx, srow = h * row;
   auto pad = [](int v) { return (v + 3) & ~3; };
   f.h = h; f.m = m; f.ns = (p - 1) * mx;
   f.ldn = pad(m); f.lds = pad(f.ns); f.ldw = pad(2 * mx);
-  f.products = best;
   const size_t RS = static_cast<size_t>(m) + 2 * mx;
   f.N.assign(p * RS * f.ldn, 0.0);
   f.W.assign(static_cast<size_t>(p) * m * f.ldw, 0.0);
@@ -909,6 +932,7 @@ static void strip_factors(const Geometry& g, const std::vector<double>& C, const
 
 static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, std::string* err) {
   const bool op_only = (o.flags & SMPM_FLAG_OPERATOR_ONLY) != 0;
+  const bool strips = !op_only && o.precond == 2 && strips_fit(g, (o.flags & SMPM_FLAG_ADJOINT) != 0);
   if (!op_only) {
     const int st = coarse_memory_check(g, (o.flags & SMPM_FLAG_ADJOINT) != 0, err);
     if (st != SMPM_OK) return st;
@@ -1108,7 +1132,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
       for (int j = 0; j < d; ++j) Hd[static_cast<size_t>(i) * d + j] = Kinv[static_cast<size_t>(i) * d + j] - s * f->uC[j];
     }
     if (!keep) f->H = std::move(Kinv);
-    if (o.precond == 2) strip_factors(g, f->C, f->H, f->uC.data(), false, &f->cs);
+    if (strips) strip_factors(g, f->C, f->H, f->uC.data(), false, &f->cs);
   }
 
   // null vectors of S and L
@@ -1213,7 +1237,7 @@ static int factor_host_body(const Geometry& g, const smpm_opts& o, Factors* f, s
       for (int j = 0; j < d; ++j)
         f->Ha[static_cast<size_t>(i) * d + j] =
             Kinv[static_cast<size_t>(j) * d + i] - v[i] * ch[j] - f->uC[i] * w[j];
-    if (o.precond == 2) strip_factors(g, f->C, f->Ha, ch.data(), true, &f->csa);
+    if (strips) strip_factors(g, f->C, f->Ha, ch.data(), true, &f->csa);
     // left null vector of the permuted S^T: Phi B1 (Phi swaps the two slots
     // facing each other across an interface; Phi B1 = B1 where B1 is constant
     // on each interface), normalised
