@@ -59,8 +59,6 @@ constexpr double kInnerTol = 1e-4;   // relative tolerance of each FP32 inner GM
 struct GState {
   double tolabs, beta0, beta, wnorm0sq, resid;
   int j, converged, breakdown, nan;
-  double g[kMaxRestart + 1];
-  double cs[kMaxRestart], sn[kMaxRestart];
   double R[(kMaxRestart + 1) * kMaxRestart];  // column j at R[j*(kMaxRestart+1)]
   double h1[kMaxRestart + 2], h2[kMaxRestart + 2];
   double y[kMaxRestart];

@@ -237,7 +237,7 @@ struct OwnedEntry {
 
 template <typename S>
 struct Smem {
-  double *h1, *h2, *hs1, *hs2, *z, *xi, *gg, *col, *invb, *misc;
+  double *h1, *h2, *hs1, *hs2, *z, *xi, *gg, *invb, *misc;
   double* cst;  // staged coarse vector c (d, and two entries of padding)
   unsigned char* wb;  // group scratch (item_bytes each)
   Resident* res;
@@ -268,7 +268,6 @@ __device__ Smem<S> carve(const GmresArgs<S>& a, unsigned char* raw) {
   s.z = d; d += m + 3;
   s.xi = d; d += m + 3;
   s.gg = d; d += m + 3;
-  s.col = d; d += m + 3;
   s.invb = d; d += m + 3;
   s.misc = d; d += 16;
   s.cst = d; d += a.g.d + 3;
@@ -300,7 +299,7 @@ inline size_t resident_bytes(int M, int n, int res_T, int res_G, int blk) {
 template <typename S>
 inline size_t gmres_smem_bytes(int m, int M, int n, int ES, int W, int basis_smem, long long d, bool w_global = false,
                                int res_T = 0, int res_G = 0, int blk = 0, int tab = 0, size_t H_bytes = 0) {
-  const size_t dbl = 9 * (size_t)(m + 3) + 16 + (size_t)d + 3;
+  const size_t dbl = 8 * (size_t)(m + 3) + 16 + (size_t)d + 3;
   size_t sel = w_global ? 0 : ES;
   if (basis_smem) sel += (size_t)(m + 1) * ES;
   return dbl * sizeof(double) + (size_t)(kGmresThreads / 32 / W) * item_bytes<S>(M, n, blk) + sel * sizeof(S) +

@@ -1736,7 +1736,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
   double acc8[8];
   CU(cudaMemcpyAsync(&herr, h->werr, sizeof(int), cudaMemcpyDeviceToHost, st));
   CU(cudaMemcpyAsync(acc8, h->wacc8, sizeof(acc8), cudaMemcpyDeviceToHost, st));
-  CU(cudaMemcpyAsync(&hs, h->wgs, offsetof(GState, g), cudaMemcpyDeviceToHost, st));
+  CU(cudaMemcpyAsync(&hs, h->wgs, offsetof(GState, R), cudaMemcpyDeviceToHost, st));
   double scal[8];
   CU(cudaMemcpyAsync(scal, reinterpret_cast<char*>(h->wgs) + offsetof(GState, scal), sizeof(scal),
                      cudaMemcpyDeviceToHost, st));
