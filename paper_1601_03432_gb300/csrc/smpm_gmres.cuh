@@ -99,6 +99,7 @@ struct GmresArgs {
   S* wscr;          // when non-null: per-CTA global scratch for w (ES per rank)
   // C^+ by element-row strips (strips.p > 0 and use_strips): see coarse_solve
   CoarseStrips<typename std::conditional<sizeof(S) == 4, float, double>::type> strips;
+  CoarseStrips<double> strips64;  // where H64 is set
   double* gsep;        // strips: 2 p mx + 1 doubles per column (sums pushed onto the separators, alpha)
   int use_strips;      // 1: the strips are the cheaper form for this team size
 };
@@ -722,12 +723,11 @@ __device__ __forceinline__ void row_dots(int r0, int r1, int longest, Get&& get,
 
 // c_hat = C^+ c, complete after the final barrier; false when a
 // barrier timed out.  cst: staging for at least d + 1 entries.
-template <typename S>
-__device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, void* cst, unsigned& epoch, const double* c, double* chat) {
-  using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
+template <typename T, typename S>
+__device__ SMPM_PHASE bool coarse_strips(const GmresArgs<S>& a, const CoarseStrips<T>& k, void* cst, unsigned& epoch,
+                                         const double* c, double* chat) {
   constexpr int V = 16 / (int)sizeof(T);
   T* xs = reinterpret_cast<T*>(cst);
-  const auto& k = a.strips;
   const int G = a.G, rank = team_rank(a), d = (int)a.g.d;
   const int srow = k.h * k.row, RS = k.m + 2 * k.mx;  // interfaces of a strip with its upper separator; rows of N
   double* alpha = a.gsep + 2 * (size_t)k.p * k.mx;
@@ -840,15 +840,16 @@ __device__ __forceinline__ void coarse_rows_in(const GmresArgs<S>& a, const T* H
         put);
   }
 }
-// The FP32 inner solves of the mixed-precision path take the FP64 inverse on small
-// grids (H64), where its products are a small part of a step, and else its FP32
-// copy with FP32 products and sums: an inner solve needs only a relative 1e-4, and
+// The FP32 inner solves of the mixed-precision path take the FP64 inverse (or its
+// strips) on small grids (H64), where its products are a small part of a step, and
+// else its FP32 copy with FP32 products and sums: an inner solve needs only a relative 1e-4, and
 // every refinement sweep recomputes the residual in FP64.
 template <typename S>
 __device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, const double* c, double* chat) {
   using T = typename std::conditional<sizeof(S) == 4, float, double>::type;
-  if (sizeof(S) == 4 && a.H64) coarse_rows_in<double>(a, a.H64, (const double*)nullptr, s.cst, c, chat);
-  else coarse_rows_in<T>(a, a.H, s.H, reinterpret_cast<T*>(s.cst), c, chat);
+  if constexpr (sizeof(S) == 4)
+    if (a.H64) return coarse_rows_in<double>(a, a.H64, (const double*)nullptr, s.cst, c, chat);
+  coarse_rows_in<T>(a, a.H, s.H, reinterpret_cast<T*>(s.cst), c, chat);
 }
 
 // c_hat = C^+ c by all CTAs of the team (strips or dense rows), complete after
@@ -856,7 +857,9 @@ __device__ SMPM_PHASE void coarse_rows(const GmresArgs<S>& a, const Smem<S>& s, 
 template <typename S>
 __device__ __forceinline__ bool coarse_solve(const GmresArgs<S>& a, const Smem<S>& s, unsigned& epoch, const double* c,
                                              double* chat) {
-  if (a.use_strips) return coarse_strips(a, s.cst, epoch, c, chat);
+  if constexpr (sizeof(S) == 4)
+    if (a.use_strips && a.H64) return coarse_strips(a, a.strips64, s.cst, epoch, c, chat);
+  if (a.use_strips) return coarse_strips(a, a.strips, s.cst, epoch, c, chat);
   coarse_rows(a, s, c, chat);
   return team_sync(a, epoch);
 }

@@ -1454,7 +1454,7 @@ bool coarse_in_fp64(smpm_handle h) {
 // Form of the coarse solve for a solve of R columns by a.G CTAs.
 template <typename S>
 void choose_coarse(GmresArgs<S>& a, double products, int R) {
-  a.use_strips = a.precond == 2 && !a.H64 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4);
+  a.use_strips = a.precond == 2 && a.strips.p > 0 && strips_pay(a.g.d, products, a.G, R, sizeof(S) == 4 && !a.H64);
 }
 
 DigitMats digit_mats(smpm_handle h, const smpm_handle_s::DigitSet& d) {
@@ -1528,6 +1528,7 @@ GmresArgs<float> gmres_args32(smpm_handle h, double tol) {
   a.base = 0;
   a.H64 = coarse_in_fp64(h) ? h->dH : nullptr;
   a.strips = h->st32;
+  a.strips64 = h->st;
   a.gsep = h->wgsep;
   choose_coarse(a, h->st_products, 1);
   return a;
