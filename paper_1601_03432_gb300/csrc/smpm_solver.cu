@@ -1419,12 +1419,17 @@ size_t refine_shape(const Geometry& g, int m, int ES, int items, size_t budget, 
   return need();
 }
 
-// Whether C^+ by strips is the cheaper form for R columns on a team of G CTAs:
-// its two extra team barriers and phase starts cost about 9,000 cycles, the
-// dense rows one cycle per product and CTA in FP64, 0.37 in FP32.  Measured
-// (SM cycles per Arnoldi step, G = 152): see the comment of coarse_solve.
+// Whether C^+ by strips is the cheaper form for R columns on a team of G CTAs: its
+// two extra team barriers and phase starts against the products that it saves per
+// CTA and step.  Measured, GMRES time per step in us, n = 6, 152 CTAs, dense rows
+// against strips (saved products per CTA):
+//   one column, FP64: 28x28 elements (13 k) 35.1 / 35.7; 32x32 (22 k) 39.2 / 37.4; 48x48 112 / 52
+//   one column, FP32: 32x32 (22 k) 42.4 / 44.6; 40x40 (54 k) 53.6 / 50.6; 48x48 71 / 54
+//   8 columns, FP64:  16x16 (10 k) 88 / 93; 20x20 (25 k) 97.6 / 98.0; 24x24 (54 k) 109 / 103
+//   8 columns, FP32:  20x20 (25 k) 112 / 116; 24x24 (54 k) 121 / 119
 bool strips_pay(long long d, double products, int G, int R, bool fp32) {
-  return R * ((double)d * d - products) / G >= (fp32 ? 24000.0 : 9000.0);
+  const double line = R > 1 ? (fp32 ? 45000.0 : 25000.0) : (fp32 ? 24000.0 : 14000.0);
+  return R * ((double)d * d - products) / G >= line;
 }
 
 // Whether black blocks are solved with their whole inverse (black_block): a
