@@ -11,7 +11,7 @@
 // runs on across its tasks.  The task's arguments are staged in shared
 // memory (header of the dynamic buffer) and the bodies carve the rest.
 #pragma once
-// Included inside the anonymous namespace of smpm_solver.cu.
+// Included inside the anonymous namespace of each translation unit that uses it.
 
 struct alignas(16) BatchTask {
   PrePostArgs P;          // FP64 pre/post arguments (all-global layout)

@@ -1,23 +1,33 @@
 // Exact fixed-point products on the tensor cores ("digits"): y = A x for small
-// dense A in FP64 or FP32 accuracy, where the FP64 pipe of this part (2 FMA
+// dense A, accurate relative to A's rows and the whole vector x, where the FP64 pipe of this part (2 FMA
 // per clock and SM) or the FP32 pipe's shared-memory loads are the bound.
 //
-// A number is held as a signed integer X = v 2^(B-e) (|X| < 2^B; B = 62 for
-// FP64, 30 for FP32) relative to an exponent e shared by a row of A or a
-// column of x, and cut into base-256 digits in [-128, 127] (ND = 8 or 4): with
+// A number is held as a signed integer X = v 2^(B-e) (|X| <= 2^B; B = 62 for
+// FP64, 30 for FP32, 94 for single products, see tile8_wide) relative to an exponent e shared by a row of A or a
+// column of x, and cut into base-256 digits in [-128, 127] (ND = 8, 4 or 12): with
 // the bias 0x80..80 added, the digits are the bytes of X, less 128.  Digits
 // are exact in fp16, their products are integers of at most 2^14, and up to
 // 8 x 128 of them add exactly in the FP32 accumulators of mma.sync (at most
-// 2^24; checked on this part).  Products of digits i and j weigh 256^(i+j);
+// 2^24; tests/test_gpu_accumulators.py).  Products of digits i and j weigh 256^(i+j);
 // those of one weight share an accumulator, and the weights below 256^GMIN
 // are left out.  The sums are put together in integers and rounded once.
 //
-// Error: the operands carry 2^-62 (2^-30) relative to the largest of their row
-// or column, the left-out weights about 2^-59 (2^-35) of row maximum times
-// column maximum; a chain of K FP64 FMAs loses up to K 2^-53 of the sum of
-// magnitudes.  mma.sync m16n8k16 rather than tcgen05: the operands are one
+// Error, for K columns, as a share of row maximum times column maximum (each at
+// least half of its power of two): the operands lose up to K 2^-60 (K 2^-28 in FP32),
+// the left-out weights up to 7 K 2^14 256^6 2^-122 = K 2^-57 (2 K 2^14 256 2^-58 = K 2^-35) if
+// all their digits are extreme and of one sign, about 2^-8 of that for digits of
+// mixed signs.  This is a bound relative to the largest entries, as a GMRES solve with
+// its normwise tolerance needs it; a chain of K FP64 FMAs loses up to K 2^-53 of the
+// sum of magnitudes of the entry itself, which is less where that sum is below
+// 2^-4 of the two maxima (solves on local and widely ranging right-hand sides end
+// with the same errors either way).  The products that are results by themselves,
+// y = S v, take operands of 94 bits (tile8_wide).
+//
+// mma.sync m16n8k16 rather than tcgen05 in the solves: the operands are one
 // element's 4n x 4n matrix and eight columns (or the eight digits of one
 // column), far below a tcgen05 tile, and each warp works on its own element.
+// The class apply of y = S v on a large grid is a contraction that would fill
+// tcgen05 tiles; that form has not been built.
 //
 // Fragments of A (host: pack_digits): tile (mt, kt) of 16 x 16 entries, lane
 // (g = lane / 4, q = lane % 4) holds rows g, g + 8 and columns 2q, 2q+1, 2q+8,

@@ -31,15 +31,15 @@
 // step: five barriers (about 3,000 SM cycles each), a dozen dependent loads
 // from L2 (about 700 each), FP64 sums at 76 cycles per operation, one packing
 // and one product of digits per element phase.  At 16 x 16 elements, n = 16,
-// on 152 CTAs a step takes 59,000 cycles (57,000 with FP64 products and a
-// step more per solve before).  On large grids, the element products, the
+// on 128 CTAs the phases and barriers of a step take 54,000 cycles of CTA 0 (57,000 with
+// FP64 products and rotations in every step, and a step more per solve).  On large grids, the element products, the
 // basis read from L2 and C^+.
 //
 // Data written by other CTAs inside the kernel is read with ld.global.cg: L1
 // is not coherent across SMs.  The barrier spins with a bound and raises an
 // error flag instead of hanging.
 #pragma once
-// Included inside the anonymous namespace of smpm_solver.cu.
+// Included inside the anonymous namespace of each translation unit that uses it.
 
 // Packed class matrices of the element products (smpm_digits.cuh): T_e per
 // element class, G_b and the four X_F per block class, with row exponents,

@@ -2,19 +2,21 @@
 // Arnoldi processes of Algorithm 2 / 3 (GMRES on S M^-1 or P S M^-1) advance
 // together, one step at a time, in ONE persistent cooperative launch, so that
 // every operator matrix (G_b, X_b, T_e, the coarse C^+) is read once per step
-// for all R columns and the five grid barriers of a step are shared.  Each
-// element product becomes a small dense GEMM: the M x M matrix times a tile of
-// eight columns.
+// for all R columns and the five team barriers of a step (seven with C^+ by strips)
+// are shared.  Each element product becomes a small dense GEMM: the M x M matrix
+// times a tile of eight columns.
 //
 // Per column, everything of the single-column kernel is kept: its own basis,
 // Hessenberg column, FP64 Givens rotations, residual estimate, convergence,
 // breakdown and NaN flags, and its own restarts.  A column that converges
 // stops (its scale is set to zero: its later basis vectors are zero and its
 // Givens state is frozen); the step loop ends when every column has stopped,
-// and a restart cycle restarts only the columns still running.  The
-// iterates of column rho are exactly those of a single-column solve of that
-// right-hand side (same phases, same CGS2 with the lazy v_j and the
-// Pythagorean norm); only the order of the atomic dot-product sums differs.
+// and a restart cycle restarts only the columns still running.  In exact
+// arithmetic the iterates of column rho are those of a single-column solve of that
+// right-hand side (same phases, same CGS2, Pythagorean norm and stopping
+// criterion).  Rounding differs: v_j is formed at the start of step j, the residual
+// norm comes from a rotation per step, the block solves run in stages where a
+// single solve may take the whole inverse, and the sums meet in another order.
 //
 // Layouts: column rho of a kp-vector at base + rho * vs; of a d-vector at
 // base + rho * ds.  The basis lives in global memory (L2 / HBM): CTA rank's
@@ -24,7 +26,8 @@
 // takes items grp, grp + ngrp, ...; an item's tiles live in the group's
 // shared scratch.
 #pragma once
-// Included inside the anonymous namespace of smpm_solver.cu, after smpm_gmres.cuh.
+// Included inside the anonymous namespace of each translation unit that uses it,
+// after smpm_gmres.cuh.
 
 constexpr int kLockMaxCols = 16;  // columns of one lockstep launch
 
@@ -367,9 +370,9 @@ __device__ SMPM_PHASE void lk_coarse_h(const LockArgs<S>& A, const HT* H) {
   }
 }
 
-// FP32 columns: the coarse inverse's FP32 copy (see coarse_rows32).  The R
+// FP32 columns: the coarse inverse's FP32 copy, FP32 products and sums.  The R
 // coarse vectors are converted to FP32 once per CTA, a chunk of dc entries of
-// every column at a time, into the idle warp tiles (converting them on every
+// every column at a time, into the groups' idle scratch (converting them on every
 // row's pass costs as much as FP64 products); each warp keeps its rows'
 // partial sums in c_hat across the chunks.
 template <typename S>
@@ -421,7 +424,7 @@ __device__ SMPM_PHASE void lk_coarse32_staged(const LockArgs<S>& A, float* cf, i
           }
       }
     }
-    __syncthreads();  // the warp tiles take the next chunk, or the next phase
+    __syncthreads();  // the scratch takes the next chunk, or the next phase
   }
 }
 

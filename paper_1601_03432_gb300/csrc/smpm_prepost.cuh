@@ -37,7 +37,7 @@
 //   Q6  dl/db = lam - u_L (u_L^T lam) written to u; dl/dg on boundary-face
 //       slots = tau_F dl/db at the face node (gg, if given)
 #pragma once
-// Included inside the anonymous namespace of smpm_solver.cu.
+// Included inside the anonymous namespace of each translation unit that uses it.
 
 // Packed fast-diagonalisation factors (smpm_digits.cuh): per x entry (a
 // face-type class, or a column of a graded grid) the digits of V and V^-1 and

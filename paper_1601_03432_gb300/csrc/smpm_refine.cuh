@@ -1,19 +1,20 @@
 // One step of GMRES-based iterative refinement (mixed precision):
-// the inner GMRES (k_gmres<float>) has solved P S M^-1 y = P r in FP32 with
-// the FP64 coarse solve; this cooperative kernel turns y into the FP64
-// correction and the next inner right-hand side:
+// the inner GMRES (k_gmres<float>) has solved P S M^-1 y = P r in FP32; this
+// cooperative kernel turns y into the FP64 correction and the next inner
+// right-hand side.  C^+ is the inner solve's own (coarse_solve): the FP64 inverse on
+// small grids, else its FP32 copy with FP32 products and sums; c and c_hat are FP64.
 //   R1  owner blocks:   t = M^-1 y                        (FP32 operator)
 //   R2  white elements: S t on the black slots, c = Z^T S t (FP64 sums)
-//   R3  c_hat = C^+ c                                      (FP64)
+//   R3  c_hat = C^+ c
 //   R4  owner entries:  x_S += t - Z (c_hat - c_hat_r)     (FP64; Eq. deflated_schur
 //                       for the correction equation S d = r); y <- 0
 //   R5  elements:       r = b_S - S x_S with the FP64 T_e (push form);
 //                       ||r||^2 and Z^T r accumulated
 //   R6  ||r|| <= tol ||P b_S||: done (all CTAs agree); otherwise
-//                       c_hat_r = C^+ Z^T r                (FP64)
+//                       c_hat_r = C^+ Z^T r
 //   R7  owner entries:  next inner right-hand side P r = r - S Z c_hat_r (FP32)
 #pragma once
-// Included inside the anonymous namespace of smpm_solver.cu.
+// Included inside the anonymous namespace of each translation unit that uses it.
 
 struct alignas(16) RefineArgs {  // 16-byte multiple: staged with 16-byte copies in batched solves
   GmresArgs<float> ga;   // FP32 operator and vectors: x = inner y, t, y, c, chat, rhs (next inner rhs)

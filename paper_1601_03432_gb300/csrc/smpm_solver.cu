@@ -2346,8 +2346,7 @@ smpm_status batch_layout(smpm_batch b, const TeamPlan& plan) {
     L.ES = basis_entries(g.M, L.nown_b);
     const bool mixed = batch_mixed(b, p);
     // the all-global needs of pre/post and refinement, then the richest
-    // GMRES layout that fits beside the argument header (resident or
-    // streamed operator matrices, resident basis)
+    // GMRES layout that fits beside the argument header (choose_layout)
     const size_t budget = budget_all;
     const int items = std::max(L.nown_b, L.nown_w);
     auto need_fixed = [&](bool wg) {
