@@ -31,7 +31,7 @@
 // step: five barriers (about 3,000 SM cycles each), a dozen dependent loads
 // from L2 (about 700 each), FP64 sums at 76 cycles per operation, one packing
 // and one product of digits per element phase.  At 16 x 16 elements, n = 16,
-// on 128 CTAs the phases and barriers of a step take 54,000 cycles of CTA 0 (57,000 with
+// on 128 CTAs the phases and barriers of a step take 55,000 cycles of CTA 0 (57,000 with
 // FP64 products and rotations in every step, and a step more per solve).  On large grids, the element products, the
 // basis read from L2 and C^+.
 //

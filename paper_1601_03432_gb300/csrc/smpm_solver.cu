@@ -1234,22 +1234,21 @@ bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
 bool class_tiles_pay(smpm_handle h) { return (long long)h->ntiles * kClassTile <= 5 * h->g.nel; }
 
 // Whether SMPM_APPLY_AUTO takes the class apply: its matrices are packed
-// (class_span), its tiles fill, and it is the faster one.  Measured, back to back,
-// FP64 / FP32 in us, best per-element kernel (T_e in L2 where it fits) against the
-// class kernel, which takes 9.5 us for M <= 64 and 14.5 / 12.3 beyond until its CTAs
-// fill the SMs several times:
-//   FP64: 16x16, n = 24 12.7 / 14.5; 20x24, n = 24 14.5 / 14.5; 32x32, n = 5 9.5 / 9.7,
-//     n = 16 16.8 / 9.8, n = 24 24.8 / 14.5; 96x96, n = 24 160 / 54; 128x128, n = 16 183 / 46:
-//     from four elements per SM on.
-//   FP32: 32x32, n = 24 9.6 / 12.4, n = 32 22.8 / 12.7; 48x48, n = 24 14.7 / 14.5; 96x96,
-//     n = 11 14.8 / 18.8, n = 24 74 / 39; 128x128, n = 8 17.6 / 18.8, n = 11 39 / 27, n = 16 60 / 33:
-//     where the matrices leave L2 (three quarters of it), or M > 96, whose
-//     per-element kernel stages them in shared memory.
+// (class_span), its tiles fill, and it is the faster one.  Measured in a CUDA graph
+// (no launch gaps, T_e in L2 where it fits), us, the per-element kernel that AUTO
+// takes else against the class kernel:
+//   FP64, elements: 608 (four per SM, one wave), n = 8 6.0 / 6.8, n = 17 9.8 / 10.3, n = 24 12.3 / 11.8;
+//     702 n = 5 6.3 / 6.8, n = 8 7.7 / 6.7, n = 16 12.3 / 7.9, n = 24 17.1 / 11.7; 1024 n = 5 7.5 / 7.0,
+//     n = 24 23 / 11.8; 5184 n = 16 69 / 19, n = 24 102 / 35
+//   FP32: 1024 n = 8 4.4 / 7.0, n = 24 7.3 / 9.6; 1296 n = 5 6.2 / 7.4, n = 10 8.5 / 8.3, n = 24 12.4 / 11.4;
+//     1600 n = 5 6.4 / 7.4, n = 8 7.3 / 7.0; 3136 n = 5 9.3 / 8.0, n = 24 47 / 18; n = 28 (staged in
+//     shared memory): 608 8.0 / 10.3, 702 10.2 / 9.3, 1600 18 / 14
 template <typename S>
-bool class_pays(smpm_handle h, int sms, int l2) {
+bool class_pays(smpm_handle h, int sms) {
   if (!class_tiles_pay(h)) return false;
-  if (sizeof(S) == 8) return h->g.nel >= 4LL * sms;
-  return (double)h->g.nel * h->g.M * h->g.M * sizeof(S) >= 0.75 * l2 || (h->g.M > 96 && h->g.nel >= 4LL * sms);
+  const long long ne = h->g.nel, M = h->g.M;
+  if (sizeof(S) == 8) return ne > 4LL * sms && (M >= 32 || ne > 6LL * sms);
+  return (ne > 8LL * sms && ne * M >= 50000) || (M > 96 && ne > 4LL * sms);
 }
 
 // y = S v with the handle's apply kernel.  SMPM_APPLY_AUTO: the class-shared
@@ -1262,12 +1261,11 @@ smpm_status launch_schur_kind(smpm_handle h, int kind, const S* v, S* y, cudaStr
   const bool fp32 = sizeof(S) == 4;
   const ElemMeta<S>* tab = reinterpret_cast<const ElemMeta<S>*>(fp32 ? (const void*)h->dtab32 : (const void*)h->dtab64);
   const S* T = reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT);
-  int dev = 0, sms = 0, l2 = 0;
+  int dev = 0, sms = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  CU(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
   const bool packed = fp32 ? h->clsT32 != nullptr : h->clsT64 != nullptr;
-  if (kind == SMPM_APPLY_AUTO && packed && class_pays<S>(h, sms, l2)) kind = SMPM_APPLY_CLASS;
+  if (kind == SMPM_APPLY_AUTO && packed && class_pays<S>(h, sms)) kind = SMPM_APPLY_CLASS;
   if (kind == SMPM_APPLY_CLASS && !packed) kind = SMPM_APPLY_AUTO;
   if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
   if (kind == SMPM_APPLY_STREAM) return launch_schur_stream<S>(h, T, v, y, st);

@@ -156,3 +156,27 @@ def test_mixed_solves_of_small_grids_keep_the_fp64_coarse_inverse(built, mx, my,
     assert coarse64 == fp64 == int(g.d * ctas <= 1 << 17)
     assert g.solve(f, um)[0]["converged"] == 1
     assert (u - um).norm() <= 1e-8 * u.norm()
+
+
+# four elements per SM and one more (FP64), eight per SM and one more (FP32, with
+# entries enough and not), more than 96 rows
+@pytest.mark.parametrize("mx,my,n", [(19, 32, 8), (29, 21, 8), (38, 32, 11), (35, 35, 11), (35, 35, 6), (29, 21, 27)])
+def test_default_apply_on_both_sides_of_its_lines(built, mx, my, n):
+    """What AUTO takes agrees with the class and per-element kernels entry by entry."""
+    g = Grid(mx, my, n, float(mx), float(my))
+    g.factor(precision=1, flags=B.FLAG_OPERATOR_ONLY)
+    M, nel = 4 * n, mx * my
+    h = Grid(3, 3, n, 3.0, 3.0)
+    h.factor_host_only()
+    T9 = h.host_factor("T").reshape(9, M, M)
+    ix, iy = np.arange(nel) % mx, np.arange(nel) // mx
+    side = lambda i, m: np.where(i == 0, 0, np.where(i == m - 1, 2, 1))  # noqa: E731
+    T = T9[3 * side(iy, my) + side(ix, mx)]
+    v = np.random.default_rng(n).standard_normal((nel, M))
+    for dtype, u in ((torch.float64, 2.0 ** -53), (torch.float32, 2.0 ** -24)):
+        vt = dev(v.ravel(), dtype)
+        vr = vt.double().cpu().numpy().reshape(nel, M)
+        bound = 2 * own_bound(T, vr, mx, my, n, u)  # either side's rounding
+        outs = [applied(g, k, vt).reshape(nel, M) for k in (B.APPLY_AUTO, B.APPLY_CLASS, B.APPLY_STREAM)]
+        for o in outs[1:]:
+            assert np.all(np.abs(o - outs[0]) <= bound + 2 * u * np.abs(o))
