@@ -330,7 +330,7 @@ def run_ours(args):
     mixed = {"value": mix_rate, "unit": "solves/s",
              "ms_per_step": mix_max / args.steps, "inner_iterations": mix_rep["iterations"],
              "refinements": mix_rep["refinements"], "schur_relres": mix_rep["schur_relres"],
-             "precision": "FP32 inner GMRES (30-bit digit operator products, FP32 coarse product; FP64 Hessenberg least squares and dot accumulation) + FP64 refinement"}
+             "precision": "FP32 inner GMRES (30-bit digit operator products; FP64 coarse product at this size, Hessenberg least squares and dot accumulation) + FP64 refinement"}
 
     # ---- Schur apply y = S v on single grids of growing size (operator-only
     # factor step: T_e only), L2 flushed before each launch (write + read
@@ -797,7 +797,7 @@ def run_batch(args, stream, hbm_peak):
 def run_profile(which):
     """Small fixed cases for ncu captures: `gmres` runs three solves of the
     bench workload (FP64), `apply` three y = S v launches each in FP32 and
-    FP64 on 32x32 elements, n = 24, `bapply` three batched FP32 applies over
+    FP64 on 32x32 elements, n = 24 (four warps per element), `bapply` three batched FP32 applies over
     the first 40 grids of the uneven batch.  Prints "ok" and no bench line."""
     import torch
     from paper_1601_03432_gb300 import Grid, inputs
@@ -853,6 +853,7 @@ def run_profile(which):
         from paper_1601_03432_gb300 import _binding as _B
         g = Grid(96, 96, 24)
         g.factor(precision=1, flags=_B.FLAG_OPERATOR_ONLY)
+        g.set_apply_kernel(_B.APPLY_WARP)
         gen = torch.Generator(device="cuda").manual_seed(7)
         for dt, fn in ((torch.float32, g.apply_schur32), (torch.float64, g.apply_schur)):
             v = torch.randn(g.kp, dtype=dt, device="cuda", generator=gen)
@@ -863,8 +864,10 @@ def run_profile(which):
         print("ok")
         return
     else:
+        from paper_1601_03432_gb300 import _binding as _B
         g = Grid(32, 32, 24)
         g.factor(tol=W["tol"], restart=W["restart"], precision=1)
+        g.set_apply_kernel(_B.APPLY_WARP4)
         gen = torch.Generator(device="cuda").manual_seed(7)
         for dt, fn in ((torch.float32, g.apply_schur32), (torch.float64, g.apply_schur)):
             v = torch.randn(g.kp, dtype=dt, device="cuda", generator=gen)
