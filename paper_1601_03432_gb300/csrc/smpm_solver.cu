@@ -1849,6 +1849,22 @@ size_t lock_shape(smpm_handle h, LockArgs<S>& A, int R, int nown_b, size_t budge
   return A.wb_bytes ? fixed + A.wb_bytes : 0;
 }
 
+constexpr size_t kLockStatic = 2048;  // the kernel stages its arguments in static shared memory
+
+// Columns of a lockstep group of at most R: halved until the layout fits (1: it does
+// not fit for two; long restart cycles hold nine values per step and column).
+int lock_columns(smpm_handle h, int R, int optin) {
+  for (; R > 1; R = (R + 1) / 2) {
+    LockArgs<double> A64{};
+    LockArgs<float> A32{};
+    const size_t budget = (size_t)optin - kLockStatic;
+    if (h->opts.precision == 1 ? lock_shape(h, A32, R, h->gm.nown_b, budget) : lock_shape(h, A64, R, h->gm.nown_b, budget))
+      return R;
+    if (R == 2) break;
+  }
+  return 1;
+}
+
 // R right-hand sides of one grid in lockstep.  FP64: k_pre_cols,
 // k_gmres_lock<double>, k_post_cols.  Mixed precision: k_pre_cols, then
 // kMaxRefine pairs (k_gmres_lock<float>, k_refine_cols) that skip the columns
@@ -1867,7 +1883,7 @@ smpm_status solve_lock(smpm_handle h, const double* f, const double* gn, double*
   CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   LockArgs<double> A64{};
   LockArgs<float> A32{};
-  const size_t budget = (size_t)optin - 2048;  // the kernel stages its arguments in static shared memory
+  const size_t budget = (size_t)optin - kLockStatic;
   const size_t smem =
       mixed ? lock_shape(h, A32, R, h->gm.nown_b, budget) : lock_shape(h, A64, R, h->gm.nown_b, budget);
   if (!smem) return fail(SMPM_EINVAL, "lockstep layout does not fit in shared memory");
@@ -3564,8 +3580,11 @@ smpm_status schur_solve(smpm_handle h, const double* f, const double* gn, double
   // several right-hand sides of an FP64 solve with block-Jacobi: lockstep
   // groups of up to kLockMaxCols columns
   const bool lock = nrhs > 1 && h->opts.precond > 0 && !(h->opts.flags & SMPM_FLAG_NO_LOCKSTEP);
-  for (int k = 0; lock && k < nrhs; k += kLockMaxCols) {
-    const int R = std::min(kLockMaxCols, nrhs - k);
+  int dev = 0, optin = 0;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  for (int k = 0, R = 1; lock && k < nrhs; k += R) {
+    R = lock_columns(h, std::min(kLockMaxCols, nrhs - k), optin);
     smpm_status s = R == 1 ? solve_one(h, f + (size_t)k * h->g.r, gn ? gn + (size_t)k * h->g.kp : nullptr,
                                        u + (size_t)k * h->g.r, t, rep ? rep + k : nullptr, st)
                            : solve_lock(h, f + (size_t)k * h->g.r, gn ? gn + (size_t)k * h->g.kp : nullptr,

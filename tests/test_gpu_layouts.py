@@ -67,3 +67,19 @@ def test_team_sizes_meet_the_single_solve(built, precision, team):
     b.close()
     assert (u - ub).norm() <= BOUND[precision] * u.norm()
     assert abs(rep["iterations"] - one["iterations"]) <= (1 if precision == 0 else 3)
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp64", "mixed"])
+def test_lockstep_groups_with_long_cycles(built, precision):
+    """Restart 190 with 14 columns of the largest order: the least squares' state leaves
+    no room for a group's digits, so the columns run in smaller groups."""
+    g = Grid(3, 2, 32)
+    g.factor(tol=1e-11, precision=precision, restart=190, maxit=400)
+    f = dev(np.stack([inputs.white_noise(g.r, 60 + k) for k in range(14)]))
+    u, one = torch.empty_like(f), torch.empty_like(f[0])
+    reps = g.solve(f, u, nrhs=14)
+    for k in range(14):
+        assert reps[k]["converged"] == 1
+        if k % 4 == 0:
+            g.solve(f[k].contiguous(), one)
+            assert (one - u[k]).norm() <= BOUND[precision] * one.norm()
