@@ -1101,10 +1101,19 @@ smpm_status host_exception() {
     CU(cudaGetLastError()); \
   } while (0)
 
+// cudaMalloc whose failure does not stay behind as the last error, which the next
+// launch's check would report as its own
+template <typename P>
+cudaError_t device_malloc(P** p, size_t bytes) {
+  const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
 template <typename P>
 smpm_status dalloc(smpm_handle h, P** p, size_t count) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(P) + 16);
+  cudaError_t e = device_malloc(&q, count * sizeof(P) + 16);
   if (e != cudaSuccess) return fail(SMPM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   h->allocs.push_back(q);
   *p = static_cast<P*>(q);
@@ -1776,7 +1785,7 @@ smpm_status solve_one(smpm_handle h, const double* f, const double* gn, double* 
 template <typename P>
 smpm_status lalloc(smpm_handle h, P** p, size_t count) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(P) + 16);
+  cudaError_t e = device_malloc(&q, count * sizeof(P) + 16);
   if (e != cudaSuccess) return fail(SMPM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   h->lk.allocs.push_back(q);
   *p = static_cast<P*>(q);
@@ -2148,7 +2157,7 @@ void batch_free_layout(smpm_batch b) {
 template <typename P>
 smpm_status balloc(smpm_batch b, P** p, size_t count) {
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(P) + 16);
+  cudaError_t e = device_malloc(&q, count * sizeof(P) + 16);
   if (e != cudaSuccess) return fail(SMPM_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   b->allocs.push_back(q);
   *p = static_cast<P*>(q);
@@ -3707,8 +3716,8 @@ smpm_status smpm_autotune_apply(smpm_handle h, int precision, int reps, int flus
     if (y) cudaFree(y);
     if (fl) cudaFree(fl);
   };
-  if (cudaMalloc(&v, h->g.kp * es) != cudaSuccess || cudaMalloc(&y, h->g.kp * es) != cudaSuccess ||
-      (flush_bytes && cudaMalloc(&fl, flush_bytes) != cudaSuccess)) {
+  if (device_malloc(&v, h->g.kp * es) != cudaSuccess || device_malloc(&y, h->g.kp * es) != cudaSuccess ||
+      (flush_bytes && device_malloc(&fl, flush_bytes) != cudaSuccess)) {
     release();
     cudaGetLastError();
     return fail(SMPM_ENOMEM, "device allocation failed in the apply autotuner");
@@ -4003,8 +4012,8 @@ smpm_status smpm_batch_create(const smpm_handle* hs, int count, const int* nrhs,
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))
     return bad(fail(SMPM_ECUDA, "no CUDA device"));
-  if (cudaMalloc(&b->dbars, sizeof(unsigned) * sms) || cudaMalloc(&b->derr, 4 * sizeof(int)) ||
-      cudaMalloc(&b->dio, sizeof(BatchIO)) || cudaMalloc(&b->drep, sizeof(TaskReport) * b->ntasks) ||
+  if (device_malloc(&b->dbars, sizeof(unsigned) * sms) || device_malloc(&b->derr, 4 * sizeof(int)) ||
+      device_malloc(&b->dio, sizeof(BatchIO)) || device_malloc(&b->drep, sizeof(TaskReport) * b->ntasks) ||
       cudaMallocHost(&b->hio, sizeof(BatchIO)) || cudaMallocHost(&b->hrep, sizeof(TaskReport) * b->ntasks) ||
       cudaMallocHost(&b->herr, 4 * sizeof(int)) || cudaStreamCreateWithFlags(&b->bs, cudaStreamNonBlocking) ||
       cudaEventCreate(&b->ein) || cudaEventCreate(&b->eout))
@@ -4054,8 +4063,8 @@ smpm_status smpm_batch_create(const smpm_handle* hs, int count, const int* nrhs,
     }
     b->nelem = (long long)t64.size();
     b->v_len = off;
-    if (cudaMalloc(&b->dtab64, t64.size() * sizeof(ElemMeta<double>)) ||
-        (all32 && cudaMalloc(&b->dtab32, t32.size() * sizeof(ElemMeta<float>))))
+    if (device_malloc(&b->dtab64, t64.size() * sizeof(ElemMeta<double>)) ||
+        (all32 && device_malloc(&b->dtab32, t32.size() * sizeof(ElemMeta<float>))))
       return bad(fail(SMPM_ENOMEM, "batch allocation failed"));
     if (cudaMemcpy(b->dtab64, t64.data(), t64.size() * sizeof(ElemMeta<double>), cudaMemcpyHostToDevice) ||
         (all32 && cudaMemcpy(b->dtab32, t32.data(), t32.size() * sizeof(ElemMeta<float>), cudaMemcpyHostToDevice)))

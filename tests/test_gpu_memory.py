@@ -32,3 +32,27 @@ def test_coarse_inverse_is_held_once(flags):
         # 31 MB per dense inverse; the rest of the factors, 14 MB, follows the grid's
         # size and the strips' height
         assert abs(used - used0) < 0.6 * 8 * d * d, (d, used, used0)
+
+
+def test_failed_allocation_leaves_nothing_behind():
+    """A factor step that finds no device memory reports ENOMEM, and the next solve of
+    another handle on the same device is unaffected."""
+    from paper_1601_03432_gb300 import SmpmError, inputs
+    from paper_1601_03432_gb300 import _binding as B
+    g, big = Grid(6, 5, 6), Grid(40, 40, 12)
+    g.factor(tol=1e-11)
+    f = torch.as_tensor(inputs.white_noise(g.r, 1), device="cuda")
+    u, u2 = torch.empty_like(f), torch.empty_like(f)
+    g.solve(f, u)
+    torch.cuda.synchronize()
+    room = 64 << 20  # the factors of the larger grid take 78 MB for one d x d matrix alone
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(SmpmError) as ei:
+            big.factor(tol=1e-11)
+        assert ei.value.status == B.SMPM_ENOMEM
+        assert g.solve(f, u2)[0]["converged"] == 1
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert (u2 - u).norm() <= 1e-9 * u.norm()
