@@ -97,11 +97,13 @@ enum { ACC_ULB = 0, ACC_USBS = 1, ACC_MEAN = 2, ACC_RES = 3, ACC_BSN = 4, ACC_RG
 // in tiles of eight shared out over the warps.  B, U, t1: n rows of fd_ld(n)
 // doubles; Bf: one packed tile per warp.
 __host__ __device__ constexpr int fd_ld(int n) { return (n + 3) / 8 * 8 + 4; }  // 4 modulo 8: rows spread over the banks
+// whether a group of W warps forms the products by threads (fd_thread_pass)
+__host__ __device__ constexpr bool fd_by_threads(int n, int W) { return n <= 8 || (n <= 12 && n * n <= 64 * W); }
 // scratch of a group: three tiles, the slot values (two times 4n), packed tiles
-// (the element's residual product takes the first W of them for its vector)
+// (none by threads; the element's residual product packs its vector there)
 __host__ __device__ inline size_t fd_item_bytes(int n, int W) {
-  const size_t tile = sizeof(uint4) * (size_t)digit_bwords<double>(n), vec = sizeof(uint4) * (size_t)digit_bwords<double>(4 * n);
-  const size_t bf = W * tile > vec ? W * tile : vec;
+  const size_t tile = fd_by_threads(n, W) ? 0 : sizeof(uint4) * (size_t)digit_bwords<double>(n);
+  const size_t vec = sizeof(uint4) * (size_t)digit_bwords<double>(4 * n), bf = W * tile > vec ? W * tile : vec;
   return bf + sizeof(double) * (3 * (size_t)n * fd_ld(n) + 8 * (size_t)n);
 }
 struct FdItem {
@@ -146,7 +148,6 @@ __device__ __noinline__ void fd_pass(const uint4* A, const short* er, uint4* Bw,
 // tile of eight columns (half of it padding) 3,500.  At n = 12 the FP64 products
 // alone cost what the tiles do, so there only where the group has a thread for
 // every other entry; from n = 16 on the digits win.
-__host__ __device__ constexpr bool fd_by_threads(int n, int W) { return n <= 8 || (n <= 12 && n * n <= 64 * W); }
 __device__ __noinline__ void fd_thread_pass(const double* __restrict__ A, int n, int tid, int nthr, const double* x, int ldk,
                                             int ldc, double* out, int ldr, int ldo, const double* __restrict__ w) {
 #pragma unroll 1
