@@ -231,7 +231,7 @@ smpm_status smpm_apply_deflation_q(smpm_handle h, const double* v, double* y, vo
  * class's elements side by side) and only the vectors stream from HBM.  The
  * paper's method keeps per-element factors (mapped elements, Sec. 1.2); this
  * is a property of uniform grids.  Where the elements fall into many small
- * classes, or a row of T_e spans more than 2^35 (FP32: 2^33) in magnitude, the
+ * classes, or a row of T_e spans more than 2^35 (FP32: 2^64) in magnitude, the
  * per-element kernels run in its place.  Errors as smpm_apply_schur. */
 smpm_status smpm_apply_schur_class(smpm_handle h, const double* v, double* y, void* stream);
 smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, void* stream);
@@ -239,8 +239,8 @@ smpm_status smpm_apply_schur_class32(smpm_handle h, const float* v, float* y, vo
 /* Kernels of y = S v (smpm_apply_schur, smpm_apply_schur32 and the S apply
  * inside the deflation entry points): AUTO takes CLASS where the elements
  * fall into few enough classes that its tiles of eight elements are at least a
- * fifth full on average and the grid is large enough for it to be the faster
- * one, else by thresholds one warp per element for 4n <= 96 (1, 2 or 4 warps by
+ * fifth full on average (FP64: and the grid is large enough for it to be the
+ * faster one), else by thresholds one warp per element for 4n <= 96 (1, 2 or 4 warps by
  * the element count) or the shared-memory stream; WARP: persistent CTAs, one
  * warp per element, T_e read column by column from global memory; WARP2 / WARP4:
  * 2 or 4 warps per element; STREAM: bulk copies of T_e into a shared-memory

@@ -855,20 +855,16 @@ __device__ __noinline__ S plain_row(const S* __restrict__ row, const S* v, int M
   return z;
 }
 
-// Digits of the class apply: FP64 vectors in twelve (tile8_wide), FP32 vectors in
-// the eight of FP64 operands: an FP32 entry then keeps its accuracy as far as
-// T_e's rows span at most 2^33 (the left-out weights are K 2^-57 of row maximum
-// times column maximum, an FP32 chain K 2^-24 of its sum of magnitudes).
-template <typename S>
-using ClassDigits = typename std::conditional<sizeof(S) == 4, double, Wide>::type;
-template <typename S>
-constexpr double kClassSpan = sizeof(S) == 4 ? 0x1p33 : 0x1p35;
+// Digits of the class apply: FP64 vectors in twelve (Wide: tile8_wide), as far as
+// T_e's rows span at most 2^35.  FP32 vectors in the eight of FP64 operands up to
+// 2^33 (the left-out weights are K 2^-57 of row maximum times column maximum, an FP32
+// chain K 2^-24 of its sum of magnitudes), in twelve up to 2^64.
+constexpr double kClassSpan64 = 0x1p35, kClassSpan32 = 0x1p33, kClassSpan32Wide = 0x1p64;
 
-template <typename S, int kThreads>
+template <typename S, typename D, int kThreads>
 __global__ void __launch_bounds__(kThreads, kThreads <= 192 ? 2 : 1) k_schur_class(DevGeo g, const uint4* __restrict__ Tdig,
                                                      const short* __restrict__ Texp, const int* __restrict__ tiles,
                                                      const int* __restrict__ elems, const S* __restrict__ T, const S* v, S* y) {
-  using D = ClassDigits<S>;
   extern __shared__ __align__(16) unsigned char raw[];
   const int M = g.M, kt_n = digit_tiles(M), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int cls = tiles[3 * blockIdx.x], start = tiles[3 * blockIdx.x + 1], cnt = tiles[3 * blockIdx.x + 2];
@@ -918,7 +914,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 192 ? 2 : 1) k_schur_cla
   const uint4* A = Tdig + (size_t)cls * digit_words<D>(M, M);
   const short* er = Texp + (size_t)cls * M;
   Tile8<double> t;
-  if constexpr (sizeof(S) == 4) {
+  if constexpr (std::is_same<D, double>::value) {
     pack_tile<double>(Bf, warp, lane, x, E);
     __syncthreads();
     t = tile8_products<double>(A, er, Bf, M, kt_n, warp, lane, E);
@@ -960,10 +956,11 @@ struct smpm_handle_s {
   bool op_factored = false;  // operator-only factor step (SMPM_FLAG_OPERATOR_ONLY): S can be applied
   // element classes (face-type masks) for the class-shared apply
   int ncls = 0, ntiles = 0;
-  // T_e per class in the digits of the class apply (null: not packed, see
-  // class_digits) and its row exponents; the FP32 one may be dig.T
-  uint4 *clsT64 = nullptr, *clsT32 = nullptr;
-  short *clsTe64 = nullptr, *clsTe32 = nullptr;
+  // T_e per class in twelve digits and its row exponents for the class apply (null: not
+  // packed), and what FP64 and FP32 vectors take: 0 no class apply, 8 dig.T, 12 clsT
+  uint4* clsT = nullptr;
+  short* clsTe = nullptr;
+  int cls64 = 0, cls32 = 0;
   int apply_kind = 0;                     // kernel of smpm_apply_schur(32): SMPM_APPLY_*
   // packed digits (smpm_digits.cuh) of one T_e per class, G_b and the four X_F
   // per block class, their row exponents, and the class of each element / block
@@ -1242,22 +1239,21 @@ bool apply_kind_ok(smpm_handle h, int kind, bool fp32) {
 // Whether the class apply's tiles of eight elements are filled to a fifth on average.
 bool class_tiles_pay(smpm_handle h) { return (long long)h->ntiles * kClassTile <= 5 * h->g.nel; }
 
-// Whether SMPM_APPLY_AUTO takes the class apply: its matrices are packed
-// (class_span), its tiles fill, and it is the faster one.  Measured in a CUDA graph
-// (no launch gaps, T_e in L2 where it fits), us, the per-element kernel that AUTO
-// takes else against the class kernel:
+// Whether SMPM_APPLY_AUTO takes the class apply where its matrices are packed
+// (class_span) and its tiles fill: in FP64 where it is the faster one, in FP32
+// always, for its accuracy: its sums are rounded once, an FP32 chain loses up to K
+// roundings (relative error of S v for random v, 4x15 to 128x128: 2.5e-8 to 3.6e-8 against 6e-8 to 1e-7).
+// Measured in a CUDA graph (no launch gaps, T_e in L2 where it fits), us, the
+// per-element kernel that AUTO takes else against the class kernel:
 //   FP64, elements: 608 (four per SM, one wave), n = 8 6.0 / 6.8, n = 17 9.8 / 10.3, n = 24 12.3 / 11.8;
 //     702 n = 5 6.3 / 6.8, n = 8 7.7 / 6.7, n = 16 12.3 / 7.9, n = 24 17.1 / 11.7; 1024 n = 5 7.5 / 7.0,
 //     n = 24 23 / 11.8; 5184 n = 16 69 / 19, n = 24 102 / 35
-//   FP32: 1024 n = 8 4.4 / 7.0, n = 24 7.3 / 9.6; 1296 n = 5 6.2 / 7.4, n = 10 8.5 / 8.3, n = 24 12.4 / 11.4;
-//     1600 n = 5 6.4 / 7.4, n = 8 7.3 / 7.0; 3136 n = 5 9.3 / 8.0, n = 24 47 / 18; n = 28 (staged in
-//     shared memory): 608 8.0 / 10.3, 702 10.2 / 9.3, 1600 18 / 14
+//   FP32: 256 n = 16 5.3 / 7.6; 1024 n = 8 4.4 / 7.0, n = 24 7.3 / 9.6; 1600 n = 5 6.4 / 7.4, n = 16 9.9 / 8.7;
+//     3136 n = 5 9.3 / 8.0, n = 24 47 / 18
 template <typename S>
 bool class_pays(smpm_handle h, int sms) {
   if (!class_tiles_pay(h)) return false;
-  const long long ne = h->g.nel, M = h->g.M;
-  if (sizeof(S) == 8) return ne > 4LL * sms && (M >= 32 || ne > 6LL * sms);
-  return (ne > 8LL * sms && ne * M >= 50000) || (M > 96 && ne > 4LL * sms);
+  return sizeof(S) == 4 || (h->g.nel > 4LL * sms && (h->g.M >= 32 || h->g.nel > 6LL * sms));
 }
 
 // y = S v with the handle's apply kernel.  SMPM_APPLY_AUTO: the class-shared
@@ -1273,7 +1269,7 @@ smpm_status launch_schur_kind(smpm_handle h, int kind, const S* v, S* y, cudaStr
   int dev = 0, sms = 0;
   CU(cudaGetDevice(&dev));
   CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const bool packed = fp32 ? h->clsT32 != nullptr : h->clsT64 != nullptr;
+  const bool packed = (fp32 ? h->cls32 : h->cls64) != 0;
   if (kind == SMPM_APPLY_AUTO && packed && class_pays<S>(h, sms)) kind = SMPM_APPLY_CLASS;
   if (kind == SMPM_APPLY_CLASS && !packed) kind = SMPM_APPLY_AUTO;
   if (kind == SMPM_APPLY_AUTO) kind = apply_kind_ok(h, SMPM_APPLY_WARP, fp32) ? -1 : SMPM_APPLY_STREAM;
@@ -1428,14 +1424,17 @@ size_t refine_shape(const Geometry& g, int m, int ES, int items, size_t budget, 
 
 // Whether C^+ by strips is the cheaper form for R columns on a team of G CTAs: its
 // two extra team barriers and phase starts against the products that it saves per
-// CTA and step.  Measured, GMRES time per step in us, n = 6, 152 CTAs, dense rows
-// against strips (saved products per CTA):
-//   one column, FP64: 28x28 elements (13 k) 35.1 / 35.7; 32x32 (22 k) 39.2 / 37.4; 48x48 112 / 52
-//   one column, FP32: 32x32 (22 k) 42.4 / 44.6; 40x40 (54 k) 53.6 / 50.6; 48x48 71 / 54
-//   8 columns, FP64:  16x16 (10 k) 88 / 93; 20x20 (25 k) 97.6 / 98.0; 24x24 (54 k) 109 / 103
-//   8 columns, FP32:  20x20 (25 k) 112 / 116; 24x24 (54 k) 121 / 119
+// CTA and step.  Measured, time of the solve kernel by strips over that by dense
+// rows, 152 CTAs, n = 6 to 14 (saved products per CTA):
+//   one column, FP64: 28x28 elements (13 k) 1.02; 30x30 (17 k) 1.00; 32x32 (22 k) 0.96; 48x48 0.46
+//   one column, FP32: 28x28 1.09; 34x34 (28 k) 1.07; 40x40 (54 k) 0.94; 48x48 0.77
+//   3 columns, FP64:  20x20 (9 k) 0.97; 26x26 (28 k) 0.69 to 0.77 (the dense rows take four columns' time)
+//   8 columns, FP64:  16x16 (9 k) 1.05; 20x20 (25 k) 0.98 to 1.00; 24x24 (53 k) 0.95
+//   3 and 8 columns, FP32: 20x20 (9 k, 25 k) 1.07, 1.00 to 1.04; 26x26 (28 k) 1.01 to 1.03; 30x30 (51 k) 0.96
 bool strips_pay(long long d, double products, int G, int R, bool fp32) {
-  const double line = R > 1 ? (fp32 ? 45000.0 : 25000.0) : (fp32 ? 24000.0 : 14000.0);
+  double line = 17000;
+  if (R == 1 && fp32) line = 40000;
+  if (R > 1) line = fp32 ? 32000 : R <= 4 ? 9000 : 25000;
   return R * ((double)d * d - products) / G >= line;
 }
 
@@ -3262,12 +3261,10 @@ smpm_status upload_classes(smpm_handle h, cudaStream_t st) {
   // the class apply's: where it can be taken, and the digits hold the rows' span
   if (!class_tiles_pay(h) && h->ncls > kClassFew) return SMPM_OK;
   const double span = class_span(g, Tcls, first);
-  if (span <= kClassSpan<double> && (s = upload_digits<Wide>(h, Tcls, g.M, &h->clsT64, &h->clsTe64, st))) return s;
-  if (mixed && span <= kClassSpan<float>) {
-    if (!h->dig.T && (s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
-    h->clsT32 = h->dig.T;
-    h->clsTe32 = h->dig.Te;
-  }
+  h->cls64 = span <= kClassSpan64 ? 12 : 0;
+  if (mixed) h->cls32 = span <= kClassSpan32 ? 8 : span <= kClassSpan32Wide ? 12 : 0;
+  if ((h->cls64 == 12 || h->cls32 == 12) && (s = upload_digits<Wide>(h, Tcls, g.M, &h->clsT, &h->clsTe, st))) return s;
+  if (h->cls32 == 8 && !h->dig.T && (s = upload_digits<double>(h, Tcls, g.M, &h->dig.T, &h->dig.Te, st))) return s;
   return SMPM_OK;
 }
 
@@ -3767,12 +3764,19 @@ namespace {
 
 template <typename S>
 smpm_status launch_schur_class(smpm_handle h, const S* v, S* y, cudaStream_t st) {
-  const bool fp32 = sizeof(S) == 4;
+  const bool fp32 = sizeof(S) == 4, small = h->g.M <= 96;
+  const S* T = reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT);
+  auto launch = [&](auto k, const uint4* D, const short* E, int words) {
+    k<<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), words * sizeof(uint4), st>>>(h->dg, D, E, h->dtiles, h->dclsel, T, v, y);
+  };
   // two CTAs per SM need at most 168 registers a thread, which M <= 96 leaves
-  const auto k = h->g.M <= 96 ? k_schur_class<S, 192> : k_schur_class<S, 256>;
-  k<<<(unsigned)h->ntiles, 32 * digit_tiles(h->g.M), digit_bwords<ClassDigits<S>>(h->g.M) * sizeof(uint4), st>>>(
-      h->dg, fp32 ? h->clsT32 : h->clsT64, fp32 ? h->clsTe32 : h->clsTe64, h->dtiles, h->dclsel,
-      reinterpret_cast<const S*>(fp32 ? (const void*)h->dT32 : (const void*)h->dT), v, y);
+  const bool eight = fp32 && h->cls32 == 8;
+  if constexpr (sizeof(S) == 4)
+    if (eight)
+      launch(small ? k_schur_class<S, double, 192> : k_schur_class<S, double, 256>, h->dig.T, h->dig.Te,
+             digit_bwords<double>(h->g.M));
+  if (!eight)
+    launch(small ? k_schur_class<S, Wide, 192> : k_schur_class<S, Wide, 256>, h->clsT, h->clsTe, digit_bwords<Wide>(h->g.M));
   CHECK_LAUNCH();
   return SMPM_OK;
 }

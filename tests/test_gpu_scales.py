@@ -158,8 +158,7 @@ def test_mixed_solves_of_small_grids_keep_the_fp64_coarse_inverse(built, mx, my,
     assert (u - um).norm() <= 1e-8 * u.norm()
 
 
-# four elements per SM and one more (FP64), eight per SM and one more (FP32, with
-# entries enough and not), more than 96 rows
+# four elements per SM and one more, rows below and above 32, more than 96
 @pytest.mark.parametrize("mx,my,n", [(19, 32, 8), (29, 21, 8), (38, 32, 11), (35, 35, 11), (35, 35, 6), (29, 21, 27)])
 def test_default_apply_on_both_sides_of_its_lines(built, mx, my, n):
     """What AUTO takes agrees with the class and per-element kernels entry by entry."""
